@@ -187,7 +187,8 @@ mone_status dalloc(T** p, size_t n) {
 }
 
 void free_state(DevState& s) {
-    void* ptrs[] = {s.W1, s.W2, s.mu1, s.mu2, s.W1b, s.W2b, s.n1, s.n2, s.sumsq, s.status, s.alpha, s.gamma,
+    // mu1 and mu2 lie in W1's and W2's allocations
+    void* ptrs[] = {s.W1, s.W2, s.W1b, s.W2b, s.n1, s.n2, s.sumsq, s.status, s.alpha, s.gamma,
                     s.w_eta, s.b_eta, s.w_beta, s.b_beta, s.gate, s.U, s.eta, s.dbeta, s.zinv, s.dHt, s.Att, s.Uq, s.Aq,
                     s.Oq, s.Amse, s.Kres, s.Vres, s.Kres32, s.Vres32, s.nc2, s.colpart};
     for (void* p : ptrs)
@@ -297,18 +298,16 @@ mone_status build_state_maps(mone_mem* m) {
     bool ok = encode_map_bf16_3d(&m->maps.W1b, s.W1b, s.d_in, s.d_hid, s.C, 64, 128) &&
               encode_map_bf16_3d(&m->maps.W2b, s.W2b, s.d_out, s.d_hid, s.C, 64, 128) &&
               encode_map_bf16_3d(&m->maps.W2m, s.W2b, s.d_out, s.d_hid, s.C, 64, 64) &&
-              encode_map_bf16_3d(&m->maps.dH, s.dHt, s.d_hid, s.T, s.C, 64, 64) &&
-              encode_map_bf16_3d(&m->maps.At, s.Att, s.d_hid, s.T, s.C, 64, 64);
+              encode_map_bf16_blocks(&m->maps.dH, s.dHt, s.d_hid, s.T, s.C, 64, 2) &&
+              encode_map_bf16_blocks(&m->maps.At, s.Att, s.d_hid, s.T, s.C, 64, 2);
     if (ok && s.Amse) ok = encode_map_bf16_3d(&m->maps.Amse, s.Amse, s.d_hid, s.T, s.C, 64, 128);
     if (ok && s.U)
         ok = encode_map_bf16_3d(&m->maps.Ua, s.U, s.d_in, s.win_rows, s.C, 64, 128) &&
-             encode_map_bf16_3d(&m->maps.Ub, s.U, s.d_in, s.win_rows, s.C, 64, 64);
+             encode_map_bf16_blocks(&m->maps.Ub, s.U, s.d_in, s.win_rows, s.C, 64, 4) &&
+             encode_map_bf16_blocks(&m->maps.Ub2, s.U, s.d_in, s.win_rows, s.C, 64, 2);
     if (ok)
-        ok = encode_map_plain_3d(&m->maps.W1s, s.W1, true, s.d_in, s.d_hid, s.C, 128, 32) &&
-             encode_map_plain_3d(&m->maps.W2s, s.W2, true, s.d_out, s.d_hid, s.C, 128, 32);
-    if (ok && s.mu1)
-        ok = encode_map_plain_3d(&m->maps.M1s, s.mu1, true, s.d_in, s.d_hid, s.C, 128, 32) &&
-             encode_map_plain_3d(&m->maps.M2s, s.mu2, true, s.d_out, s.d_hid, s.C, 128, 32);
+        ok = encode_map_state(&m->maps.W1s, s.W1, s.mu1, s.d_in, s.d_hid, s.C) &&
+             encode_map_state(&m->maps.W2s, s.W2, s.mu2, s.d_out, s.d_hid, s.C);
     return ok ? MONE_OK : MONE_ERR_CUDA;
 }
 
@@ -317,12 +316,15 @@ mone_status build_input_maps(const DevState& s, TcInputMaps* in, const void* X, 
                              long long rows, int chains) {
     const int dh = s.d_out / 2;
     bool ok = encode_map_bf16_3d(&in->Ka, K, dh, rows, chains, 64, 128) &&
-              encode_map_bf16_3d(&in->Kb, K, dh, rows, chains, 64, 64) &&
+              encode_map_bf16_blocks(&in->Kb, K, dh, rows, chains, 64, 4) &&
+              encode_map_bf16_blocks(&in->Kb2, K, dh, rows, chains, 64, 2) &&
               encode_map_bf16_3d(&in->Va, V, dh, rows, chains, 64, 128) &&
-              encode_map_bf16_3d(&in->Vb, V, dh, rows, chains, 64, 64);
+              encode_map_bf16_blocks(&in->Vb, V, dh, rows, chains, 64, 4) &&
+              encode_map_bf16_blocks(&in->Vb2, V, dh, rows, chains, 64, 2);
     if (ok && s.mode == MONE_PLAIN)
         ok = encode_map_bf16_3d(&in->Xa, X, s.d_in, rows, chains, 64, 128) &&
-             encode_map_bf16_3d(&in->Xb, X, s.d_in, rows, chains, 64, 64);
+             encode_map_bf16_blocks(&in->Xb, X, s.d_in, rows, chains, 64, 4) &&
+             encode_map_bf16_blocks(&in->Xb2, X, s.d_in, rows, chains, 64, 2);
     return ok ? MONE_OK : MONE_ERR_CUDA;
 }
 
@@ -501,6 +503,7 @@ mone_status run_segments(mone_mem* m, SegWork w, long long N, cudaStream_t st) {
             if (s.mode == MONE_PLAIN) {  // U stays the caller's X
                 rin[g].Xa = gin[g].Xa;
                 rin[g].Xb = gin[g].Xb;
+                rin[g].Xb2 = gin[g].Xb2;
             }
         }
         off += n;
@@ -615,11 +618,12 @@ mone_status mone_mem_init(const mone_config* cfg, const float* W1_0, const float
     const size_t r1 = w1_rows(s);  // rows of W1 over all chains (and heads): sizes the row tables
     mone_status rc = MONE_OK;
     auto step = [&](mone_status r) { if (rc == MONE_OK) rc = r; };
-    step(dalloc(&s.W1, n1));
-    step(dalloc(&s.W2, n2));
-    if (s.momentum) {
-        step(dalloc(&s.mu1, n1));
-        step(dalloc(&s.mu2, n2));
+    // the momentum of a matrix follows its weights in one allocation: one tensor map covers both
+    step(dalloc(&s.W1, n1 * (s.momentum ? 2 : 1)));
+    step(dalloc(&s.W2, n2 * (s.momentum ? 2 : 1)));
+    if (rc == MONE_OK && s.momentum) {
+        s.mu1 = s.W1 + n1;
+        s.mu2 = s.W2 + n2;
     }
     if (s.dtype == MONE_BF16) {
         step(dalloc(&s.W1b, n1));

@@ -177,14 +177,15 @@ cudaError_t launch_attention(const DevState& s, int n_layers, const void* Q, int
 // ---- kernels in ttl_tc.cu (bf16 tcgen05 path)
 struct TcMaps {
     CUtensorMap W1b, W2b;        // K-major boxes {64, 128}
-    CUtensorMap dH, At;          // MN-major boxes {64, 64} over [C][T][d_hid]
-    CUtensorMap Ua, Ub;          // scratch U: K-major {64,128} and MN {64,64}
-    CUtensorMap W1s, W2s, M1s, M2s;  // fp32 state chunks {128 cols, 32 rows}, no swizzle
+    CUtensorMap dH, At;          // phase B's A operand, MN-major blocks of 128 hidden units over [C][T][d_hid]
+    CUtensorMap Ua, Ub, Ub2;     // scratch U: K-major {64,128}; MN-major blocks of 256 columns, of 128 (CTA pairs)
+    CUtensorMap W1s, W2s;            // fp32 state chunks of W and, with momentum, mu in one box
     CUtensorMap W2m;                 // bf16 W2 copy, MN-major boxes {64 outputs, 64 hidden} (memory read)
     CUtensorMap Amse;                // squared-error activations, K-major {64, 128}
 };
 struct TcInputMaps {
-    CUtensorMap Xa, Xb, Ka, Kb, Va, Vb;  // per call: K-major {64,128} (a) and MN {64,64} (b)
+    // per call: K-major {64,128} (a), MN-major blocks of 256 columns (b) and of 128 (b2, CTA pairs)
+    CUtensorMap Xa, Xb, Xb2, Ka, Kb, Kb2, Va, Vb, Vb2;
 };
 cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                               cudaStream_t st);
@@ -207,6 +208,15 @@ bool encode_map_bf16_3d(CUtensorMap* map, const void* base, uint64_t inner, uint
                         uint32_t box_inner, uint32_t box_rows);
 bool encode_map_plain_3d(CUtensorMap* map, const void* base, bool f32, uint64_t inner, uint64_t rows,
                          uint64_t chains, uint32_t box_inner, uint32_t box_rows);
+// The MN-major operand form of a bf16 [chains][rows][inner] array (inner a multiple of 64): (64, rows,
+// inner / 64, chains), one box = box_rows rows x box_blocks consecutive 64-column blocks, written to
+// shared memory block after block.  x is always 0 and the third coordinate counts blocks.
+bool encode_map_bf16_blocks(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint64_t chains,
+                            uint32_t box_rows, uint32_t box_blocks);
+// fp32 state chunks: W [chains][rows][inner] and, when mu is not null, mu of the same shape in the
+// same allocation above W, as (32, rows, inner / 32, chains, 2), 128-byte swizzle; a box takes 32 rows x
+// 64 columns of both, as [matrix][32-column block][row][128 bytes] in shared memory.
+bool encode_map_state(CUtensorMap* map, const float* W, const float* mu, uint64_t inner, uint64_t rows, uint64_t chains);
 // 4-D bf16 map, 128-byte swizzle: dims[0] innermost, byte strides of dims 1..3.
 bool encode_map_bf16_4d(CUtensorMap* map, const void* base, const uint64_t dims[4], const uint64_t strides[3],
                         const uint32_t box[4]);

@@ -12,13 +12,12 @@
 //     Writes dH and At row-major (bf16 [token][hidden]) and the loss partial
 //     sum_t sum_h A_th R_th = sum_t y_t . M(u_t).
 //
-//   phase B, tile = (chain, 128 columns of [W1 | W2], 256 hidden units)
-//       G1^T = U^T dH         K = T'        (gradient of W1, transposed)
-//       G2^T = Y^T At         K = T'        (gradient of W2, transposed)
+//   phase B, tile = (chain, 128 hidden units, 256 columns of W1 or of a half of W2)
+//       G1 = dH^T U           K = T'        (gradient of W1)
+//       G2 = At^T Y           K = T'        (gradient of W2)
 //     Both operands are read MN-major straight from the row-major buffers.
-//     The accumulator is transposed (TMEM lane = weight column) so the fused
-//     update epilogue (Eq. 8, App. A) walks the fp32 state row by row with
-//     128-byte coalesced loads and stores: mu = beta mu + G; W = s W_raw - mu
+//     TMEM lane = hidden unit, so in the fused update epilogue (Eq. 8, App. A) a
+//     lane owns a row of the fp32 state: mu = beta mu + G; W = s W_raw - mu
 //     (s = the previous segment's pending row renormalisation); it writes W,
 //     mu, the bf16 operand copy and the new row sums of squares.
 //
@@ -47,7 +46,6 @@ constexpr int A_BM = 128, A_BN = 128, A_STAGES = 6;
 constexpr int A_STAGE = (A_BM + A_BN) * BK * 2;           // 32 KB
 // phase B
 constexpr int B_BM = 128, B_BN = 256;
-constexpr int B_STAGE = (B_BM + B_BN) * BK * 2;           // 48 KB
 constexpr int BOX = 64 * BK * 2;                          // one 64 x 64 MN-major box, 8 KB
 
 template <int STAGES, int STAGE, int TABLE>
@@ -86,6 +84,7 @@ struct TcArgs {
     int* status;
     int r_only;                 // phase A pairs: At and c SiLU'(x) / |z| come from the squared-error
                                 // pre-pass (the latter in dH); accumulate R only and form dH in place
+    int store_lag;              // phase B: state stores in flight (4 or 2 of the ring's 8 slots)
     unsigned long long wait_ns; // limit of every mbarrier wait of the launch (kWaitLimitNs)
     int stall;                  // test knob (phase A): the producer issues no loads, so the first
                                 // wait for a full stage runs out; nothing is in flight when it does
@@ -684,69 +683,94 @@ tc_phase_a_pair_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_con
 
 // ------------------------------------------------------------------ phase B
 //
-// Warps: 0 operand producer (TMA), 1 MMA issuer, 2..9 epilogue in two groups of
-// four (one warp per TMEM lane quarter; thread = one weight column), 10 state
-// producer.  The fp32 state of a tile (256 rows x 128 columns of W and mu) moves
-// in chunks of 32 rows through a 4-slot shared-memory ring: the state producer
-// TMA-loads chunks ahead of time; the two epilogue groups take alternate chunks,
-// update a chunk in place and TMA-store it back (the bf16 copy goes out with
-// coalesced 64-byte warp stores), and hand the slot back once the store has read it.
+// Tile = 128 hidden rows x 256 weight columns of W1, or of the K or V half of W2 (128 columns
+// where a width leaves that remainder), accumulated with TMEM lane = hidden row: D = dH^T U or
+// At^T Y, both operands MN-major, one TMA box per operand and 64-token k-block.
 //
-// PAIR: clusters of 2 CTAs run tcgen05.mma.cta_group::2 over 256 weight columns x 256
-// hidden rows.  CTA r stages its own 128 columns of U (or Y) and rows r*128 .. +127 of the
-// tile's 256 rows of dH (or At) per 64-token k-block, so each SM takes in 32 KB of operands
-// a k-block instead of 48 KB for the same 128 x 256 accumulator.  Both CTAs' loads complete
-// on rank 0's full barrier, rank 0 issues the MMAs, each commit arrives on both CTAs'
-// barriers, and the 16 epilogue warps of the pair release an accumulator buffer on rank 0's
-// tempty barrier.  Each CTA updates the state of its own 128 columns exactly as the one-CTA
-// kernel does.  A pair's 256 columns lie in one matrix (d_in and d_out multiples of 256).
+// Warps: 0 operand producer (TMA), 1 MMA issuer, 2..9 update, 10 state producer, 11 store warp.
+// The fp32 state of a tile moves in chunks of 32 rows x 64 columns of W and mu (16 KB, one TMA box)
+// through an 8-slot shared-memory ring.  A chunk belongs to one update warp: its rows are the warp's
+// TMEM lane quarter, so a lane owns one hidden row of the chunk.  It holds the row's
+// renormalisation scale in a register, reads and writes its part of the row 16 bytes at a time
+// (128-byte swizzle: conflict-free), sums the row's squares without a shuffle, and writes the bf16
+// copy in whole 32-byte sectors.  No barrier joins the update warps; each waits for its own chunks.
+//
+// What bounds it: with many chains the state's HBM traffic (18 B per parameter: 128 chains of
+// 2048 -> 1024 -> 1024 at T = 256 run at 0.97 of the HBM copy rate), with one chain the latency of a tile.
+// The lane-per-row form replaced one with lane = weight column, whose update (scalar shared-memory
+// accesses, a 31-shuffle row reduction, 2-byte stores, two barriers a chunk) took a one-chain launch
+// (96 tiles, one a CTA) from 18.4 to 21.2 us; merging its six operand boxes a k-block into two changed nothing.
+//
+// PAIR: clusters of 2 CTAs run tcgen05.mma.cta_group::2 over 256 hidden rows x 256 columns.  CTA r
+// stages its own 128 hidden rows of dH (or At) and columns r*128 .. +127 of U (or Y) per k-block,
+// so each SM takes in 32 KB of operands a k-block instead of 48 KB for the same 128 x 256
+// accumulator.  Both CTAs' loads complete on rank 0's full barrier, rank 0 issues the MMAs, each
+// commit arrives on both CTAs' barriers, and the 16 update warps of the pair release an
+// accumulator buffer on rank 0's tempty barrier.
 
-constexpr int S_ROWS = 32;                                 // hidden rows per state chunk
-constexpr int S_SLOTS = 4;
-constexpr int S_F32 = S_ROWS * B_BM * 4;                   // 16 KB
-constexpr int S_SLOT = 2 * S_F32;                          // W and mu: 32 KB
+constexpr int S_ROWS = 32, S_COLS = 64;                    // state chunk: hidden rows x weight columns
+constexpr int S_SLOTS = 8;
+constexpr int S_F32 = S_ROWS * S_COLS * 4;                 // 8 KB
+constexpr int S_SLOT = 2 * S_F32;                          // W and mu: 16 KB
 constexpr int B_THREADS = 12 * 32;
-constexpr int B_EPI_THREADS = 4 * 32;     // per epilogue group
 constexpr int B_STATE_WARP = 10;          // TMA loads of state chunks
 constexpr int B_STORE_WARP = 11;          // TMA stores of updated chunks, slot release
 
 template <bool PAIR>
 struct LayoutBT {
-    // operand stages: one CTA 48 KB (128 columns + 256 hidden rows); a pair member 32 KB
-    // (128 columns + its 128 hidden rows), three of them in the same space as two
-    static constexpr int STAGE = PAIR ? (B_BM + B_BN / 2) * BK * 2 : B_STAGE;
+    // operand stages: one CTA 48 KB (128 hidden rows + 256 columns); a pair member 32 KB (its 128
+    // hidden rows + 128 columns), three of them in the same space as two
+    static constexpr int A_BYTES = B_BM * BK * 2;
+    static constexpr int STAGE = A_BYTES + (PAIR ? B_BN / 2 : B_BN) * BK * 2;
     static constexpr int STAGES = PAIR ? 3 : 2;
     static constexpr int RING = STAGES * STAGE;
     static constexpr int STATE = RING;
     static constexpr int BARS = STATE + S_SLOTS * S_SLOT;  // full[S] empty[S] tfull[2] tempty[2] sfull/sdone/sempty[N]
     static constexpr int NBARS = 2 * STAGES + 4 + 3 * S_SLOTS;
     static constexpr int SLOT = BARS + NBARS * 8;
-    static constexpr int FLAG = SLOT + 16;
-    static constexpr int TAB = FLAG + 16;                  // per group: [B_BN/2] renorm scales + [4] decay partials
-    static constexpr int END = TAB + 2 * (B_BN / 2 + 4) * 4;
+    static constexpr int END = SLOT + 16;
     static constexpr int DYN = END + 1024;
 };
 using LayoutB = LayoutBT<false>;
 using LayoutB2 = LayoutBT<true>;
 static_assert(LayoutB::DYN <= 227 * 1024 && LayoutB2::DYN <= 227 * 1024, "phase B shared memory budget");
 
-// The tiles one CTA of phase B walks: t = first, first + step, ... < count, each giving
-// (chain of the launch, first hidden row, first weight column of this CTA).
+// Column tiles of [W1 | W2]: each lies in W1, or in the K or the V half of W2.
+__host__ __device__ constexpr int b_col_tiles(int d_in, int d_out) {
+    return (d_in + B_BN - 1) / B_BN + 2 * ((d_out / 2 + B_BN - 1) / B_BN);
+}
+
+// The tiles one CTA of phase B walks: t = first, first + step, ... < count.
 template <bool PAIR>
 struct BTiles {
-    int first, step, count, n_ht, n_ct, rank;
+    int first, step, count, n_ht, n_ct, n1, nk, rank, d_in, dhalf;
     __device__ BTiles(const TcArgs& a) {
-        n_ht = a.d_hid / B_BN;
-        n_ct = (a.d_in + a.d_out) / (PAIR ? 2 * B_BM : B_BM);
+        d_in = a.d_in;
+        dhalf = a.d_out / 2;
+        n_ht = a.d_hid / (PAIR ? 2 * B_BM : B_BM);
+        n1 = (d_in + B_BN - 1) / B_BN;
+        nk = (dhalf + B_BN - 1) / B_BN;
+        n_ct = n1 + 2 * nk;
         count = a.nc * n_ht * n_ct;
         rank = PAIR ? (int)cluster_ctarank() : 0;
         first = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
         step = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     }
-    __device__ void decode(int t, int& cz, int& h0, int& col0) const {
-        cz = t / (n_ht * n_ct);
-        h0 = ((t / n_ct) % n_ht) * B_BN;
-        col0 = (t % n_ct) * (PAIR ? 2 * B_BM : B_BM) + rank * B_BM;
+    // tile t: chain of the launch, this CTA's first hidden row, source of the columns (0: U, W1;
+    // 1: K, 2: V, of W2), first column within the source and within its matrix, live columns
+    struct Tile {
+        int cz, h0, src, scol, mcol, ncol;
+    };
+    __device__ Tile decode(int t) const {
+        Tile x;
+        x.cz = t / (n_ht * n_ct);
+        x.h0 = ((t / n_ct) % n_ht) * (PAIR ? 2 * B_BM : B_BM) + rank * B_BM;
+        const int c = t % n_ct;
+        x.src = c < n1 ? 0 : (c < n1 + nk ? 1 : 2);
+        x.scol = (x.src == 0 ? c : (c - n1) % nk) * B_BN;
+        x.mcol = x.scol + (x.src == 2 ? dhalf : 0);
+        x.ncol = min(B_BN, (x.src == 0 ? d_in : dhalf) - x.scol);
+        return x;
     }
 };
 
@@ -757,8 +781,7 @@ __global__ void __launch_bounds__(B_THREADS, 1)
 tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constant__ CUtensorMap tmKb,
                   const __grid_constant__ CUtensorMap tmVb, const __grid_constant__ CUtensorMap tmDH,
                   const __grid_constant__ CUtensorMap tmAT, const __grid_constant__ CUtensorMap tmW1s,
-                  const __grid_constant__ CUtensorMap tmW2s, const __grid_constant__ CUtensorMap tmM1s,
-                  const __grid_constant__ CUtensorMap tmM2s, const TcArgs a) {
+                  const __grid_constant__ CUtensorMap tmW2s, const TcArgs a) {
     extern __shared__ uint8_t smem_raw[];
     using L = LayoutBT<PAIR>;
     constexpr int NS = L::STAGES;
@@ -773,6 +796,7 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
     auto sdone = [&](int k) { return bars + 8 * (2 * NS + 4 + 2 * S_SLOTS + k); };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const BTiles<PAIR> tl(a);
+    using Tile = typename BTiles<PAIR>::Tile;
     if (threadIdx.x == 0) {
         for (int i = 0; i < NS; ++i) {
             mbar_init(full(i), 1);
@@ -780,12 +804,12 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(tfull(b), 1);
-            mbar_init(tempty(b), PAIR ? 16 : 8);  // every epilogue warp (of both CTAs of a pair)
+            mbar_init(tempty(b), PAIR ? 16 : 8);  // every update warp (of both CTAs of a pair)
         }
         for (int k = 0; k < S_SLOTS; ++k) {
             mbar_init(sfull(k), 1);
             mbar_init(sempty(k), 1);
-            mbar_init(sdone(k), 4);  // the four warps of the epilogue group that updated the chunk
+            mbar_init(sdone(k), 1);  // the update warp that owns the chunk
         }
         fence_mbar_init();
     }
@@ -807,8 +831,13 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
     const uint32_t tmem = *reinterpret_cast<uint32_t*>(base + L::SLOT);
 
     const int KB = (a.Tp + BK - 1) / BK;  // tokens beyond T' carry zero dH / At
-    const int dhalf = a.d_out / 2;
     const int chunk_bytes = a.momentum ? 2 * S_F32 : S_F32;
+    // chunk i of a tile: columns (i >> 3) * 128 + (i & 1) * 64, rows ((i >> 1) & 3) * 32.  A chunk is
+    // updated by the warp of that quarter and column half, so every warp takes one chunk of eight in
+    // a row and a ring slot always belongs to the same warp; two consecutive boxes cover 512
+    // contiguous bytes of each row (with 256 bytes at a time the 128-chain step lost 5% to DRAM).
+    auto chunk_col = [](int i) { return (i >> 3) * 128 + (i & 1) * S_COLS; };
+    auto chunk_row = [](int i) { return ((i >> 1) & 3) * S_ROWS; };
 
     if (warp == 0) {
         if (lane == 0) {
@@ -820,57 +849,28 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
             uint32_t kc = 0;
             bool ok = true;
             for (int t = tl.first; t < tl.count && ok; t += tl.step) {
-                int cz, h0, col0;
-                tl.decode(t, cz, h0, col0);
-                const int cs = a.c0 + cz;
-                const bool isW1 = col0 < a.d_in;
-                // this CTA's share of the tile's hidden rows: all 256, or 128 of a pair
-                const int hrow = h0 + (PAIR ? tl.rank * (B_BN / 2) : 0);
-                constexpr int HB = (PAIR ? B_BN / 2 : B_BN) / 64;  // 64-row boxes of hidden rows
+                const Tile x = tl.decode(t);
+                const CUtensorMap* ma = x.src == 0 ? &tmDH : &tmAT;
+                const CUtensorMap* mb = x.src == 0 ? &tmUb : (x.src == 1 ? &tmKb : &tmVb);
+                const int y0 = x.src == 0 ? a.u_row0 : a.y_row0, z = x.src == 0 ? a.u_chain0 + x.cz : x.cz;
+                // this CTA's share of the columns: all 256 (blocks past the source read as zeros), or 128 of a pair
+                const int blk = (x.scol + (PAIR ? tl.rank * (B_BN / 2) : 0)) / 64;
                 for (int kb = 0; kb < KB; ++kb, ++kc) {
                     const int s = kc % NS;
                     if (kc >= NS && !mbar_wait(empty(s), ((kc / NS) - 1) & 1, a.status, a.wait_ns)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t sa = smem_u32(base + s * L::STAGE), sb = sa + B_BM * BK * 2;
-                    uint32_t fb = full(s);
+                    const uint32_t sa = smem_u32(base + s * L::STAGE), sb = sa + L::A_BYTES;
                     if constexpr (PAIR) {
-                        fb = map_to_cta(full(s), 0);  // both CTAs' loads complete on rank 0's barrier
+                        const uint32_t fb = map_to_cta(full(s), 0);  // both CTAs' loads complete on rank 0's barrier
                         if (tl.rank == 0) mbar_expect_tx(full(s), 2 * L::STAGE);
+                        tma_load_4d_pair(sa, ma, fb, 0, kb * BK, x.h0 / 64, a.c0 + x.cz);
+                        tma_load_4d_pair(sb, mb, fb, 0, y0 + kb * BK, blk, z);
                     } else {
-                        mbar_expect_tx(fb, L::STAGE);
-                    }
-#pragma unroll
-                    for (int bx = 0; bx < B_BM / 64; ++bx) {
-                        const uint32_t dst = sa + bx * BOX;
-                        const CUtensorMap* map;
-                        int x, y, z;
-                        if (isW1) {
-                            map = &tmUb;
-                            x = col0 + bx * 64;
-                            y = a.u_row0 + kb * BK;
-                            z = a.u_chain0 + cz;
-                        } else {
-                            const int o = col0 - a.d_in + bx * 64;
-                            map = o < dhalf ? &tmKb : &tmVb;
-                            x = o < dhalf ? o : o - dhalf;
-                            y = a.y_row0 + kb * BK;
-                            z = cz;
-                        }
-                        // a tiled copy's innermost coordinate must be 16-byte aligned (8 bf16)
-                        if (!MONE_DCHECK((x & 7) == 0, a.status, DS_TMA_X)) continue;
-                        if constexpr (PAIR)
-                            tma_load_3d_pair(dst, map, fb, x, y, z);
-                        else
-                            tma_load_3d(dst, map, fb, x, y, z);
-                    }
-#pragma unroll
-                    for (int bx = 0; bx < HB; ++bx) {
-                        if constexpr (PAIR)
-                            tma_load_3d_pair(sb + bx * BOX, isW1 ? &tmDH : &tmAT, fb, hrow + bx * 64, kb * BK, cs);
-                        else
-                            tma_load_3d(sb + bx * BOX, isW1 ? &tmDH : &tmAT, fb, hrow + bx * 64, kb * BK, cs);
+                        mbar_expect_tx(full(s), L::STAGE);
+                        tma_load_4d(sa, ma, full(s), 0, kb * BK, x.h0 / 64, a.c0 + x.cz);
+                        tma_load_4d(sb, mb, full(s), 0, y0 + kb * BK, blk, z);
                     }
                 }
             }
@@ -887,7 +887,7 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
                 const int b = local & 1;
                 if (local >= 2 && !mbar_wait(tempty(b), ((local >> 1) - 1) & 1, a.status, a.wait_ns)) break;
                 tc_fence_after();
-                const uint32_t d = tmem + b * 256;
+                const uint32_t d = tmem + b * B_BN;
                 for (int kb = 0; kb < KB; ++kb, ++kc) {
                     const int s = kc % NS;
                     if (!mbar_wait(full(s), (kc / NS) & 1, a.status, a.wait_ns)) {
@@ -895,15 +895,14 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(base + s * L::STAGE), sb = sa + B_BM * BK * 2;
+                    const uint32_t sa = smem_u32(base + s * L::STAGE), sb = sa + L::A_BYTES;
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
+                        const uint64_t da = sdesc_sw128(sa + k * 16 * 128, BOX), db = sdesc_sw128(sb + k * 16 * 128, BOX);
                         if constexpr (PAIR)
-                            umma_bf16_pair(d, sdesc_sw128(sa + k * 16 * 128, BOX), sdesc_sw128(sb + k * 16 * 128, BOX),
-                                           idesc, (kb == 0 && k == 0) ? 0u : 1u);
+                            umma_bf16_pair(d, da, db, idesc, (kb == 0 && k == 0) ? 0u : 1u);
                         else
-                            umma_bf16(d, sdesc_sw128(sa + k * 16 * 128, BOX), sdesc_sw128(sb + k * 16 * 128, BOX), idesc,
-                                      (kb == 0 && k == 0) ? 0u : 1u);
+                            umma_bf16(d, da, db, idesc, (kb == 0 && k == 0) ? 0u : 1u);
                     }
                     if constexpr (PAIR)
                         umma_commit_pair(empty(s), 0x3);
@@ -920,32 +919,29 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
         }
         __syncwarp();
     } else if (warp == B_STATE_WARP) {
-        // ---- state producer: W (and mu) chunks of every tile, in epilogue order
+        // ---- state producer: W (and mu) chunks of every tile, in update order
         if (lane == 0) {
             tma_prefetch_map(&tmW1s);
             tma_prefetch_map(&tmW2s);
-            if (a.momentum) {
-                tma_prefetch_map(&tmM1s);
-                tma_prefetch_map(&tmM2s);
-            }
             uint32_t seq = 0;
             bool ok = true;
             for (int t = tl.first; t < tl.count && ok; t += tl.step) {
-                int cz, h0, col0;
-                tl.decode(t, cz, h0, col0);
-                const int cs = a.c0 + cz;
-                const bool isW1 = col0 < a.d_in;
-                const int cl = isW1 ? col0 : col0 - a.d_in;
-                for (int g = 0; g < B_BN / S_ROWS; ++g, ++seq) {
+                const Tile x = tl.decode(t);
+                for (int i = 0; i < x.ncol / 16; ++i, ++seq) {
                     const int k = seq % S_SLOTS;
                     if (seq >= S_SLOTS && !mbar_wait(sempty(k), ((seq / S_SLOTS) - 1) & 1, a.status, a.wait_ns)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t dst = smem_u32(base + L::STATE + k * S_SLOT);
+                    const int col = x.mcol + chunk_col(i);
+                    // the chunk lies inside the matrix (a tiled copy's block coordinate counts 32 columns)
+                    if (!MONE_DCHECK((col & 31) == 0 && col + S_COLS <= (x.src ? a.d_out : a.d_in), a.status, DS_TMA_X)) {
+                        ok = false;
+                        break;
+                    }
                     mbar_expect_tx(sfull(k), chunk_bytes);
-                    tma_load_3d(dst, isW1 ? &tmW1s : &tmW2s, sfull(k), cl, h0 + g * S_ROWS, cs);
-                    if (a.momentum) tma_load_3d(dst + S_F32, isW1 ? &tmM1s : &tmM2s, sfull(k), cl, h0 + g * S_ROWS, cs);
+                    tma_load_5d(smem_u32(base + L::STATE + k * S_SLOT), x.src ? &tmW2s : &tmW1s, sfull(k), 0,
+                                x.h0 + chunk_row(i), col / 32, a.c0 + x.cz, 0);
                 }
             }
         }
@@ -956,147 +952,125 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
             uint32_t seq = 0;
             bool ok = true;
             for (int t = tl.first; t < tl.count && ok; t += tl.step) {
-                int cz, h0, col0;
-                tl.decode(t, cz, h0, col0);
-                const int cs = a.c0 + cz;
-                const bool isW1 = col0 < a.d_in;
-                const int cl = isW1 ? col0 : col0 - a.d_in;
-                for (int g = 0; g < B_BN / S_ROWS; ++g, ++seq) {
+                const Tile x = tl.decode(t);
+                for (int i = 0; i < x.ncol / 16; ++i, ++seq) {
                     const int k = seq % S_SLOTS;
                     if (!mbar_wait(sdone(k), (seq / S_SLOTS) & 1, a.status, a.wait_ns)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t src = smem_u32(base + L::STATE + k * S_SLOT);
-                    tma_store_3d(isW1 ? &tmW1s : &tmW2s, src, cl, h0 + g * S_ROWS, cs);
-                    if (a.momentum) tma_store_3d(isW1 ? &tmM1s : &tmM2s, src + S_F32, cl, h0 + g * S_ROWS, cs);
+                    tma_store_5d(x.src ? &tmW2s : &tmW1s, smem_u32(base + L::STATE + k * S_SLOT), 0,
+                                 x.h0 + chunk_row(i), (x.mcol + chunk_col(i)) / 32, a.c0 + x.cz, 0);
                     bulk_commit();
-                    bulk_wait_read_all();  // the store has read the slot: hand it back
-                    mbar_arrive(sempty(k));
+                    // hand back the slot of the store `lag` before this one, which has been read by now: the
+                    // ring's slots are split between lag stores and S_SLOTS - lag loads in flight
+                    if (a.store_lag == 4)
+                        bulk_wait_read<4>();
+                    else
+                        bulk_wait_read<2>();
+                    if (seq >= (uint32_t)a.store_lag) mbar_arrive(sempty((seq - a.store_lag) % S_SLOTS));
                 }
             }
             bulk_wait_all();
         }
         __syncwarp();
     } else {
-        // ---- epilogue warps 2..9: group grp takes the tile's chunks grp, grp+2, grp+4, grp+6;
-        //      within a group, TMEM lane quarter q = 32 weight columns
-        const int grp = (warp - 2) >> 2, q = warp & 3, et = threadIdx.x - 64 - grp * B_EPI_THREADS;
-        const uint32_t bar_id = 1 + grp;
-        // Single-buffered per-tile tables: a warp writes tile i+1's entries only after
-        // every warp of its group has passed the last chunk barrier of tile i.
-        float* tab = reinterpret_cast<float*>(base + L::TAB) + grp * (B_BN / 2 + 4);  // [B_BN/2]
-        float* bred = tab + B_BN / 2;                                                  // [4]
-        int* flag = reinterpret_cast<int*>(base + L::FLAG) + grp * 2;
+        // ---- update warps 2..9: TMEM lane quarter q (32 hidden rows, one per lane), column half
+        const int q = warp & 3, half = (warp - 2) >> 2;
         const uint32_t tempty_rank0 = PAIR ? map_to_cta(tempty(0), 0) : tempty(0);
+        const uint64_t wpol = l2_evict_last_policy();  // phase A of the next segment reads the copy
         bool finite = true;
-        float step = 0.f;        // sum of mu_s^2 over this thread's elements of the current tile
         uint32_t tile_seq0 = 0;  // chunk sequence number of the current tile's first chunk
         int local = 0;
-        for (int t = tl.first; t < tl.count; t += tl.step, ++local, tile_seq0 += B_BN / S_ROWS) {
-            int cz, h0, col0;
-            tl.decode(t, cz, h0, col0);
-            const int cs = a.c0 + cz;
-            const bool isW1 = col0 < a.d_in;
-            const int which = isW1 ? 0 : 1;
-            const int cl = isW1 ? col0 : col0 - a.d_in;
-            const int width = isW1 ? a.d_in : a.d_out;
-            const int b = local & 1;
+        for (int t = tl.first; t < tl.count; t += tl.step, ++local) {
+            const Tile x = tl.decode(t);
+            const int cs = a.c0 + x.cz, which = x.src ? 1 : 0, width = x.src ? a.d_out : a.d_in;
+            const int b = local & 1, row = x.h0 + q * 32 + lane;
             // the tile's rows and columns lie inside the chain's W (index check of MONE_DEBUG builds)
-            const bool wr = MONE_DCHECK(cs < a.C && h0 + B_BN <= a.d_hid && cl + B_BM <= width, a.status,
-                                        DS_PHASE_B_TILE);
-            const float* n0 = (isW1 ? a.n1 : a.n2) + (size_t)cs * a.d_hid;
-            const float* prevss = ss_row(a, a.parity ^ 1, which, cs);
-            {   // scales of this group's 4 chunks x 32 rows
-                const int i = et >> 5, j = et & 31;
-                const int row = h0 + (2 * i + grp) * S_ROWS + j;
-                tab[et] = a.renorm_pending ? renorm_scale(n0[row], prevss[row]) : 1.f;
-            }
-            if (a.momentum) {
+            const bool wr = MONE_DCHECK(cs < a.C && row < a.d_hid && x.mcol + x.ncol <= width, a.status, DS_PHASE_B_TILE);
+            float sc = 1.f, beta = 0.f;
+            if (a.renorm_pending && wr)
+                sc = renorm_scale((x.src ? a.n2 : a.n1)[(size_t)cs * a.d_hid + row], ss_row(a, a.parity ^ 1, which, cs)[row]);
+            if (a.momentum) {  // beta_s = sigmoid(mean_t w_beta . x_t + b_beta)
+                const float* db = a.dbeta + (size_t)cs * a.win + a.tok0;
                 float v = 0.f;
-                for (int tk = et; tk < a.Tp; tk += B_EPI_THREADS) v += a.dbeta[(size_t)cs * a.win + a.tok0 + tk];
-                v = warp_sum(v);
-                if (lane == 0) bred[q] = v;
+#pragma unroll 4
+                for (int tk = lane; tk < a.Tp; tk += 32) v += db[tk];
+                beta = sigmoidf_(warp_sum(v) / (float)a.Tp + a.b_beta[cs]);
             }
-            if (et == 0) flag[0] = mbar_wait(tfull(b), (local >> 1) & 1, a.status, a.wait_ns) ? 1 : 0;
-            __syncwarp();
-            named_bar_sync(bar_id, B_EPI_THREADS);
-            if (!flag[0]) break;
+            const int ncg = x.ncol / 128;
+            bool ok = __all_sync(0xffffffffu, mbar_wait(tfull(b), (local >> 1) & 1, a.status, a.wait_ns));
+            if (!ok) break;
             tc_fence_after();
-            float beta = 0.f;
-            if (a.momentum) beta = sigmoidf_((bred[0] + bred[1] + bred[2] + bred[3]) / (float)a.Tp + a.b_beta[cs]);
-            float* cur = ss_row(a, a.parity, which, cs);
-            const int col = q * 32 + lane;  // column within the tile (= TMEM lane)
-            bf16* Wb = (isW1 ? a.W1b : a.W2b) + (size_t)cs * a.d_hid * width + cl + col;
-            const uint64_t wpol = l2_evict_last_policy();  // phase A of the next segment reads the copy
-            const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + b * 256;
-            bool ok = true;
+            const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + b * B_BN + half * S_COLS;
+            float ss = 0.f, step = 0.f;  // sums of squares of this lane's part of its row of W, and of mu
+            bf16* wrow = (x.src ? a.W2b : a.W1b) + ((size_t)cs * a.d_hid + row) * width + x.mcol + half * S_COLS;
 #pragma unroll 1
-            for (int i = 0; i < B_BN / S_ROWS / 2; ++i) {
-                const int c = 2 * i + grp;
-                const uint32_t seq = tile_seq0 + c;
+            for (int cg = 0; cg < ncg; ++cg) {
+                const uint32_t seq = tile_seq0 + cg * S_SLOTS + q * 2 + half;
                 const int k = seq % S_SLOTS;
-                const int r0 = h0 + c * S_ROWS;
-                float gv[32];
-                tmem_ld32(lane_base + c * S_ROWS, gv);
-                if (i == B_BN / S_ROWS / 2 - 1) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if constexpr (PAIR)
-                            mbar_arrive_remote(tempty_rank0 + 8 * b);
-                        else
-                            mbar_arrive(tempty(b));
+                ok = __all_sync(0xffffffffu, mbar_wait(sfull(k), (seq / S_SLOTS) & 1, a.status, a.wait_ns));
+                if (!ok) break;
+                uint8_t* slot = base + L::STATE + k * S_SLOT + lane * 128;
+#pragma unroll
+                for (int blk = 0; blk < S_COLS / 32; ++blk) {
+                    float g[32];
+                    tmem_ld32(lane_base + cg * 128 + blk * 32, g);
+                    if (cg == ncg - 1 && blk == S_COLS / 32 - 1) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if constexpr (PAIR)
+                                mbar_arrive_remote(tempty_rank0 + 8 * b);
+                            else
+                                mbar_arrive(tempty(b));
+                        }
+                    }
+                    uint8_t* wp = slot + blk * 4096;
+                    uint32_t pk[16];
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) {
+                        const int off = (p ^ (lane & 7)) << 4;
+                        float4 w = *reinterpret_cast<const float4*>(wp + off);
+                        float4 m = make_float4(g[4 * p], g[4 * p + 1], g[4 * p + 2], g[4 * p + 3]);
+                        if (a.momentum) {
+                            float4* mp = reinterpret_cast<float4*>(wp + S_F32 + off);
+                            const float4 mo = *mp;
+                            m.x = fmaf(beta, mo.x, m.x);
+                            m.y = fmaf(beta, mo.y, m.y);
+                            m.z = fmaf(beta, mo.z, m.z);
+                            m.w = fmaf(beta, mo.w, m.w);
+                            *mp = m;
+                        }
+                        w.x = fmaf(sc, w.x, -m.x);
+                        w.y = fmaf(sc, w.y, -m.y);
+                        w.z = fmaf(sc, w.z, -m.z);
+                        w.w = fmaf(sc, w.w, -m.w);
+                        *reinterpret_cast<float4*>(wp + off) = w;
+                        ss = fmaf(w.x, w.x, fmaf(w.y, w.y, fmaf(w.z, w.z, fmaf(w.w, w.w, ss))));
+                        if constexpr (STEP)
+                            step = fmaf(m.x, m.x, fmaf(m.y, m.y, fmaf(m.z, m.z, fmaf(m.w, m.w, step))));
+                        pk[2 * p] = pack_bf16(w.x, w.y);
+                        pk[2 * p + 1] = pack_bf16(w.z, w.w);
+                    }
+                    if (wr) {
+                        st_32b_hint(wrow + cg * 128 + blk * 32, pk, wpol);
+                        st_32b_hint(wrow + cg * 128 + blk * 32 + 16, pk + 8, wpol);
                     }
                 }
-                if (et == 0) flag[1] = mbar_wait(sfull(k), (seq / S_SLOTS) & 1, a.status, a.wait_ns) ? 1 : 0;
-                __syncwarp();
-                named_bar_sync(bar_id, B_EPI_THREADS);
-                if (!flag[1]) {
-                    ok = false;
-                    break;
-                }
-                uint8_t* slot = base + L::STATE + k * S_SLOT;
-                float* Ws = reinterpret_cast<float*>(slot);
-                float* Ms = reinterpret_cast<float*>(slot + S_F32);
-                bf16* bp = Wb + (size_t)r0 * width;
-                float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float sc = tab[i * S_ROWS + j];
-                    const float m = a.momentum ? Ms[j * B_BM + col] : 0.f;
-                    const float mn = fmaf(beta, m, gv[j]);
-                    const float wn = fmaf(sc, Ws[j * B_BM + col], -mn);
-                    Ws[j * B_BM + col] = wn;
-                    if (a.momentum) Ms[j * B_BM + col] = mn;
-                    if (wr) st_bf16_hint(bp + j * width, __float2bfloat16_rn(wn), wpol);
-                    v[j] = wn * wn;  // a NaN or Inf weight makes its row's sum non-finite
-                    if constexpr (STEP) step = fmaf(mn, mn, step);
-                }
-                // transpose-reduce: afterwards lane j holds this warp's 32-column partial of row j
-#pragma unroll
-                for (int sft = 16; sft >= 1; sft >>= 1) {
-                    const bool upper = (lane & sft) != 0;
-#pragma unroll
-                    for (int u = 0; u < sft; ++u) {
-                        const float send = upper ? v[u] : v[u + sft];
-                        const float keep = upper ? v[u + sft] : v[u];
-                        v[u] = keep + __shfl_xor_sync(0xffffffffu, send, sft);
-                    }
-                }
-                finite = finite && isfinite(v[0]);
-                if (wr) atomicAdd(&cur[r0 + lane], v[0]);
                 // make this warp's shared-memory writes visible to the TMA store, then tell the store warp
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(sdone(k));
             }
             if (!ok) break;
+            finite = finite && isfinite(ss);  // a NaN or Inf weight makes its row's sum non-finite
+            if (wr) atomicAdd(&ss_row(a, a.parity, which, cs)[row], ss);
             if constexpr (STEP) {  // per-segment metric: the tile's share of |mu_s|^2
-                const float t = warp_sum(step);
-                if (lane == 0) atomicAdd(&a.step_sq[cz], t);
-                step = 0.f;
+                step = warp_sum(step);
+                if (lane == 0) atomicAdd(&a.step_sq[x.cz], step);
             }
+            tile_seq0 += x.ncol / 16;
         }
         if (!finite) atomicOr(a.status, DEV_NONFINITE);
     }
@@ -1801,15 +1775,21 @@ cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputM
                               cudaStream_t st) {
     cudaError_t e = ensure_attrs();
     if (e != cudaSuccess) return e;
-    const TcArgs a = make_args(s, w);
+    TcArgs a = make_args(s, w);
+    // The state ring's 8 slots: with short segments the state stream alone sets the pace and four
+    // stores with four loads in flight suit HBM best (128 chains, T = 256, 2K tokens: 14.95 ms with 2
+    // stores in flight, 14.93 with 3, 14.32 with 4, 18.1 with 6); from T = 512 on more loads in
+    // flight win (16 chains, T = 512, 32K tokens: 13.81 / 13.74 / 14.14 ms with 2 / 3 / 4).
+    a.store_lag = s.T <= 256 ? 4 : 2;
     const CUtensorMap& U = s.mode == 1 ? m.Ub : in.Xb;
-    // CTA pairs over 256-column x 256-hidden tiles (a pair's columns lie in one matrix) from
-    // T = 1024 on: there a tile's operand stream (768 KB a CTA) rivals its state stream, and the
-    // pair halves the dH / At share of it.  At T = 512 the pair's coupled loads and accumulator
-    // release cost more than they save (measured: 57.2 vs 54.8 ms a step on l16_d2048_128k).
+    const CUtensorMap& U2 = s.mode == 1 ? m.Ub2 : in.Xb2;
+    const int col_tiles = b_col_tiles(s.d_in, s.d_out);
+    // CTA pairs over 256-hidden x 256-column tiles (a tile's columns all live) from T = 1024 on:
+    // there a tile's operand stream (768 KB a CTA) rivals its state stream, and the pair takes a
+    // third off it.  At T = 512 the pair's coupled loads and accumulator release cost more than they save.
     constexpr int PAIR_MIN_T = 1024;
-    if (s.T >= PAIR_MIN_T && s.d_in % (2 * B_BM) == 0 && s.d_out % (2 * B_BM) == 0 && g_pairb_clusters > 0) {
-        const int npairs = w.nc * ((s.d_in + s.d_out) / (2 * B_BM)) * (s.d_hid / B_BN);
+    if (s.T >= PAIR_MIN_T && s.d_in % B_BN == 0 && (s.d_out / 2) % B_BN == 0 && g_pairb_clusters > 0) {
+        const int npairs = w.nc * col_tiles * (s.d_hid / (2 * B_BM));
         const int maxc = g_pairb_clusters - (s.reserve_sms + 1) / 2;
         const int clusters = npairs < maxc ? npairs : maxc;
         cudaLaunchConfig_t cfg = {};
@@ -1824,21 +1804,16 @@ cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputM
         cfg.stream = st;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        if (a.step_sq)
-            return cudaLaunchKernelEx(&cfg, tc_phase_b_kernel<true, true>, U, in.Kb, in.Vb, m.dH, m.At, m.W1s, m.W2s,
-                                      m.M1s, m.M2s, a);
-        return cudaLaunchKernelEx(&cfg, tc_phase_b_kernel<true, false>, U, in.Kb, in.Vb, m.dH, m.At, m.W1s, m.W2s,
-                                  m.M1s, m.M2s, a);
+        return cudaLaunchKernelEx(&cfg, a.step_sq ? tc_phase_b_kernel<true, true> : tc_phase_b_kernel<true, false>, U2,
+                                  in.Kb2, in.Vb2, m.dH, m.At, m.W1s, m.W2s, a);
     }
-    const int ntiles = w.nc * ((s.d_in + s.d_out) / B_BM) * (s.d_hid / B_BN);
+    const int ntiles = w.nc * col_tiles * (s.d_hid / B_BM);
     const int sms = g_sms - s.reserve_sms;
     const int grid = ntiles < sms ? ntiles : sms;
     if (a.step_sq)
-        tc_phase_b_kernel<false, true><<<grid, B_THREADS, LayoutB::DYN, st>>>(U, in.Kb, in.Vb, m.dH, m.At, m.W1s,
-                                                                              m.W2s, m.M1s, m.M2s, a);
+        tc_phase_b_kernel<false, true><<<grid, B_THREADS, LayoutB::DYN, st>>>(U, in.Kb, in.Vb, m.dH, m.At, m.W1s, m.W2s, a);
     else
-        tc_phase_b_kernel<false, false><<<grid, B_THREADS, LayoutB::DYN, st>>>(U, in.Kb, in.Vb, m.dH, m.At, m.W1s,
-                                                                               m.W2s, m.M1s, m.M2s, a);
+        tc_phase_b_kernel<false, false><<<grid, B_THREADS, LayoutB::DYN, st>>>(U, in.Kb, in.Vb, m.dH, m.At, m.W1s, m.W2s, a);
     return cudaGetLastError();
 }
 
@@ -1968,6 +1943,26 @@ bool encode_map_bf16_3d(CUtensorMap* map, const void* base, uint64_t inner, uint
     const cuuint32_t box[3] = {box_inner, box_rows, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool encode_map_bf16_blocks(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint64_t chains,
+                            uint32_t box_rows, uint32_t box_blocks) {
+    const uint64_t dims[4] = {64, rows, inner / 64, chains}, strides[3] = {inner * 2, 128, inner * rows * 2};
+    const uint32_t box[4] = {64, box_rows, box_blocks, 1};
+    return encode_map_bf16_4d(map, base, dims, strides, box);
+}
+
+bool encode_map_state(CUtensorMap* map, const float* W, const float* mu, uint64_t inner, uint64_t rows,
+                      uint64_t chains) {
+    if (!encoder() || !map || (mu && mu <= W)) return false;
+    const cuuint64_t dims[5] = {32, rows, inner / 32, chains, mu ? 2u : 1u};
+    const cuuint64_t strides[4] = {inner * 4, 128, inner * rows * 4,
+                                   mu ? (cuuint64_t)(mu - W) * 4 : (cuuint64_t)(inner * rows * chains * 4)};
+    const cuuint32_t box[5] = {32, 32, 2, 1, mu ? 2u : 1u};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float*>(W), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
