@@ -3,9 +3,10 @@
 // tokens visible to every query token and the query tokens causal among themselves;
 // query head h reads key/value head h / (n_q / n_kv) (grouped heads).
 //
-// Two forms.  bf16 with 16-byte-aligned rows runs on the tensor cores
-// (attention_tc_kernel: S = Q K^T and O = P V as tcgen05 MMAs with TMEM accumulators, the
-// softmax one row per thread in between).  fp32, and bf16 caches with other strides, run
+// Three forms.  bf16 with 16-byte-aligned rows runs on the tensor cores: many query rows in
+// attention_prefill_kernel (S = Q K^T and O = P V as tcgen05 MMAs with TMEM accumulators, the
+// softmax one row per thread in between), few in attention_decode_kernel (the keys split over
+// warps and a cluster of CTAs).  fp32, and bf16 caches with other strides, run
 // on the CUDA cores in flash-decode form: a CTA takes one (chain, key/value head, tile of
 // query tokens) and stages the cache rows its tokens can see through shared memory in
 // chunks of KC = 64 positions (converted to fp32 once, shared by every query head of the
@@ -35,7 +36,7 @@ struct AttnArgs {
     int L, n_q, n_kv, group, Lq, n_mem, rows;  // rows: query tokens per CTA (group * rows <= ATT_ITEMS)
     float scale;            // 1 / sqrt(hd)
     int vec;                // caches 16-byte aligned (base and every stride): stage with 16-byte loads
-    int* status;            // device status word (bounded waits of the tensor-core form)
+    int* status;            // device status word (bounded waits of the prefill form)
 };
 
 // Stage cache positions [j0, j0 + nk) of one head into shared memory as fp32 rows of HD
@@ -207,57 +208,6 @@ __global__ void __launch_bounds__(ATT_WARPS * 32, 2) attention_kernel(const Attn
     }
 }
 
-// ---------------------------------------------------------------- tensor-core form (bf16)
-// One CTA of 512 threads per (chain, key/value head, tile of query tokens).  Its 128 rows are
-// (query head of the group, token) pairs, `rows` = 128 / group tokens of each of the group's
-// heads, so the group's heads share every staged key and value row.  Keys are taken in chunks
-// of up to AT_NC positions: S = Q K^T accumulates in TMEM columns [0, AT_NC).  Four threads
-// share a row (TMEM lane): each reads its 32-key blocks of the row, the row max is exchanged
-// through shared memory, and each writes its bf16 probabilities to shared memory and
-// keeps its own part of the row sum.  O_c = P V accumulates in TMEM columns [AT_NC, AT_NC + HD),
-// of which each of the four threads takes hd / 4; the running max rescales the output columns
-// and the partial sums from one chunk to the next, and the partial sums meet once at the end.
-// Q, K and V reach shared memory through 16-byte asynchronous copies (cp.async, zero-filled
-// past the last key), all in flight at once, written in the 128-byte-swizzled layout the MMA
-// descriptors read: Q, K and P as K-major operands, V as the MN-major B operand of P V (a value
-// row holds 64 dimensions per 128-byte line, the same bytes as a key row).  S = Q K^T is issued
-// once the queries and keys have landed, with the values still in flight.
-constexpr int AT_THREADS = 512;
-constexpr int AT_GROUPS = AT_THREADS / 128;  // threads per row, each with its own columns
-constexpr int AT_NC = 256;     // key positions per chunk: S's MMA N and TMEM columns
-constexpr int AT_TMEM = 512;   // S (AT_NC columns) + O (HD <= 128 columns), a power of two
-
-template <int HD>
-struct AtSmem {
-    static constexpr int SLAB_Q = 128 * 128;    // one 64-dimension slab of the 128 query rows
-    static constexpr int SLAB_K = AT_NC * 128;  // one 64-dimension slab of AT_NC key (or value) rows
-    static constexpr int SLAB_P = 128 * 128;    // one 64-key slab of the 128 probability rows
-    static constexpr int Q_OFF = 0;
-    static constexpr int K_OFF = Q_OFF + (HD / 64) * SLAB_Q;
-    static constexpr int V_OFF = K_OFF + (HD / 64) * SLAB_K;
-    // hd 128: the probabilities take the key buffer (the same size; keys are dead once S is in TMEM)
-    static constexpr int P_OFF = HD == 128 ? K_OFF : V_OFF + (HD / 64) * SLAB_K;
-    static constexpr int RED_OFF = HD == 128 ? V_OFF + (HD / 64) * SLAB_K : P_OFF + (AT_NC / 64) * SLAB_P;
-    static constexpr int BAR_OFF = RED_OFF + AT_GROUPS * 128 * 4;
-    static constexpr int DYN = BAR_OFF + 64 + 1024;  // + barriers, TMEM slot, flag; + alignment slack
-};
-static_assert(AtSmem<128>::DYN <= 227 * 1024 && AtSmem<64>::DYN <= 227 * 1024, "attention tile exceeds shared memory");
-
-// Issue the copies of n_pad rows of HD bf16 into 64-dimension slabs `slab` bytes apart; row r
-// comes from row_ptr(r) (16-byte aligned) when r < n and row_ptr(r) is non-null, else it is
-// zero-filled (from `any`, a valid global address of which no byte is read).  Nothing waits
-// here: every copy of the tile is in flight at once.
-template <int HD, typename RowPtr>
-__device__ __forceinline__ void at_stage(uint8_t* dst, int slab, int n, int n_pad, const bf16* any, RowPtr row_ptr) {
-    constexpr int VPR = HD / 8;  // 16-byte pieces per row
-    const uint32_t d0 = smem_u32(dst);
-    for (int e = threadIdx.x; e < n_pad * VPR; e += AT_THREADS) {
-        const int r = e / VPR, v = e - r * VPR;
-        const bf16* p = r < n ? row_ptr(r) : nullptr;
-        cpa16(d0 + (v >> 3) * slab + sw128_off(r, v & 7), p ? p + v * 8 : any, p ? 16 : 0);
-    }
-}
-
 // 2^x on the special-function unit (PTX ex2.approx), whose error is far below the bf16
 // rounding of the probabilities it feeds (the parity tests bound the result at 1e-2).
 __device__ __forceinline__ float at_exp2(float x) {
@@ -266,190 +216,525 @@ __device__ __forceinline__ float at_exp2(float x) {
     return y;
 }
 
+// ---------------------------------------------------------------- prefill form (bf16, tcgen05)
+// One CTA per (chain, key/value head, tile of query tokens), two CTAs an SM.  A tile's 128 MMA rows are
+// (query head of the group, token) pairs, rt = 128 / group tokens of each of the group's heads, so
+// the group's heads share every staged key and value row.
+//
+// Warps 0-7: the softmax, two threads per row (= TMEM lane), one for each half of a chunk's keys.
+// Warp 8: the loader; keys and values arrive in chunks of NK positions, in the order they are consumed,
+// through a ring of NS slots, by TMA with the caller's strides (positions past the last key read as
+// zeros).  Warp 9: the MMA issuer.  Per chunk: S = Q K^T into one of two TMEM buffers; the softmax
+// takes the row max (exchanged between a row's two threads), writes its bf16 probabilities over the
+// scores, where P V takes its A operand from, and keeps the row sum; O += P V accumulates in TMEM over all
+// chunks.  The next chunk's S is there before the softmax asks for it.  O is rescaled in TMEM only when
+// a row's max has grown by more than 2^8 (bf16 keeps its relative precision at any scale; the sums are
+// fp32), which after the first chunks hardly ever happens.
+//
+// What bounds it: the softmax's instructions (scale, ex2, bf16, and the sum of the rounded values: about
+// five an element), at 55% of the issue slots; the max exchange and the waits around it leave the rest.
+// 16 chains x 8 heads x 4, 2048 + 64 keys, hd 64: 437 us, 2.23 M visible pairs a head at 668 TFLOP/s (the
+// one-CTA form it replaced, which took S, the softmax and P V of a 256-key chunk in turn: 1140 us); 4 chains,
+// hd 128: 171 us (389).  Measured on the way: P through shared memory, two tiles a CTA 699 us; P in TMEM
+// 565; loads by TMA instead of cp.async 490; one thread per row with two S buffers of 64 keys 463.
+constexpr float FA_SLACK = 8.f;              // growth of the row max, in powers of two, that leaves O alone
+
 template <int HD>
-__global__ void __launch_bounds__(AT_THREADS, 1) attention_tc_kernel(const AttnArgs a) {
-    using SM = AtSmem<HD>;
-    constexpr int OC = HD / AT_GROUPS;  // output columns per thread
+struct FaSmem {
+    static constexpr int LOAD_WARP = 8, MMA_WARP = 9, THREADS = 10 * 32;
+    static constexpr int NK = HD == 64 ? 96 : 64;          // key positions per chunk: 2 NK + HD TMEM columns
+    static constexpr int TMEM = 256;                       // two CTAs an SM
+    static constexpr int Q_SLAB = 128 * 128;               // 128 query rows x 64 bf16
+    static constexpr int SLAB = NK * 128;                  // NK keys x 64 bf16
+    static constexpr int TILE = (HD / 64) * SLAB;          // NK keys x HD
+    static constexpr int NS = HD == 64 ? 7 : 4;            // ring slots, one K or V chunk each
+    static constexpr int Q_OFF = 0;
+    static constexpr int KV_OFF = Q_OFF + (HD / 64) * Q_SLAB;
+    static constexpr int X_OFF = KV_OFF + NS * TILE;       // [2][2][128] floats: row max (or sum) of each half
+    static constexpr int BAR_OFF = X_OFF + 2 * 2 * 128 * 4;  // qfull full[NS] empty[NS] sfull[2] odone[2] pready[2]
+    static constexpr int SLOT_OFF = BAR_OFF + (2 * NS + 7) * 8;
+    static constexpr int DYN = SLOT_OFF + 16 + 1024;       // + TMEM slot, + alignment slack
+};
+static_assert(2 * (FaSmem<64>::DYN + 1024) <= 228 * 1024 && 2 * (FaSmem<128>::DYN + 1024) <= 228 * 1024,
+              "two attention CTAs an SM");
+
+// Packed fp32 pairs (one instruction for two lanes of arithmetic).
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack_f32x2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// N probabilities 2^(v k2 + moff) of a row in bf16 to N / 2 TMEM columns at `tp`.  Returns their sum as
+// the MMA sees them (bf16-rounded).
+template <int N>
+__device__ __forceinline__ float fa_probs(const float (&v)[N], uint64_t k2, uint64_t moff, uint32_t tp) {
+    uint64_t sum[2] = {0, 0};
+#pragma unroll
+    for (int b = 0; b < N; b += 16) {
+        uint32_t pk[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float2 x = unpack_f32x2(fma_f32x2(pack_f32x2(v[b + 2 * j], v[b + 2 * j + 1]), k2, moff));
+            pk[j] = pack_bf16(at_exp2(x.x), at_exp2(x.y));
+            sum[j & 1] = add_f32x2(sum[j & 1], pack_f32x2(__uint_as_float(pk[j] << 16), __uint_as_float(pk[j] & 0xffff0000u)));
+        }
+        tmem_st8(tp + b / 2, pk);
+    }
+    const float2 s = unpack_f32x2(add_f32x2(sum[0], sum[1]));
+    return s.x + s.y;
+}
+
+template <int HD>
+__global__ void __launch_bounds__(FaSmem<HD>::THREADS, 2)
+attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                         const __grid_constant__ CUtensorMap tmV, const AttnArgs a) {
+    using SM = FaSmem<HD>;
+    constexpr int NS = SM::NS, NK = SM::NK, NE = NK / 2;  // NE: keys of a chunk per softmax thread
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* Qs = base + SM::Q_OFF;
-    uint8_t* Ks = base + SM::K_OFF;
-    uint8_t* Vs = base + SM::V_OFF;
-    uint8_t* Ps = base + SM::P_OFF;
-    float* red = reinterpret_cast<float*>(base + SM::RED_OFF);  // [AT_GROUPS][128] per-row partials
-    const uint32_t bar_s = smem_u32(base + SM::BAR_OFF), bar_o = bar_s + 8;
-    uint32_t* slot = reinterpret_cast<uint32_t*>(base + SM::BAR_OFF + 16);
-    int* abort_flag = reinterpret_cast<int*>(base + SM::BAR_OFF + 24);
-    const int tid = threadIdx.x, warp = tid >> 5;
-    // thread -> (row, column group): a warp reaches TMEM lanes 32 (warp % 4) .. + 31, so the four
-    // warps of a lane quarter share its 32 rows and split the columns
-    const int row = (warp & 3) * 32 + (tid & 31), grp = warp >> 2;
+    const uint32_t bars = smem_u32(base + SM::BAR_OFF);
+    const uint32_t qfull = bars;
+    auto full = [&](int s) { return bars + 8 * (1 + s); };
+    auto empty = [&](int s) { return bars + 8 * (1 + NS + s); };
+    // of chunk j, phase j >> 1: two of each, since the softmax may be a chunk ahead of the issuer's P V
+    auto sfull = [&](int j) { return bars + 8 * (1 + 2 * NS + (j & 1)); };
+    auto odone = [&](int j) { return bars + 8 * (3 + 2 * NS + (j & 1)); };
+    auto pready = [&](int j) { return bars + 8 * (5 + 2 * NS + (j & 1)); };
+    uint32_t* slot = reinterpret_cast<uint32_t*>(base + SM::SLOT_OFF);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
-        mbar_init(bar_s, 1);
-        mbar_init(bar_o, 1);
-        *abort_flag = 0;
+        mbar_init(qfull, 1);
+        for (int s = 0; s < NS; ++s) {
+            mbar_init(full(s), 1);
+            mbar_init(empty(s), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(sfull(b), 1);
+            mbar_init(odone(b), 1);
+            mbar_init(pready(b), 8);  // the eight softmax warps
+        }
         fence_mbar_init();
     }
-    if (warp == 0) {
-        tmem_alloc(smem_u32(slot), AT_TMEM);
+    if (warp == SM::MMA_WARP) {
+        tmem_alloc(smem_u32(slot), SM::TMEM);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *slot;
-    const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16);  // this thread's TMEM lane = its row
+    const uint32_t tmem = *slot, t_out = tmem + 2 * NK;  // two S (and P) buffers, then O
 
-    const int c = blockIdx.z, g = blockIdx.y, rt = a.rows, r0 = blockIdx.x * rt;
-    const bf16* Qb = static_cast<const bf16*>(a.Q);
-    const long long kv_off = (long long)(c / a.L) * a.s0 + (long long)(c % a.L) * a.s1 + (long long)g * a.s2;
-    const bf16* Kc = static_cast<const bf16*>(a.K) + kv_off;
-    const bf16* Vc = static_cast<const bf16*>(a.V) + kv_off;
-    // row r of the tile: query head g * group + r / rt of the group, token r0 + r % rt
-    auto q_row = [&](int r) -> const bf16* {
-        const int hr = r / rt, ir = r0 + r % rt;
-        if (hr >= a.group || ir >= a.Lq) return nullptr;
-        return Qb + (((size_t)c * a.n_q + g * a.group + hr) * a.Lq + ir) * HD;
-    };
-    const int hg = row / rt, i = r0 + row % rt;
-    const bool live = hg < a.group && i < a.Lq;
-    const int vis = live ? a.n_mem + i + 1 : 0;     // keys this row sees (causal among the query tokens)
-    const int keys = a.n_mem + min(a.Lq, r0 + rt);  // keys the tile's last token sees
-    const float k2 = a.scale * 1.4426950408889634f;  // softmax scale in base 2: exp(s x) = 2^(s log2(e) x)
+    // token tiles: the last first (causal: it has the most keys)
+    const int c = blockIdx.z, g = blockIdx.y, rt = a.rows, r0 = (gridDim.x - 1 - blockIdx.x) * rt;
+    const int n = (a.n_mem + min(a.Lq, r0 + rt) + NK - 1) / NK;  // chunks the tile's last token sees
 
-    at_stage<HD>(Qs, SM::SLAB_Q, 128, 128, Qb, q_row);
-    float o[OC];
+    if (warp == SM::LOAD_WARP) {
+        if (lane == 0) {
+            tma_prefetch_map(&tmQ);
+            tma_prefetch_map(&tmK);
+            tma_prefetch_map(&tmV);
+            mbar_expect_tx(qfull, (HD / 64) * a.group * rt * 128);
 #pragma unroll
-    for (int d = 0; d < OC; ++d) o[d] = 0.f;
-    float m_run = -INFINITY, l_part = 0.f;  // row max so far; this thread's share of the row sum
-    bool ok = true;
-    int chunk = 0;
-    for (int j0 = 0; j0 < keys; j0 += AT_NC, ++chunk) {
-        const int nk = min(AT_NC, keys - j0), nc = (nk + 15) & ~15;
-        // copy groups: (the queries and) the keys, then the values, which S = Q K^T does not wait for
-        at_stage<HD>(Ks, SM::SLAB_K, nk, nc, Kc, [&](int r) { return Kc + (long long)(j0 + r) * a.s3; });
-        cpa_commit();
-        at_stage<HD>(Vs, SM::SLAB_K, nk, nc, Vc, [&](int r) { return Vc + (long long)(j0 + r) * a.s3; });
-        cpa_commit();
-        cpa_wait(1);
-        fence_proxy_async_smem();
-        tc_fence_before();
-        __syncthreads();
-        if (tid == 0) {  // S = Q K^T over HD (K-major both)
-            tc_fence_after();
-            const uint32_t idesc = idesc_bf16_f32(128, nc, false, false);
+            for (int kb = 0; kb < HD / 64; ++kb)  // the query rows, [head of the group][token]
+                tma_load_4d(smem_u32(base + SM::Q_OFF) + kb * SM::Q_SLAB, &tmQ, qfull, 64 * kb, r0, g * a.group, c);
+            const int ctx = c / a.L, layer = c % a.L;
+            int s = 0, ph = 1;  // slot, and the phase of its release (the first round passes)
+            auto load = [&](const CUtensorMap* m, int j) {
+                if (!mbar_wait(empty(s), ph, a.status)) return false;
+                const uint32_t dst = smem_u32(base + SM::KV_OFF + s * SM::TILE);
+                mbar_expect_tx(full(s), SM::TILE);
 #pragma unroll
-            for (int kb = 0; kb < HD / 64; ++kb)
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    umma_bf16(tmem, sdesc_sw128(smem_u32(Qs + kb * SM::SLAB_Q) + k * 32, 16),
-                              sdesc_sw128(smem_u32(Ks + kb * SM::SLAB_K) + k * 32, 16), idesc, (kb | k) ? 1u : 0u);
-            umma_commit(bar_s);
-        }
-        if (!mbar_wait(bar_s, chunk & 1, a.status)) atomicOr(abort_flag, 1);
-        __syncthreads();
-        if (*abort_flag) {
-            ok = false;
-            break;
-        }
-        tc_fence_after();
-        // this thread's 32-key blocks of the chunk: cb = 32 (grp + AT_GROUPS k); its row sees keys [0, nv)
-        const int nv = min(max(vis - j0, 0), nc);
-        float cm = -INFINITY;
-#pragma unroll
-        for (int k = 0; k < AT_NC / (32 * AT_GROUPS); ++k) {
-            const int cb = 32 * (grp + AT_GROUPS * k);
-            if (cb < nc) {  // uniform over the warp
-                float v[32];
-                tmem_ld32(t_row + cb, v);
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (cb + j < nv) cm = fmaxf(cm, v[j]);
-            }
-        }
-        red[grp * 128 + row] = cm;
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < AT_GROUPS; ++q) cm = fmaxf(cm, red[q * 128 + row]);
-        const float mn = fmaxf(m_run, cm);
-        // rescale of what earlier chunks accumulated (none yet: m_run = -inf gives 0)
-        const float corr = mn == -INFINITY ? 1.f : at_exp2((m_run - mn) * k2);
-        const float moff = mn == -INFINITY ? 0.f : -mn * k2;
-        float ps = 0.f;
-#pragma unroll
-        for (int k = 0; k < AT_NC / (32 * AT_GROUPS); ++k) {
-            const int cb = 32 * (grp + AT_GROUPS * k);
-            if (cb < nc) {
-                float v[32];  // the scores again (a TMEM reload is cheaper than holding them over the exchange)
-                tmem_ld32(t_row + cb, v);
-                uint32_t pk[16];
-#pragma unroll
-                for (int j = 0; j < 32; j += 2) {
-                    const float p0 = cb + j < nv ? at_exp2(fmaf(v[j], k2, moff)) : 0.f;
-                    const float p1 = cb + j + 1 < nv ? at_exp2(fmaf(v[j + 1], k2, moff)) : 0.f;
-                    const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
-                    const float2 pr = __bfloat1622float2(pb);  // the sum takes the probabilities the MMA sees
-                    ps += pr.x + pr.y;
-                    pk[j / 2] = *reinterpret_cast<const uint32_t*>(&pb);
+                for (int kb = 0; kb < HD / 64; ++kb)
+                    tma_load_5d(dst + kb * SM::SLAB, m, full(s), 64 * kb, j * NK, g, layer, ctx);
+                if (++s == NS) {
+                    s = 0;
+                    ph ^= 1;
                 }
-                uint8_t* prow = Ps + (cb >> 6) * SM::SLAB_P;
+                return true;
+            };
+            // K0 K1 V0 K2 V1 .. K(n-1) V(n-2) V(n-1)
+            bool ok = load(&tmK, 0);
+            for (int j = 0; ok && j < n; ++j) ok = (j + 1 >= n || load(&tmK, j + 1)) && load(&tmV, j);
+        }
+        __syncwarp();
+    } else if (warp == SM::MMA_WARP) {
+        if (lane == 0) {
+            const uint32_t id_s = idesc_bf16_f32(128, NK, false, false), id_o = idesc_bf16_f32(128, HD, false, true);
+            // descriptors of the queries and of the ring's first slot as K and as V
+            const uint64_t dq = sdesc_sw128(smem_u32(base + SM::Q_OFF), 16), dk0 = sdesc_sw128(smem_u32(base + SM::KV_OFF), 16),
+                           dv0 = sdesc_sw128(smem_u32(base + SM::KV_OFF), SM::SLAB);
+            int s = 0, ph = 0;  // the ring's next slot and its phase
+            auto next = [&]() {
+                if (++s == NS) {
+                    s = 0;
+                    ph ^= 1;
+                }
+            };
+            auto issue_s = [&](int j) {  // S = Q K^T over HD (K-major both)
+                if (!mbar_wait(full(s), ph, a.status)) return false;
+                tc_fence_after();
+                const uint64_t dk = sdesc_step(dk0, s * SM::TILE);
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    *reinterpret_cast<uint4*>(prow + sw128_off(row, ((cb & 63) >> 3) + u)) =
-                        make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2], pk[4 * u + 3]);
+                for (int kb = 0; kb < HD / 64; ++kb)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        umma_bf16(tmem + (j & 1) * NK, sdesc_step(dq, kb * SM::Q_SLAB + u * 32),
+                                  sdesc_step(dk, kb * SM::SLAB + u * 32), id_s, (kb | u) ? 1u : 0u);
+                umma_commit(sfull(j));
+                umma_commit(empty(s));
+                next();
+                return true;
+            };
+            bool ok = mbar_wait(qfull, 0, a.status) && issue_s(0) && (n < 2 || issue_s(1));
+            for (int j = 0; ok && j < n; ++j) {
+                // P of chunk j is in TMEM
+                ok = mbar_wait(full(s), ph, a.status) && mbar_wait(pready(j), (j >> 1) & 1, a.status);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t dv = sdesc_step(dv0, s * SM::TILE);
+#pragma unroll
+                for (int kk = 0; kk < NK / 16; ++kk)  // O += P V over the chunk's keys (P in TMEM, V MN-major)
+                    umma_bf16_ta(t_out, tmem + (j & 1) * NK + kk * 8, sdesc_step(dv, kk * 16 * 128), id_o, (j | kk) ? 1u : 0u);
+                umma_commit(odone(j));
+                umma_commit(empty(s));
+                next();
+                // S of chunk j + 2 goes over the P that P V has to have read
+                if (j + 2 < n) ok = mbar_wait(odone(j), (j >> 1) & 1, a.status) && issue_s(j + 2);
             }
         }
-        l_part = fmaf(l_part, corr, ps);
-        cpa_wait(0);  // this thread's value copies
-        fence_proxy_async_smem();
-        tc_fence_before();
-        __syncthreads();
-        if (tid == 0) {  // O_c = P V over the chunk's keys (P K-major, V MN-major)
+        __syncwarp();
+    } else {
+        // ---- softmax: row = TMEM lane, half = keys NE half .. of every chunk
+        const int quarter = warp & 3, half = warp >> 2, row = quarter * 32 + lane;
+        const int hr = row / rt, i = r0 + row % rt;
+        const bool live = hr < a.group && i < a.Lq;
+        const int vis = a.n_mem + (live ? i : r0) + 1;   // keys the row sees (a row of padding: any)
+        const float k2 = a.scale * 1.4426950408889634f;  // softmax scale in base 2: exp(s x) = 2^(s log2(e) x)
+        const uint32_t lane_off = (uint32_t)(quarter * 32) << 16, t_o = t_out + lane_off + half * (HD / 2);
+        float* xch = reinterpret_cast<float*>(base + SM::X_OFF);
+        float m_run = -INFINITY, l = 0.f;
+        bool ok = true;
+        for (int j = 0; j < n; ++j) {
+            const uint32_t t_s = tmem + lane_off + (j & 1) * NK;
+            ok = __all_sync(0xffffffffu, mbar_wait(sfull(j), (j >> 1) & 1, a.status));
             tc_fence_after();
-            const uint32_t idesc = idesc_bf16_f32(128, HD, false, true);
-            for (int kk = 0; kk < nc / 16; ++kk)
-                umma_bf16(tmem + AT_NC, sdesc_sw128(smem_u32(Ps + (kk >> 2) * SM::SLAB_P) + (kk & 3) * 32, 16),
-                          sdesc_sw128(smem_u32(Vs) + kk * 16 * 128, SM::SLAB_K), idesc, kk ? 1u : 0u);
-            umma_commit(bar_o);
-        }
-        if (!mbar_wait(bar_o, chunk & 1, a.status)) atomicOr(abort_flag, 1);
-        __syncthreads();
-        if (*abort_flag) {
-            ok = false;
-            break;
-        }
-        tc_fence_after();
-        {  // this thread's OC output columns
-            float w[OC];
-            if constexpr (OC == 32)
-                tmem_ld32(t_row + AT_NC + grp * OC, w);
+            float v[NE];
+            if constexpr (NE == 48)
+                tmem_ld48(t_s + half * NE, v);
             else
-                tmem_ld16(t_row + AT_NC + grp * OC, w);
+                tmem_ld32(t_s + half * NE, v);
+            if ((j + 1) * NK > a.n_mem + r0 + 1) {      // some row does not see the whole chunk:
+                const int nv = vis - j * NK - half * NE;  // a hidden key's score of -inf gives it a probability of 0
 #pragma unroll
-            for (int d = 0; d < OC; ++d) o[d] = fmaf(o[d], corr, w[d]);
+                for (int u = 0; u < NE; ++u) v[u] = u < nv ? v[u] : -INFINITY;
+            }
+            float c4[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+            for (int u = 4; u < NE; u += 4)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) c4[k] = fmaxf(c4[k], v[u + k]);
+            float cm = fmaxf(fmaxf(c4[0], c4[1]), fmaxf(c4[2], c4[3]));
+            float* x = xch + (j & 1) * 256;
+            x[half * 128 + row] = cm;
+            // The two warps of the rows meet, all their scores read (P goes over them); after a wait that ran
+            // out both leave here.
+            tc_fence_before();
+            ok = named_bar_and(1 + quarter, 64, ok);
+            if (!ok) break;
+            tc_fence_after();
+            cm = fmaxf(cm, x[(half ^ 1) * 128 + row]);
+            if (j == 0) {
+                m_run = cm;
+            } else {
+                const bool grown = (cm - m_run) * k2 > FA_SLACK;
+                if (__any_sync(0xffffffffu, grown)) {  // the same in both warps: each rescales its half of O
+                    // O up to the last chunk (on this barrier the phase before is done: S of this chunk waited for it)
+                    const bool in = __all_sync(0xffffffffu, mbar_wait(odone(j - 1), ((j - 1) >> 1) & 1, a.status));
+                    tc_fence_after();
+                    const float corr = grown ? at_exp2((m_run - cm) * k2) : 1.f;
+                    if (grown) m_run = cm;
+                    l *= corr;
+#pragma unroll 1
+                    for (int cb = 0; in && cb < HD / 2; cb += 16) {
+                        float ov[16];
+                        uint32_t on[16];
+                        tmem_ld16(t_o + cb, ov);
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) on[u] = __float_as_uint(ov[u] * corr);
+                        tmem_st16(t_o + cb, on);
+                    }
+                }
+            }
+            const float moff = -m_run * k2;
+            l += fa_probs(v, pack_f32x2(k2, k2), pack_f32x2(moff, moff), t_s + half * (NE / 2));
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(pready(j));
         }
-        m_run = mn;
-        // the next chunk restages K, V (and P) and rewrites red: the MMAs that read the buffers
-        // have completed and every thread passed the barrier after its last read of red
-    }
-    red[grp * 128 + row] = l_part;
-    __syncthreads();
-    if (ok && live) {
-        float l = 0.f;
+        float* x = xch + (n & 1) * 256;
+        x[half * 128 + row] = l;
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(odone(n - 1), ((n - 1) >> 1) & 1, a.status));
+        ok = named_bar_and(1 + quarter, 64, ok);
+        if (ok) {
+            tc_fence_after();
+            const float inv = 1.f / (l + x[(half ^ 1) * 128 + row]);
+            bf16* orow = static_cast<bf16*>(a.out) +
+                         (((size_t)c * a.n_q + g * a.group + (live ? hr : 0)) * a.Lq + (live ? i : 0)) * HD + half * (HD / 2);
 #pragma unroll
-        for (int q = 0; q < AT_GROUPS; ++q) l += red[q * 128 + row];
-        const float inv = 1.f / l;
-        bf16* orow = static_cast<bf16*>(a.out) + (((size_t)c * a.n_q + g * a.group + hg) * a.Lq + i) * HD + grp * OC;
+            for (int cb = 0; cb < HD / 2; cb += 32) {
+                float v[32];
+                tmem_ld32(t_o + cb, v);
+                if (live) {
 #pragma unroll
-        for (int v8 = 0; v8 < OC / 8; ++v8)
-            *reinterpret_cast<uint4*>(orow + v8 * 8) =
-                make_uint4(pack_bf16(o[8 * v8] * inv, o[8 * v8 + 1] * inv), pack_bf16(o[8 * v8 + 2] * inv, o[8 * v8 + 3] * inv),
-                           pack_bf16(o[8 * v8 + 4] * inv, o[8 * v8 + 5] * inv),
-                           pack_bf16(o[8 * v8 + 6] * inv, o[8 * v8 + 7] * inv));
+                    for (int u = 0; u < 32; u += 8)
+                        *reinterpret_cast<uint4*>(orow + cb + u) =
+                            make_uint4(pack_bf16(v[u] * inv, v[u + 1] * inv), pack_bf16(v[u + 2] * inv, v[u + 3] * inv),
+                                       pack_bf16(v[u + 4] * inv, v[u + 5] * inv), pack_bf16(v[u + 6] * inv, v[u + 7] * inv));
+                }
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, AT_TMEM);
+    tc_fence_after();
+    if (warp == SM::MMA_WARP) tmem_dealloc(tmem, SM::TMEM);
+}
+
+// ---------------------------------------------------------------- decode form (bf16, few rows)
+// Few (query head, token) rows per key/value head: the caches are read once and little is computed,
+// so the kernel is a stream over keys and values, bound by HBM, or at short caches by latency.  A
+// cluster of `splits` CTAs takes (chain, key/value head, 16 rows); the keys' 32-position blocks are
+// split over the CTAs and their warps.  Each warp runs an online softmax of its own with
+// mma.m16n8k16 on operands loaded from global memory straight into fragment order (a 128-row
+// tcgen05 tile would be 1/8 to 1/32 full, and its staging would cost more than the arithmetic): the
+// contraction over hd and the order of output columns are free, so they are permuted to let every
+// thread load 16 contiguous bytes (K: dims 32 p + 8 t .. + 7 of key g; V: dims 64 p + 8 g .. + 7 of keys
+// 2 t, 2 t + 1, 2 t + 8, 2 t + 9; lane = 4 g + t).  The warps' partial results meet in shared memory, the
+// CTAs' through distributed shared memory.
+constexpr int DE_WARPS = 4, DE_ROWS = 16;
+// This form is taken up to 16 rows per key/value head, and beyond that while its row tiles over all
+// heads stay few: it re-reads the caches for each 16 rows but splits the keys, the prefill form does
+// neither.  1 chain x 8 heads x 4, 4000 keys: 16 / 64 / 128 rows take 7.9 / 9.5 / 14.0 us here and 37 us
+// in the prefill form; 16 chains, 1000 keys: 16 rows 10.4 and 12.5 us, 20 rows 14.9 and 12.7 us.
+constexpr int DE_MAX_TILES = 128;
+
+template <int HD>
+struct DeSmem {
+    // per warp, then once for the CTA: O [16][HD], then max and sum per row
+    static constexpr int PART = DE_ROWS * HD + 2 * DE_ROWS;
+    static constexpr int FLOATS = (DE_WARPS + 1) * PART;
+};
+
+__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&A)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(b0), "r"(b1));
+}
+
+// fp32 of CTA `rank` of the cluster at the place of `p` in this one
+__device__ __forceinline__ float ld_cluster_f32(const float* p, uint32_t rank) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(map_to_cta(smem_u32(p), rank)) : "memory");
+    return v;
+}
+
+template <int HD>
+__global__ void __launch_bounds__(DE_WARPS * 32, HD == 64 ? 4 : 3) attention_decode_kernel(const AttnArgs a, int splits) {
+    constexpr int NP = HD / 32, NV = HD / 64;  // 16-byte pieces of a key per thread; of a value
+    constexpr int KB = HD == 64 ? 32 : 16;     // keys per step
+    extern __shared__ float de_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gq = lane >> 2, t = lane & 3;
+    const int c = blockIdx.z, g = blockIdx.y, rank = blockIdx.x % splits, row0 = blockIdx.x / splits * DE_ROWS;
+    const int R = a.group * a.Lq, keys = a.n_mem + a.Lq;
+    const long long kv_off = (long long)(c / a.L) * a.s0 + (long long)(c % a.L) * a.s1 + (long long)g * a.s2;
+    const bf16* Kc = static_cast<const bf16*>(a.K) + kv_off + 8 * t;
+    const bf16* Vc = static_cast<const bf16*>(a.V) + kv_off + 8 * gq;
+    // rows row0 + gq and + 8: row r is token r % Lq of the group's head r / Lq
+    uint32_t qa[HD / 16][4];
+    int vis[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r = row0 + gq + 8 * h;
+        vis[h] = r < R ? a.n_mem + r % a.Lq + 1 : 0;
+        const bf16* q = static_cast<const bf16*>(a.Q) + ((size_t)c * a.n_q + (size_t)g * a.group) * a.Lq * HD + (size_t)r * HD + 8 * t;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const uint4 v = r < R ? *reinterpret_cast<const uint4*>(q + 32 * p) : make_uint4(0, 0, 0, 0);
+            qa[2 * p][h] = v.x;
+            qa[2 * p][2 + h] = v.y;
+            qa[2 * p + 1][h] = v.z;
+            qa[2 * p + 1][2 + h] = v.w;
+        }
+    }
+    const float k2 = a.scale * 1.4426950408889634f;
+    float o[8 * NV][4], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < 8 * NV; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
+    const int nb = (keys + KB - 1) / KB;
+    const int b1 = (int)((long long)nb * (rank + 1) / splits);
+    for (int b = (int)((long long)nb * rank / splits) + warp; b < b1; b += DE_WARPS) {
+        const int j0 = b * KB;
+        uint4 kr[KB / 8][NP], vr[KB / 16][4][NV];
+#pragma unroll
+        for (int nt = 0; nt < KB / 8; ++nt) {
+            const int key = j0 + 8 * nt + gq;
+#pragma unroll
+            for (int p = 0; p < NP; ++p)
+                kr[nt][p] = key < keys ? __ldg(reinterpret_cast<const uint4*>(Kc + (long long)key * a.s3 + 32 * p))
+                                       : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int kk = 0; kk < KB / 16; ++kk)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int key = j0 + 16 * kk + 2 * t + (u & 1) + 8 * (u >> 1);
+#pragma unroll
+                for (int p = 0; p < NV; ++p)
+                    vr[kk][u][p] = key < keys ? __ldg(reinterpret_cast<const uint4*>(Vc + (long long)key * a.s3 + 64 * p))
+                                              : make_uint4(0, 0, 0, 0);
+            }
+        float s[KB / 8][4];
+        float cm[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+        for (int nt = 0; nt < KB / 8; ++nt) {
+            s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                mma_16816(s[nt], qa[2 * p], kr[nt][p].x, kr[nt][p].y);
+                mma_16816(s[nt], qa[2 * p + 1], kr[nt][p].z, kr[nt][p].w);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {  // e: row half e >> 1, key 2 t + (e & 1)
+                const bool in = j0 + 8 * nt + 2 * t + (e & 1) < vis[e >> 1];
+                cm[e >> 1] = in ? fmaxf(cm[e >> 1], s[nt][e]) : cm[e >> 1];
+            }
+        }
+        float moff[2], corr[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            cm[h] = fmaxf(cm[h], __shfl_xor_sync(0xffffffffu, cm[h], 1));
+            cm[h] = fmaxf(cm[h], __shfl_xor_sync(0xffffffffu, cm[h], 2));
+            const float mn = fmaxf(m[h], cm[h]);
+            corr[h] = mn == -INFINITY ? 1.f : at_exp2((m[h] - mn) * k2);
+            moff[h] = mn == -INFINITY ? 0.f : -mn * k2;
+            m[h] = mn;
+            l[h] *= corr[h];
+        }
+#pragma unroll
+        for (int j = 0; j < 8 * NV; ++j) {
+            o[j][0] *= corr[0];
+            o[j][1] *= corr[0];
+            o[j][2] *= corr[1];
+            o[j][3] *= corr[1];
+        }
+#pragma unroll
+        for (int kk = 0; kk < KB / 16; ++kk) {
+            uint32_t pa[4];  // rows g / g + 8 x keys (2t, 2t + 1), then the same of the next eight keys
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int nt = 2 * kk + (q >> 1), h = q & 1, key = j0 + 8 * nt + 2 * t;
+                const float e0 = key < vis[h] ? at_exp2(fmaf(s[nt][2 * h], k2, moff[h])) : 0.f;
+                const float e1 = key + 1 < vis[h] ? at_exp2(fmaf(s[nt][2 * h + 1], k2, moff[h])) : 0.f;
+                pa[q] = pack_bf16(e0, e1);
+                // the sum takes the probabilities the MMA sees
+                l[h] += __uint_as_float(pa[q] << 16) + __uint_as_float(pa[q] & 0xffff0000u);
+            }
+#pragma unroll
+            for (int p = 0; p < NV; ++p) {
+                const uint32_t* v0 = reinterpret_cast<const uint32_t*>(&vr[kk][0][p]);
+                const uint32_t* v1 = reinterpret_cast<const uint32_t*>(&vr[kk][1][p]);
+                const uint32_t* v2 = reinterpret_cast<const uint32_t*>(&vr[kk][2][p]);
+                const uint32_t* v3 = reinterpret_cast<const uint32_t*>(&vr[kk][3][p]);
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    mma_16816(o[8 * p + 2 * w], pa, __byte_perm(v0[w], v1[w], 0x5410), __byte_perm(v2[w], v3[w], 0x5410));
+                    mma_16816(o[8 * p + 2 * w + 1], pa, __byte_perm(v0[w], v1[w], 0x7632), __byte_perm(v2[w], v3[w], 0x7632));
+                }
+            }
+        }
+    }
+    // partial results of the warps: column n of output tile j of piece p is dimension 64 p + 8 n + j
+    float* part = de_smem + warp * DeSmem<HD>::PART;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        l[h] += __shfl_xor_sync(0xffffffffu, l[h], 1);
+        l[h] += __shfl_xor_sync(0xffffffffu, l[h], 2);
+        const int r = gq + 8 * h;
+        if (t == 0) {
+            part[DE_ROWS * HD + r] = m[h];
+            part[DE_ROWS * HD + DE_ROWS + r] = l[h];
+        }
+#pragma unroll
+        for (int p = 0; p < NV; ++p)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int j = 0; j < 8; j += 4)
+                    *reinterpret_cast<float4*>(part + r * HD + 64 * p + 8 * (2 * t + e) + j) =
+                        make_float4(o[8 * p + j][2 * h + e], o[8 * p + j + 1][2 * h + e], o[8 * p + j + 2][2 * h + e],
+                                    o[8 * p + j + 3][2 * h + e]);
+    }
+    __syncthreads();
+    // the CTA's result: max, sum and O over its warps
+    float* sum = de_smem + DE_WARPS * DeSmem<HD>::PART;
+    const float* ml = de_smem + DE_ROWS * HD;
+    for (int e = threadIdx.x; e < DE_ROWS * HD; e += DE_WARPS * 32) {
+        const int r = e / HD;
+        float mx = -INFINITY, lt = 0.f, ot = 0.f;
+#pragma unroll
+        for (int w = 0; w < DE_WARPS; ++w) mx = fmaxf(mx, ml[w * DeSmem<HD>::PART + r]);
+#pragma unroll
+        for (int w = 0; w < DE_WARPS; ++w) {
+            const float mw = ml[w * DeSmem<HD>::PART + r];
+            const float f = mw == -INFINITY ? 0.f : at_exp2((mw - mx) * k2);
+            lt = fmaf(f, ml[w * DeSmem<HD>::PART + DE_ROWS + r], lt);
+            ot = fmaf(f, de_smem[w * DeSmem<HD>::PART + e], ot);
+        }
+        sum[e] = ot;
+        if (e % HD == 0) {
+            sum[DE_ROWS * HD + r] = mx;
+            sum[DE_ROWS * HD + DE_ROWS + r] = lt;
+        }
+    }
+    if (splits > 1)
+        cluster_sync();
+    else
+        __syncthreads();
+    // every CTA of the cluster finishes a share of the rows' outputs, two dimensions a thread
+    for (int e = 2 * (rank * DE_WARPS * 32 + threadIdx.x); e < DE_ROWS * HD; e += 2 * splits * DE_WARPS * 32) {
+        const int r = e / HD, d = e - r * HD;
+        if (row0 + r >= R) break;
+        float mx = -INFINITY, lt = 0.f, o0 = 0.f, o1 = 0.f;
+        for (int k = 0; k < splits; ++k) mx = fmaxf(mx, ld_cluster_f32(sum + DE_ROWS * HD + r, k));
+        for (int k = 0; k < splits; ++k) {
+            const float mk = ld_cluster_f32(sum + DE_ROWS * HD + r, k);
+            const float f = mk == -INFINITY ? 0.f : at_exp2((mk - mx) * k2);
+            lt = fmaf(f, ld_cluster_f32(sum + DE_ROWS * HD + DE_ROWS + r, k), lt);
+            o0 = fmaf(f, ld_cluster_f32(sum + e, k), o0);
+            o1 = fmaf(f, ld_cluster_f32(sum + e + 1, k), o1);
+        }
+        const float inv = 1.f / lt;
+        bf16* out = static_cast<bf16*>(a.out) + ((size_t)c * a.n_q + (size_t)g * a.group) * a.Lq * HD + (size_t)(row0 + r) * HD + d;
+        *reinterpret_cast<uint32_t*>(out) = pack_bf16(o0 * inv, o1 * inv);
+    }
+    if (splits > 1) cluster_sync();  // no CTA leaves while another reads its shared memory
 }
 
 std::mutex g_attr_mu;
@@ -483,14 +768,58 @@ cudaError_t launch_t(const AttnArgs& a, int C, cudaStream_t st) {
 }
 
 template <int HD>
-cudaError_t launch_tc(AttnArgs a, int C, cudaStream_t st) {
+cudaError_t launch_prefill(AttnArgs a, int n_ctx, int C, cudaStream_t st) {
     static bool done[64] = {};
-    cudaError_t e = smem_opt_in(attention_tc_kernel<HD>, AtSmem<HD>::DYN, done);
+    cudaError_t e = smem_opt_in(attention_prefill_kernel<HD>, FaSmem<HD>::DYN, done);
     if (e != cudaSuccess) return e;
+    const int rows0 = a.rows;
     a.rows = 128 / a.group;  // tokens per tile: the group's heads x rows fill the 128 MMA rows
+    const uint64_t Lq = a.Lq, keys = (uint64_t)a.n_mem + Lq;
+    CUtensorMap mq, mk, mv;
+    const uint64_t qd[4] = {HD, Lq, (uint64_t)a.n_q, (uint64_t)C}, qs[3] = {HD * 2, Lq * HD * 2, a.n_q * Lq * HD * 2};
+    const uint32_t qb[4] = {64, (uint32_t)a.rows, (uint32_t)a.group, 1};
+    // the caller's strides (a dimension of one element takes any stride)
+    const uint64_t kd[5] = {HD, keys, (uint64_t)a.n_kv, (uint64_t)a.L, (uint64_t)n_ctx};
+    const uint64_t s3 = a.s3 * 2;
+    const uint64_t ks[4] = {s3, a.n_kv > 1 ? a.s2 * 2 : s3, a.L > 1 ? a.s1 * 2 : s3, n_ctx > 1 ? a.s0 * 2 : s3};
+    const uint32_t kb[5] = {64, FaSmem<HD>::NK, 1, 1, 1};
+    const bool broadcast = std::min({ks[0], ks[1], ks[2], ks[3]}) == 0;
+    if (broadcast || !encode_map_bf16_4d(&mq, a.Q, qd, qs, qb) || !encode_map_bf16_5d(&mk, a.K, kd, ks, kb) ||
+        !encode_map_bf16_5d(&mv, a.V, kd, ks, kb)) {
+        a.rows = rows0;  // strides a tensor map does not take (0, or past its range): the CUDA-core form
+        return launch_t<bf16, HD>(a, C, st);
+    }
     dim3 grid((a.Lq + a.rows - 1) / a.rows, a.n_kv, C);
-    attention_tc_kernel<HD><<<grid, AT_THREADS, AtSmem<HD>::DYN, st>>>(a);
+    attention_prefill_kernel<HD><<<grid, FaSmem<HD>::THREADS, FaSmem<HD>::DYN, st>>>(mq, mk, mv, a);
     return cudaGetLastError();
+}
+
+template <int HD>
+cudaError_t launch_decode(const AttnArgs& a, int C, cudaStream_t st) {
+    static bool done[64] = {};
+    constexpr size_t smem = DeSmem<HD>::FLOATS * sizeof(float);
+    cudaError_t e = smem_opt_in(attention_decode_kernel<HD>, smem, done);
+    if (e != cudaSuccess) return e;
+    const int row_tiles = (a.group * a.Lq + DE_ROWS - 1) / DE_ROWS;
+    // split the keys over a cluster until the grid fills the SMs' CTA slots, or a CTA's warps would
+    // have no block of keys each
+    const long long ctas = (long long)row_tiles * a.n_kv * C;
+    const int blocks = (a.n_mem + a.Lq + 31) / 32;
+    constexpr int slots = (HD == 64 ? 4 : 3) * 152;
+    const int splits = (int)std::max(1ll, std::min({8ll, slots / ctas, (long long)blocks / DE_WARPS}));
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = splits;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(splits * row_tiles, a.n_kv, C);
+    cfg.blockDim = dim3(DE_WARPS * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, attention_decode_kernel<HD>, a, splits);
 }
 
 }  // namespace
@@ -511,8 +840,12 @@ cudaError_t launch_attention(const DevState& s, int n_layers, const void* Q, int
         return s.hd == 64 ? launch_t<float, 64>(a, s.C, st) : launch_t<float, 128>(a, s.C, st);
     // bf16 on the tensor cores when every row it stages is 16-byte aligned (the queries and the
     // output are dense rows of hd elements); other cache layouts take the CUDA-core kernel
-    if (a.vec && ((reinterpret_cast<uintptr_t>(Q) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0)
-        return s.hd == 64 ? launch_tc<64>(a, s.C, st) : launch_tc<128>(a, s.C, st);
+    if (a.vec && ((reinterpret_cast<uintptr_t>(Q) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0) {
+        const long long row_tiles = ((long long)a.group * Lq + DE_ROWS - 1) / DE_ROWS;
+        if (row_tiles == 1 || row_tiles * a.n_kv * s.C <= DE_MAX_TILES)
+            return s.hd == 64 ? launch_decode<64>(a, s.C, st) : launch_decode<128>(a, s.C, st);
+        return s.hd == 64 ? launch_prefill<64>(a, s.C / n_layers, s.C, st) : launch_prefill<128>(a, s.C / n_layers, s.C, st);
+    }
     return s.hd == 64 ? launch_t<bf16, 64>(a, s.C, st) : launch_t<bf16, 128>(a, s.C, st);
 }
 

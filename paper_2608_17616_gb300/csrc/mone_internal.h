@@ -221,4 +221,8 @@ bool encode_map_state(CUtensorMap* map, const float* W, const float* mu, uint64_
 bool encode_map_bf16_4d(CUtensorMap* map, const void* base, const uint64_t dims[4], const uint64_t strides[3],
                         const uint32_t box[4]);
 
+// 5-D bf16 map, 128-byte swizzle, as above.
+bool encode_map_bf16_5d(CUtensorMap* map, const void* base, const uint64_t dims[5], const uint64_t strides[4],
+                        const uint32_t box[5]);
+
 }  // namespace mone

@@ -1979,6 +1979,18 @@ bool encode_map_bf16_4d(CUtensorMap* map, const void* base, const uint64_t dims[
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool encode_map_bf16_5d(CUtensorMap* map, const void* base, const uint64_t dims[5], const uint64_t strides[4],
+                        const uint32_t box[5]) {
+    if (!encoder() || !map) return false;
+    const cuuint64_t d[5] = {dims[0], dims[1], dims[2], dims[3], dims[4]};
+    const cuuint64_t st[4] = {strides[0], strides[1], strides[2], strides[3]};
+    const cuuint32_t b[5] = {box[0], box[1], box[2], box[3], box[4]};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), d, st, b, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool encode_map_plain_3d(CUtensorMap* map, const void* base, bool f32, uint64_t inner, uint64_t rows,
                          uint64_t chains, uint32_t box_inner, uint32_t box_rows) {
     if (!encoder() || !map) return false;

@@ -1,0 +1,91 @@
+"""GPU parity of the two bf16 tensor-core attention forms at the edges of their tiles.
+
+Prefill form (many rows over all heads): 128-row tiles, chunks of 96 keys (64 at hd 128) through a
+ring, an output rescale when a row's max grows.  Decode form (up to 16 rows per head, or few row tiles
+in all): 16-row tiles, keys split over warps and clusters.  Tolerance 1e-2 as in test_attention_gpu.py (bf16
+probabilities and outputs, 2^-9 each, fp32 sums).
+"""
+import pytest
+import torch
+
+import oracle as O
+import paper_2608_17616_gb300 as mone
+import workloads as wk
+from harness import DeviceRun, rel_fro
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2608_17616_gb300 import build
+    build.build()
+    assert torch.cuda.is_available()
+    mone.lib()
+
+
+def run_case(group, Lq, n_mem, hd, n_layers=2, n_kv=2, late_scale=1.0):
+    """late_scale: factor on the keys of the last third of the cache, so later chunks raise the row max."""
+    d_out = max(256, 2 * n_kv * hd)
+    wl = wk.Workload("attn_forms", 41, 1, n_layers, 256, 256, d_out, d_out // (2 * hd), hd, 128, 128, 8, "bf16", wk.PLAIN)
+    run = DeviceRun(wl)
+    n_kv, S = wl.n_kv_heads, n_mem + Lq
+    g = torch.Generator(device="cuda").manual_seed(group * 1000 + Lq * 10 + n_mem + hd)
+    K = torch.randn(1, n_layers, n_kv, S, hd, generator=g, device="cuda")
+    K[..., 2 * S // 3:, :] *= late_scale
+    K, V = K.bfloat16(), torch.randn(K.shape, generator=g, device="cuda").bfloat16()
+    Q = torch.randn(1, n_layers, group * n_kv, Lq, hd, generator=g, device="cuda").bfloat16()
+    out = torch.full_like(Q, 7.0)
+    mone.mone_attention(run.h, Q, group * n_kv, Lq, K, V, K.stride()[:4], n_mem, out)
+    mone.mone_mem_sync(run.h)
+    run.close()
+    for layer in sorted({0, n_layers // 2, n_layers - 1}):
+        ref = O.attention(Q[0, layer].cpu(), K[0, layer].cpu(), V[0, layer].cpu(), n_mem)
+        assert rel_fro(out[0, layer].float().cpu(), ref) <= 1e-2, layer
+
+
+@pytest.mark.parametrize("group,Lq,n_mem,hd,late_scale", [
+    (4, 200, 70, 64, 1.0),    # 32-token tiles, the last ragged
+    (1, 300, 513, 64, 1.0),   # 128-token tiles; nine chunks, a ring wrap
+    (2, 33, 1000, 64, 1.0),   # one tile of 66 rows over eleven chunks
+    (64, 2, 94, 64, 1.0),     # the largest group: 2 tokens a tile; exactly one chunk of keys
+    (64, 2, 95, 64, 1.0),     # one key past it
+    (3, 150, 0, 128, 1.0),    # padded rows (126 of 128), no memory, hd 128
+    (4, 129, 383, 128, 1.0),  # hd 128: 64-key chunks, eight of them exactly, one token past the tiles
+    (4, 100, 300, 64, 9.0),   # the row max grows past the slack in later chunks: O is rescaled
+    (2, 140, 200, 128, 9.0),
+])
+def test_prefill_form(group, Lq, n_mem, hd, late_scale):
+    run_case(group, Lq, n_mem, hd, n_layers=20, late_scale=late_scale)
+
+
+def test_prefill_form_many_tiles_repeat():
+    """More CTAs than the SMs hold at once, repeated: every wait is met and the output repeats bit for bit."""
+    n_kv, group, hd, Lq, n_mem, L = 8, 4, 128, 400, 64, 16
+    wl = wk.Workload("attn_forms", 42, 1, L, 256, 256, 2 * n_kv * hd, n_kv, hd, 128, 128, 8, "bf16", wk.PLAIN)
+    run = DeviceRun(wl)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    K = torch.randn(1, L, n_kv, n_mem + Lq, hd, generator=g, device="cuda").bfloat16()
+    V = torch.randn(K.shape, generator=g, device="cuda").bfloat16()
+    Q = torch.randn(1, L, group * n_kv, Lq, hd, generator=g, device="cuda").bfloat16()
+    outs = [torch.full_like(Q, 7.0) for _ in range(2)]
+    for i in range(40):
+        mone.mone_attention(run.h, Q, group * n_kv, Lq, K, V, K.stride()[:4], n_mem, outs[i % 2])
+    mone.mone_mem_sync(run.h)
+    run.close()
+    assert torch.equal(*outs)
+
+
+@pytest.mark.parametrize("group,Lq,n_mem,hd,n_layers", [
+    (1, 1, 0, 64, 2),        # one row, one key
+    (4, 1, 31, 64, 2),       # one whole 32-key block
+    (4, 1, 32, 64, 2),       # one key past it
+    (7, 2, 5000, 64, 1),     # a cluster of eight, 14 rows
+    (8, 3, 700, 64, 3),      # 24 rows: two row tiles, causal rows
+    (16, 32, 100, 64, 1),    # 512 rows: 32 row tiles of two heads
+    (4, 1, 15, 128, 2),      # hd 128: one whole 16-key block
+    (4, 1, 16, 128, 2),      # one key past it
+    (5, 5, 3000, 128, 1),    # 25 rows over a cluster
+])
+def test_decode_form(group, Lq, n_mem, hd, n_layers):
+    run_case(group, Lq, n_mem, hd, n_layers=n_layers, late_scale=3.0)
