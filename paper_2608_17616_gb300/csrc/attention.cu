@@ -258,28 +258,6 @@ struct FaSmem {
 static_assert(2 * (FaSmem<64>::DYN + 1024) <= 228 * 1024 && 2 * (FaSmem<128>::DYN + 1024) <= 228 * 1024,
               "two attention CTAs an SM");
 
-// Packed fp32 pairs (one instruction for two lanes of arithmetic).
-__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpack_f32x2(uint64_t v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
 // N probabilities 2^(v k2 + moff) of a row in bf16 to N / 2 TMEM columns at `tp`.  Returns their sum as
 // the MMA sees them (bf16-rounded).
 template <int N>

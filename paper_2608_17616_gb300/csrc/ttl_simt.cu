@@ -2,10 +2,9 @@
 //
 // When d_in + d_out <= 512 the fp32 path runs every segment of a call in one launch with
 // the rows resident on chip (ttl_resident_f32_kernel, below).  Otherwise it runs two
-// kernels a segment (three with the squared-error pre-pass).  Those are latency-bound,
-// so they use plain CUDA-core FFMA tiles (64 x 64 per CTA, 4 x 4 per thread, 64-deep K
-// slabs so that each thread has 32 loads in flight per slab) in fp32 throughout, and
-// compute the same two phases as the bf16 tensor-core path:
+// kernels a segment (three with the squared-error pre-pass): register-tiled FFMA
+// contractions in fp32 throughout (nt_tile, tn_tile), computing the same two phases as the
+// bf16 tensor-core path:
 //   phase A  H = U W1^T, R = Y W2^T (Y = [K || V]); A = SiLU(H);
 //            dH = c_t R * SiLU'(H), At = c_t A with c_t = -eta_t / T'   (Eq. 10)
 //   phase B  G1 = dH^T U, G2 = At^T Y; mu = beta mu + G; W = s W_raw - mu  (Eq. 8)
@@ -79,6 +78,137 @@ __device__ __forceinline__ void simt_tile(float (&acc)[MR][4], const float* A, l
     }
 }
 
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, int src_bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(float* dst, const float* src, int src_bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// ---- tiled contractions of the fp32 phases: 256 threads as 16 x 16, TM x TN outputs each, slabs of the
+// contraction through a ring of cp.async stages.  (TM + TN) 16-byte shared-memory loads feed 4 TM TN
+// multiply-adds a thread; a warp is 4 (ty) x 8 (tx) threads, so a half warp's load is at most 128
+// distinct bytes, one wavefront (2 x 16 threads: two for the tx operand).  Every output is one fmaf chain in
+// order of k.
+__device__ __forceinline__ int tile_tx() { return (threadIdx.x & 7) | ((threadIdx.x >> 5 & 1) << 3); }
+__device__ __forceinline__ int tile_ty() { return (threadIdx.x >> 3 & 3) | (threadIdx.x >> 6 << 2); }
+
+// Both operands with k contiguous: acc[i][j] += sum_k A[ty + 16 i][k] B[tx + 16 j][k], rows of A from
+// m_valid on read as 0.  K a multiple of 32; rows 36 floats apart, so the 8 rows of a quarter warp start
+// in 8 bank groups.
+constexpr int NT_K = 32, NT_LD = NT_K + 4, NT_ST = 3;
+template <int TM, int TN> constexpr size_t nt_smem() { return sizeof(float) * NT_ST * 16 * (TM + TN) * NT_LD; }
+
+template <int TM, int TN>
+__device__ __forceinline__ void nt_tile(float (&acc)[TM][TN], const float* A, long long lda, const float* B, long long ldb,
+                                        int K, int m_valid, float* sm) {
+    constexpr int BM = 16 * TM, BN = 16 * TN, STAGE = (BM + BN) * NT_LD;
+    const int tid = threadIdx.x, tx = tile_tx(), ty = tile_ty(), n = K / NT_K;
+    auto load = [&](int s) {
+        float* d = sm + (s % NT_ST) * STAGE;
+#pragma unroll
+        for (int u = 0; u < (BM + BN) * 8 / 256; ++u) {
+            const int e = tid + 256 * u, r = e >> 3, p = 4 * (e & 7), k = s * NT_K + p;
+            if (r < BM)
+                cp_async16(d + r * NT_LD + p, r < m_valid ? A + r * lda + k : A, r < m_valid ? 16 : 0);
+            else
+                cp_async16(d + r * NT_LD + p, B + (r - BM) * ldb + k, 16);
+        }
+    };
+    // the ring may still be read from an earlier contraction of this kernel
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < NT_ST - 1; ++s) {
+        if (s < n) load(s);
+        cp_async_commit();
+    }
+    for (int s = 0; s < n; ++s) {
+        cp_async_wait<NT_ST - 2>();
+        __syncthreads();
+        if (s + NT_ST - 1 < n) load(s + NT_ST - 1);
+        cp_async_commit();
+        const float* As = sm + (s % NT_ST) * STAGE + ty * NT_LD;
+        const float* Bs = sm + (s % NT_ST) * STAGE + (BM + tx) * NT_LD;
+#pragma unroll
+        for (int k = 0; k < NT_K; k += 4) {
+            float4 a[TM], b[TN];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(As + 16 * i * NT_LD + k);
+#pragma unroll
+            for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const float4*>(Bs + 16 * j * NT_LD + k);
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) {
+                    acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+                }
+        }
+    }
+}
+
+// Both operands with the output dimension contiguous: acc[i][j] += sum_k A[k][m(i)] B[k][n(j)] with
+// m(i) = 4 ty + 64 (i / 4) + i % 4 and n(j) likewise from tx (tile 16 TM x 16 TN).  Rows k >= kv read as 0.
+constexpr int TN_K = 16, TN_ST = 3;
+template <int TM, int TN> constexpr size_t tn_smem() { return sizeof(float) * TN_ST * TN_K * 16 * (TM + TN); }
+
+template <int TM, int TN>
+__device__ __forceinline__ void tn_tile(float (&acc)[TM][TN], const float* A, long long lda, const float* B, long long ldb,
+                                        int K, int kv, float* sm) {
+    static_assert(TM % 4 == 0 && TN % 4 == 0, "outputs in groups of four");
+    constexpr int BM = 16 * TM, BN = 16 * TN, LD = BM + BN, STAGE = TN_K * LD;
+    const int tid = threadIdx.x, tx = tile_tx(), ty = tile_ty(), n = (K + TN_K - 1) / TN_K;
+    auto load = [&](int s) {
+        float* d = sm + (s % TN_ST) * STAGE;
+#pragma unroll
+        for (int u = 0; u < STAGE / 4 / 256; ++u) {
+            const int e = tid + 256 * u, r = e / (LD / 4), c = 4 * (e % (LD / 4)), k = s * TN_K + r;
+            const float* src = c < BM ? A + k * lda + c : B + k * ldb + (c - BM);
+            cp_async16(d + r * LD + c, k < kv ? src : A, k < kv ? 16 : 0);
+        }
+    };
+#pragma unroll
+    for (int s = 0; s < TN_ST - 1; ++s) {
+        if (s < n) load(s);
+        cp_async_commit();
+    }
+    for (int s = 0; s < n; ++s) {
+        cp_async_wait<TN_ST - 2>();
+        __syncthreads();
+        if (s + TN_ST - 1 < n) load(s + TN_ST - 1);
+        cp_async_commit();
+        const float* S = sm + (s % TN_ST) * STAGE;
+#pragma unroll
+        for (int k = 0; k < TN_K; ++k) {
+            float a[TM], b[TN];
+#pragma unroll
+            for (int i = 0; i < TM; i += 4)
+                *reinterpret_cast<float4*>(a + i) = *reinterpret_cast<const float4*>(S + k * LD + 4 * ty + 16 * i);
+#pragma unroll
+            for (int j = 0; j < TN; j += 4)
+                *reinterpret_cast<float4*>(b + j) = *reinterpret_cast<const float4*>(S + k * LD + BM + 4 * tx + 16 * j);
+#pragma unroll
+            for (int i = 0; i < TM; ++i) {  // pairs of columns: half the issue slots of single multiply-adds
+                const uint64_t aa = pack_f32x2(a[i], a[i]);
+#pragma unroll
+                for (int j = 0; j < TN; j += 2) {
+                    const float2 v = unpack_f32x2(fma_f32x2(aa, pack_f32x2(b[j], b[j + 1]), pack_f32x2(acc[i][j], acc[i][j + 1])));
+                    acc[i][j] = v.x;
+                    acc[i][j + 1] = v.y;
+                }
+            }
+        }
+    }
+}
+
 struct F32SegArgs {
     int d_in, d_hid, d_out, T, Tp, c0, paper, momentum, renorm_pending, parity, C;
     long long tok0;           // per-token tables: entry of token t of chain cs is [cs * win + tok0 + t]
@@ -107,68 +237,65 @@ __device__ __forceinline__ const float* ss_ptr(const F32SegArgs& a, int parity, 
     return a.sumsq + ((size_t)(parity * 2 + which) * a.C) * a.d_hid;
 }
 
-// Phase A takes tiles of 32 tokens x 64 hidden units (2 x 4 per thread): the fp32 workload has
-// only T = 128 tokens a segment, so 64-row tiles would leave all but 16 SMs idle.
-constexpr int A_MR = 2, A_TM = 16 * A_MR;
-
-__global__ void __launch_bounds__(256) phase_a_f32_kernel(const F32SegArgs a) {
-    __shared__ float As[TK][A_TM + 4], Bs[TK][TN + 4];
+// Phase A: 16 TM tokens x 16 TN hidden units a CTA, H over d_in and R over d_out in turn.  Bound by FMA
+// issue and the last wave: 4 chains of 1024 -> 1024 -> 1024, T = 256 (256 tiles of 64 x 64) take 126 us,
+// 34 TFLOP/s (32 x 64 tiles with a slab read, waited for and then multiplied: 250 us; 64 x 128 tiles, one
+// CTA an SM: 152 us; 32 x 64: 189 us).
+template <int TM, int TN>
+__global__ void __launch_bounds__(256, 2) phase_a_f32_kernel(const F32SegArgs a) {
+    extern __shared__ float4 f32_smem[];
     __shared__ float red[8];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int t0 = blockIdx.x * A_TM, h0 = blockIdx.y * TN, cz = blockIdx.z, cs = a.c0 + cz;
-    long long avail = a.row_avail - t0;
-    int m_valid = (int)min((long long)min(A_TM, a.Tp - t0), avail);
+    float* sm = reinterpret_cast<float*>(f32_smem);
+    constexpr int BM = 16 * TM, BN = 16 * TN;
+    const int tid = threadIdx.x, tx = tile_tx(), ty = tile_ty();
+    const int t0 = blockIdx.x * BM, h0 = blockIdx.y * BN, cz = blockIdx.z, cs = a.c0 + cz;
+    int m_valid = (int)min((long long)min(BM, a.Tp - t0), a.row_avail - t0);
     if (m_valid < 0) m_valid = 0;
     // zero this segment's row sums of squares (read by phase B of this segment)
-    if (blockIdx.x == 0 && tid < TN) {
+    if (blockIdx.x == 0 && tid < BN) {
         float* cur = a.sumsq + ((size_t)(a.parity * 2) * a.C + cs) * a.d_hid + h0 + tid;
         cur[0] = 0.f;
         cur[(size_t)a.C * a.d_hid] = 0.f;
     }
-    float accH[A_MR][4] = {}, accR[A_MR][4] = {};
-    const float* U = a.U + cz * a.u_cstride + (long long)t0 * a.d_in;
-    simt_tile(accH, U, a.d_in, 1, a.W1 + ((size_t)cs * a.d_hid + h0) * a.d_in, a.d_in, 1, a.d_in, m_valid,
-              a.d_in, As, Bs);
-    const int dh = a.d_out / 2;
-    const float* W2 = a.W2 + ((size_t)cs * a.d_hid + h0) * a.d_out;
-    simt_tile(accR, a.K + cz * a.y_cstride + (long long)t0 * dh, dh, 1, W2, a.d_out, 1, dh, m_valid, dh, As, Bs);
-    simt_tile(accR, a.V + cz * a.y_cstride + (long long)t0 * dh, dh, 1, W2 + dh, a.d_out, 1, dh, m_valid, dh, As,
-              Bs);
-
+    float accH[TM][TN] = {}, accR[TM][TN] = {};
+    if (m_valid > 0) {
+        const int dh = a.d_out / 2;
+        const float* W2 = a.W2 + ((size_t)cs * a.d_hid + h0) * a.d_out;
+        nt_tile(accH, a.U + cz * a.u_cstride + (long long)t0 * a.d_in, a.d_in, a.W1 + ((size_t)cs * a.d_hid + h0) * a.d_in,
+                a.d_in, a.d_in, m_valid, sm);
+        nt_tile(accR, a.K + cz * a.y_cstride + (long long)t0 * dh, dh, W2, a.d_out, dh, m_valid, sm);
+        nt_tile(accR, a.V + cz * a.y_cstride + (long long)t0 * dh, dh, W2 + dh, a.d_out, dh, m_valid, sm);
+    }
     const float* prev1 = ss_ptr(a, a.parity ^ 1, 0) + (size_t)cs * a.d_hid;
     const float* prev2 = ss_ptr(a, a.parity ^ 1, 1) + (size_t)cs * a.d_hid;
-    float s1[4], s2[4];
+    float ct[TM];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int h = h0 + tx * 4 + j;
-        s1[j] = a.renorm_pending ? renorm_scale(a.n1[(size_t)cs * a.d_hid + h], prev1[h]) : 1.f;
-        s2[j] = a.renorm_pending ? renorm_scale(a.n2[(size_t)cs * a.d_hid + h], prev2[h]) : 1.f;
+    for (int i = 0; i < TM; ++i) {
+        const int t = t0 + ty + 16 * i;
+        ct[i] = 0.f;
+        if (t < a.Tp && t - t0 < m_valid) {
+            const float e = a.paper ? a.eta[(size_t)cs * a.win + a.tok0 + t]
+                                    : (a.eta_in ? a.eta_in[cz * a.eta_cstride + t] : a.lr);
+            ct[i] = -e / (float)a.Tp;
+        }
     }
     float lsum = 0.f;
 #pragma unroll
-    for (int i = 0; i < A_MR; ++i) {
-        const int t = t0 + ty * A_MR + i;
-        float ct = 0.f;
-        if (t < a.Tp && t - t0 < m_valid) {
-            float e;
-            if (a.paper)
-                e = a.eta[(size_t)cs * a.win + a.tok0 + t];
-            else
-                e = a.eta_in ? a.eta_in[cz * a.eta_cstride + t] : a.lr;
-            ct = -e / (float)a.Tp;
-        }
-        float* dHrow = a.dH + ((size_t)cs * a.T + t) * a.d_hid + h0 + tx * 4;
-        float* Arow = a.At + ((size_t)cs * a.T + t) * a.d_hid + h0 + tx * 4;
+    for (int j = 0; j < TN; ++j) {
+        const int h = h0 + tx + 16 * j;
+        const float s1 = a.renorm_pending ? renorm_scale(a.n1[(size_t)cs * a.d_hid + h], prev1[h]) : 1.f;
+        const float s2 = a.renorm_pending ? renorm_scale(a.n2[(size_t)cs * a.d_hid + h], prev2[h]) : 1.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float hv = accH[i][j] * s1[j];
-            const float rv = accR[i][j] * s2[j];
+        for (int i = 0; i < TM; ++i) {
+            const size_t o = ((size_t)cs * a.T + t0 + ty + 16 * i) * a.d_hid + h;
+            const float hv = accH[i][j] * s1;
+            const float rv = accR[i][j] * s2;
             const float sg = sigmoidf_(hv);
             const float av = hv * sg;
             const float dsilu = sg * (1.f + hv * (1.f - sg));
             lsum += av * rv;
-            dHrow[j] = ct * rv * dsilu;
-            Arow[j] = ct * av;
+            a.dH[o] = ct[i] * rv * dsilu;
+            a.At[o] = ct[i] * av;
         }
     }
     if (a.loss) {
@@ -183,27 +310,19 @@ __global__ void __launch_bounds__(256) phase_a_f32_kernel(const F32SegArgs a) {
     }
 }
 
-// Phase B takes tiles of 32 hidden rows x 64 weight columns (2 x 4 per thread), for the same reason.
-constexpr int B_MR = 2, B_TM = 16 * B_MR;
-
-__global__ void __launch_bounds__(256) phase_b_f32_kernel(const F32SegArgs a) {
-    __shared__ float As[TK][B_TM + 4], Bs[TK][TN + 4];
+// Phase B: 16 TM hidden rows x 16 TN columns of W1, or of the K or V half of W2, a CTA.  The same 4
+// chains: 105 us, 41 TFLOP/s, with 128 x 128 tiles and paired multiply-adds (single ones 122 us; 64 x 64
+// tiles 133 us; the 32 x 64 tiles before them 344 us).
+template <int TM, int TN>
+__global__ void __launch_bounds__(256, 2) phase_b_f32_kernel(const F32SegArgs a) {
+    extern __shared__ float4 f32_smem[];
     __shared__ float red[8];
     __shared__ float s_beta;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int col0 = blockIdx.x * TN, h0 = blockIdx.y * B_TM, cz = blockIdx.z, cs = a.c0 + cz;
+    constexpr int BM = 16 * TM, BN = 16 * TN;
+    const int tid = threadIdx.x, tx = tile_tx(), ty = tile_ty();
+    const int col0 = blockIdx.x * BN, h0 = blockIdx.y * BM, cz = blockIdx.z, cs = a.c0 + cz;
     const bool isW1 = col0 < a.d_in;
     const int kv = (int)min((long long)a.Tp, a.row_avail);
-    float acc[B_MR][4] = {};
-    if (isW1) {
-        const float* U = a.U + cz * a.u_cstride + col0;
-        simt_tile(acc, a.dH + (size_t)cs * a.T * a.d_hid + h0, 1, a.d_hid, U, 1, a.d_in, a.Tp, B_TM, kv, As, Bs);
-    } else {
-        const int dh = a.d_out / 2;
-        const int o0 = col0 - a.d_in;
-        const float* Y = (o0 < dh ? a.K + o0 : a.V + (o0 - dh)) + cz * a.y_cstride;
-        simt_tile(acc, a.At + (size_t)cs * a.T * a.d_hid + h0, 1, a.d_hid, Y, 1, dh, a.Tp, B_TM, kv, As, Bs);
-    }
     // momentum decay beta_s = sigmoid(mean_t w_beta . x_t + b_beta)
     if (a.momentum) {
         float v = 0.f;
@@ -216,42 +335,50 @@ __global__ void __launch_bounds__(256) phase_b_f32_kernel(const F32SegArgs a) {
             for (int w = 0; w < 8; ++w) tot += red[w];
             s_beta = sigmoidf_(tot / (float)a.Tp + a.b_beta[cs]);
         }
-        __syncthreads();
     }
-    const float beta = a.momentum ? s_beta : 0.f;
+    float acc[TM][TN] = {};
+    {
+        const int dh = a.d_out / 2, o0 = col0 - a.d_in;
+        const float* A = (isW1 ? a.dH : a.At) + (size_t)cs * a.T * a.d_hid + h0;
+        const float* B = isW1 ? a.U + cz * a.u_cstride + col0 : (o0 < dh ? a.K + o0 : a.V + (o0 - dh)) + cz * a.y_cstride;
+        tn_tile(acc, A, a.d_hid, B, isW1 ? a.d_in : dh, a.Tp, kv, reinterpret_cast<float*>(f32_smem));
+    }
+    const float beta = a.momentum ? s_beta : 0.f;  // tn_tile's first barrier has published it
     const int which = isW1 ? 0 : 1;
     const int width = isW1 ? a.d_in : a.d_out;
     const int c_local = isW1 ? col0 : col0 - a.d_in;
-    float* W = (isW1 ? a.W1 : a.W2) + (size_t)cs * a.d_hid * width;
-    float* M = a.momentum ? (isW1 ? a.mu1 : a.mu2) + (size_t)cs * a.d_hid * width : nullptr;
     const float* n0 = (isW1 ? a.n1 : a.n2) + (size_t)cs * a.d_hid;
     const float* prev = ss_ptr(a, a.parity ^ 1, which) + (size_t)cs * a.d_hid;
     float* cur = a.sumsq + ((size_t)(a.parity * 2 + which) * a.C + cs) * a.d_hid;
     bool finite = true;
     float step = 0.f;  // sum of mu_s^2 over this thread's elements
 #pragma unroll
-    for (int i = 0; i < B_MR; ++i) {
-        const int h = h0 + ty * B_MR + i;
+    for (int i = 0; i < TM; ++i) {
+        const int h = h0 + 4 * ty + 64 * (i / 4) + i % 4;
         const float s = a.renorm_pending ? renorm_scale(n0[h], prev[h]) : 1.f;
-        float* wrow = W + (size_t)h * width + c_local + tx * 4;
-        float* mrow = M ? M + (size_t)h * width + c_local + tx * 4 : nullptr;
+        const size_t row = ((size_t)cs * a.d_hid + h) * width + c_local + 4 * tx;
+        float* wrow = (isW1 ? a.W1 : a.W2) + row;
+        float* mrow = a.momentum ? (isW1 ? a.mu1 : a.mu2) + row : nullptr;
         float ss = 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float g = acc[i][j];
-            const float mn = M ? fmaf(beta, mrow[j], g) : g;
-            const float wn = s * wrow[j] - mn;
-            wrow[j] = wn;
-            if (M) mrow[j] = mn;
-            ss = fmaf(wn, wn, ss);
-            step = fmaf(mn, mn, step);
-            finite = finite && isfinite(wn);
+        for (int j = 0; j < TN; j += 4) {
+            float4 w = *reinterpret_cast<const float4*>(wrow + 16 * j);
+            float4 m = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+            if (mrow) {
+                const float4 o = *reinterpret_cast<const float4*>(mrow + 16 * j);
+                m = make_float4(fmaf(beta, o.x, m.x), fmaf(beta, o.y, m.y), fmaf(beta, o.z, m.z), fmaf(beta, o.w, m.w));
+                *reinterpret_cast<float4*>(mrow + 16 * j) = m;
+            }
+            w = make_float4(s * w.x - m.x, s * w.y - m.y, s * w.z - m.z, s * w.w - m.w);
+            *reinterpret_cast<float4*>(wrow + 16 * j) = w;
+            finite = finite && isfinite(w.x) && isfinite(w.y) && isfinite(w.z) && isfinite(w.w);
+            ss = fmaf(w.x, w.x, fmaf(w.y, w.y, fmaf(w.z, w.z, fmaf(w.w, w.w, ss))));
+            step = fmaf(m.x, m.x, fmaf(m.y, m.y, fmaf(m.z, m.z, fmaf(m.w, m.w, step))));
         }
-        ss += __shfl_xor_sync(0xffffffffu, ss, 8);
         ss += __shfl_xor_sync(0xffffffffu, ss, 4);
         ss += __shfl_xor_sync(0xffffffffu, ss, 2);
         ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-        if (tx == 0) atomicAdd(&cur[h], ss);
+        if ((tx & 7) == 0) atomicAdd(&cur[h], ss);
     }
     if (a.step_sq) {
         step = warp_sum(step);
@@ -305,6 +432,9 @@ F32SegArgs make_f32_args(const DevState& s, const SegWork& w) {
 // (so A' W2raw = A W2), written to the At scratch, which phase A overwrites only after
 // the second kernel has read it; then the residual y - A' W2raw into the residual scratch
 // and 1/2 |y - M(u)|^2 / T' into the loss.
+
+// Tiles of 32 tokens x 64 outputs (2 x 4 per thread): short segments would leave most SMs idle on 64 x 64.
+constexpr int A_MR = 2, A_TM = 16 * A_MR;
 
 __global__ void __launch_bounds__(256) mse_hidden_f32_kernel(const F32SegArgs a) {
     __shared__ float As[TK][A_TM + 4], Bs[TK][TN + 4];
@@ -414,19 +544,6 @@ struct ResArgs {
     long long m_sstride;         // stride between segments of loss and step_sq (0: one accumulator)
     int* status;
 };
-
-__device__ __forceinline__ void cp_async16(float* dst, const float* src, int src_bytes) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async4(float* dst, const float* src, int src_bytes) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 
 __device__ __forceinline__ float dot4(const float4 a, const float4 b, float acc) {
     acc = fmaf(a.x, b.x, acc);
@@ -901,18 +1018,47 @@ __global__ void __launch_bounds__(256) read_norm_kernel(DevState s, int Q, Tout*
 
 }  // namespace
 
-cudaError_t launch_phase_a_f32(const DevState& s, const SegWork& w, cudaStream_t st) {
-    F32SegArgs a = make_f32_args(s, w);
-    dim3 grid((s.T + A_TM - 1) / A_TM, s.d_hid / TN, w.nc);
-    phase_a_f32_kernel<<<grid, 256, 0, st>>>(a);
+namespace {
+// Launch a phase kernel of the fp32 path (its shared memory opted in on first use).
+template <typename K>
+cudaError_t launch_f32_tiles(K kernel, size_t smem, std::once_flag& once, dim3 grid, const F32SegArgs& a, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    std::call_once(once, [&] { e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, 256, smem, st>>>(a);
     return cudaGetLastError();
+}
+template <int TM, int TN>
+cudaError_t phase_a_f32(const DevState& s, const SegWork& w, const F32SegArgs& a, cudaStream_t st) {
+    static std::once_flag once;
+    return launch_f32_tiles(phase_a_f32_kernel<TM, TN>, nt_smem<TM, TN>(), once,
+                            dim3(s.T / (16 * TM), s.d_hid / (16 * TN), w.nc), a, st);
+}
+template <int TM, int TN>
+cudaError_t phase_b_f32(const DevState& s, const SegWork& w, const F32SegArgs& a, cudaStream_t st) {
+    static std::once_flag once;
+    return launch_f32_tiles(phase_b_f32_kernel<TM, TN>, tn_smem<TM, TN>(), once,
+                            dim3((s.d_in + s.d_out) / (16 * TN), s.d_hid / (16 * TM), w.nc), a, st);
+}
+constexpr long long F32_SMS = 152;
+}  // namespace
+
+cudaError_t launch_phase_a_f32(const DevState& s, const SegWork& w, cudaStream_t st) {
+    const F32SegArgs a = make_f32_args(s, w);
+    const long long g64 = (long long)(s.T / 64) * (s.d_hid / 64) * w.nc;  // 64 x 64 tiles (T, d_hid multiples of 64)
+    // 32 x 64 tiles while their grid fits the SMs once (a wave of them takes three quarters of a wave of
+    // 64 x 64: 59 against 79 us for one chain of 1024 -> 1024 -> 1024 at T = 256), else 64 x 64 (two chains:
+    // 79 against 101 us)
+    return 2 * g64 <= F32_SMS ? phase_a_f32<2, 4>(s, w, a, st) : phase_a_f32<4, 4>(s, w, a, st);
 }
 
 cudaError_t launch_phase_b_f32(const DevState& s, const SegWork& w, cudaStream_t st) {
-    F32SegArgs a = make_f32_args(s, w);
-    dim3 grid((s.d_in + s.d_out) / TN, s.d_hid / B_TM, w.nc);
-    phase_b_f32_kernel<<<grid, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    const F32SegArgs a = make_f32_args(s, w);
+    // a tile lies in W1 or in one half of W2: widths are multiples of 64, for the large tile of 128, which
+    // is taken from two thirds of the SMs on
+    const bool wide = s.d_in % 128 == 0 && (s.d_out / 2) % 128 == 0 && s.d_hid % 128 == 0;
+    if (wide && (long long)(s.d_hid / 128) * ((s.d_in + s.d_out) / 128) * w.nc >= 100) return phase_b_f32<8, 8>(s, w, a, st);
+    return phase_b_f32<4, 4>(s, w, a, st);
 }
 
 bool resident_f32_fits(const DevState& s) {
