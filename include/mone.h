@@ -170,10 +170,11 @@ mone_status mone_ttl_context(mone_mem* m, const void* X, const void* K, const vo
  * host's page tables (Grace), any host memory.  The caller guarantees that each tensor's
  * whole range is allocated: the library checks its first and last bytes only.
  * The context is learned in chunks of chunk_tokens tokens (a multiple of seg_T; 0 lets
- * the library choose about 512 MB of X, K and V per chunk): the library gathers chunk
- * k+1 into one of two device windows (owned by the handle, grown on demand; growing
- * synchronises the stream) on its own staging stream while chunk k is learned on
- * `stream`, so the result equals mone_ttl_context on the same tokens.  Asynchronous:
+ * the library choose: about an eighth of the context, at least two segments and 32 MB of
+ * X, K and V, at most 512 MB): the library gathers chunk k+1 into one of two device windows
+ * (owned by the handle, grown on demand; growing synchronises the stream) on its own
+ * staging stream while chunk k is learned on `stream`, so the result equals
+ * mone_ttl_context on the same tokens.  Asynchronous:
  * the host buffers must stay valid and unchanged until `stream` has passed the call
  * (mone_mem_sync or a stream synchronisation).  Kernel kind 8 times the gathers.
  * Errors: INVALID_ARG (null or unaligned pointer, device or managed memory, a range
