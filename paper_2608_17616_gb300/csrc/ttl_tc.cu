@@ -1114,7 +1114,7 @@ TcArgs make_args(const DevState& s, const SegWork& w) {
 // ------------------------------------------------------------------ memory read (Eq. 4)
 //
 // The read of generate_kv on the bf16 path, on the tensor cores, in two kernels:
-//   hidden:  A_q = SiLU(U_q W1^T)    tile = (128 queries, 128 hidden units, chain), K = d_in
+//   hidden:  A_q = SiLU(Z_q W1^T / |z_q|)  tile = (128 queries, 128 hidden units, chain), K = d_in
 //   out:     O = A_q W2, then per output head h of width hd: g_h o_h / sqrt(mean(o_h^2) + eps)
 //            written into the caller's K / V layout   tile = (128 queries, 128 outputs, chain), K = d_hid
 // One tile per CTA: warp 0 streams the query rows and the bf16 weight copy with TMA,
@@ -1173,12 +1173,12 @@ struct ReadArgs {
     float lr;
     const float *eta, *eta_in;
     long long eta_cstride;
-    const float* qzinv;    // read with the weights as M: 1/|z| per query [C][Q] (paper mode), or null
+    const float* qzinv;    // read: 1/|z| per query [C][Q] (paper mode), or null
 };
 
 enum { READ_HIDDEN = 0, MSE_HIDDEN = 1, MSE_OUT = 2 };  // other MODEs: read out with heads of width MODE
 
-// MODE READ_HIDDEN: A_q = SiLU(U_q W1^T).  MODE 64 / 128: the read's out kernel with heads
+// MODE READ_HIDDEN: A_q = SiLU(Z_q W1^T / |z_q|).  MODE 64 / 128: the read's out kernel with heads
 // of that width.  MODE MSE_HIDDEN: A' = SiLU(s1 (1/|z_t|) H) s2, the segment's activations
 // with the pending renorm scales (s2 folded in, so A' W2raw = A W2).  MODE MSE_OUT: the
 // residual target y_t - M(u_t) = y_t - A'_t W2raw (and the segment's squared-error loss).
@@ -1355,10 +1355,13 @@ tc_read_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 bf16* row0 = a.Aq + ((size_t)c * a.Q + qw) * a.d_hid + n0;
                 // the tile's columns of A_q lie inside [Q][d_hid] (index check of MONE_DEBUG builds)
                 const bool wr = MONE_DCHECK(n0 + 128 <= a.d_hid, a.status, DS_READ_TILE);
+                const float zi = a.qzinv && qw + lane < a.Q ? a.qzinv[(size_t)c * a.Q + qw + lane] : 1.f;
 #pragma unroll 1
                 for (int cc = 0; cc < 4; ++cc) {
                     float hv[32];
                     tmem_ld32(lane_base + cc * 32, hv);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) hv[j] *= zi;
                     uint32_t pk[16];
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
@@ -1862,13 +1865,8 @@ cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, v
     cudaError_t e = ensure_attrs();
     if (e != cudaSuccess) return e;
     if (s.hd != 64 && s.hd != 128) return cudaErrorInvalidValue;
-    // the query side: unnormalised z and 1/|z| for the read with the weights as M (Q <= 256),
-    // the normalised u for the 128-query form
-    if (Q <= RT_MAX_NT)
-        e = launch_query_z(s, Xq, Q, Uq, zq, st);
-    else
-        e = launch_query_transform(s, Xq, Q, Uq, true, st);
-    if (e != cudaSuccess) return e;
+    // the query side: unnormalised z and 1/|z|, which the hidden kernel applies
+    if ((e = launch_query_z(s, Xq, Q, Uq, zq, st)) != cudaSuccess) return e;
     CUtensorMap mu, ma;
     if (!encode_map_bf16_3d(&mu, Uq, s.d_in, Q, s.C, 64, 128) || !encode_map_bf16_3d(&ma, Aq, s.d_hid, Q, s.C, 64, 128))
         return cudaErrorInvalidValue;
@@ -1881,8 +1879,8 @@ cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, v
     a.Vout = static_cast<bf16*>(V_out);
     a.s0 = strides[0]; a.s1 = strides[1]; a.s2 = strides[2]; a.s3 = strides[3];
     a.status = s.status;
+    a.qzinv = s.mode == 1 ? zq : nullptr;
     if (Q <= RT_MAX_NT) {  // weights as the 128-row operand, the queries as N
-        a.qzinv = s.mode == 1 ? zq : nullptr;
         const int NT = (Q + 31) / 32 * 32;
         CUtensorMap tu, ta;
         if (!encode_map_bf16_3d(&tu, Uq, s.d_in, Q, s.C, 64, NT) || !encode_map_bf16_3d(&ta, Aq, s.d_hid, Q, s.C, 64, NT))
