@@ -211,11 +211,11 @@ swiglu_a_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(c.base + s * (48 * 1024)), sb = sa + 128 * 128;
+                    const uint64_t da = sdesc_sw128(smem_u32(c.base + s * (48 * 1024)), 16), db = sdesc_step(da, 128 * 128);
                     const bool u_part = kb < KU;
     #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        umma_bf16(u_part ? tmem : tmem + 256, sdesc_sw128(sa + k * 32, 16), sdesc_sw128(sb + k * 32, 16),
+                        umma_bf16(u_part ? tmem : tmem + 256, sdesc_step(da, k * 32), sdesc_step(db, k * 32),
                                   u_part ? id_pg : id_r, ((kb == 0 || kb == KU) && k == 0) ? 0u : 1u);
                     umma_commit(c.empty(s));
                 }
@@ -476,11 +476,11 @@ swiglu_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constant_
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(base + s * SWB_STAGE), sb = sa + 2 * SW_BOX;
+                    const uint64_t da = sdesc_sw128(smem_u32(base + s * SWB_STAGE), SW_BOX), db = sdesc_step(da, 2 * SW_BOX);
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        umma_bf16(d, sdesc_sw128(sa + k * 16 * 128, SW_BOX), sdesc_sw128(sb + k * 16 * 128, SW_BOX),
-                                  idesc, (kb == 0 && k == 0) ? 0u : 1u);
+                        umma_bf16(d, sdesc_step(da, k * 16 * 128), sdesc_step(db, k * 16 * 128), idesc,
+                                  (kb == 0 && k == 0) ? 0u : 1u);
                     umma_commit(empty(s));
                 }
                 if (ok) umma_commit(tfull(b));

@@ -468,12 +468,13 @@ tc_phase_a_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(c.base + s * A_STAGE), sb = sa + A_BM * BK * 2;
+                    const uint32_t sa = smem_u32(c.base + s * A_STAGE);
+                    const uint64_t da = sdesc_sw128(sa, 16), db = sdesc_step(da, A_BM * BK * 2);
                     const bool first = (kb == 0 || kb == KB1);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
-                        umma_bf16(kb < KB1 ? dH : dR, sdesc_sw128(sa + k * 32, 16), sdesc_sw128(sb + k * 32, 16),
-                                  idesc, (first && k == 0) ? 0u : 1u);
+                        umma_bf16(kb < KB1 ? dH : dR, sdesc_step(da, k * 32), sdesc_step(db, k * 32), idesc,
+                                  (first && k == 0) ? 0u : 1u);
                     umma_commit(c.empty(s, A_STAGES));
                 }
                 umma_commit(c.tfull(b, A_STAGES));
@@ -633,12 +634,13 @@ tc_phase_a_pair_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_con
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(c.base + s * P_STAGE), sb = sa + P_A;
+                    const uint32_t sa = smem_u32(c.base + s * P_STAGE);
+                    const uint64_t da = sdesc_sw128(sa, 16), db = sdesc_step(da, P_A);
                     const bool first = (kb == 0 || kb == KB1);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
-                        umma_bf16_pair(kb < KB1 ? dH : dR, sdesc_sw128(sa + k * 32, 16),
-                                       sdesc_sw128(sb + k * 32, 16), idesc, (first && k == 0) ? 0u : 1u);
+                        umma_bf16_pair(kb < KB1 ? dH : dR, sdesc_step(da, k * 32), sdesc_step(db, k * 32), idesc,
+                                       (first && k == 0) ? 0u : 1u);
                     umma_commit_pair(c.empty(s, P_STAGES), 0x3);
                     if (kb == KB1 - 1) umma_commit_pair(c.tfull(1, P_STAGES), 0x3);  // H complete
                 }
@@ -895,10 +897,10 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(base + s * L::STAGE), sb = sa + L::A_BYTES;
+                    const uint64_t da0 = sdesc_sw128(smem_u32(base + s * L::STAGE), BOX), db0 = sdesc_step(da0, L::A_BYTES);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
-                        const uint64_t da = sdesc_sw128(sa + k * 16 * 128, BOX), db = sdesc_sw128(sb + k * 16 * 128, BOX);
+                        const uint64_t da = sdesc_step(da0, k * 16 * 128), db = sdesc_step(db0, k * 16 * 128);
                         if constexpr (PAIR)
                             umma_bf16_pair(d, da, db, idesc, (kb == 0 && k == 0) ? 0u : 1u);
                         else
@@ -1243,11 +1245,11 @@ tc_read_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     break;
                 }
                 tc_fence_after();
-                const uint32_t sa = smem_u32(base + s * R_STAGE), sb = sa + 128 * BK * 2;
+                const uint32_t sa = smem_u32(base + s * R_STAGE);
+                const uint64_t da = sdesc_sw128(sa, 16), db = sdesc_sw128(sa + 128 * BK * 2, OUT ? BOX : 16);
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
-                    umma_bf16(tmem, sdesc_sw128(sa + k * 32, 16),
-                              OUT ? sdesc_sw128(sb + k * 16 * 128, BOX) : sdesc_sw128(sb + k * 32, 16), idesc,
+                    umma_bf16(tmem, sdesc_step(da, k * 32), sdesc_step(db, OUT ? k * 16 * 128 : k * 32), idesc,
                               (kb == 0 && k == 0) ? 0u : 1u);
                 umma_commit(empty(s));
             }
@@ -1532,11 +1534,12 @@ tc_read_t_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     break;
                 }
                 tc_fence_after();
-                const uint32_t sa = smem_u32(base + s * STAGE), sb = sa + RT_A;
+                const uint32_t sa = smem_u32(base + s * STAGE);
+                const uint64_t da = sdesc_sw128(sa, OUT ? BOX : 16), db = sdesc_sw128(sa + RT_A, 16);
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
-                    umma_bf16(tmem, OUT ? sdesc_sw128(sa + k * 16 * 128, BOX) : sdesc_sw128(sa + k * 32, 16),
-                              sdesc_sw128(sb + k * 32, 16), idesc, (kb == 0 && k == 0) ? 0u : 1u);
+                    umma_bf16(tmem, sdesc_step(da, OUT ? k * 16 * 128 : k * 32), sdesc_step(db, k * 32), idesc,
+                              (kb == 0 && k == 0) ? 0u : 1u);
                 umma_commit(empty(s));
             }
             if (ok) umma_commit(tfull);
