@@ -300,6 +300,9 @@ mone_status build_state_maps(mone_mem* m) {
               encode_map_bf16_3d(&m->maps.W2m, s.W2b, s.d_out, s.d_hid, s.C, 64, 64) &&
               encode_map_bf16_blocks(&m->maps.dH, s.dHt, s.d_hid, s.T, s.C, 64, 2) &&
               encode_map_bf16_blocks(&m->maps.At, s.Att, s.d_hid, s.T, s.C, 64, 2);
+    for (int k = 1; k <= 2; ++k)
+        ok = ok && encode_map_bf16_blocks(&m->maps.W1r[k - 1], s.W1b, s.d_in, s.d_hid, s.C, 128, k) &&
+             encode_map_bf16_blocks(&m->maps.W2r[k - 1], s.W2b, s.d_out, s.d_hid, s.C, 64 * k, 2);
     if (ok && s.Amse) ok = encode_map_bf16_3d(&m->maps.Amse, s.Amse, s.d_hid, s.T, s.C, 64, 128);
     if (ok && s.U)
         ok = encode_map_bf16_3d(&m->maps.Ua, s.U, s.d_in, s.win_rows, s.C, 64, 128) &&

@@ -181,6 +181,7 @@ struct TcMaps {
     CUtensorMap Ua, Ub, Ub2;     // scratch U: K-major {64,128}; MN-major blocks of 256 columns, of 128 (CTA pairs)
     CUtensorMap W1s, W2s;            // fp32 state chunks of W and, with momentum, mu in one box
     CUtensorMap W2m;                 // bf16 W2 copy, MN-major boxes {64 outputs, 64 hidden} (memory read)
+    CUtensorMap W1r[2], W2r[2];      // read: bf16 weight tiles of one k-block and of two, in one box
     CUtensorMap Amse;                // squared-error activations, K-major {64, 128}
 };
 struct TcInputMaps {

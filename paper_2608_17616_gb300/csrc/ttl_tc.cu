@@ -1435,17 +1435,23 @@ tc_read_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 constexpr int RT_THREADS = 6 * 32;
 constexpr int RT_MAX_NT = 256;
 constexpr int RT_A = 128 * BK * 2;  // 16 KB: the weight tile of one k-block
-__host__ __device__ constexpr int rt_stage(int nt) { return RT_A + nt * BK * 2; }
 // Ring budget: 192 KB (one CTA per SM) when the grid fits in one wave; 96 KB (two CTAs per SM,
 // one's epilogue overlapping the other's loads) when it takes several.
 constexpr int RT_RING_1 = 192 * 1024, RT_RING_2 = 96 * 1024;
+// A stage holds two k-blocks, each operand's in one TMA box (d_in and d_hid are multiples of 128), where
+// three such stages fit the ring, else one.  A box costs the SM nearly the same at half the size, and
+// with one CTA an SM the boxes set its pace: 64 queries of 16 chains of 2048 -> 1024 -> 1024 went from
+// 41.3 to 38.8 us, of one chain from 36.2 to 30.8, of 4 chains of 3072 -> 2048 -> 2048 from 51.3 to 43.0 (200
+// queries, where two of the larger stages fit: 66.3 to 67.7).
+__host__ __device__ constexpr int rt_kblocks(int nt, int ring) { return ring / (2 * (RT_A + nt * BK * 2)) >= 3 ? 2 : 1; }
+__host__ __device__ constexpr int rt_stage(int nt, int ring) { return rt_kblocks(nt, ring) * (RT_A + nt * BK * 2); }
 __host__ __device__ constexpr int rt_stages(int nt, int ring = RT_RING_1) {
-    return ring / rt_stage(nt) < 8 ? ring / rt_stage(nt) : 8;
+    return ring / rt_stage(nt, ring) < 8 ? ring / rt_stage(nt, ring) : 8;
 }
 // shared memory after the ring: barriers, TMEM slot and flag, then the epilogue's buffers:
 // 4 warps x 2 KB transposes and the queries' 1/|z| (hidden), or 4 x NT column partial sums +
 // 2 x NT scales (out)
-__host__ __device__ constexpr int rt_bars(int nt, int ring = RT_RING_1) { return rt_stages(nt, ring) * rt_stage(nt); }
+__host__ __device__ constexpr int rt_bars(int nt, int ring = RT_RING_1) { return rt_stages(nt, ring) * rt_stage(nt, ring); }
 __host__ __device__ constexpr int rt_epi(int nt, int ring = RT_RING_1) { return rt_bars(nt, ring) + 256; }
 __host__ __device__ constexpr int rt_dyn(int nt, int ring = RT_RING_1) {
     return rt_epi(nt, ring) + (4 * 2048 + RT_MAX_NT * 4 > 6 * nt * 4 ? 4 * 2048 + RT_MAX_NT * 4 : 6 * nt * 4) + 1024;
@@ -1462,7 +1468,7 @@ tc_read_t_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     constexpr bool OUT = HD != 0;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const int NST = rt_stages(NT, ring), STAGE = rt_stage(NT);
+    const int NST = rt_stages(NT, ring), STAGE = rt_stage(NT, ring), KPS = rt_kblocks(NT, ring);
     const uint32_t bars = smem_u32(base + rt_bars(NT, ring));
     auto full = [&](int s) { return bars + 8 * s; };
     auto empty = [&](int s) { return bars + 8 * (8 + s); };
@@ -1495,31 +1501,29 @@ tc_read_t_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         if (lane == 0) {
             tma_prefetch_map(&tmW);
             tma_prefetch_map(&tmQ);
-            auto load_w = [&](int kb, uint32_t sa, uint32_t fb) {
-                if (OUT) {  // W2 rows kb*64.. as [64 hidden][64 outputs] boxes: the MN-major A operand
-                    tma_load_3d(sa, &tmW, fb, n0, kb * BK, a.b_chain0 + c);
-                    tma_load_3d(sa + BOX, &tmW, fb, n0 + 64, kb * BK, a.b_chain0 + c);
-                } else {
-                    tma_load_3d(sa, &tmW, fb, kb * BK, n0, a.b_chain0 + c);
-                }
+            // stage i: k-blocks KPS i ..; W1 as [k-block][128 rows], W2 (MN-major) as [64 outputs][KPS 64 hidden rows]
+            auto load_w = [&](int i, uint32_t sa, uint32_t fb) {
+                if (OUT)
+                    tma_load_4d(sa, &tmW, fb, 0, i * KPS * BK, n0 / 64, a.b_chain0 + c);
+                else
+                    tma_load_4d(sa, &tmW, fb, 0, n0, i * KPS, a.b_chain0 + c);
             };
             // the first stages' weight tiles, then the wait for the kernel that writes the queries
-            const int pre = KB < NST ? KB : NST;
-            for (int kb = 0; kb < pre; ++kb) {
-                const uint32_t sa = smem_u32(base + kb * STAGE), fb = full(kb);
-                mbar_expect_tx(fb, STAGE);
-                load_w(kb, sa, fb);
+            const int n = KB / KPS, pre = n < NST ? n : NST;
+            for (int i = 0; i < pre; ++i) {
+                mbar_expect_tx(full(i), STAGE);
+                load_w(i, smem_u32(base + i * STAGE), full(i));
             }
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            for (int kb = 0; kb < KB; ++kb) {
-                const int s = kb % NST;
-                const uint32_t sa = smem_u32(base + s * STAGE), sb = sa + RT_A, fb = full(s);
-                if (kb >= pre) {
-                    if (!mbar_wait(empty(s), ((kb / NST) - 1) & 1, a.status)) break;
+            for (int i = 0; i < n; ++i) {
+                const int s = i % NST;
+                const uint32_t sa = smem_u32(base + s * STAGE), fb = full(s);
+                if (i >= pre) {
+                    if (!mbar_wait(empty(s), ((i / NST) - 1) & 1, a.status)) break;
                     mbar_expect_tx(fb, STAGE);
-                    load_w(kb, sa, fb);
+                    load_w(i, sa, fb);
                 }
-                tma_load_3d(sb, &tmQ, fb, kb * BK, a.a_row0 + q0, a.a_chain0 + c);
+                tma_load_4d(sa + KPS * RT_A, &tmQ, fb, 0, a.a_row0 + q0, i * KPS, a.a_chain0 + c);
             }
         }
         __syncwarp();
@@ -1527,19 +1531,23 @@ tc_read_t_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16_f32(128, NT, OUT, false);
             bool ok = true;
-            for (int kb = 0; kb < KB; ++kb) {
-                const int s = kb % NST;
-                if (!mbar_wait(full(s), (kb / NST) & 1, a.status)) {
+            for (int i = 0; i < KB / KPS; ++i) {
+                const int s = i % NST;
+                if (!mbar_wait(full(s), (i / NST) & 1, a.status)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t sa = smem_u32(base + s * STAGE);
-                const uint64_t da = sdesc_sw128(sa, OUT ? BOX : 16), db = sdesc_sw128(sa + RT_A, 16);
+                const uint64_t da0 = sdesc_sw128(sa, OUT ? KPS * BOX : 16), db0 = sdesc_sw128(sa + KPS * RT_A, 16);
+                for (int kb = 0; kb < KPS; ++kb) {
+                    // the k-block's weights: 64 further rows of both output blocks (W2), or the next tile (W1)
+                    const uint64_t da = sdesc_step(da0, kb * (OUT ? BOX : RT_A)), db = sdesc_step(db0, kb * NT * BK * 2);
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    umma_bf16(tmem, sdesc_step(da, OUT ? k * 16 * 128 : k * 32), sdesc_step(db, k * 32), idesc,
-                              (kb == 0 && k == 0) ? 0u : 1u);
+                    for (int k = 0; k < BK / 16; ++k)
+                        umma_bf16(tmem, sdesc_step(da, OUT ? k * 16 * 128 : k * 32), sdesc_step(db, k * 32), idesc,
+                                  (i | kb | k) ? 1u : 0u);
+                }
                 umma_commit(empty(s));
             }
             if (ok) umma_commit(tfull);
@@ -1870,9 +1878,6 @@ cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, v
     if (s.hd != 64 && s.hd != 128) return cudaErrorInvalidValue;
     // the query side: unnormalised z and 1/|z|, which the hidden kernel applies
     if ((e = launch_query_z(s, Xq, Q, Uq, zq, st)) != cudaSuccess) return e;
-    CUtensorMap mu, ma;
-    if (!encode_map_bf16_3d(&mu, Uq, s.d_in, Q, s.C, 64, 128) || !encode_map_bf16_3d(&ma, Aq, s.d_hid, Q, s.C, 64, 128))
-        return cudaErrorInvalidValue;
     ReadArgs a{};
     a.Q = Q; a.d_in = s.d_in; a.d_hid = s.d_hid; a.d_out = s.d_out; a.n_kv = s.n_kv; a.L = n_layers;
     a.eps = s.rms_eps;
@@ -1885,8 +1890,12 @@ cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, v
     a.qzinv = s.mode == 1 ? zq : nullptr;
     if (Q <= RT_MAX_NT) {  // weights as the 128-row operand, the queries as N
         const int NT = (Q + 31) / 32 * 32;
+        // one CTA per SM with the deep ring when a kernel's tiles fit in one wave, else two
+        const int ring1 = (long long)(s.d_hid / 128) * s.C <= g_sms ? RT_RING_1 : RT_RING_2;
+        const int ring2 = (long long)(s.d_out / 128) * s.C <= g_sms ? RT_RING_1 : RT_RING_2;
+        const int k1 = rt_kblocks(NT, ring1), k2 = rt_kblocks(NT, ring2);
         CUtensorMap tu, ta;
-        if (!encode_map_bf16_3d(&tu, Uq, s.d_in, Q, s.C, 64, NT) || !encode_map_bf16_3d(&ta, Aq, s.d_hid, Q, s.C, 64, NT))
+        if (!encode_map_bf16_blocks(&tu, Uq, s.d_in, Q, s.C, NT, k1) || !encode_map_bf16_blocks(&ta, Aq, s.d_hid, Q, s.C, NT, k2))
             return cudaErrorInvalidValue;
         // programmatic stream serialisation: each kernel may start before the one it follows ends
         cudaLaunchConfig_t cfg = {};
@@ -1897,17 +1906,17 @@ cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, v
         cfg.stream = st;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        // one CTA per SM with the deep ring when a kernel's tiles fit in one wave, else two
-        const int ring1 = (long long)(s.d_hid / 128) * s.C <= g_sms ? RT_RING_1 : RT_RING_2;
-        const int ring2 = (long long)(s.d_out / 128) * s.C <= g_sms ? RT_RING_1 : RT_RING_2;
         cfg.gridDim = dim3(1, s.d_hid / 128, s.C);
         cfg.dynamicSmemBytes = rt_dyn(NT, ring1);
-        if ((e = cudaLaunchKernelEx(&cfg, tc_read_t_kernel<0>, m.W1b, tu, a, NT, ring1)) != cudaSuccess) return e;
+        if ((e = cudaLaunchKernelEx(&cfg, tc_read_t_kernel<0>, m.W1r[k1 - 1], tu, a, NT, ring1)) != cudaSuccess) return e;
         cfg.gridDim = dim3(1, s.d_out / 128, s.C);
         cfg.dynamicSmemBytes = rt_dyn(NT, ring2);
-        if (s.hd == 64) return cudaLaunchKernelEx(&cfg, tc_read_t_kernel<64>, m.W2m, ta, a, NT, ring2);
-        return cudaLaunchKernelEx(&cfg, tc_read_t_kernel<128>, m.W2m, ta, a, NT, ring2);
+        if (s.hd == 64) return cudaLaunchKernelEx(&cfg, tc_read_t_kernel<64>, m.W2r[k2 - 1], ta, a, NT, ring2);
+        return cudaLaunchKernelEx(&cfg, tc_read_t_kernel<128>, m.W2r[k2 - 1], ta, a, NT, ring2);
     }
+    CUtensorMap mu, ma;
+    if (!encode_map_bf16_3d(&mu, Uq, s.d_in, Q, s.C, 64, 128) || !encode_map_bf16_3d(&ma, Aq, s.d_hid, Q, s.C, 64, 128))
+        return cudaErrorInvalidValue;
     const int nq = (Q + 127) / 128;
     if ((e = launch_read_kernel<0>(dim3(nq, s.d_hid / 128, s.C), mu, m.W1b, a, st)) != cudaSuccess) return e;
     if (s.hd == 64) return launch_read_kernel<64>(dim3(nq, s.d_out / 128, s.C), ma, m.W2m, a, st);
