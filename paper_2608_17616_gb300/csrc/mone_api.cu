@@ -430,6 +430,7 @@ mone_status run_segment_loop(mone_mem* m, SegWork* gw, TcInputMaps* gin, TcInput
             x.parity = (int)(i & 1);
             x.renorm_pending = (s.renorm && i > 0) ? 1 : 0;
             x.u_off = u_off;
+            x.first = i == 0 && s.mode != MONE_PAPER;  // paper mode: the input transform comes first
             if (x.loss0) x.loss = x.loss0 + i * x.mstride;
             if (x.step0) x.step_sq = x.step0 + i * x.mstride;
             if (s.memory == MONE_MEM_SWIGLU) {
@@ -468,7 +469,7 @@ mone_status run_segment_loop(mone_mem* m, SegWork* gw, TcInputMaps* gin, TcInput
         if (s.memory == MONE_MEM_SWIGLU)
             MONE_TRY(timed(m, K_FINALIZE, st, 1, [&] { return launch_swiglu_rows(s, 1, par, w.c0, w.nc, st); }));
         else
-            MONE_TRY(timed(m, K_FINALIZE, st, 1, [&] { return launch_finalize(s, w.c0, w.nc, par, 1, st); }));
+            MONE_TRY(timed(m, K_FINALIZE, st, 1, [&] { return launch_finalize(s, w.c0, w.nc, par, 1, st, G == 1 && s.dtype == MONE_BF16); }));
     }
     return MONE_OK;
 }
@@ -485,6 +486,7 @@ mone_status run_segments(mone_mem* m, SegWork w, long long N, cudaStream_t st) {
         gw[g] = w;
         gw[g].c0 = w.c0 + off;
         gw[g].nc = n;
+        gw[g].single = G == 1;
         gw[g].X = static_cast<const uint8_t*>(w.X) + (size_t)off * w.x_cstride * el;
         gw[g].K = static_cast<const uint8_t*>(w.K) + (size_t)off * w.y_cstride * el;
         gw[g].V = static_cast<const uint8_t*>(w.V) + (size_t)off * w.y_cstride * el;
@@ -751,7 +753,10 @@ mone_status mone_ttl_segment(mone_mem* m, int ctx, int layer, const void* X, con
     w.eta_in = eta;
     w.eta_cstride = 0;
     w.loss = loss_out;
-    if (loss_out) MONE_CUDA(cudaMemsetAsync(loss_out, 0, sizeof(float), st));
+    if (s.mode == MONE_PAPER)
+        w.zero_loss = loss_out;  // by the input transform, the call's first kernel
+    else if (loss_out)
+        MONE_CUDA(cudaMemsetAsync(loss_out, 0, sizeof(float), st));
     return run_segments(m, w, n_tok, st);
 }
 

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 namespace mone {
 
 using bf16 = __nv_bfloat16;
@@ -90,9 +92,12 @@ struct SegWork {
     int renorm_pending;          // previous segment's renorm scale still to apply
     float* loss;                 // [C] loss accumulator of this segment or null
     float* step_sq;              // [C] squared norm of this segment's Eq. 8 step, or null
+    float* zero_loss;            // loss scalar that the input transform sets to 0 (one segment), or null
     // per-segment metrics of a whole call: segment i of chain c at [i * mstride + c], or null
     float *loss0, *step0;
     long long mstride;
+    int single;                  // the call runs on one stream: its kernels may chain by programmatic launch
+    int first;                   // ... and this segment's first kernel is the call's first
     int y_scratch;               // targets are the residual scratch (rows from 0), not the caller's K, V
 };
 
@@ -115,7 +120,8 @@ cudaError_t launch_mse_f32(const DevState& s, const SegWork& w, cudaStream_t st)
 // weights renormalised, so no finalize follows.  w: the call's chains, row0 / u_off of the window.
 bool resident_f32_fits(const DevState& s);
 cudaError_t launch_resident_f32(const DevState& s, const SegWork& w, long long n_tok, cudaStream_t st);
-cudaError_t launch_finalize(const DevState& s, int c0, int nc, int parity, int apply_scale, cudaStream_t st);
+cudaError_t launch_finalize(const DevState& s, int c0, int nc, int parity, int apply_scale, cudaStream_t st,
+                            bool pdl = false);
 cudaError_t launch_row_norms(const DevState& s, cudaStream_t st);
 // Output-channel renormalisation: every column of W2 of chains [c0, c0 + nc) rescaled to its norm
 // in W_0 (fp32 masters and, on the bf16 path, the operand copy).  Two kernels.
@@ -225,5 +231,30 @@ bool encode_map_bf16_4d(CUtensorMap* map, const void* base, const uint64_t dims[
 // 5-D bf16 map, 128-byte swizzle, as above.
 bool encode_map_bf16_5d(CUtensorMap* map, const void* base, const uint64_t dims[5], const uint64_t strides[4],
                         const uint32_t box[5]);
+
+// Launch a kernel; pdl: with programmatic stream serialisation (it may start before the kernel ahead
+// of it in the stream ends, and waits for it with griddepcontrol.wait); cluster: CTAs per cluster (x).
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, int cluster,
+                          A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    if (cluster > 1) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[cfg.numAttrs].val.clusterDim.x = cluster;
+        at[cfg.numAttrs].val.clusterDim.y = 1;
+        at[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
+    if (pdl) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 }  // namespace mone

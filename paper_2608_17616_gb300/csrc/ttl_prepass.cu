@@ -37,6 +37,7 @@ struct PrepassArgs {
     float* eta;           // [C][rows]
     float* dbeta;         // [C][rows]
     float* zinv;          // [C][rows] 1/|z_t|; when set, U receives the unnormalised z (one pass)
+    float* zero;          // scalar to set to 0 (a segment's loss accumulator), or null
 };
 
 // 16-byte vector of inputs: 8 bf16 or 4 fp32 values, kept packed in registers.
@@ -92,15 +93,15 @@ template <typename T> __device__ __forceinline__ float sig(float z);
 template <> __device__ __forceinline__ float sig<bf16>(float z) { return sigmoid_fast(z); }
 template <> __device__ __forceinline__ float sig<float>(float z) { return sigmoidf_(z); }
 
-constexpr int RPW = 2;                 // token rows per warp, processed together
-constexpr int PRE_ROWS = 8 * RPW;      // token rows per CTA
-
 // Each warp transforms RPW token rows at once with 16-byte vector loads, so every
 // load of the chain's meta-parameters (alpha, gamma, w_eta, w_beta) serves RPW
 // rows.  Statistics first; the output pass re-reads the rows (L1/L2 hits).
-template <typename Tin, typename Tout>
+template <typename Tin, typename Tout, int RPW>
 __global__ void __launch_bounds__(256) prepass_kernel(const PrepassArgs a) {
-    constexpr int V = Vec<Tin>::N;
+    constexpr int V = Vec<Tin>::N, PRE_ROWS = 8 * RPW;  // rows per CTA
+    pdl_wait();
+    pdl_trigger();
+    if (a.zero && (blockIdx.x | blockIdx.y | threadIdx.x) == 0) *a.zero = 0.f;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cz = blockIdx.y;
     const int cs = a.c0 + cz;
@@ -264,8 +265,12 @@ __global__ void __launch_bounds__(256) prepass_kernel(const PrepassArgs a) {
 
 template <typename Tin, typename Tout>
 cudaError_t launch_one(const PrepassArgs& a, int nchains, cudaStream_t st) {
-    dim3 grid((a.rows + PRE_ROWS - 1) / PRE_ROWS, nchains);
-    prepass_kernel<Tin, Tout><<<grid, 256, 0, st>>>(a);
+    // two rows a warp share the meta-parameter loads; few rows are spread one a warp instead (512 rows of
+    // one chain, d_in = 2048, caches cold: 11.1 -> 9.2 us)
+    if ((long long)((a.rows + 15) / 16) * nchains >= 2 * 152)
+        prepass_kernel<Tin, Tout, 2><<<dim3((a.rows + 15) / 16, nchains), 256, 0, st>>>(a);
+    else
+        prepass_kernel<Tin, Tout, 1><<<dim3((a.rows + 7) / 8, nchains), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -295,6 +300,7 @@ cudaError_t launch_prepass(const DevState& s, const SegWork& w, cudaStream_t st)
     a.U = s.U;
     a.eta = s.eta;
     a.dbeta = s.dbeta;
+    a.zero = w.zero_loss;
     a.zinv = s.dtype == 1 ? s.zinv : nullptr;  // bf16 path: unnormalised z + row scale
     return s.dtype == 0 ? launch_one<float, float>(a, w.nc, st) : launch_one<bf16, bf16>(a, w.nc, st);
 }

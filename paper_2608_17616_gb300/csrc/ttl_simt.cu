@@ -823,6 +823,8 @@ template <int RB> constexpr size_t res_smem_bytes(int D) {
 __global__ void __launch_bounds__(256) finalize_kernel(DevState s, int c0, int parity, int apply_scale) {
     const int h = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int cs = c0 + blockIdx.y, which = blockIdx.z;
+    pdl_wait();
+    pdl_trigger();
     if (h >= s.d_hid) return;
     const int width = which ? s.d_out : s.d_in;
     float* w = (which ? s.W2 : s.W1) + ((size_t)cs * s.d_hid + h) * width;
@@ -1123,9 +1125,8 @@ cudaError_t launch_mse_f32(const DevState& s, const SegWork& w, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(const DevState& s, int c0, int nc, int parity, int apply_scale, cudaStream_t st) {
-    finalize_kernel<<<dim3((s.d_hid + 7) / 8, nc, 2), 256, 0, st>>>(s, c0, parity, apply_scale);
-    return cudaGetLastError();
+cudaError_t launch_finalize(const DevState& s, int c0, int nc, int parity, int apply_scale, cudaStream_t st, bool pdl) {
+    return launch_kernel(finalize_kernel, dim3((s.d_hid + 7) / 8, nc, 2), 256, 0, st, pdl, 1, s, c0, parity, apply_scale);
 }
 
 cudaError_t launch_col_renorm(const DevState& s, int c0, int nc, cudaStream_t st) {
