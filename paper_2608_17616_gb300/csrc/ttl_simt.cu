@@ -13,6 +13,7 @@
 // The loss L_s = -(1/T') sum_t sum_h A_th R_th equals Eq. 7's segment mean
 // because sum_h A_th R_th = y_t . (A_t W2) = y_t . M(u_t).
 #include <mutex>
+#include <type_traits>
 
 #include "mone_common.cuh"
 
@@ -503,24 +504,28 @@ __global__ void __launch_bounds__(256) mse_out_f32_kernel(const F32SegArgs a, fl
 // When a chain's rows fit on chip, a whole call runs in one launch with the fast
 // weights resident.  A CTA owns RB hidden units of one chain: their rows of W1 and
 // W2, kept side by side as [W1 | W2] (width D = d_in + d_out) in shared memory, and
-// their momentum and gradient in registers.  Hidden units do not interact within a
+// their momentum too, with the gradient in registers.  Hidden units do not interact within a
 // step: H[:, r] = U W1[r]^T and R[:, r] = Y W2[r]^T use only row r, dL/dO does not
 // depend on W (Eq. 10), the gradient rows dW1[r] = dH[:, r]^T U and dW2[r] =
 // At[:, r]^T Y use only column r of dH and At, and Eq. 8's renormalisation is per
 // row.  So a CTA takes its rows through every segment of the call without waiting
 // for any other CTA, and the weights cross HBM once per call instead of once per
 // segment.  Each segment streams its rows [U | K | V] once, RC tokens at a time,
-// through a double-buffered cp.async stage: forward (H, R), the backward epilogue
+// into a double buffer (three bulk copies a chunk): forward (H, R), the backward epilogue
 // (dH, At), then the gradient accumulation from the same staged rows.  At the end
 // of the segment the update (momentum, W -= mu) and the row renormalisation are
 // applied in place.
 //
-// 512 threads (16 warps), so that shared-memory and FMA latencies are hidden.  Forward: half
-// of the CTA contracts U with the W1 rows (H), the other half Y with the W2 rows (R); an
-// output group is 2 tokens x 2 hidden units, its contraction split over KS = 32 / RB lanes
-// (float4 steps over interleaved columns) and summed by shuffles; one thread per (token,
-// hidden unit) then finishes the epilogue.  Backward: thread i owns column i of [W1 | W2]
-// for all RB rows.
+// 512 threads.  Forward: a warp takes two tokens of a chunk, lane l the columns 4 l + 128 i of [U | Y], with
+// the W values of these columns in registers (RB = 4; from shared memory for RB = 8) and even and odd columns
+// as packed pairs; the partial sums of H and R over the lanes are added by a transpose-reduction (16 shuffles
+// for 16 sums), and the same warp finishes the epilogue.  Backward: a thread takes two columns of [W1 | W2]
+// for all RB rows and one half of the chunk's tokens.  So a staged value is read from shared memory once in
+// each direction.  The two phases of a chunk, each a chain of shared-memory and shuffle latencies between
+// barriers with four warps a scheduler, bound it (49% of the issue slots used, 44% of the shared-memory rate).
+// 4096 tokens of 256 -> 512 -> 256, T = 128: 406 us with the rows staged by a 16-byte copy a thread and scalar
+// FFMA (16,500 warp instructions a chunk), 336 so (10,400).  Eight warps that take two tokens through both
+// directions with the gradient of all four rows in registers, added up once a segment: 364 us.
 constexpr int RES_RC = 32;                                             // tokens per streamed chunk
 __host__ __device__ constexpr int res_ld(int D) { return (D + 31) / 32 * 32 + 16; }  // row pitch, floats
 
@@ -568,43 +573,43 @@ __device__ __forceinline__ float block_sum_res(float v, float* red) {
 
 template <int RB>
 __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResArgs a) {
-    constexpr int RC = RES_RC, KS = 32 / RB, RH = RB / 2, NW = RES_NW;
+    constexpr int RC = RES_RC, NW = RES_NW, NV = 4 * RB;  // NV: sums of a warp's two tokens (H and R)
     static_assert(RB == 4 || RB == 8, "rows per CTA");
+    static_assert(RC == 2 * NW, "two tokens a warp");
     extern __shared__ float4 res_smem[];
     const int D = a.d_in + a.d_out, LD = res_ld(D), dh = a.d_out / 2;
     float* Ws = reinterpret_cast<float*>(res_smem);  // [RB][LD]
-    float* Xs = Ws + RB * LD;                        // [2][RC][LD]: rows [U | K | V] of a chunk
-    float* Gs = Xs + 2 * RC * LD;                    // [RC][2][RB]: c dH, c A of the chunk
-    float* HQ = Gs + RC * 2 * RB;                    // [2][RC][RB]: H and R of the chunk
-    float* red = HQ + 2 * RC * RB;                   // [NW][2 RB]
+    float* Ps = Ws + RB * LD;                        // [RB][LD]: gradient rows from the second token half
+    float* Ms = Ps + RB * LD;                        // [RB][LD]: momentum
+    float* Xs = Ms + RB * LD;                        // [2][RC][D]: a chunk's U [RC][d_in], K and V [RC][dh]
+    float* Gs = Xs + 2 * RC * D;                     // [RC][2][RB][2]: c dH, c A of the chunk, each twice (a packed pair)
+    float* red = Gs + RC * 4 * RB;                   // [NW][2 RB]
     float* scl = red + NW * 2 * RB;                  // [2 RB] row scales, then beta
     float* etaS = scl + 2 * RB + 4;                  // [2][RC] rates of the chunk's tokens
     float* dbS = etaS + 2 * RC;                      // [2][RC] w_beta . x of the chunk's tokens
     float* nS = dbS + 2 * RC;                        // [2 RB] renormalisation targets
+    __shared__ alignas(8) uint64_t bars[2];          // a chunk's rows have landed in buffer b
+    const uint32_t full = smem_u32(bars);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int h0 = blockIdx.x * RB, cz = blockIdx.y, cs = a.c0 + cz;
     const float* Uc = a.U + cz * a.u_cstride;
     const float* Kc = a.K + cz * a.y_cstride;
     const float* Vc = a.V + cz * a.y_cstride;
 
-    // stage RC token rows of segment seg, chunk ch into buffer b (a warp per row, lanes over
-    // columns), with the tokens' rates and w_beta . x terms; rows past the segment read as 0
+    // stage up to RC token rows of segment seg, chunk ch into buffer b: three copies of whole rows
+    // (thread 0 of the last warp), and the tokens' rates and w_beta . x terms.  Rows past the
+    // segment keep what the buffer held: their rate is 0 and no gradient sum reads them
     auto issue = [&](int seg, int ch, int b) {
         const long long t_seg = (long long)seg * a.T;
         const int Tp = (int)min((long long)a.T, a.n_tok - t_seg);
         const int nvalid = min(RC, Tp - ch * RC);
         const long long r0 = t_seg + ch * RC;
-        for (int t = warp; t < RC; t += NW) {
-            const bool v = t < nvalid;
-            const long long r = r0 + (v ? t : 0);
-            const float* ur = Uc + r * a.d_in;
-            const float* kr = Kc + r * dh;
-            const float* vr = Vc + r * dh;
-            float* dr = Xs + (b * RC + t) * LD;
-            for (int c = 4 * lane; c < D; c += 128) {
-                const float* src = c < a.d_in ? ur + c : c < a.d_in + dh ? kr + (c - a.d_in) : vr + (c - a.d_in - dh);
-                cp_async16(dr + c, src, v ? 16 : 0);
-            }
+        if (tid == RES_NT - 32) {
+            float* d = Xs + b * RC * D;
+            mbar_expect_tx(full + 8 * b, (uint32_t)(nvalid * D * 4));
+            bulk_load(smem_u32(d), Uc + r0 * a.d_in, (uint32_t)(nvalid * a.d_in * 4), full + 8 * b);
+            bulk_load(smem_u32(d + RC * a.d_in), Kc + r0 * dh, (uint32_t)(nvalid * dh * 4), full + 8 * b);
+            bulk_load(smem_u32(d + RC * (a.d_in + dh)), Vc + r0 * dh, (uint32_t)(nvalid * dh * 4), full + 8 * b);
         }
         if (tid < 2 * RC) {
             const int t = tid & (RC - 1);
@@ -624,138 +629,200 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
         }
     };
 
-    // resident rows, and the momentum of the thread's column (registers)
+    if (tid == 0) {
+        mbar_init(full, 1);
+        mbar_init(full + 8, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    issue(0, 0, 0);
+    cp_async_commit();
+    // resident rows
     for (int i = tid; i < RB * (D / 4); i += RES_NT) {
         const int r = i / (D / 4), c = 4 * (i - r * (D / 4));
         const size_t row = (size_t)cs * a.d_hid + h0 + r;
-        const float* src = c < a.d_in ? a.W1 + row * a.d_in + c : a.W2 + row * a.d_out + (c - a.d_in);
-        *reinterpret_cast<float4*>(Ws + r * LD + c) = *reinterpret_cast<const float4*>(src);
+        const size_t o = c < a.d_in ? row * a.d_in + c : row * a.d_out + (c - a.d_in);
+        *reinterpret_cast<float4*>(Ws + r * LD + c) = *reinterpret_cast<const float4*>((c < a.d_in ? a.W1 : a.W2) + o);
+        if (a.momentum) *reinterpret_cast<float4*>(Ms + r * LD + c) = *reinterpret_cast<const float4*>((c < a.d_in ? a.mu1 : a.mu2) + o);
     }
     if (tid < 2 * RB) nS[tid] = (tid < RB ? a.n1 : a.n2)[(size_t)cs * a.d_hid + h0 + tid % RB];
     const float b_beta = a.momentum ? a.b_beta[cs] : 0.f;
-    const int cb = tid;                          // owned column of [W1 | W2]
-    const bool own = cb < D;
-    const int kind = cb < a.d_in ? 0 : 1;
-    float mu[RB], acc[RB];
+    const int cb = 2 * (tid & 255), th = tid >> 8;  // backward: columns cb, cb + 1, tokens 16 th .. + 15 of a chunk
+    const bool own = cb < D;                        // widths are even: both columns or none
+    const int kind = cb < a.d_in ? 0 : 1;           // both in one matrix
+    // the columns' place in a staged chunk: offset of token 0, and the floats between tokens
+    auto x_col = [&](int c, int& stride) {
+        stride = c < a.d_in ? a.d_in : dh;
+        return c < a.d_in ? c : c < a.d_in + dh ? RC * a.d_in + (c - a.d_in) : RC * (a.d_in + dh) + (c - a.d_in - dh);
+    };
+    int bs;
+    int bo = x_col(cb, bs);
+    bo += th * (RC / 2) * bs;
+    uint64_t acc[RB];  // packed pairs
 #pragma unroll
-    for (int r = 0; r < RB; ++r) {
-        mu[r] = 0.f;
-        acc[r] = 0.f;
-        if (own && a.momentum) {
-            const size_t row = (size_t)cs * a.d_hid + h0 + r;
-            mu[r] = kind == 0 ? a.mu1[row * a.d_in + cb] : a.mu2[row * a.d_out + (cb - a.d_in)];
-        }
+    for (int r = 0; r < RB; ++r) acc[r] = 0;
+    __syncthreads();
+    // forward: the lane's weights, columns 4 lane + 128 i
+    constexpr int NI = 4;  // D <= 512
+    int fo[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        int stride;
+        fo[i] = x_col(4 * lane + 128 * i, stride);
+        fo[i] += 2 * warp * stride;
     }
+    ulonglong2 w[RB == 4 ? NI : 1][RB == 4 ? RB : 1];  // two packed pairs each
+    auto load_w = [&]() {
+        if constexpr (RB == 4) {
+#pragma unroll
+            for (int i = 0; i < NI; ++i)
+                if (4 * lane + 128 * i < D)
+#pragma unroll
+                    for (int r = 0; r < RB; ++r) w[i][r] = *reinterpret_cast<const ulonglong2*>(Ws + r * LD + 4 * lane + 128 * i);
+        }
+    };
+    load_w();
 
-    // forward mapping: half 0 contracts U with W1 (H), half 1 Y with W2 (R); within a half an
-    // output group og = (token pair tp, row pair rp) and a contraction lane ks
-    const int half = tid >> 8, ht = tid & 255;
-    const int ks = ht % KS, og = ht / KS, rp = og % RH, tp = og / RH;
-    const int c_lo = half ? a.d_in : 0, c_hi = half ? D : a.d_in;
     bool finite = true;
     int buf = 0;
-    issue(0, 0, 0);
-    cp_async_commit();
+    uint32_t phase = 0;  // a buffer is filled every second chunk
     for (int seg = 0; seg < a.n_seg; ++seg) {
         const long long t_seg = (long long)seg * a.T;
         const int Tp = (int)min((long long)a.T, a.n_tok - t_seg);
         const int nch = (Tp + RC - 1) / RC;
         float lsum = 0.f, dbsum = 0.f;
         for (int ch = 0; ch < nch; ++ch) {
+            cp_async_wait<0>();
+            const bool landed = mbar_wait(full + 8 * buf, phase, a.status);
+            if (!__syncthreads_and(landed)) return;  // the chunk has landed; everyone is done with the other buffer and Gs
             if (ch + 1 < nch)
                 issue(seg, ch + 1, buf ^ 1);
             else if (seg + 1 < a.n_seg)
                 issue(seg + 1, 0, buf ^ 1);
             cp_async_commit();
-            cp_async_wait<1>();
-            __syncthreads();
-            const float* Xb = Xs + buf * RC * LD;
-            // tokens (tp, tp + 16) x rows (rp, rp + RH) of H (half 0) or R (half 1)
-            float p[2][2] = {};
-            {
-                const float* x0 = Xb + tp * LD;
-                const float* x1 = Xb + (tp + 16) * LD;
-                const float* w0 = Ws + rp * LD;
-                const float* w1 = Ws + (rp + RH) * LD;
-#pragma unroll 2
-                for (int c = c_lo + 4 * ks; c < c_hi; c += 4 * KS) {
-                    const float4 u0 = *reinterpret_cast<const float4*>(x0 + c);
-                    const float4 u1 = *reinterpret_cast<const float4*>(x1 + c);
-                    const float4 b0 = *reinterpret_cast<const float4*>(w0 + c);
-                    const float4 b1 = *reinterpret_cast<const float4*>(w1 + c);
-                    p[0][0] = dot4(u0, b0, p[0][0]);
-                    p[0][1] = dot4(u0, b1, p[0][1]);
-                    p[1][0] = dot4(u1, b0, p[1][0]);
-                    p[1][1] = dot4(u1, b1, p[1][1]);
+            const float* Xb = Xs + buf * RC * D;
+            {   // ---- forward of tokens 2 warp, 2 warp + 1: v[(matrix 2 + token) RB + row]
+                uint64_t p[NV] = {};  // even and odd columns packed
+#pragma unroll
+                for (int i = 0; i < NI; ++i) {
+                    const int c = 4 * lane + 128 * i;
+                    if (c >= D) continue;
+                    const ulonglong2 xa = *reinterpret_cast<const ulonglong2*>(Xb + fo[i]);
+                    const ulonglong2 xb = *reinterpret_cast<const ulonglong2*>(Xb + fo[i] + (c < a.d_in ? a.d_in : dh));
+                    auto add = [&](auto mat) {
+                        constexpr int o = decltype(mat)::value * 2 * RB;
+#pragma unroll
+                        for (int r = 0; r < RB; ++r) {
+                            ulonglong2 wr;
+                            if constexpr (RB == 4)
+                                wr = w[i][r];
+                            else
+                                wr = *reinterpret_cast<const ulonglong2*>(Ws + r * LD + c);
+                            p[o + r] = fma_f32x2(xa.y, wr.y, fma_f32x2(xa.x, wr.x, p[o + r]));
+                            p[o + RB + r] = fma_f32x2(xb.y, wr.y, fma_f32x2(xb.x, wr.x, p[o + RB + r]));
+                        }
+                    };
+                    if (c < a.d_in)
+                        add(std::integral_constant<int, 0>{});
+                    else
+                        add(std::integral_constant<int, 1>{});
                 }
-            }
+                float v[NV];
 #pragma unroll
-            for (int o = 1; o < KS; o <<= 1)
+                for (int u = 0; u < NV; ++u) {
+                    const float2 f = unpack_f32x2(p[u]);
+                    v[u] = f.x + f.y;
+                }
+                // add the lanes' sums: afterwards the lanes whose top bits spell j hold sum j
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
+                for (int n = NV, sft = 16; n > 1; n >>= 1, sft >>= 1) {
+                    const bool upper = (lane & sft) != 0;
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) p[i][j] += __shfl_xor_sync(0xffffffffu, p[i][j], o);
-            if (ks == 0) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) HQ[(half * RC + tp + 16 * i) * RB + rp + RH * j] = p[i][j];
+                    for (int u = 0; u < n / 2; ++u) {
+                        const float send = upper ? v[u] : v[u + n / 2], keep = upper ? v[u + n / 2] : v[u];
+                        v[u] = keep + __shfl_xor_sync(0xffffffffu, send, sft);
+                    }
+                }
+                if (NV == 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+                // epilogue of output (token, row): c_t = -eta_t / T' (Eq. 10), A = SiLU(H); H is in the
+                // lower lanes, R sixteen above
+                const float rv = __shfl_down_sync(0xffffffffu, v[0], 16);
+                constexpr int LPV = 32 / NV;  // lanes holding a sum
+                const int j = lane / LPV, t = 2 * warp + j / RB, r = j % RB, ts = ch * RC + t;
+                if (lane < 16 && lane % LPV == 0) {
+                    const float hv = v[0];
+                    const float ct = ts < Tp ? -etaS[buf * RC + t] / (float)Tp : 0.f;
+                    const float sg = sigmoidf_(hv);
+                    const float av = hv * sg;
+                    const float ds = sg * (1.f + hv * (1.f - sg));
+                    if (ts < Tp) lsum = fmaf(av, rv, lsum);
+                    const float gh = ct * rv * ds, ga = ct * av;
+                    *reinterpret_cast<float2*>(Gs + 2 * ((t * 2 + 0) * RB + r)) = make_float2(gh, gh);
+                    *reinterpret_cast<float2*>(Gs + 2 * ((t * 2 + 1) * RB + r)) = make_float2(ga, ga);
+                }
             }
             if (a.momentum && warp == 0) dbsum += warp_sum(lane < Tp - ch * RC ? dbS[buf * RC + lane] : 0.f);
             __syncthreads();
-            if (tid < RC * RB) {
-                // epilogue of output (t, r): c_t = -eta_t / T' (Eq. 10), A = SiLU(H)
-                const int t = tid / RB, r = tid % RB;
-                const float hv = HQ[t * RB + r], rv = HQ[(RC + t) * RB + r];
-                const int ts = ch * RC + t;  // token within the segment
-                const float ct = ts < Tp ? -etaS[buf * RC + t] / (float)Tp : 0.f;
-                const float sg = sigmoidf_(hv);
-                const float av = hv * sg;
-                const float ds = sg * (1.f + hv * (1.f - sg));
-                if (ts < Tp) lsum = fmaf(av, rv, lsum);
-                Gs[(t * 2 + 0) * RB + r] = ct * rv * ds;
-                Gs[(t * 2 + 1) * RB + r] = ct * av;
-            }
-            __syncthreads();
-            // gradient rows: acc[r] += sum_t G[t][kind][r] * X[t][cb]
+            // ---- gradient rows: acc[r] += sum_t G[t][kind][r] * X[t][cb, cb + 1] over the thread's token half
             if (own) {
-                const int nv = min(RC, Tp - ch * RC);
-                const float* gk = Gs + kind * RB;
-#pragma unroll 4
-                for (int t = 0; t < nv; ++t) {
-                    const float x = Xb[t * LD + cb];
+                const int nv = min(RC / 2, Tp - ch * RC - th * (RC / 2));
+                const float* gk = Gs + 2 * (th * (RC / 2) * 2 + kind) * RB;
+                const float* xk = Xb + bo;
+                auto add = [&](int t) {
+                    const uint64_t x = *reinterpret_cast<const uint64_t*>(xk + t * bs);
 #pragma unroll
-                    for (int r4 = 0; r4 < RB; r4 += 4) {
-                        const float4 g4 = *reinterpret_cast<const float4*>(gk + t * 2 * RB + r4);
-                        acc[r4] = fmaf(g4.x, x, acc[r4]);
-                        acc[r4 + 1] = fmaf(g4.y, x, acc[r4 + 1]);
-                        acc[r4 + 2] = fmaf(g4.z, x, acc[r4 + 2]);
-                        acc[r4 + 3] = fmaf(g4.w, x, acc[r4 + 3]);
+                    for (int r = 0; r < RB; r += 2) {
+                        const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(gk + t * 4 * RB + 2 * r);
+                        acc[r] = fma_f32x2(g.x, x, acc[r]);
+                        acc[r + 1] = fma_f32x2(g.y, x, acc[r + 1]);
                     }
+                };
+                if (nv == RC / 2) {
+#pragma unroll
+                    for (int t = 0; t < RC / 2; ++t) add(t);
+                } else {
+                    for (int t = 0; t < nv; ++t) add(t);
                 }
             }
-            __syncthreads();
+            phase ^= buf;
             buf ^= 1;
         }
-        // end of segment: Eq. 8 update, then the row renormalisation to the norms of W_0
-        float beta = 0.f;
-        if (a.momentum) {  // beta_s = sigmoid(mean_t w_beta . x_t + b_beta); warp 0 holds the sum
-            if (tid == 0) scl[2 * RB] = sigmoidf_(dbsum / (float)Tp + b_beta);
-            __syncthreads();
-            beta = scl[2 * RB];
+        // ---- end of segment: the token halves' gradients together, the Eq. 8 update, then the row
+        //      renormalisation to the norms of W_0
+        if (own && th == 1) {
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                *reinterpret_cast<uint64_t*>(Ps + r * LD + cb) = acc[r];
+                acc[r] = 0;
+            }
         }
+        if (a.momentum && tid == 0)  // beta_s = sigmoid(mean_t w_beta . x_t + b_beta); warp 0 holds the sum
+            scl[2 * RB] = sigmoidf_(dbsum / (float)Tp + b_beta);
+        __syncthreads();
+        const float beta = a.momentum ? scl[2 * RB] : 0.f;
         if (a.loss) {
             const float tot = block_sum_res(lsum, red);
             if (tid == 0) atomicAdd(&a.loss[seg * a.m_sstride + cz], -tot / (float)Tp);
         }
-        float wn[RB], step = 0.f;
+        float2 wn[RB];
+        float step = 0.f;
+        const bool upd = own && th == 0;
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
-            const float mn = a.momentum ? fmaf(beta, mu[r], acc[r]) : acc[r];
-            mu[r] = mn;
-            acc[r] = 0.f;
-            wn[r] = own ? Ws[r * LD + cb] - mn : 0.f;
-            step = own ? fmaf(mn, mn, step) : step;
+            wn[r] = make_float2(0.f, 0.f);
+            if (upd) {
+                const float2 p = *reinterpret_cast<const float2*>(Ps + r * LD + cb), wo = *reinterpret_cast<const float2*>(Ws + r * LD + cb);
+                const float2 g = unpack_f32x2(acc[r]);
+                float2 m = make_float2(g.x + p.x, g.y + p.y);
+                if (a.momentum) {
+                    float2* mu = reinterpret_cast<float2*>(Ms + r * LD + cb);
+                    m = make_float2(fmaf(beta, mu->x, m.x), fmaf(beta, mu->y, m.y));
+                    *mu = m;
+                }
+                acc[r] = 0;
+                wn[r] = make_float2(wo.x - m.x, wo.y - m.y);
+                step = fmaf(m.x, m.x, fmaf(m.y, m.y, step));
+            }
         }
         if (a.step_sq) {
             __syncthreads();  // red may still be read by block_sum_res above
@@ -769,26 +836,28 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
             for (int k = 0; k < 2; ++k)
 #pragma unroll
                 for (int r = 0; r < RB; ++r) {
-                    const float v = warp_sum(kind == k ? wn[r] * wn[r] : 0.f);
+                    const float v = warp_sum(kind == k ? fmaf(wn[r].x, wn[r].x, wn[r].y * wn[r].y) : 0.f);
                     if (lane == 0) red[warp * 2 * RB + k * RB + r] = v;
                 }
             __syncthreads();
             if (tid < 2 * RB) {
                 float tot = 0.f;
-                for (int w = 0; w < NW; ++w) tot += red[w * 2 * RB + tid];
+                for (int i = 0; i < NW; ++i) tot += red[i * 2 * RB + tid];
                 scl[tid] = renorm_scale(nS[tid], tot);
             }
             __syncthreads();
         }
-        if (own) {
+        if (upd) {
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
-                const float wv = wn[r] * (a.renorm ? scl[kind * RB + r] : 1.f);
-                finite = finite && isfinite(wv);
-                Ws[r * LD + cb] = wv;
+                const float sc = a.renorm ? scl[kind * RB + r] : 1.f;
+                const float2 wv = make_float2(wn[r].x * sc, wn[r].y * sc);
+                finite = finite && isfinite(wv.x) && isfinite(wv.y);
+                *reinterpret_cast<float2*>(Ws + r * LD + cb) = wv;
             }
         }
         __syncthreads();
+        load_w();
     }
     cp_async_wait<0>();
     // write the rows and the momentum back (the CTA's rows lie inside the chain: index check of
@@ -797,22 +866,16 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
     for (int i = tid; i < RB * (D / 4); i += RES_NT) {
         const int r = i / (D / 4), c = 4 * (i - r * (D / 4));
         const size_t row = (size_t)cs * a.d_hid + h0 + r;
-        float* dst = c < a.d_in ? a.W1 + row * a.d_in + c : a.W2 + row * a.d_out + (c - a.d_in);
-        *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(Ws + r * LD + c);
-    }
-    if (own && a.momentum) {
-#pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            const size_t row = (size_t)cs * a.d_hid + h0 + r;
-            (kind == 0 ? a.mu1[row * a.d_in + cb] : a.mu2[row * a.d_out + (cb - a.d_in)]) = mu[r];
-        }
+        const size_t o = c < a.d_in ? row * a.d_in + c : row * a.d_out + (c - a.d_in);
+        *reinterpret_cast<float4*>((c < a.d_in ? a.W1 : a.W2) + o) = *reinterpret_cast<const float4*>(Ws + r * LD + c);
+        if (a.momentum) *reinterpret_cast<float4*>((c < a.d_in ? a.mu1 : a.mu2) + o) = *reinterpret_cast<const float4*>(Ms + r * LD + c);
     }
     if (!finite) atomicOr(a.status, DEV_NONFINITE);
 }
 
 template <int RB> constexpr size_t res_smem_bytes(int D) {
-    return sizeof(float) * ((size_t)(RB + 2 * RES_RC) * res_ld(D) + RES_RC * 2 * RB + 2 * RES_RC * RB +
-                            RES_NW * 2 * RB + 2 * RB + 4 + 4 * RES_RC + 2 * RB);
+    return sizeof(float) * ((size_t)3 * RB * res_ld(D) + (size_t)2 * RES_RC * D + RES_RC * 4 * RB + RES_NW * 2 * RB + 2 * RB + 4 +
+                            4 * RES_RC + 2 * RB);
 }
 
 // ------------------------------------------------------------------ state upkeep
@@ -1102,17 +1165,18 @@ cudaError_t launch_resident_f32(const DevState& s, const SegWork& w, long long n
     if (e != cudaSuccess) return e;
     // four rows a CTA while that still fits the chains in one wave, else eight (less re-streaming)
     const int D = s.d_in + s.d_out;
-    if ((long long)w.nc * (s.d_hid / 4) <= sms) {
-        const size_t bytes = res_smem_bytes<4>(D);
-        e = cudaFuncSetAttribute(ttl_resident_f32_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        ttl_resident_f32_kernel<4><<<dim3(s.d_hid / 4, w.nc), RES_NT, bytes, st>>>(a);
-    } else {
-        const size_t bytes = res_smem_bytes<8>(D);
-        e = cudaFuncSetAttribute(ttl_resident_f32_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        ttl_resident_f32_kernel<8><<<dim3(s.d_hid / 8, w.nc), RES_NT, bytes, st>>>(a);
-    }
+    static std::once_flag once;
+    std::call_once(once, [&] {
+        e = cudaFuncSetAttribute(ttl_resident_f32_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_smem_bytes<4>(512));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(ttl_resident_f32_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)res_smem_bytes<8>(512));
+    });
+    if (e != cudaSuccess) return e;
+    if ((long long)w.nc * (s.d_hid / 4) <= sms)
+        ttl_resident_f32_kernel<4><<<dim3(s.d_hid / 4, w.nc), RES_NT, res_smem_bytes<4>(D), st>>>(a);
+    else
+        ttl_resident_f32_kernel<8><<<dim3(s.d_hid / 8, w.nc), RES_NT, res_smem_bytes<8>(D), st>>>(a);
     return cudaGetLastError();
 }
 
