@@ -550,13 +550,6 @@ struct ResArgs {
     int* status;
 };
 
-__device__ __forceinline__ float dot4(const float4 a, const float4 b, float acc) {
-    acc = fmaf(a.x, b.x, acc);
-    acc = fmaf(a.y, b.y, acc);
-    acc = fmaf(a.z, b.z, acc);
-    return fmaf(a.w, b.w, acc);
-}
-
 constexpr int RES_NT = 512, RES_NW = RES_NT / 32;  // threads and warps of a resident CTA
 
 // Sum of v over the CTA; every thread gets the total.  red: RES_NW floats.
