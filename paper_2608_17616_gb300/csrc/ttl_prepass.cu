@@ -305,33 +305,38 @@ cudaError_t launch_prepass(const DevState& s, const SegWork& w, cudaStream_t st)
     return s.dtype == 0 ? launch_one<float, float>(a, w.nc, st) : launch_one<bf16, bf16>(a, w.nc, st);
 }
 
-// Query side of the read on the bf16 path, in one pass: one warp per (chain, query token).
+// Query side of the read on the bf16 path, in one pass: a warp to one or two query tokens of a chain.
 // Paper mode: z = SiLU(alpha x + gamma), stored in bf16 unnormalised, and 1/|z| per token into
 // zinv (the read scales each query's pre-activation by it: the row scale commutes with the
 // contraction over d_in, Sec. 3.3's L2 normalisation); plain mode: z = x.  A lane's x, alpha
 // and gamma loads of a 4-vector group are all issued before any arithmetic.
+// A warp takes R rows of one chain, so that alpha and gamma (8 bytes an element against a row's 4 in and
+// out, from L2) are read once for all of them, and G 16-byte vectors a lane and row at a time.
+template <int R, int G>
 __global__ void __launch_bounds__(256) query_z_kernel(const bf16* X, int Q, int d, int paper, const float* alpha,
-                                                      const float* gamma, bf16* Z, float* zinv, int total) {
+                                                      const float* gamma, bf16* Z, float* zinv, int groups) {
     // the read's hidden kernel, launched after this one with programmatic stream serialisation,
     // may start now; it waits for this grid's completion before it reads Z or zinv
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (row >= total) return;
-    const int c = row / Q;
-    const bf16* x = X + (size_t)row * d;
-    bf16* z = Z + (size_t)row * d;
+    const int grp = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (grp >= groups) return;
+    const int gpc = (Q + R - 1) / R, c = grp / gpc, q0 = (grp - c * gpc) * R, nr = min(R, Q - q0);
+    const size_t row0 = (size_t)c * Q + q0;
+    const bf16* x = X + row0 * d;
+    bf16* z = Z + row0 * d;
     const float* al = paper ? alpha + (size_t)c * d : nullptr;
     const float* ga = paper ? gamma + (size_t)c * d : nullptr;
-    float ss = 0.f;
-    constexpr int G = 4;  // 16-byte vectors of a group
+    float ss[R] = {};
     for (int base = lane * 8; base < d; base += G * 256) {
-        uint4 xr[G];
+        uint4 xr[G][R];
         float4 av[G][2], gv[G][2];
 #pragma unroll
         for (int q = 0; q < G; ++q) {
             const int i0 = base + q * 256;
             if (i0 < d) {
-                xr[q] = __ldg(reinterpret_cast<const uint4*>(x + i0));
+#pragma unroll
+                for (int r = 0; r < R; ++r)  // a row past the chain's last: the last again, not stored
+                    xr[q][r] = __ldg(reinterpret_cast<const uint4*>(x + (size_t)min(r, nr - 1) * d + i0));
                 if (paper) {
                     av[q][0] = __ldg(reinterpret_cast<const float4*>(al + i0));
                     av[q][1] = __ldg(reinterpret_cast<const float4*>(al + i0 + 4));
@@ -344,36 +349,50 @@ __global__ void __launch_bounds__(256) query_z_kernel(const bf16* X, int Q, int 
         for (int q = 0; q < G; ++q) {
             const int i0 = base + q * 256;
             if (i0 >= d) break;
-            if (!paper) {
-                *reinterpret_cast<uint4*>(z + i0) = xr[q];
-                continue;
-            }
-            float xv[8];
-            Vec<bf16>::unpack(xr[q], xv);
             const float a8[8] = {av[q][0].x, av[q][0].y, av[q][0].z, av[q][0].w,
                                  av[q][1].x, av[q][1].y, av[q][1].z, av[q][1].w};
             const float g8[8] = {gv[q][0].x, gv[q][0].y, gv[q][0].z, gv[q][0].w,
                                  gv[q][1].x, gv[q][1].y, gv[q][1].z, gv[q][1].w};
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float zp = fmaf(a8[e], xv[e], g8[e]);
-                xv[e] = zp * sig<bf16>(zp);
-                ss = fmaf(xv[e], xv[e], ss);
+            for (int r = 0; r < R; ++r) {
+                if (r >= nr) break;
+                if (!paper) {
+                    *reinterpret_cast<uint4*>(z + (size_t)r * d + i0) = xr[q][r];
+                    continue;
+                }
+                float xv[8];
+                Vec<bf16>::unpack(xr[q][r], xv);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const float zp = fmaf(a8[e], xv[e], g8[e]);
+                    xv[e] = zp * sig<bf16>(zp);
+                    ss[r] = fmaf(xv[e], xv[e], ss[r]);
+                }
+                store_vec<bf16, 8>(z + (size_t)r * d + i0, xv);
             }
-            store_vec<bf16, 8>(z + i0, xv);
         }
     }
     if (paper) {
-        ss = warp_sum(ss);
-        if (lane == 0) zinv[row] = 1.0f / sqrtf(ss + 1e-12f);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float s = warp_sum(ss[r]);
+            if (lane == 0 && r < nr) zinv[row0 + r] = 1.0f / sqrtf(s + 1e-12f);
+        }
     }
 }
 
 cudaError_t launch_query_z(const DevState& s, const void* Xq, int Q, void* Z, float* zinv, cudaStream_t st) {
-    const int total = s.C * Q;
-    query_z_kernel<<<(total + 7) / 8, 256, 0, st>>>(static_cast<const bf16*>(Xq), Q, s.d_in, s.mode == 1, s.alpha,
-                                                    s.gamma, static_cast<bf16*>(Z), zinv, total);
-    return cudaGetLastError();
+    auto run = [&](auto kernel, int R) {
+        const int groups = s.C * ((Q + R - 1) / R);
+        kernel<<<(groups + 7) / 8, 256, 0, st>>>(static_cast<const bf16*>(Xq), Q, s.d_in, s.mode == 1, s.alpha, s.gamma,
+                                                 static_cast<bf16*>(Z), zinv, groups);
+        return cudaGetLastError();
+    };
+    // Two rows a warp once that leaves enough warps to fill the GPU.  Whole reads, one and two rows a warp: 4112
+    // rows of 2048 70.7 and 70.9 us, 5200 rows 72.7 and 71.6, 16,000 rows 134 and 127, 28,000 rows of 3072 457
+    // and 438, 128,000 rows of 256 207 and 162; 1000 rows of 2048 36.9 and 39.0.
+    if (Q > 1 && (long long)s.C * Q > 4608) return run(query_z_kernel<2, 1>, 2);
+    return run(query_z_kernel<1, 4>, 1);
 }
 
 // Query side of the read, normalised (the SwiGLU read, the fp32 read and the 128-query form):

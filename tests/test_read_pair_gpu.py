@@ -21,7 +21,8 @@ def _built():
 
 @pytest.mark.parametrize("Q,hd,mode", [(1000, 64, wk.PAPER), (1025, 128, wk.PAPER), (513, 64, wk.PLAIN), (900, 128, wk.PLAIN)])
 def test_read_of_many_tiles(Q, hd, mode):
-    # 10 chains x 4 tiles of hidden units (and of outputs) x ceil(Q / 128) query tiles
+    # 10 chains x 4 tiles of hidden units (and of outputs) x ceil(Q / 128) query tiles; more than 4608 query
+    # rows, so the input transform takes two a warp (an odd Q leaves a warp with one)
     wl = wk.Workload("read_pair", 14, 2, 5, 256, 512, 512, 512 // (2 * hd), hd, 128, 160, Q, "bf16", mode)
     run = DeviceRun(wl)
     run.ttl_context()
