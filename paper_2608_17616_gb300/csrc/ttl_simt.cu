@@ -92,36 +92,40 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// ---- tiled contractions of the fp32 phases: 256 threads as 16 x 16, TM x TN outputs each, slabs of the
+// ---- tiled contractions of the fp32 phases: threads as TY (ty) x 16 (tx), TM x TN outputs each, slabs of the
 // contraction through a ring of cp.async stages.  (TM + TN) 16-byte shared-memory loads feed 4 TM TN
 // multiply-adds a thread; a warp is 4 (ty) x 8 (tx) threads, so a half warp's load is at most 128
-// distinct bytes, one wavefront (2 x 16 threads: two for the tx operand).  Every output is one fmaf chain in
-// order of k.
+// distinct bytes, one wavefront (2 x 16 threads: two for the tx operand).  Multiply-adds are packed pairs: of
+// even and odd k in nt_tile, of neighbouring columns in tn_tile.
 __device__ __forceinline__ int tile_tx() { return (threadIdx.x & 7) | ((threadIdx.x >> 5 & 1) << 3); }
 __device__ __forceinline__ int tile_ty() { return (threadIdx.x >> 3 & 3) | (threadIdx.x >> 6 << 2); }
 
-// Both operands with k contiguous: acc[i][j] += sum_k A[ty + 16 i][k] B[tx + 16 j][k], rows of A from
+// Both operands with k contiguous: acc[i][j] += sum_k A[ty + TY i][k] B[tx + 16 j][k], rows of A from
 // m_valid on read as 0.  K a multiple of 32; rows 36 floats apart, so the 8 rows of a quarter warp start
 // in 8 bank groups.
 constexpr int NT_K = 32, NT_LD = NT_K + 4, NT_ST = 3;
-template <int TM, int TN> constexpr size_t nt_smem() { return sizeof(float) * NT_ST * 16 * (TM + TN) * NT_LD; }
+template <int TM, int TN, int TY> constexpr size_t nt_smem() { return sizeof(float) * NT_ST * (TY * TM + 16 * TN) * NT_LD; }
 
-template <int TM, int TN>
+template <int TM, int TN, int TY>
 __device__ __forceinline__ void nt_tile(float (&acc)[TM][TN], const float* A, long long lda, const float* B, long long ldb,
                                         int K, int m_valid, float* sm) {
-    constexpr int BM = 16 * TM, BN = 16 * TN, STAGE = (BM + BN) * NT_LD;
+    constexpr int BM = TY * TM, BN = 16 * TN, STAGE = (BM + BN) * NT_LD;
     const int tid = threadIdx.x, tx = tile_tx(), ty = tile_ty(), n = K / NT_K;
+    // the thread's 16-byte pieces of a slab: rows r0 + 2 TY u (of A, then of B), columns p0
+    const int r0 = tid >> 3, p0 = 4 * (tid & 7);
+    const float *ga = A + r0 * lda + p0, *gb = B + r0 * ldb + p0;
     auto load = [&](int s) {
-        float* d = sm + (s % NT_ST) * STAGE;
+        float* d = sm + (s % NT_ST) * STAGE + r0 * NT_LD + p0;
 #pragma unroll
-        for (int u = 0; u < (BM + BN) * 8 / 256; ++u) {
-            const int e = tid + 256 * u, r = e >> 3, p = 4 * (e & 7), k = s * NT_K + p;
-            if (r < BM)
-                cp_async16(d + r * NT_LD + p, r < m_valid ? A + r * lda + k : A, r < m_valid ? 16 : 0);
-            else
-                cp_async16(d + r * NT_LD + p, B + (r - BM) * ldb + k, 16);
+        for (int u = 0; u < BM / (2 * TY); ++u) {
+            const bool v = r0 + 2 * TY * u < m_valid;
+            cp_async16(d + 2 * TY * u * NT_LD, v ? ga + 2 * TY * u * lda + s * NT_K : A, v ? 16 : 0);
         }
+#pragma unroll
+        for (int u = 0; u < BN / (2 * TY); ++u)
+            cp_async16(d + (BM + 2 * TY * u) * NT_LD, gb + 2 * TY * u * ldb + s * NT_K, 16);
     };
+    uint64_t p[TM][TN] = {};  // sums over even and odd k
     // the ring may still be read from an earlier contraction of this kernel
     __syncthreads();
 #pragma unroll
@@ -138,40 +142,46 @@ __device__ __forceinline__ void nt_tile(float (&acc)[TM][TN], const float* A, lo
         const float* Bs = sm + (s % NT_ST) * STAGE + (BM + tx) * NT_LD;
 #pragma unroll
         for (int k = 0; k < NT_K; k += 4) {
-            float4 a[TM], b[TN];
+            ulonglong2 a[TM], b[TN];  // two packed pairs of k each
 #pragma unroll
-            for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(As + 16 * i * NT_LD + k);
+            for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(As + TY * i * NT_LD + k);
 #pragma unroll
-            for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const float4*>(Bs + 16 * j * NT_LD + k);
+            for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const ulonglong2*>(Bs + 16 * j * NT_LD + k);
 #pragma unroll
             for (int i = 0; i < TM; ++i)
 #pragma unroll
-                for (int j = 0; j < TN; ++j) {
-                    acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-                    acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-                    acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-                    acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
-                }
+                for (int j = 0; j < TN; ++j) p[i][j] = fma_f32x2(a[i].x, b[j].x, p[i][j]);
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) p[i][j] = fma_f32x2(a[i].y, b[j].y, p[i][j]);
         }
     }
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            const float2 v = unpack_f32x2(p[i][j]);
+            acc[i][j] += v.x + v.y;
+        }
 }
 
 // Both operands with the output dimension contiguous: acc[i][j] += sum_k A[k][m(i)] B[k][n(j)] with
-// m(i) = 4 ty + 64 (i / 4) + i % 4 and n(j) likewise from tx (tile 16 TM x 16 TN).  Rows k >= kv read as 0.
+// m(i) = 4 ty + 4 TY (i / 4) + i % 4 and n(j) = 4 tx + 64 (j / 4) + j % 4 (tile TY TM x 16 TN).  Rows k >= kv read as 0.
 constexpr int TN_K = 16, TN_ST = 3;
-template <int TM, int TN> constexpr size_t tn_smem() { return sizeof(float) * TN_ST * TN_K * 16 * (TM + TN); }
+template <int TM, int TN, int TY> constexpr size_t tn_smem() { return sizeof(float) * TN_ST * TN_K * (TY * TM + 16 * TN); }
 
-template <int TM, int TN>
+template <int TM, int TN, int TY>
 __device__ __forceinline__ void tn_tile(float (&acc)[TM][TN], const float* A, long long lda, const float* B, long long ldb,
                                         int K, int kv, float* sm) {
     static_assert(TM % 4 == 0 && TN % 4 == 0, "outputs in groups of four");
-    constexpr int BM = 16 * TM, BN = 16 * TN, LD = BM + BN, STAGE = TN_K * LD;
+    constexpr int BM = TY * TM, BN = 16 * TN, LD = BM + BN, STAGE = TN_K * LD;
     const int tid = threadIdx.x, tx = tile_tx(), ty = tile_ty(), n = (K + TN_K - 1) / TN_K;
     auto load = [&](int s) {
         float* d = sm + (s % TN_ST) * STAGE;
 #pragma unroll
-        for (int u = 0; u < STAGE / 4 / 256; ++u) {
-            const int e = tid + 256 * u, r = e / (LD / 4), c = 4 * (e % (LD / 4)), k = s * TN_K + r;
+        for (int u = 0; u < STAGE / 4 / (16 * TY); ++u) {
+            const int e = tid + 16 * TY * u, r = e / (LD / 4), c = 4 * (e % (LD / 4)), k = s * TN_K + r;
             const float* src = c < BM ? A + k * lda + c : B + k * ldb + (c - BM);
             cp_async16(d + r * LD + c, k < kv ? src : A, k < kv ? 16 : 0);
         }
@@ -192,7 +202,7 @@ __device__ __forceinline__ void tn_tile(float (&acc)[TM][TN], const float* A, lo
             float a[TM], b[TN];
 #pragma unroll
             for (int i = 0; i < TM; i += 4)
-                *reinterpret_cast<float4*>(a + i) = *reinterpret_cast<const float4*>(S + k * LD + 4 * ty + 16 * i);
+                *reinterpret_cast<float4*>(a + i) = *reinterpret_cast<const float4*>(S + k * LD + 4 * ty + TY * i);
 #pragma unroll
             for (int j = 0; j < TN; j += 4)
                 *reinterpret_cast<float4*>(b + j) = *reinterpret_cast<const float4*>(S + k * LD + BM + 4 * tx + 16 * j);
@@ -238,16 +248,17 @@ __device__ __forceinline__ const float* ss_ptr(const F32SegArgs& a, int parity, 
     return a.sumsq + ((size_t)(parity * 2 + which) * a.C) * a.d_hid;
 }
 
-// Phase A: 16 TM tokens x 16 TN hidden units a CTA, H over d_in and R over d_out in turn.  Bound by FMA
-// issue and the last wave: 4 chains of 1024 -> 1024 -> 1024, T = 256 (256 tiles of 64 x 64) take 126 us,
-// 34 TFLOP/s (32 x 64 tiles with a slab read, waited for and then multiplied: 250 us; 64 x 128 tiles, one
-// CTA an SM: 152 us; 32 x 64: 189 us).
-template <int TM, int TN>
-__global__ void __launch_bounds__(256, 2) phase_a_f32_kernel(const F32SegArgs a) {
+// Phase A: TY TM tokens x 16 TN hidden units a CTA, H over d_in and R over d_out in turn.  Bound by shared
+// memory (TM = 4) or FMA issue (TM = 8) and the last wave: 4 chains of 1024 -> 1024 -> 1024, T = 256 (256
+// tiles of 64 x 64) take 123 us, 35 TFLOP/s (with 256 threads of 4 x 4 outputs: single multiply-adds 126 us,
+// paired 130; 32 x 64 tiles with a slab read, waited for and then multiplied: 250 us; 64 x 128 tiles, one CTA an
+// SM: 152 us).
+template <int TM, int TN, int TY>
+__global__ void __launch_bounds__(16 * TY, 2) phase_a_f32_kernel(const F32SegArgs a) {
     extern __shared__ float4 f32_smem[];
     __shared__ float red[8];
     float* sm = reinterpret_cast<float*>(f32_smem);
-    constexpr int BM = 16 * TM, BN = 16 * TN;
+    constexpr int BM = TY * TM, BN = 16 * TN;
     const int tid = threadIdx.x, tx = tile_tx(), ty = tile_ty();
     const int t0 = blockIdx.x * BM, h0 = blockIdx.y * BN, cz = blockIdx.z, cs = a.c0 + cz;
     int m_valid = (int)min((long long)min(BM, a.Tp - t0), a.row_avail - t0);
@@ -262,17 +273,17 @@ __global__ void __launch_bounds__(256, 2) phase_a_f32_kernel(const F32SegArgs a)
     if (m_valid > 0) {
         const int dh = a.d_out / 2;
         const float* W2 = a.W2 + ((size_t)cs * a.d_hid + h0) * a.d_out;
-        nt_tile(accH, a.U + cz * a.u_cstride + (long long)t0 * a.d_in, a.d_in, a.W1 + ((size_t)cs * a.d_hid + h0) * a.d_in,
+        nt_tile<TM, TN, TY>(accH, a.U + cz * a.u_cstride + (long long)t0 * a.d_in, a.d_in, a.W1 + ((size_t)cs * a.d_hid + h0) * a.d_in,
                 a.d_in, a.d_in, m_valid, sm);
-        nt_tile(accR, a.K + cz * a.y_cstride + (long long)t0 * dh, dh, W2, a.d_out, dh, m_valid, sm);
-        nt_tile(accR, a.V + cz * a.y_cstride + (long long)t0 * dh, dh, W2 + dh, a.d_out, dh, m_valid, sm);
+        nt_tile<TM, TN, TY>(accR, a.K + cz * a.y_cstride + (long long)t0 * dh, dh, W2, a.d_out, dh, m_valid, sm);
+        nt_tile<TM, TN, TY>(accR, a.V + cz * a.y_cstride + (long long)t0 * dh, dh, W2 + dh, a.d_out, dh, m_valid, sm);
     }
     const float* prev1 = ss_ptr(a, a.parity ^ 1, 0) + (size_t)cs * a.d_hid;
     const float* prev2 = ss_ptr(a, a.parity ^ 1, 1) + (size_t)cs * a.d_hid;
     float ct[TM];
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
-        const int t = t0 + ty + 16 * i;
+        const int t = t0 + ty + TY * i;
         ct[i] = 0.f;
         if (t < a.Tp && t - t0 < m_valid) {
             const float e = a.paper ? a.eta[(size_t)cs * a.win + a.tok0 + t]
@@ -288,7 +299,7 @@ __global__ void __launch_bounds__(256, 2) phase_a_f32_kernel(const F32SegArgs a)
         const float s2 = a.renorm_pending ? renorm_scale(a.n2[(size_t)cs * a.d_hid + h], prev2[h]) : 1.f;
 #pragma unroll
         for (int i = 0; i < TM; ++i) {
-            const size_t o = ((size_t)cs * a.T + t0 + ty + 16 * i) * a.d_hid + h;
+            const size_t o = ((size_t)cs * a.T + t0 + ty + TY * i) * a.d_hid + h;
             const float hv = accH[i][j] * s1;
             const float rv = accR[i][j] * s2;
             const float sg = sigmoidf_(hv);
@@ -305,21 +316,21 @@ __global__ void __launch_bounds__(256, 2) phase_a_f32_kernel(const F32SegArgs a)
         __syncthreads();
         if (tid == 0) {
             float tot = 0.f;
-            for (int w = 0; w < 8; ++w) tot += red[w];
+            for (int w = 0; w < TY / 2; ++w) tot += red[w];
             atomicAdd(&a.loss[cz], -tot / (float)a.Tp);
         }
     }
 }
 
-// Phase B: 16 TM hidden rows x 16 TN columns of W1, or of the K or V half of W2, a CTA.  The same 4
+// Phase B: TY TM hidden rows x 16 TN columns of W1, or of the K or V half of W2, a CTA.  The same 4
 // chains: 105 us, 41 TFLOP/s, with 128 x 128 tiles and paired multiply-adds (single ones 122 us; 64 x 64
 // tiles 133 us; the 32 x 64 tiles before them 344 us).
-template <int TM, int TN>
-__global__ void __launch_bounds__(256, 2) phase_b_f32_kernel(const F32SegArgs a) {
+template <int TM, int TN, int TY>
+__global__ void __launch_bounds__(16 * TY, 32 / TY) phase_b_f32_kernel(const F32SegArgs a) {
     extern __shared__ float4 f32_smem[];
     __shared__ float red[8];
     __shared__ float s_beta;
-    constexpr int BM = 16 * TM, BN = 16 * TN;
+    constexpr int BM = TY * TM, BN = 16 * TN;
     const int tid = threadIdx.x, tx = tile_tx(), ty = tile_ty();
     const int col0 = blockIdx.x * BN, h0 = blockIdx.y * BM, cz = blockIdx.z, cs = a.c0 + cz;
     const bool isW1 = col0 < a.d_in;
@@ -327,13 +338,13 @@ __global__ void __launch_bounds__(256, 2) phase_b_f32_kernel(const F32SegArgs a)
     // momentum decay beta_s = sigmoid(mean_t w_beta . x_t + b_beta)
     if (a.momentum) {
         float v = 0.f;
-        for (int t = tid; t < a.Tp; t += 256) v += a.dbeta[(size_t)cs * a.win + a.tok0 + t];
+        for (int t = tid; t < a.Tp; t += 16 * TY) v += a.dbeta[(size_t)cs * a.win + a.tok0 + t];
         v = warp_sum(v);
         if ((tid & 31) == 0) red[tid >> 5] = v;
         __syncthreads();
         if (tid == 0) {
             float tot = 0.f;
-            for (int w = 0; w < 8; ++w) tot += red[w];
+            for (int w = 0; w < TY / 2; ++w) tot += red[w];
             s_beta = sigmoidf_(tot / (float)a.Tp + a.b_beta[cs]);
         }
     }
@@ -342,7 +353,7 @@ __global__ void __launch_bounds__(256, 2) phase_b_f32_kernel(const F32SegArgs a)
         const int dh = a.d_out / 2, o0 = col0 - a.d_in;
         const float* A = (isW1 ? a.dH : a.At) + (size_t)cs * a.T * a.d_hid + h0;
         const float* B = isW1 ? a.U + cz * a.u_cstride + col0 : (o0 < dh ? a.K + o0 : a.V + (o0 - dh)) + cz * a.y_cstride;
-        tn_tile(acc, A, a.d_hid, B, isW1 ? a.d_in : dh, a.Tp, kv, reinterpret_cast<float*>(f32_smem));
+        tn_tile<TM, TN, TY>(acc, A, a.d_hid, B, isW1 ? a.d_in : dh, a.Tp, kv, reinterpret_cast<float*>(f32_smem));
     }
     const float beta = a.momentum ? s_beta : 0.f;  // tn_tile's first barrier has published it
     const int which = isW1 ? 0 : 1;
@@ -355,7 +366,7 @@ __global__ void __launch_bounds__(256, 2) phase_b_f32_kernel(const F32SegArgs a)
     float step = 0.f;  // sum of mu_s^2 over this thread's elements
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
-        const int h = h0 + 4 * ty + 64 * (i / 4) + i % 4;
+        const int h = h0 + 4 * ty + 4 * TY * (i / 4) + i % 4;
         const float s = a.renorm_pending ? renorm_scale(n0[h], prev[h]) : 1.f;
         const size_t row = ((size_t)cs * a.d_hid + h) * width + c_local + 4 * tx;
         float* wrow = (isW1 ? a.W1 : a.W2) + row;
@@ -1079,24 +1090,25 @@ __global__ void __launch_bounds__(256) read_norm_kernel(DevState s, int Q, Tout*
 namespace {
 // Launch a phase kernel of the fp32 path (its shared memory opted in on first use).
 template <typename K>
-cudaError_t launch_f32_tiles(K kernel, size_t smem, std::once_flag& once, dim3 grid, const F32SegArgs& a, cudaStream_t st) {
+cudaError_t launch_f32_tiles(K kernel, int threads, size_t smem, std::once_flag& once, dim3 grid, const F32SegArgs& a,
+                             cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     std::call_once(once, [&] { e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
     if (e != cudaSuccess) return e;
-    kernel<<<grid, 256, smem, st>>>(a);
+    kernel<<<grid, threads, smem, st>>>(a);
     return cudaGetLastError();
 }
-template <int TM, int TN>
+template <int TM, int TN, int TY>
 cudaError_t phase_a_f32(const DevState& s, const SegWork& w, const F32SegArgs& a, cudaStream_t st) {
     static std::once_flag once;
-    return launch_f32_tiles(phase_a_f32_kernel<TM, TN>, nt_smem<TM, TN>(), once,
-                            dim3(s.T / (16 * TM), s.d_hid / (16 * TN), w.nc), a, st);
+    return launch_f32_tiles(phase_a_f32_kernel<TM, TN, TY>, 16 * TY, nt_smem<TM, TN, TY>(), once,
+                            dim3(s.T / (TY * TM), s.d_hid / (16 * TN), w.nc), a, st);
 }
-template <int TM, int TN>
+template <int TM, int TN, int TY>
 cudaError_t phase_b_f32(const DevState& s, const SegWork& w, const F32SegArgs& a, cudaStream_t st) {
     static std::once_flag once;
-    return launch_f32_tiles(phase_b_f32_kernel<TM, TN>, tn_smem<TM, TN>(), once,
-                            dim3((s.d_in + s.d_out) / (16 * TN), s.d_hid / (16 * TM), w.nc), a, st);
+    return launch_f32_tiles(phase_b_f32_kernel<TM, TN, TY>, 16 * TY, tn_smem<TM, TN, TY>(), once,
+                            dim3((s.d_in + s.d_out) / (16 * TN), s.d_hid / (TY * TM), w.nc), a, st);
 }
 constexpr long long F32_SMS = 152;
 }  // namespace
@@ -1104,10 +1116,12 @@ constexpr long long F32_SMS = 152;
 cudaError_t launch_phase_a_f32(const DevState& s, const SegWork& w, cudaStream_t st) {
     const F32SegArgs a = make_f32_args(s, w);
     const long long g64 = (long long)(s.T / 64) * (s.d_hid / 64) * w.nc;  // 64 x 64 tiles (T, d_hid multiples of 64)
-    // 32 x 64 tiles while their grid fits the SMs once (a wave of them takes three quarters of a wave of
-    // 64 x 64: 59 against 79 us for one chain of 1024 -> 1024 -> 1024 at T = 256), else 64 x 64 (two chains:
-    // 79 against 101 us)
-    return 2 * g64 <= F32_SMS ? phase_a_f32<2, 4>(s, w, a, st) : phase_a_f32<4, 4>(s, w, a, st);
+    // 32 x 64 tiles, but 64 x 64 (8 x 4 outputs a thread) where halving the tiles saves nothing of the last wave.
+    // 1024 -> 1024 -> 1024, T = 256, 32 x 64 and 64 x 64 tiles: one chain (64 tiles of 64 x 64) 48 and 73 us,
+    // three 102 and 123, four (256) 135 and 123, five 163 and 180, eight 223 and 234
+    const auto waves = [](long long tiles) { return (tiles + F32_SMS - 1) / F32_SMS; };
+    if (g64 > F32_SMS && waves(2 * g64) == 2 * waves(g64)) return phase_a_f32<8, 4, 8>(s, w, a, st);
+    return phase_a_f32<4, 4, 8>(s, w, a, st);
 }
 
 cudaError_t launch_phase_b_f32(const DevState& s, const SegWork& w, cudaStream_t st) {
@@ -1115,8 +1129,11 @@ cudaError_t launch_phase_b_f32(const DevState& s, const SegWork& w, cudaStream_t
     // a tile lies in W1 or in one half of W2: widths are multiples of 64, for the large tile of 128, which
     // is taken from two thirds of the SMs on
     const bool wide = s.d_in % 128 == 0 && (s.d_out / 2) % 128 == 0 && s.d_hid % 128 == 0;
-    if (wide && (long long)(s.d_hid / 128) * ((s.d_in + s.d_out) / 128) * w.nc >= 100) return phase_b_f32<8, 8>(s, w, a, st);
-    return phase_b_f32<4, 4>(s, w, a, st);
+    if (wide && (long long)(s.d_hid / 128) * ((s.d_in + s.d_out) / 128) * w.nc >= 100) return phase_b_f32<8, 8, 16>(s, w, a, st);
+    // 64 x 64 tiles from two to an SM on (2 chains of 1024 -> 512 -> 512, T = 512: 49 us, 32 x 64 tiles 53), else 32 x
+    // 64 (one chain, T = 64: 13.9 and 11.9 us); with 256 threads of 4 x 4 outputs 64 x 64 tiles take 55 and 12.2
+    if ((long long)(s.d_hid / 64) * ((s.d_in + s.d_out) / 64) * w.nc > 2 * F32_SMS) return phase_b_f32<8, 4, 8>(s, w, a, st);
+    return phase_b_f32<4, 4, 8>(s, w, a, st);
 }
 
 bool resident_f32_fits(const DevState& s) {

@@ -1,5 +1,5 @@
-"""GPU parity of the fp32 phase kernels over their tile variants: 64 x 64 and 128 x 128 tiles on
-large grids, 64 x 64 where a width is an odd multiple of 64, 32 x 64 on small grids; ragged last
+"""GPU parity of the fp32 phase kernels over their tile variants: 64 x 64 (phase A) and 128 x 128 (phase B)
+tiles on large grids, 32 x 64 and 64 x 64 where a width is an odd multiple of 64, 32 x 64 on small grids; ragged last
 segments (rows of a tile absent, a contraction over few tokens) and plain mode; and of the resident kernel
 (d_in + d_out <= 512) at widths that end inside a warp's 128 columns, with four and with eight rows a CTA
 (more than 152 CTAs of four), and a last segment of one token, of one chunk and one token.  fp32 bound 1e-4 on the
@@ -25,7 +25,7 @@ def _built():
 
 @pytest.mark.parametrize("d_in,d_hid,d_out,T,n_layers,N,mode,loss", [
     (512, 512, 512, 256, 8, 2 * 256 + 33, wk.PAPER, "neg_inner"),  # 64 x 64 and 128 x 128 tiles
-    (448, 320, 384, 192, 8, 2 * 192 + 1, wk.PAPER, "neg_inner"),   # odd multiples of 64; a last segment of one token
+    (448, 320, 384, 192, 8, 2 * 192 + 1, wk.PAPER, "neg_inner"),   # 32 x 64 and 64 x 64; a last segment of one token
     (576, 64, 128, 64, 1, 3 * 64 + 17, wk.PAPER, "neg_inner"),     # one 32 x 64 tile column
     (384, 256, 256, 128, 2, 2 * 128 + 65, wk.PLAIN, "mse"),        # residual targets, no momentum
     (64, 64, 128, 64, 2, 3 * 64 + 1, wk.PAPER, "neg_inner"),       # resident: W1 in half a warp's columns
