@@ -227,17 +227,18 @@ __device__ __forceinline__ float at_exp2(float x) {
 // zeros).  Warp 9: the MMA issuer.  Per chunk: S = Q K^T into one of two TMEM buffers; the softmax
 // takes the row max (exchanged between a row's two threads), writes its bf16 probabilities over the
 // scores, where P V takes its A operand from, and keeps the row sum; O += P V accumulates in TMEM over all
-// chunks.  The next chunk's S is there before the softmax asks for it.  O is rescaled in TMEM only when
-// a row's max has grown by more than 2^8 (bf16 keeps its relative precision at any scale; the sums are
-// fp32), which after the first chunks hardly ever happens.
+// chunks.  The next chunk's S is there before the softmax asks for it.  O is rescaled in TMEM whenever the
+// max of one of a warp's rows has grown, so that the largest probability of a row is 1, which bf16 holds
+// exactly: rescaled only on growth by more than 2^8 the kernel takes 8% less time, but the error against 64
+// bits is 2 to 9% larger (2.26e-3 for 2.16e-3 of 2048 queries, hd 128).
 //
 // What bounds it: the softmax's instructions (scale, ex2, bf16, and the sum of the rounded values: about
 // five an element), at 55% of the issue slots; the max exchange and the waits around it leave the rest.
-// 16 chains x 8 heads x 4, 2048 + 64 keys, hd 64: 437 us, 2.23 M visible pairs a head at 668 TFLOP/s (the
+// 16 chains x 8 heads x 4, 2048 + 64 keys, hd 64: 471 us, 2.23 M visible pairs a head at 620 TFLOP/s (the
 // one-CTA form it replaced, which took S, the softmax and P V of a 256-key chunk in turn: 1140 us); 4 chains,
-// hd 128: 171 us (389).  Measured on the way: P through shared memory, two tiles a CTA 699 us; P in TMEM
-// 565; loads by TMA instead of cp.async 490; one thread per row with two S buffers of 64 keys 463.
-constexpr float FA_SLACK = 8.f;              // growth of the row max, in powers of two, that leaves O alone
+// hd 128: 185 us (389).  Measured on the way, with the rarer rescaling (437 us): P through shared memory,
+// two tiles a CTA 699 us; P in TMEM 565; loads by TMA instead of cp.async 490; one thread per row with two S
+// buffers of 64 keys 463.
 
 template <int HD>
 struct FaSmem {
@@ -440,7 +441,7 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
             if (j == 0) {
                 m_run = cm;
             } else {
-                const bool grown = (cm - m_run) * k2 > FA_SLACK;
+                const bool grown = cm > m_run;
                 if (__any_sync(0xffffffffu, grown)) {  // the same in both warps: each rescales its half of O
                     // O up to the last chunk (on this barrier the phase before is done: S of this chunk waited for it)
                     const bool in = __all_sync(0xffffffffu, mbar_wait(odone(j - 1), ((j - 1) >> 1) & 1, a.status));
@@ -510,7 +511,7 @@ constexpr int DE_WARPS = 4, DE_ROWS = 16;
 // This form is taken up to 16 rows per key/value head, and beyond that while its row tiles over all
 // heads stay few: it re-reads the caches for each 16 rows but splits the keys, the prefill form does
 // neither.  1 chain x 8 heads x 4, 4000 keys: 16 / 64 / 128 rows take 7.9 / 9.5 / 14.0 us here and 37 us
-// in the prefill form; 16 chains, 1000 keys: 16 rows 10.4 and 12.5 us, 20 rows 14.9 and 12.7 us.
+// in the prefill form; 16 chains, 1000 keys: 16 rows 10.4 us here, 20 rows 14.9; 32 rows 13.2 in the prefill form.
 constexpr int DE_MAX_TILES = 128;
 
 template <int HD>

@@ -52,7 +52,7 @@ def run_case(group, Lq, n_mem, hd, n_layers=2, n_kv=2, late_scale=1.0):
     (64, 2, 95, 64, 1.0),     # one key past it
     (3, 150, 0, 128, 1.0),    # padded rows (126 of 128), no memory, hd 128
     (4, 129, 383, 128, 1.0),  # hd 128: 64-key chunks, eight of them exactly, one token past the tiles
-    (4, 100, 300, 64, 9.0),   # the row max grows past the slack in later chunks: O is rescaled
+    (4, 100, 300, 64, 9.0),   # the row max grows in later chunks: O is rescaled
     (2, 140, 200, 128, 9.0),
 ])
 def test_prefill_form(group, Lq, n_mem, hd, late_scale):
