@@ -319,11 +319,9 @@ mone_status build_input_maps(const DevState& s, TcInputMaps* in, const void* X, 
                              long long rows, int chains) {
     const int dh = s.d_out / 2;
     bool ok = encode_map_bf16_3d(&in->Ka, K, dh, rows, chains, 64, 128) &&
-              encode_map_bf16_blocks(&in->Kb, K, dh, rows, chains, 64, 4) &&
-              encode_map_bf16_blocks(&in->Kb2, K, dh, rows, chains, 64, 2) &&
+              encode_map_bf16_blocks(&in->Kb, K, dh, rows, chains, 64, 2) &&
               encode_map_bf16_3d(&in->Va, V, dh, rows, chains, 64, 128) &&
-              encode_map_bf16_blocks(&in->Vb, V, dh, rows, chains, 64, 4) &&
-              encode_map_bf16_blocks(&in->Vb2, V, dh, rows, chains, 64, 2);
+              encode_map_bf16_blocks(&in->Vb, V, dh, rows, chains, 64, 2);
     if (ok && s.mode == MONE_PLAIN)
         ok = encode_map_bf16_3d(&in->Xa, X, s.d_in, rows, chains, 64, 128) &&
              encode_map_bf16_blocks(&in->Xb, X, s.d_in, rows, chains, 64, 4) &&

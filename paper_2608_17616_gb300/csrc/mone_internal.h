@@ -191,8 +191,8 @@ struct TcMaps {
     CUtensorMap Amse;                // squared-error activations, K-major {64, 128}
 };
 struct TcInputMaps {
-    // per call: K-major {64,128} (a), MN-major blocks of 256 columns (b) and of 128 (b2, CTA pairs)
-    CUtensorMap Xa, Xb, Xb2, Ka, Kb, Kb2, Va, Vb, Vb2;
+    // per call: K-major {64,128} (a), MN-major blocks (b): 256 columns of X, 128 of X (b2, CTA pairs), K and V
+    CUtensorMap Xa, Xb, Xb2, Ka, Kb, Va, Vb;
 };
 cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                               cudaStream_t st);

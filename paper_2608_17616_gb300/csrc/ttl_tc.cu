@@ -84,7 +84,7 @@ struct TcArgs {
     int* status;
     int r_only;                 // phase A pairs: At and c SiLU'(x) / |z| come from the squared-error
                                 // pre-pass (the latter in dH); accumulate R only and form dH in place
-    int store_lag;              // phase B: state stores in flight (4 or 2 of the ring's 8 slots)
+    int store_mode;             // phase B: when the state ring's slots are handed back (S_LAG3, ..)
     unsigned long long wait_ns; // limit of every mbarrier wait of the launch (kWaitLimitNs)
     int stall;                  // test knob (phase A): the producer issues no loads, so the first
                                 // wait for a full stage runs out; nothing is in flight when it does
@@ -901,9 +901,10 @@ tc_phase_a_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_co
 
 // ------------------------------------------------------------------ phase B
 //
-// Tile = 128 hidden rows x 256 weight columns of W1, or of the K or V half of W2 (128 columns
-// where a width leaves that remainder), accumulated with TMEM lane = hidden row: D = dH^T U or
-// At^T Y, both operands MN-major, one TMA box per operand and 64-token k-block.
+// Tile = 128 hidden rows x 256 weight columns of W1 or of W2 (128 columns of W1 where d_in leaves that
+// remainder), accumulated with TMEM lane = hidden row: D = dH^T U or
+// At^T Y, both operands MN-major, per 64-token k-block one TMA box of dH or At and of U, two of Y (a tile of W2 may
+// take 128 columns from K and 128 from V).
 //
 // Warps: 0 operand producer (TMA), 1 MMA issuer, 2..9 update, 10 state producer, 11 store warp.
 // The fp32 state of a tile moves in chunks of 32 rows x 64 columns of W and mu (16 KB, one TMA box)
@@ -928,6 +929,8 @@ tc_phase_a_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_co
 
 constexpr int S_ROWS = 32, S_COLS = 64;                    // state chunk: hidden rows x weight columns
 constexpr int S_SLOTS = 8;
+// when slots are handed back: one, three stores later; two at a time, three or one later
+enum { S_LAG3 = 0, S_PAIRS3 = 1, S_PAIRS1 = 2 };
 constexpr int S_F32 = S_ROWS * S_COLS * 4;                 // 8 KB
 constexpr int S_SLOT = 2 * S_F32;                          // W and mu: 16 KB
 constexpr int B_THREADS = 12 * 32;
@@ -953,41 +956,37 @@ using LayoutB = LayoutBT<false>;
 using LayoutB2 = LayoutBT<true>;
 static_assert(LayoutB::DYN <= 227 * 1024 && LayoutB2::DYN <= 227 * 1024, "phase B shared memory budget");
 
-// Column tiles of [W1 | W2]: each lies in W1, or in the K or the V half of W2.
-__host__ __device__ constexpr int b_col_tiles(int d_in, int d_out) {
-    return (d_in + B_BN - 1) / B_BN + 2 * ((d_out / 2 + B_BN - 1) / B_BN);
-}
+// Column tiles of [W1 | W2]: each lies in W1 or in W2 (a tile of W2 may take half its columns from K and half
+// from V: d_out is a multiple of 256, its half of 128).
+__host__ __device__ constexpr int b_col_tiles(int d_in, int d_out) { return (d_in + B_BN - 1) / B_BN + d_out / B_BN; }
 
 // The tiles one CTA of phase B walks: t = first, first + step, ... < count.
 template <bool PAIR>
 struct BTiles {
-    int first, step, count, n_ht, n_ct, n1, nk, rank, d_in, dhalf;
+    int first, step, count, n_ht, n_ct, n1, rank, d_in;
     __device__ BTiles(const TcArgs& a) {
         d_in = a.d_in;
-        dhalf = a.d_out / 2;
         n_ht = a.d_hid / (PAIR ? 2 * B_BM : B_BM);
         n1 = (d_in + B_BN - 1) / B_BN;
-        nk = (dhalf + B_BN - 1) / B_BN;
-        n_ct = n1 + 2 * nk;
+        n_ct = b_col_tiles(a.d_in, a.d_out);
         count = a.nc * n_ht * n_ct;
         rank = PAIR ? (int)cluster_ctarank() : 0;
         first = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
         step = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     }
-    // tile t: chain of the launch, this CTA's first hidden row, source of the columns (0: U, W1;
-    // 1: K, 2: V, of W2), first column within the source and within its matrix, live columns
+    // tile t: chain of the launch, this CTA's first hidden row, matrix (0: U, W1; 1: Y, W2), first column within
+    // it, live columns
     struct Tile {
-        int cz, h0, src, scol, mcol, ncol;
+        int cz, h0, m, col, ncol;
     };
     __device__ Tile decode(int t) const {
         Tile x;
         x.cz = t / (n_ht * n_ct);
         x.h0 = ((t / n_ct) % n_ht) * (PAIR ? 2 * B_BM : B_BM) + rank * B_BM;
         const int c = t % n_ct;
-        x.src = c < n1 ? 0 : (c < n1 + nk ? 1 : 2);
-        x.scol = (x.src == 0 ? c : (c - n1) % nk) * B_BN;
-        x.mcol = x.scol + (x.src == 2 ? dhalf : 0);
-        x.ncol = min(B_BN, (x.src == 0 ? d_in : dhalf) - x.scol);
+        x.m = c < n1 ? 0 : 1;
+        x.col = (x.m ? c - n1 : c) * B_BN;
+        x.ncol = x.m ? B_BN : min(B_BN, d_in - x.col);
         return x;
     }
 };
@@ -1069,11 +1068,13 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
             bool ok = true;
             for (int t = tl.first; t < tl.count && ok; t += tl.step) {
                 const Tile x = tl.decode(t);
-                const CUtensorMap* ma = x.src == 0 ? &tmDH : &tmAT;
-                const CUtensorMap* mb = x.src == 0 ? &tmUb : (x.src == 1 ? &tmKb : &tmVb);
-                const int y0 = x.src == 0 ? a.u_row0 : a.y_row0, z = x.src == 0 ? a.u_chain0 + x.cz : x.cz;
-                // this CTA's share of the columns: all 256 (blocks past the source read as zeros), or 128 of a pair
-                const int blk = (x.scol + (PAIR ? tl.rank * (B_BN / 2) : 0)) / 64;
+                const CUtensorMap* ma = x.m ? &tmAT : &tmDH;
+                // this CTA's share of the columns: all 256, or 128 of a pair; of W2 128 at a time from K or V
+                const int col = x.col + (PAIR ? tl.rank * (B_BN / 2) : 0), dhalf = a.d_out / 2;
+                auto load_y = [&](int c, auto&& load) {
+                    const bool v = c >= dhalf;
+                    load(v ? &tmVb : &tmKb, (v ? c - dhalf : c) / 64);
+                };
                 for (int kb = 0; kb < KB; ++kb, ++kc) {
                     const int s = kc % NS;
                     if (kc >= NS && !mbar_wait(empty(s), ((kc / NS) - 1) & 1, a.status, a.wait_ns)) {
@@ -1085,11 +1086,24 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
                         const uint32_t fb = map_to_cta(full(s), 0);  // both CTAs' loads complete on rank 0's barrier
                         if (tl.rank == 0) mbar_expect_tx(full(s), 2 * L::STAGE);
                         tma_load_4d_pair(sa, ma, fb, 0, kb * BK, x.h0 / 64, a.c0 + x.cz);
-                        tma_load_4d_pair(sb, mb, fb, 0, y0 + kb * BK, blk, z);
+                        if (x.m)
+                            load_y(col, [&](const CUtensorMap* mb, int blk) {
+                                tma_load_4d_pair(sb, mb, fb, 0, a.y_row0 + kb * BK, blk, x.cz);
+                            });
+                        else
+                            tma_load_4d_pair(sb, &tmUb, fb, 0, a.u_row0 + kb * BK, col / 64, a.u_chain0 + x.cz);
                     } else {
                         mbar_expect_tx(full(s), L::STAGE);
                         tma_load_4d(sa, ma, full(s), 0, kb * BK, x.h0 / 64, a.c0 + x.cz);
-                        tma_load_4d(sb, mb, full(s), 0, y0 + kb * BK, blk, z);
+                        if (x.m) {
+#pragma unroll
+                            for (int hb = 0; hb < 2; ++hb)
+                                load_y(col + hb * 128, [&](const CUtensorMap* mb, int blk) {
+                                    tma_load_4d(sb + hb * 2 * BOX, mb, full(s), 0, a.y_row0 + kb * BK, blk, x.cz);
+                                });
+                        } else {  // blocks past d_in read as zeros
+                            tma_load_4d(sb, &tmUb, full(s), 0, a.u_row0 + kb * BK, col / 64, a.u_chain0 + x.cz);
+                        }
                     }
                 }
             }
@@ -1153,14 +1167,14 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
                         ok = false;
                         break;
                     }
-                    const int col = x.mcol + chunk_col(i);
+                    const int col = x.col + chunk_col(i);
                     // the chunk lies inside the matrix (a tiled copy's block coordinate counts 32 columns)
-                    if (!MONE_DCHECK((col & 31) == 0 && col + S_COLS <= (x.src ? a.d_out : a.d_in), a.status, DS_TMA_X)) {
+                    if (!MONE_DCHECK((col & 31) == 0 && col + S_COLS <= (x.m ? a.d_out : a.d_in), a.status, DS_TMA_X)) {
                         ok = false;
                         break;
                     }
                     mbar_expect_tx(sfull(k), chunk_bytes);
-                    tma_load_5d(smem_u32(base + L::STATE + k * S_SLOT), x.src ? &tmW2s : &tmW1s, sfull(k), 0,
+                    tma_load_5d(smem_u32(base + L::STATE + k * S_SLOT), x.m ? &tmW2s : &tmW1s, sfull(k), 0,
                                 x.h0 + chunk_row(i), col / 32, a.c0 + x.cz, 0);
                 }
             }
@@ -1179,16 +1193,28 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
                         ok = false;
                         break;
                     }
-                    tma_store_5d(x.src ? &tmW2s : &tmW1s, smem_u32(base + L::STATE + k * S_SLOT), 0,
-                                 x.h0 + chunk_row(i), (x.mcol + chunk_col(i)) / 32, a.c0 + x.cz, 0);
+                    tma_store_5d(x.m ? &tmW2s : &tmW1s, smem_u32(base + L::STATE + k * S_SLOT), 0,
+                                 x.h0 + chunk_row(i), (x.col + chunk_col(i)) / 32, a.c0 + x.cz, 0);
                     bulk_commit();
-                    // hand back the slot of the store `lag` before this one, which has been read by now: the
-                    // ring's slots are split between lag stores and S_SLOTS - lag loads in flight
-                    if (a.store_lag == 4)
-                        bulk_wait_read<4>();
-                    else
-                        bulk_wait_read<2>();
-                    if (seq >= (uint32_t)a.store_lag) mbar_arrive(sempty((seq - a.store_lag) % S_SLOTS));
+                    // hand slots back whose stores have read them: the ring's slots are split between stores
+                    // and loads in flight
+                    if (a.store_mode == S_LAG3) {
+                        bulk_wait_read<3>();
+                        if (seq >= 3) mbar_arrive(sempty((seq - 3) % S_SLOTS));
+                    } else if (!(seq & 1) && seq) {  // two slots at a time
+                        uint32_t done;  // stores up to this one have been read
+                        if (a.store_mode == S_PAIRS3) {
+                            bulk_wait_read<3>();
+                            done = seq - 3;
+                        } else {
+                            bulk_wait_read<1>();
+                            done = seq - 1;
+                        }
+                        if ((int)done > 0) {
+                            mbar_arrive(sempty((done - 1) % S_SLOTS));
+                            mbar_arrive(sempty(done % S_SLOTS));
+                        }
+                    }
                 }
             }
             bulk_wait_all();
@@ -1206,13 +1232,13 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
         int local = 0;
         for (int t = tl.first; t < tl.count; t += tl.step, ++local) {
             const Tile x = tl.decode(t);
-            const int cs = a.c0 + x.cz, which = x.src ? 1 : 0, width = x.src ? a.d_out : a.d_in;
+            const int cs = a.c0 + x.cz, which = x.m ? 1 : 0, width = x.m ? a.d_out : a.d_in;
             const int b = local & 1, row = x.h0 + q * 32 + lane;
             // the tile's rows and columns lie inside the chain's W (index check of MONE_DEBUG builds)
-            const bool wr = MONE_DCHECK(cs < a.C && row < a.d_hid && x.mcol + x.ncol <= width, a.status, DS_PHASE_B_TILE);
+            const bool wr = MONE_DCHECK(cs < a.C && row < a.d_hid && x.col + x.ncol <= width, a.status, DS_PHASE_B_TILE);
             float sc = 1.f, beta = 0.f;
             if (a.renorm_pending && wr)
-                sc = renorm_scale((x.src ? a.n2 : a.n1)[(size_t)cs * a.d_hid + row], ss_row(a, a.parity ^ 1, which, cs)[row]);
+                sc = renorm_scale((x.m ? a.n2 : a.n1)[(size_t)cs * a.d_hid + row], ss_row(a, a.parity ^ 1, which, cs)[row]);
             if (a.momentum) {  // beta_s = sigmoid(mean_t w_beta . x_t + b_beta)
                 const float* db = a.dbeta + (size_t)cs * a.win + a.tok0;
                 float v = 0.f;
@@ -1226,7 +1252,7 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
             tc_fence_after();
             const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + b * B_BN + half * S_COLS;
             float ss = 0.f, step = 0.f;  // sums of squares of this lane's part of its row of W, and of mu
-            bf16* wrow = (x.src ? a.W2b : a.W1b) + ((size_t)cs * a.d_hid + row) * width + x.mcol + half * S_COLS;
+            bf16* wrow = (x.m ? a.W2b : a.W1b) + ((size_t)cs * a.d_hid + row) * width + x.col + half * S_COLS;
 #pragma unroll 1
             for (int cg = 0; cg < ncg; ++cg) {
                 const uint32_t seq = tile_seq0 + cg * S_SLOTS + q * 2 + half;
@@ -2193,24 +2219,31 @@ cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputM
     cudaError_t e = ensure_attrs();
     if (e != cudaSuccess) return e;
     TcArgs a = make_args(s, w);
-    // The state ring's 8 slots: with short segments the state stream alone sets the pace and four
-    // stores with four loads in flight suit HBM best (128 chains, T = 256, 2K tokens: 14.95 ms with 2
-    // stores in flight, 14.93 with 3, 14.32 with 4, 18.1 with 6); from T = 512 on more loads in
-    // flight win (16 chains, T = 512, 32K tokens: 13.81 / 13.74 / 14.14 ms with 2 / 3 / 4).
-    a.store_lag = s.T <= 256 ? 4 : 2;
-    const CUtensorMap& U = s.mode == 1 ? m.Ub : in.Xb;
-    const CUtensorMap& U2 = s.mode == 1 ? m.Ub2 : in.Xb2;
-    const int col_tiles = b_col_tiles(s.d_in, s.d_out);
     // CTA pairs over 256-hidden x 256-column tiles (a tile's columns all live) from T = 1024 on:
     // there a tile's operand stream (768 KB a CTA) rivals its state stream, and the pair takes a
     // third off it.  At T = 512 the pair's coupled loads and accumulator release cost more than they save.
     constexpr int PAIR_MIN_T = 1024;
-    if (s.T >= PAIR_MIN_T && s.d_in % B_BN == 0 && (s.d_out / 2) % B_BN == 0 && g_pairb_clusters > 0) {
+    const bool pairs = s.T >= PAIR_MIN_T && s.d_in % B_BN == 0 && g_pairb_clusters > 0;
+    // When the state ring's slots are handed back, by what was fastest: how stores and loads alternate
+    // decides how much of HBM the stream gets.  With no momentum, on CTA pairs, for one chain, or with W and mu of
+    // the whole handle in L2, two at a time, one store later (ms, against one by one three stores later: 64 plain chains of
+    // 2048 -> 1024 -> 1024, T = 256: 7.68 and 8.13; 28 chains, T = 1024, 4K tokens: 7.91 and 7.99; 4 chains 1.33 and
+    // 1.36).  With a large state from T = 256 on two at a time, three stores later (56 chains, T = 512: 9.81 and
+    // 10.41; 30 chains 3.86 and 3.98), else one by one (16 chains, T = 512: 5.22 and 5.39; 28 chains, T = 128: 9.74
+    // and 10.1).
+    const long long state = (long long)s.C * s.d_hid * (s.d_in + s.d_out) * 8;
+    a.store_mode = pairs || !s.momentum || w.single || state < 128000000 ? S_PAIRS1
+                   : s.T >= 256 && state > (s.T >= 512 ? 740000000 : 800000000) ? S_PAIRS3
+                                                                               : S_LAG3;
+    const CUtensorMap& U = s.mode == 1 ? m.Ub : in.Xb;
+    const CUtensorMap& U2 = s.mode == 1 ? m.Ub2 : in.Xb2;
+    const int col_tiles = b_col_tiles(s.d_in, s.d_out);
+    if (pairs) {
         const int npairs = w.nc * col_tiles * (s.d_hid / (2 * B_BM));
         const int maxc = g_pairb_clusters - (s.reserve_sms + 1) / 2;
         const int clusters = npairs < maxc ? npairs : maxc;
         return launch_kernel(a.step_sq ? tc_phase_b_kernel<true, true> : tc_phase_b_kernel<true, false>, dim3(2 * clusters),
-                             dim3(B_THREADS), LayoutB2::DYN, st, w.single != 0, 2, U2, in.Kb2, in.Vb2, m.dH, m.At, m.W1s,
+                             dim3(B_THREADS), LayoutB2::DYN, st, w.single != 0, 2, U2, in.Kb, in.Vb, m.dH, m.At, m.W1s,
                              m.W2s, a);
     }
     const int ntiles = w.nc * col_tiles * (s.d_hid / B_BM);

@@ -1,7 +1,7 @@
 """GPU parity of phase B where its column tiles and state ring can go wrong: widths that leave a
-128-column tile in W1 and in the halves of W2, launches of more than one tile per CTA (wide and narrow
-tiles through the same ring), both splits of the ring (T <= 256 and above), plain mode (no momentum
-in the ring) and the CTA-pair form.  Bounds as in test_parity_gpu.py: 2e-2 on the weights and on
+128-column tile in W1, tiles of W2 that take half their columns from K and half from V, launches of
+more than one tile per CTA (wide and narrow tiles through the same ring), the three ways the ring's slots
+are handed back (plain mode, CTA pairs and a small state; a large state; the rest) and the CTA-pair form.  Bounds as in test_parity_gpu.py: 2e-2 on the weights and on
 their change."""
 import pytest
 import torch
@@ -22,16 +22,19 @@ def _built():
     mone.lib()
 
 
-@pytest.mark.parametrize("d_in,d_out,T,n_layers,N,mode", [
-    (128, 256, 128, 2, 300, wk.PAPER),      # every tile narrow
-    (384, 768, 128, 30, 300, wk.PAPER),     # 256 + 128 columns in W1, K and V; 180 tiles a launch
-    (384, 768, 512, 30, 700, wk.PAPER),     # the other split of the ring
-    (640, 256, 256, 3, 513, wk.PLAIN),      # W alone in the ring; a last segment of one token
-    (512, 512, 1024, 3, 1024 + 65, wk.PAPER),  # CTA pairs
-    (512, 768, 1024, 3, 1024 + 65, wk.PAPER),  # T = 1024 with a narrow tile: one-CTA tiles
+@pytest.mark.parametrize("d_in,d_hid,d_out,T,n_layers,N,mode", [
+    (128, 256, 256, 128, 2, 300, wk.PAPER),      # a narrow tile of W1, one of W2 from K and V
+    (384, 256, 768, 128, 30, 300, wk.PAPER),     # 256 + 128 columns in W1; 150 tiles a launch, two launches
+    (384, 256, 768, 512, 30, 700, wk.PAPER),     # the same in longer segments
+    (384, 768, 768, 256, 20, 600, wk.PAPER),     # a state above 128 MB: slots one by one; several tiles a CTA
+    (1152, 2048, 1280, 256, 22, 513, wk.PAPER),  # a state above 800 MB: slots two at a time, three stores later
+    (640, 256, 256, 256, 3, 513, wk.PLAIN),      # W alone in the ring; a last segment of one token
+    (512, 256, 512, 1024, 3, 1024 + 65, wk.PAPER),  # CTA pairs
+    (512, 256, 768, 1024, 3, 1024 + 65, wk.PAPER),  # CTA pairs, a tile from K and V
+    (640, 256, 768, 1024, 3, 1024 + 65, wk.PAPER),  # T = 1024 with a narrow tile: one-CTA tiles
 ])
-def test_phase_b_tiles(d_in, d_out, T, n_layers, N, mode):
-    wl = wk.Workload("phase_b", 12, 1, n_layers, d_in, 256, d_out, d_out // 128, 64, T, N, 8, "bf16", mode,
+def test_phase_b_tiles(d_in, d_hid, d_out, T, n_layers, N, mode):
+    wl = wk.Workload("phase_b", 12, 1, n_layers, d_in, d_hid, d_out, d_out // 128, 64, T, N, 8, "bf16", mode,
                      0.3 if mode == wk.PAPER else 0.05)
     run = DeviceRun(wl)
     run.ttl_context()
