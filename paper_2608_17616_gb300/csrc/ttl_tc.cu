@@ -12,7 +12,7 @@
 //     Writes dH and At row-major (bf16 [token][hidden]) and the loss partial
 //     sum_t sum_h A_th R_th = sum_t y_t . M(u_t).
 //
-//   phase B, tile = (chain, 128 hidden units, 256 columns of W1 or of a half of W2)
+//   phase B, tile = (chain, 128 hidden units, 256 columns of W1 or of W2)
 //       G1 = dH^T U           K = T'        (gradient of W1)
 //       G2 = At^T Y           K = T'        (gradient of W2)
 //     Both operands are read MN-major straight from the row-major buffers.
@@ -21,7 +21,8 @@
 //     (s = the previous segment's pending row renormalisation); it writes W,
 //     mu, the bf16 operand copy and the new row sums of squares.
 //
-// Both kernels: one CTA per SM, persistent over a static tile schedule, 10 warps.
+// Both kernels: one CTA per SM, persistent over a static tile schedule, 10 warps (phase B two more, which move
+// the fp32 state).
 // Warp 0 lane 0 streams operand tiles with TMA into a shared-memory ring
 // (128-byte swizzle), warp 1 lane 0 issues tcgen05.mma into one of two TMEM
 // accumulator buffers, warps 2..9 drain the other buffer, so the epilogue of
