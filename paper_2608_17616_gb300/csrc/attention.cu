@@ -18,6 +18,7 @@
 #include <mutex>
 
 #include "mone_common.cuh"
+#include "per_device.h"
 
 namespace mone {
 
@@ -716,30 +717,11 @@ __global__ void __launch_bounds__(DE_WARPS * 32, HD == 64 ? 4 : 3) attention_dec
     if (splits > 1) cluster_sync();  // no CTA leaves while another reads its shared memory
 }
 
-std::mutex g_attr_mu;
-
-// The shared-memory opt-in belongs to a device: set it once per device and kernel (a driver
-// call on every launch would cost more than the kernel).
-template <typename K>
-cudaError_t smem_opt_in(K kernel, size_t smem, bool (&done)[64]) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lk(g_attr_mu);
-    if (!done[dev]) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        done[dev] = true;
-    }
-    return cudaSuccess;
-}
-
 template <typename T, int HD>
 cudaError_t launch_t(const AttnArgs& a, int C, cudaStream_t st) {
     const size_t smem = AttnSmem<T, HD>::FLOATS * sizeof(float);
-    static bool done[64] = {};
-    cudaError_t e = smem_opt_in(attention_kernel<T, HD>, smem, done);
+    static PerDevice<SmemOptIn> once;
+    cudaError_t e = smem_opt_in(reinterpret_cast<const void*>(attention_kernel<T, HD>), smem, once);
     if (e != cudaSuccess) return e;
     dim3 grid((a.Lq + a.rows - 1) / a.rows, a.n_kv, C);
     attention_kernel<T, HD><<<grid, ATT_WARPS * 32, smem, st>>>(a);
@@ -748,8 +730,8 @@ cudaError_t launch_t(const AttnArgs& a, int C, cudaStream_t st) {
 
 template <int HD>
 cudaError_t launch_prefill(AttnArgs a, int n_ctx, int C, cudaStream_t st) {
-    static bool done[64] = {};
-    cudaError_t e = smem_opt_in(attention_prefill_kernel<HD>, FaSmem<HD>::DYN, done);
+    static PerDevice<SmemOptIn> once;
+    cudaError_t e = smem_opt_in(reinterpret_cast<const void*>(attention_prefill_kernel<HD>), FaSmem<HD>::DYN, once);
     if (e != cudaSuccess) return e;
     const int rows0 = a.rows;
     a.rows = 128 / a.group;  // tokens per tile: the group's heads x rows fill the 128 MMA rows
@@ -775,9 +757,9 @@ cudaError_t launch_prefill(AttnArgs a, int n_ctx, int C, cudaStream_t st) {
 
 template <int HD>
 cudaError_t launch_decode(const AttnArgs& a, int C, cudaStream_t st) {
-    static bool done[64] = {};
+    static PerDevice<SmemOptIn> once;
     constexpr size_t smem = DeSmem<HD>::FLOATS * sizeof(float);
-    cudaError_t e = smem_opt_in(attention_decode_kernel<HD>, smem, done);
+    cudaError_t e = smem_opt_in(reinterpret_cast<const void*>(attention_decode_kernel<HD>), smem, once);
     if (e != cudaSuccess) return e;
     const int row_tiles = (a.group * a.Lq + DE_ROWS - 1) / DE_ROWS;
     // split the keys over a cluster until the grid fills the SMs' CTA slots, or a CTA's warps would

@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "mone_common.cuh"
+#include "per_device.h"
 
 namespace mone {
 
@@ -1088,25 +1089,24 @@ __global__ void __launch_bounds__(256) read_norm_kernel(DevState s, int Q, Tout*
 }  // namespace
 
 namespace {
-// Launch a phase kernel of the fp32 path (its shared memory opted in on first use).
+// Launch a phase kernel of the fp32 path.
 template <typename K>
-cudaError_t launch_f32_tiles(K kernel, int threads, size_t smem, std::once_flag& once, dim3 grid, const F32SegArgs& a,
+cudaError_t launch_f32_tiles(K kernel, int threads, size_t smem, PerDevice<SmemOptIn>& once, dim3 grid, const F32SegArgs& a,
                              cudaStream_t st) {
-    cudaError_t e = cudaSuccess;
-    std::call_once(once, [&] { e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
+    const cudaError_t e = smem_opt_in(reinterpret_cast<const void*>(kernel), smem, once);
     if (e != cudaSuccess) return e;
     kernel<<<grid, threads, smem, st>>>(a);
     return cudaGetLastError();
 }
 template <int TM, int TN, int TY>
 cudaError_t phase_a_f32(const DevState& s, const SegWork& w, const F32SegArgs& a, cudaStream_t st) {
-    static std::once_flag once;
+    static PerDevice<SmemOptIn> once;
     return launch_f32_tiles(phase_a_f32_kernel<TM, TN, TY>, 16 * TY, nt_smem<TM, TN, TY>(), once,
                             dim3(s.T / (TY * TM), s.d_hid / (16 * TN), w.nc), a, st);
 }
 template <int TM, int TN, int TY>
 cudaError_t phase_b_f32(const DevState& s, const SegWork& w, const F32SegArgs& a, cudaStream_t st) {
-    static std::once_flag once;
+    static PerDevice<SmemOptIn> once;
     return launch_f32_tiles(phase_b_f32_kernel<TM, TN, TY>, 16 * TY, tn_smem<TM, TN, TY>(), once,
                             dim3((s.d_in + s.d_out) / (16 * TN), s.d_hid / (TY * TM), w.nc), a, st);
 }
@@ -1169,19 +1169,13 @@ cudaError_t launch_resident_f32(const DevState& s, const SegWork& w, long long n
     a.step_sq = w.step0;
     a.m_sstride = w.loss0 || w.step0 ? w.mstride : 0;
     a.status = s.status;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
     // four rows a CTA while that still fits the chains in one wave, else eight (less re-streaming)
     const int D = s.d_in + s.d_out;
-    static std::once_flag once;
-    std::call_once(once, [&] {
-        e = cudaFuncSetAttribute(ttl_resident_f32_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_smem_bytes<4>(512));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(ttl_resident_f32_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)res_smem_bytes<8>(512));
-    });
+    static PerDevice<SmemOptIn> once4, once8;
+    if (e == cudaSuccess) e = smem_opt_in(reinterpret_cast<const void*>(ttl_resident_f32_kernel<4>), res_smem_bytes<4>(512), once4);
+    if (e == cudaSuccess) e = smem_opt_in(reinterpret_cast<const void*>(ttl_resident_f32_kernel<8>), res_smem_bytes<8>(512), once8);
     if (e != cudaSuccess) return e;
     if ((long long)w.nc * (s.d_hid / 4) <= sms)
         ttl_resident_f32_kernel<4><<<dim3(s.d_hid / 4, w.nc), RES_NT, res_smem_bytes<4>(D), st>>>(a);

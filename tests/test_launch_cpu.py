@@ -1,0 +1,57 @@
+"""Host code of the launches, on a CUDA runtime without a GPU: two devices in one process."""
+import shutil
+
+import pytest
+
+import paper_2608_17616_gb300 as mone
+from fakert import Fake, build_fake
+
+P = 1 << 30  # a made-up, aligned device address
+
+
+@pytest.fixture()
+def fake(tmp_path, monkeypatch, built):
+    # a copy of its own for each test: the library's per-process state starts empty
+    path = shutil.copy(built, tmp_path / "libmone_fakert.so")
+    f = Fake(str(path))
+    monkeypatch.setattr(mone, "_lib", mone.lib(str(path)))
+    return f
+
+
+@pytest.fixture(scope="module")
+def built(tmp_path_factory):
+    return build_fake(tmp_path_factory.mktemp("fakert"))
+
+
+def init(n_layers, d_in, d_hid, d_out, T, dtype, mode=mone.MONE_PLAIN, n_ctx=1, hd=64, **kw):
+    meta = {k: P for k in ("alpha", "gamma", "w_eta", "b_eta", "w_beta", "b_beta", "gate")} if mode == mone.MONE_PAPER else None
+    cfg = mone.make_config(n_ctx, n_layers, d_in, d_hid, d_out, d_out // (2 * hd), hd, T, dtype, mode, 1e-2, **kw)
+    return mone.mone_mem_init(cfg, P, P, meta, 0)
+
+
+F32_SHAPES = [
+    (1, 256, 512, 256, 128),     # resident chain, four rows a CTA
+    (8, 256, 512, 256, 128),     # resident chain, eight rows
+    (4, 1024, 1024, 1024, 256),  # 64 x 64 tiles of phase A (55,296 bytes), 128 x 128 of phase B
+]
+
+
+@pytest.mark.parametrize("shape", F32_SHAPES)
+def test_fp32_learning_on_either_device(fake, shape):
+    for dev in (0, 1, 0):
+        fake.device(dev)
+        h = init(*shape, mone.MONE_FP32)
+        mone.mone_ttl_context(h, P, P, P, 1000, 0)
+        launches, _ = fake.drain()
+        assert launches and {x["dev"] for x in launches} == {dev}
+        mone.mone_mem_free(h)
+
+
+@pytest.mark.parametrize("shape", F32_SHAPES)
+def test_a_failed_opt_in_is_reported_and_tried_again(fake, shape):
+    h = init(*shape, mone.MONE_FP32)
+    fake.fail_opt_ins(1)
+    with pytest.raises(mone.MoneError):
+        mone.mone_ttl_context(h, P, P, P, 1000, 0)
+    mone.mone_ttl_context(h, P, P, P, 1000, 0)
+    mone.mone_mem_free(h)
