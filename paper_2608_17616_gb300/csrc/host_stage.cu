@@ -13,9 +13,8 @@
 // SM has beside any learning CTA (at least 195 KB), and while mone_ttl_context_host runs the
 // persistent learning kernels leave ST_GRID SMs free (DevState::reserve_sms).  8 CTAs of 512
 // threads, 8 loads in flight each, reach 210 GB/s alone.
-#include <mutex>
-
 #include "mone_common.cuh"
+#include "per_device.h"
 
 namespace mone {
 
@@ -80,18 +79,9 @@ cudaError_t launch_stage_rows(const void* const src[3], void* const dst[3], cons
     a.r0 = r0;
     a.nr = nr;
     a.C = C;
-    static std::mutex mu;
-    static bool opted_in[64] = {};  // the shared-memory opt-in belongs to a device
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static PerDevice<SmemOptIn> once;
+    const cudaError_t e = smem_opt_in(reinterpret_cast<const void*>(stage_rows_kernel), ST_SMEM, once);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lk(mu);
-    if (!opted_in[dev]) {
-        e = cudaFuncSetAttribute(stage_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM);
-        if (e != cudaSuccess) return e;
-        opted_in[dev] = true;
-    }
     stage_rows_kernel<<<ST_GRID, ST_THREADS, ST_SMEM, st>>>(a);
     return cudaGetLastError();
 }

@@ -24,9 +24,8 @@
 //                    norm kernel, since an output head of width hd may straddle two memory heads).
 // Head slices of [..][H * dh] rows are 4-D tensor maps (dh, heads, rows, chains): a box that
 // runs past a head's dh columns, or past F hidden rows, reads zeros.
-#include <mutex>
-
 #include "mone_common.cuh"
+#include "per_device.h"
 
 namespace mone {
 
@@ -829,36 +828,24 @@ __global__ void __launch_bounds__(256) swiglu_rows_kernel(SwArgs a, int mode, in
     }
 }
 
-// SM count of the current device (grid of the persistent phase A).
-int sw_sms() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) !=
-                                                      cudaSuccess || v <= 0)
-            return 1;
-        n = v;
-    }
-    return n;
-}
-
-std::once_flag g_sw_once;
-cudaError_t g_sw_err = cudaSuccess;
-
-cudaError_t sw_attrs() {
-    std::call_once(g_sw_once, [] {
-        const void* kb[] = {reinterpret_cast<const void*>(swiglu_b_kernel<false>),
-                            reinterpret_cast<const void*>(swiglu_b_kernel<true>)};
-        const void* ks[] = {reinterpret_cast<const void*>(swiglu_a_kernel), reinterpret_cast<const void*>(swiglu_rh_kernel),
-                            reinterpret_cast<const void*>(swiglu_ro_kernel)};
-        for (const void* k : kb)
-            if (g_sw_err == cudaSuccess)
-                g_sw_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SwLayoutB::DYN);
-        for (const void* k : ks)
-            if (g_sw_err == cudaSuccess)
-                g_sw_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SwLayout::DYN);
+// The current device's SM count; the first call for a device opts every kernel in to its shared memory.
+cudaError_t sw_device(int* sms) {
+    static PerDevice<int> devices;
+    const int* n;
+    const cudaError_t r = devices.get(&n, [](int& v) {
+        cudaError_t e = sm_count(&v);
+        auto opt_in = [&](auto kernel, int dyn) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+        };
+        opt_in(swiglu_b_kernel<false>, SwLayoutB::DYN);
+        opt_in(swiglu_b_kernel<true>, SwLayoutB::DYN);
+        opt_in(swiglu_a_kernel, SwLayout::DYN);
+        opt_in(swiglu_rh_kernel, SwLayout::DYN);
+        opt_in(swiglu_ro_kernel, SwLayout::DYN);
+        return e;
     });
-    return g_sw_err;
+    if (r == cudaSuccess) *sms = *n;
+    return r;
 }
 
 SwArgs sw_args(const DevState& s, const SegWork& w) {
@@ -886,12 +873,13 @@ SwArgs sw_args(const DevState& s, const SegWork& w) {
 
 cudaError_t launch_swiglu_phase_a(const DevState& s, const SwMaps& m, const SwInputMaps& in, const SegWork& w,
                                   cudaStream_t st) {
-    cudaError_t e = sw_attrs();
+    int n_sms;
+    cudaError_t e = sw_device(&n_sms);
     if (e != cudaSuccess) return e;
     SwArgs a = sw_args(s, w);
     a.nc_launch = w.nc;
     const int ntiles = (s.T / 128) * ((a.F + 127) / 128) * w.nc * a.H;
-    const int sms = sw_sms() - s.reserve_sms;  // leave the host-input gather's SMs free
+    const int sms = n_sms - s.reserve_sms;  // leave the host-input gather's SMs free
     const int grid = ntiles < sms ? ntiles : sms;
     swiglu_a_kernel<<<grid, SW_THREADS, SwLayout::DYN, st>>>(s.mode == 1 ? m.Ua : in.Xa, in.Ka, in.Va, m.W1a, m.W2a, a);
     return cudaGetLastError();
@@ -899,12 +887,13 @@ cudaError_t launch_swiglu_phase_a(const DevState& s, const SwMaps& m, const SwIn
 
 cudaError_t launch_swiglu_phase_b(const DevState& s, const SwMaps& m, const SwInputMaps& in, const SegWork& w,
                                   cudaStream_t st) {
-    cudaError_t e = sw_attrs();
+    int n_sms;
+    cudaError_t e = sw_device(&n_sms);
     if (e != cudaSuccess) return e;
     SwArgs a = sw_args(s, w);
     a.nc_launch = w.nc;
     const int ntiles = w.nc * a.H * 3 * ((a.F + SWB_N - 1) / SWB_N) * ((a.dh + 127) / 128);
-    const int sms = sw_sms() - s.reserve_sms;  // leave the host-input gather's SMs free
+    const int sms = n_sms - s.reserve_sms;  // leave the host-input gather's SMs free
     const int grid = ntiles < sms ? ntiles : sms;
     if (a.step_sq)
         swiglu_b_kernel<true><<<grid, SWB_THREADS, SwLayoutB::DYN, st>>>(s.mode == 1 ? m.Ub : in.Xb, in.Kb, in.Vb, m.PG,
@@ -925,7 +914,8 @@ cudaError_t launch_swiglu_rows(const DevState& s, int mode, int parity, int c0, 
 }
 
 cudaError_t launch_swiglu_read(const DevState& s, const SwMaps& m, const void* Uq, void* Zq, int Q, cudaStream_t st) {
-    cudaError_t e = sw_attrs();
+    int n_sms;
+    cudaError_t e = sw_device(&n_sms);
     if (e != cudaSuccess) return e;
     SegWork w{};
     w.c0 = 0;

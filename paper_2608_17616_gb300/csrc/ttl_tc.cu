@@ -31,6 +31,7 @@
 #include <mutex>
 
 #include "mone_common.cuh"
+#include "per_device.h"
 
 namespace mone {
 
@@ -2062,26 +2063,20 @@ tc_read_t_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     if (warp == 0) tmem_dealloc(tmem, RT_MAX_NT);
 }
 
-std::once_flag g_attr_once;
-cudaError_t g_attr_err = cudaSuccess;
-int g_sms = 0;
-int g_pair_clusters = 0;   // co-resident CTA pairs of the phase A pair kernel (0: use the one-CTA kernel)
-int g_pairb_clusters = 0;  // the same for the phase B pair kernel
-int g_split4 = 0, g_split2 = 0;  // co-resident clusters of the phase A split kernels
-
-template <int MODE>
-cudaError_t read_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(tc_read_kernel<MODE, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, LR::DYN);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc_read_kernel<MODE, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, LR6::DYN);
-    return e;
-}
+// What the launches need to know of a device.
+struct TcDevice {
+    int sms;
+    int pair_clusters;   // co-resident CTA pairs of the phase A pair kernel (0: use the one-CTA kernel)
+    int pairb_clusters;  // the same for the phase B pair kernel
+    int split4, split2;  // co-resident clusters of the phase A split kernels
+};
+PerDevice<TcDevice> g_devices;
 
 // Launch a read-structured kernel with the stage count that suits its grid (see LRT).
 template <int MODE>
-cudaError_t launch_read_kernel(dim3 grid, const CUtensorMap& A, const CUtensorMap& B, const ReadArgs& a,
+cudaError_t launch_read_kernel(const TcDevice& dev, dim3 grid, const CUtensorMap& A, const CUtensorMap& B, const ReadArgs& a,
                                cudaStream_t st) {
-    if ((long long)grid.x * grid.y * grid.z <= g_sms)
+    if ((long long)grid.x * grid.y * grid.z <= dev.sms)
         tc_read_kernel<MODE, 6><<<grid, R_THREADS, LR6::DYN, st>>>(A, B, a);
     else
         tc_read_kernel<MODE, 3><<<grid, R_THREADS, LR::DYN, st>>>(A, B, a);
@@ -2092,94 +2087,75 @@ cudaError_t launch_read_kernel(dim3 grid, const CUtensorMap& A, const CUtensorMa
 // an SM.  Chains of 2048 -> 1024 -> 1024 (whole reads, CTA pairs and one-CTA tiles): 64 tiles 42.5 and 36.9 us,
 // 288 tiles 53.2 and 53.5, 352 tiles 71.6 and 85.2; 288 tiles of 512 -> 256 -> 256 45.7 and 43.1.
 template <int MODE>
-cudaError_t launch_read_many(dim3 grid, const CUtensorMap& A, const CUtensorMap& B, const ReadArgs& a, cudaStream_t st) {
-    if ((long long)grid.x * grid.y * grid.z <= 2 * g_sms) return launch_read_kernel<MODE>(grid, A, B, a, st);
+cudaError_t launch_read_many(const TcDevice& dev, dim3 grid, const CUtensorMap& A, const CUtensorMap& B, const ReadArgs& a,
+                             cudaStream_t st) {
+    if ((long long)grid.x * grid.y * grid.z <= 2 * dev.sms) return launch_read_kernel<MODE>(dev, grid, A, B, a, st);
     const long long tiles = (long long)((grid.x + 1) / 2) * (grid.y / 2) * grid.z;
-    return launch_kernel(tc_read_pair_kernel<MODE>, dim3(2 * (unsigned)std::min<long long>(tiles, g_sms / 2)), dim3(RP_THREADS),
+    return launch_kernel(tc_read_pair_kernel<MODE>, dim3(2 * (unsigned)std::min<long long>(tiles, dev.sms / 2)), dim3(RP_THREADS),
                          LRP::DYN, st, false, 2, A, B, a);
 }
 
-cudaError_t ensure_attrs() {
-    std::call_once(g_attr_once, [] {
-        int dev = 0;
-        g_attr_err = cudaGetDevice(&dev);
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaFuncSetAttribute(tc_phase_a_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LA::DYN);
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaFuncSetAttribute(tc_phase_b_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              LayoutB::DYN);
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaFuncSetAttribute(tc_phase_b_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              LayoutB::DYN);
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaFuncSetAttribute(tc_phase_b_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              LayoutB2::DYN);
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaFuncSetAttribute(tc_phase_b_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              LayoutB2::DYN);
-        if (g_attr_err == cudaSuccess)
-            g_attr_err =
-                cudaFuncSetAttribute(tc_phase_a_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LP::DYN);
-        if (g_attr_err == cudaSuccess) g_attr_err = read_attrs<0>();
-        if (g_attr_err == cudaSuccess) g_attr_err = read_attrs<64>();
-        if (g_attr_err == cudaSuccess) g_attr_err = read_attrs<128>();
-        if (g_attr_err == cudaSuccess) g_attr_err = read_attrs<MSE_HIDDEN>();
-        if (g_attr_err == cudaSuccess) g_attr_err = read_attrs<MSE_OUT>();
-        for (auto fn : {tc_read_pair_kernel<READ_HIDDEN>, tc_read_pair_kernel<64>, tc_read_pair_kernel<128>})
-            if (g_attr_err == cudaSuccess) g_attr_err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, LRP::DYN);
-        for (auto fn : {tc_read_t_kernel<0>, tc_read_t_kernel<64>, tc_read_t_kernel<128>})
-            if (g_attr_err == cudaSuccess)
-                g_attr_err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, rt_dyn(RT_MAX_NT));
-        if (g_attr_err == cudaSuccess) {
+// The current device's TcDevice; the first call for a device opts every kernel in to its shared memory.
+cudaError_t tc_device(const TcDevice** out) {
+    return g_devices.get(out, [](TcDevice& d) {
+        cudaError_t e = sm_count(&d.sms);
+        auto opt_in = [&](auto kernel, int dyn) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+        };
+        opt_in(tc_phase_a_kernel, LA::DYN);
+        opt_in(tc_phase_a_pair_kernel, LP::DYN);
+        opt_in(tc_phase_a_split_kernel<4>, LSplit<4>::DYN);
+        opt_in(tc_phase_a_split_kernel<2>, LSplit<2>::DYN);
+        opt_in(tc_phase_b_kernel<false, false>, LayoutB::DYN);
+        opt_in(tc_phase_b_kernel<false, true>, LayoutB::DYN);
+        opt_in(tc_phase_b_kernel<true, false>, LayoutB2::DYN);
+        opt_in(tc_phase_b_kernel<true, true>, LayoutB2::DYN);
+        for (auto fn : {tc_read_kernel<0, 3>, tc_read_kernel<64, 3>, tc_read_kernel<128, 3>, tc_read_kernel<MSE_HIDDEN, 3>,
+                        tc_read_kernel<MSE_OUT, 3>})
+            opt_in(fn, LR::DYN);
+        for (auto fn : {tc_read_kernel<0, 6>, tc_read_kernel<64, 6>, tc_read_kernel<128, 6>, tc_read_kernel<MSE_HIDDEN, 6>,
+                        tc_read_kernel<MSE_OUT, 6>})
+            opt_in(fn, LR6::DYN);
+        for (auto fn : {tc_read_pair_kernel<READ_HIDDEN>, tc_read_pair_kernel<64>, tc_read_pair_kernel<128>}) opt_in(fn, LRP::DYN);
+        for (auto fn : {tc_read_t_kernel<0>, tc_read_t_kernel<64>, tc_read_t_kernel<128>}) opt_in(fn, rt_dyn(RT_MAX_NT));
+        if (e != cudaSuccess) return e;
+        // the forms on clusters are left out where they cannot run
+        auto clusters = [&](auto kernel, int size, int threads, int dyn, int& n) {
             cudaLaunchConfig_t cfg = {};
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = 2;
+            at[0].val.clusterDim.x = size;
             at[0].val.clusterDim.y = 1;
             at[0].val.clusterDim.z = 1;
-            cfg.gridDim = dim3(2 * (g_sms / 2));
-            cfg.blockDim = dim3(THREADS);
-            cfg.dynamicSmemBytes = LP::DYN;
+            cfg.gridDim = dim3(size * (d.sms / size));
+            cfg.blockDim = dim3(threads);
+            cfg.dynamicSmemBytes = dyn;
             cfg.attrs = at;
             cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&g_pair_clusters, tc_phase_a_pair_kernel, &cfg) != cudaSuccess) {
+            if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
                 cudaGetLastError();
-                g_pair_clusters = 0;
+                n = 0;
             }
-            cfg.blockDim = dim3(B_THREADS);
-            cfg.dynamicSmemBytes = LayoutB2::DYN;
-            if (cudaOccupancyMaxActiveClusters(&g_pairb_clusters, tc_phase_b_kernel<true, false>, &cfg) != cudaSuccess) {
-                cudaGetLastError();
-                g_pairb_clusters = 0;
-            }
-            auto split = [&](auto kernel, int S, int dyn, int& n) {
-                if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess) return;
-                at[0].val.clusterDim.x = S;
-                cfg.gridDim = dim3(S * (g_sms / S));
-                cfg.blockDim = dim3(THREADS);
-                cfg.dynamicSmemBytes = dyn;
-                if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
-            };
-            split(tc_phase_a_split_kernel<4>, 4, LSplit<4>::DYN, g_split4);
-            split(tc_phase_a_split_kernel<2>, 2, LSplit<2>::DYN, g_split2);
-            cudaGetLastError();
-        }
+        };
+        clusters(tc_phase_a_pair_kernel, 2, THREADS, LP::DYN, d.pair_clusters);
+        clusters(tc_phase_b_kernel<true, false>, 2, B_THREADS, LayoutB2::DYN, d.pairb_clusters);
+        clusters(tc_phase_a_split_kernel<4>, 4, THREADS, LSplit<4>::DYN, d.split4);
+        clusters(tc_phase_a_split_kernel<2>, 2, THREADS, LSplit<2>::DYN, d.split2);
+        return cudaSuccess;
     });
-    return g_attr_err;
 }
 
 // Whether phase A runs on CTA pairs (256-token x 256-hidden tiles) for this handle's shape.
-bool phase_a_pairs(const DevState& s) {
-    return (s.T / A_BM) % 2 == 0 && s.d_hid % P_BN == 0 && g_pair_clusters > 0;
+bool phase_a_pairs(const DevState& s, const TcDevice& dev) {
+    return (s.T / A_BM) % 2 == 0 && s.d_hid % P_BN == 0 && dev.pair_clusters > 0;
 }
 
 }  // namespace
 
 cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                               cudaStream_t st) {
-    cudaError_t e = ensure_attrs();
+    const TcDevice* dev;
+    cudaError_t e = tc_device(&dev);
     if (e != cudaSuccess) return e;
     TcArgs a = make_args(s, w);
     if (s.fault_stall > 0) {  // test knob: this launch's waits run out after 1 ms with nothing in flight
@@ -2192,24 +2168,24 @@ cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputM
     // few tiles of a call on one stream (its other kernels leave the SMs to this one): clusters of 4 or 2 a tile
     const int tiles = w.nc * (s.T / A_BM) * (s.d_hid / A_BN);
     if (w.single && s.loss == 0) {
-        if (tiles <= g_split4 && s.d_in >= 4 * BK && s.d_out >= 4 * BK)
+        if (tiles <= dev->split4 && s.d_in >= 4 * BK && s.d_out >= 4 * BK)
             return launch_kernel(tc_phase_a_split_kernel<4>, dim3(4 * tiles), dim3(THREADS), LSplit<4>::DYN, st, pdl, 4, U,
                                  in.Ka, in.Va, m.W1b, m.W2b, a);
-        if (tiles <= g_split2)
+        if (tiles <= dev->split2)
             return launch_kernel(tc_phase_a_split_kernel<2>, dim3(2 * tiles), dim3(THREADS), LSplit<2>::DYN, st, pdl, 2, U,
                                  in.Ka, in.Va, m.W1b, m.W2b, a);
     }
-    if (phase_a_pairs(s)) {
+    if (phase_a_pairs(s, *dev)) {
         // squared-error segments: the pre-pass wrote At and c SiLU'(x) / |z|, only R is left
         a.r_only = (s.loss == 1) ? 1 : 0;  // 1: MONE_LOSS_MSE
         // CTA pairs over 256-token x 256-hidden tiles
         const int npairs = w.nc * (s.T / (2 * A_BM)) * (s.d_hid / P_BN);
-        const int maxc = g_pair_clusters - (s.reserve_sms + 1) / 2;  // leave reserved SMs free
+        const int maxc = dev->pair_clusters - (s.reserve_sms + 1) / 2;  // leave reserved SMs free
         const int clusters = npairs < maxc ? npairs : maxc;
         return launch_kernel(tc_phase_a_pair_kernel, dim3(2 * clusters), dim3(THREADS), LP::DYN, st, pdl && !a.r_only, 2, U,
                              in.Ka, in.Va, m.W1b, m.W2b, a);
     }
-    const int sms = g_sms - s.reserve_sms;
+    const int sms = dev->sms - s.reserve_sms;
     const int grid = tiles < sms ? tiles : sms;
     return launch_kernel(tc_phase_a_kernel, dim3(grid), dim3(THREADS), LA::DYN, st, pdl && s.loss == 0, 1, U, in.Ka, in.Va,
                          m.W1b, m.W2b, a);
@@ -2217,14 +2193,15 @@ cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputM
 
 cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                               cudaStream_t st) {
-    cudaError_t e = ensure_attrs();
+    const TcDevice* dev;
+    cudaError_t e = tc_device(&dev);
     if (e != cudaSuccess) return e;
     TcArgs a = make_args(s, w);
     // CTA pairs over 256-hidden x 256-column tiles (a tile's columns all live) from T = 1024 on:
     // there a tile's operand stream (768 KB a CTA) rivals its state stream, and the pair takes a
     // third off it.  At T = 512 the pair's coupled loads and accumulator release cost more than they save.
     constexpr int PAIR_MIN_T = 1024;
-    const bool pairs = s.T >= PAIR_MIN_T && s.d_in % B_BN == 0 && g_pairb_clusters > 0;
+    const bool pairs = s.T >= PAIR_MIN_T && s.d_in % B_BN == 0 && dev->pairb_clusters > 0;
     // When the state ring's slots are handed back, by what was fastest: how stores and loads alternate
     // decides how much of HBM the stream gets.  With no momentum, on CTA pairs, for one chain, or with W and mu of
     // the whole handle in L2, two at a time, one store later (ms, against one by one three stores later: 64 plain chains of
@@ -2241,14 +2218,14 @@ cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputM
     const int col_tiles = b_col_tiles(s.d_in, s.d_out);
     if (pairs) {
         const int npairs = w.nc * col_tiles * (s.d_hid / (2 * B_BM));
-        const int maxc = g_pairb_clusters - (s.reserve_sms + 1) / 2;
+        const int maxc = dev->pairb_clusters - (s.reserve_sms + 1) / 2;
         const int clusters = npairs < maxc ? npairs : maxc;
         return launch_kernel(a.step_sq ? tc_phase_b_kernel<true, true> : tc_phase_b_kernel<true, false>, dim3(2 * clusters),
                              dim3(B_THREADS), LayoutB2::DYN, st, w.single != 0, 2, U2, in.Kb, in.Vb, m.dH, m.At, m.W1s,
                              m.W2s, a);
     }
     const int ntiles = w.nc * col_tiles * (s.d_hid / B_BM);
-    const int sms = g_sms - s.reserve_sms;
+    const int sms = dev->sms - s.reserve_sms;
     const int grid = ntiles < sms ? ntiles : sms;
     return launch_kernel(a.step_sq ? tc_phase_b_kernel<false, true> : tc_phase_b_kernel<false, false>, dim3(grid),
                          dim3(B_THREADS), LayoutB::DYN, st, w.single != 0, 1, U, in.Kb, in.Vb, m.dH, m.At, m.W1s, m.W2s, a);
@@ -2258,7 +2235,8 @@ int tc_kernels_per_segment() { return 2; }
 
 cudaError_t launch_mse_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                           cudaStream_t st) {
-    cudaError_t e = ensure_attrs();
+    const TcDevice* dev;
+    cudaError_t e = tc_device(&dev);
     if (e != cudaSuccess) return e;
     const bool paper = s.mode == 1;
     ReadArgs a{};
@@ -2272,7 +2250,7 @@ cudaError_t launch_mse_tc(const DevState& s, const TcMaps& m, const TcInputMaps&
     a.Kres = s.Kres; a.Vres = s.Vres;
     a.loss = w.loss;
     a.Aq = s.Amse;
-    if (phase_a_pairs(s)) {  // phase A runs in its R-only form: write At and c SiLU'(x) / |z| here
+    if (phase_a_pairs(s, *dev)) {  // phase A runs in its R-only form: write At and c SiLU'(x) / |z| here
         a.At = reinterpret_cast<bf16*>(s.Att);
         a.Sp = reinterpret_cast<bf16*>(s.dHt);
         a.paper = paper ? 1 : 0;
@@ -2286,17 +2264,18 @@ cudaError_t launch_mse_tc(const DevState& s, const TcMaps& m, const TcInputMaps&
     a.a_row0 = paper ? (int)w.u_off : (int)w.row0;
     a.a_chain0 = paper ? w.c0 : 0;
     a.b_chain0 = w.c0;
-    e = launch_read_kernel<MSE_HIDDEN>(dim3(s.T / 128, s.d_hid / 128, w.nc), paper ? m.Ua : in.Xa, m.W1b, a, st);
+    e = launch_read_kernel<MSE_HIDDEN>(*dev, dim3(s.T / 128, s.d_hid / 128, w.nc), paper ? m.Ua : in.Xa, m.W1b, a, st);
     if (e != cudaSuccess) return e;
     // out: the activations of the same chains (absolute), W2 MN-major
     a.a_row0 = 0;
     a.a_chain0 = w.c0;
-    return launch_read_kernel<MSE_OUT>(dim3(s.T / 128, s.d_out / 128, w.nc), m.Amse, m.W2m, a, st);
+    return launch_read_kernel<MSE_OUT>(*dev, dim3(s.T / 128, s.d_out / 128, w.nc), m.Amse, m.W2m, a, st);
 }
 
 cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, void* Uq, void* Aq, float* zq, int Q,
                            int n_layers, void* K_out, void* V_out, const long long* strides, cudaStream_t st) {
-    cudaError_t e = ensure_attrs();
+    const TcDevice* dev;
+    cudaError_t e = tc_device(&dev);
     if (e != cudaSuccess) return e;
     if (s.hd != 64 && s.hd != 128) return cudaErrorInvalidValue;
     // the query side: unnormalised z and 1/|z|, which the hidden kernel applies
@@ -2314,8 +2293,8 @@ cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, v
     if (Q <= RT_MAX_NT) {  // weights as the 128-row operand, the queries as N
         const int NT = (Q + 31) / 32 * 32;
         // one CTA per SM with the deep ring when a kernel's tiles fit in one wave, else two
-        const int ring1 = (long long)(s.d_hid / 128) * s.C <= g_sms ? RT_RING_1 : RT_RING_2;
-        const int ring2 = (long long)(s.d_out / 128) * s.C <= g_sms ? RT_RING_1 : RT_RING_2;
+        const int ring1 = (long long)(s.d_hid / 128) * s.C <= dev->sms ? RT_RING_1 : RT_RING_2;
+        const int ring2 = (long long)(s.d_out / 128) * s.C <= dev->sms ? RT_RING_1 : RT_RING_2;
         const int k1 = rt_kblocks(NT, ring1), k2 = rt_kblocks(NT, ring2);
         CUtensorMap tu, ta;
         if (!encode_map_bf16_blocks(&tu, Uq, s.d_in, Q, s.C, NT, k1) || !encode_map_bf16_blocks(&ta, Aq, s.d_hid, Q, s.C, NT, k2))
@@ -2342,9 +2321,9 @@ cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, v
     if (!encode_map_bf16_3d(&mu, Uq, s.d_in, Q, s.C, 64, 128) || !encode_map_bf16_3d(&ma, Aq, s.d_hid, Q, s.C, 64, 128))
         return cudaErrorInvalidValue;
     const int nq = (Q + 127) / 128;
-    if ((e = launch_read_many<READ_HIDDEN>(dim3(nq, s.d_hid / 128, s.C), mu, m.W1b, a, st)) != cudaSuccess) return e;
-    if (s.hd == 64) return launch_read_many<64>(dim3(nq, s.d_out / 128, s.C), ma, m.W2m, a, st);
-    return launch_read_many<128>(dim3(nq, s.d_out / 128, s.C), ma, m.W2m, a, st);
+    if ((e = launch_read_many<READ_HIDDEN>(*dev, dim3(nq, s.d_hid / 128, s.C), mu, m.W1b, a, st)) != cudaSuccess) return e;
+    if (s.hd == 64) return launch_read_many<64>(*dev, dim3(nq, s.d_out / 128, s.C), ma, m.W2m, a, st);
+    return launch_read_many<128>(*dev, dim3(nq, s.d_out / 128, s.C), ma, m.W2m, a, st);
 }
 
 // ------------------------------------------------------------------ tensor maps

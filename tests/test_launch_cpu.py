@@ -55,3 +55,34 @@ def test_a_failed_opt_in_is_reported_and_tried_again(fake, shape):
         mone.mone_ttl_context(h, P, P, P, 1000, 0)
     mone.mone_ttl_context(h, P, P, P, 1000, 0)
     mone.mone_mem_free(h)
+
+
+BF16_SHAPES = [  # d_in, d_hid, d_out, T, layers, options
+    (512, 512, 512, 256, 4, {}),                               # phase A on CTA pairs
+    (512, 512, 512, 128, 4, {}),                               # one-CTA phase A
+    (512, 512, 512, 1024, 4, {}),                              # phase B on CTA pairs
+    (512, 512, 512, 128, 1, {}),                               # one chain: phase A over clusters
+    (512, 512, 512, 256, 4, dict(loss=mone.MONE_LOSS_MSE)),
+    (896, 224, 896, 512, 2, dict(memory=mone.MONE_MEM_SWIGLU, mem_heads=4)),
+]
+
+
+@pytest.mark.parametrize("d_in,d_hid,d_out,T,layers,kw", BF16_SHAPES)
+def test_bf16_calls_on_either_device(fake, d_in, d_hid, d_out, T, layers, kw):
+    for dev, sms in ((0, 152), (1, 100), (0, 152)):
+        fake.device(dev)
+        h = init(layers, d_in, d_hid, d_out, T, mone.MONE_BF16, mone.MONE_PAPER, **kw)
+        fake.drain()
+        mone.mone_ttl_context_host(h, P, P, P, 3 * T + 1, T, 0)
+        launches, _ = fake.drain()
+        assert {x["dev"] for x in launches} == {dev}
+        for x in launches:  # the persistent learning kernels stay within the device's SMs
+            if "phase_" in x["name"] or "swiglu_a" in x["name"] or "swiglu_b" in x["name"]:
+                assert x["grid"][0] <= sms, x
+        mone.mone_ttl_context(h, P, P, P, 3 * T + 1, 0)
+        for Q in (3, 300, 4000):
+            mone.mone_mem_generate_kv(h, P, Q, P, P, (0, 0, 0, 64), 0)
+        for Lq in (1, 2000):
+            mone.mone_attention(h, P, d_out // 128, Lq, P, P, mone.kv_strides(layers, d_out // 128, Lq + 8, 64), 8, P, 0)
+        assert {x["dev"] for x in fake.drain()[0]} == {dev}
+        mone.mone_mem_free(h)
