@@ -766,7 +766,9 @@ cudaError_t launch_decode(const AttnArgs& a, int C, cudaStream_t st) {
     // have no block of keys each
     const long long ctas = (long long)row_tiles * a.n_kv * C;
     const int blocks = (a.n_mem + a.Lq + 31) / 32;
-    constexpr int slots = (HD == 64 ? 4 : 3) * 152;
+    int sms = 0;
+    if ((e = sm_count(&sms)) != cudaSuccess) return e;
+    const int slots = (HD == 64 ? 4 : 3) * sms;
     const int splits = (int)std::max(1ll, std::min({8ll, slots / ctas, (long long)blocks / DE_WARPS}));
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];

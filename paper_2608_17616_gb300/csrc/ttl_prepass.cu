@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "mone_common.cuh"
+#include "per_device.h"
 
 namespace mone {
 
@@ -265,9 +266,12 @@ __global__ void __launch_bounds__(256) prepass_kernel(const PrepassArgs a) {
 
 template <typename Tin, typename Tout>
 cudaError_t launch_one(const PrepassArgs& a, int nchains, cudaStream_t st) {
-    // two rows a warp share the meta-parameter loads; few rows are spread one a warp instead (512 rows of
-    // one chain, d_in = 2048, caches cold: 11.1 -> 9.2 us)
-    if ((long long)((a.rows + 15) / 16) * nchains >= 2 * 152)
+    // two rows a warp share the meta-parameter loads; few rows (less than two CTAs an SM that way) are spread
+    // one a warp instead (512 rows of one chain, d_in = 2048, caches cold: 11.1 -> 9.2 us)
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    if ((long long)((a.rows + 15) / 16) * nchains >= 2 * sms)
         prepass_kernel<Tin, Tout, 2><<<dim3((a.rows + 15) / 16, nchains), 256, 0, st>>>(a);
     else
         prepass_kernel<Tin, Tout, 1><<<dim3((a.rows + 7) / 8, nchains), 256, 0, st>>>(a);

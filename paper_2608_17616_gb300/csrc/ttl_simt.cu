@@ -1110,29 +1110,35 @@ cudaError_t phase_b_f32(const DevState& s, const SegWork& w, const F32SegArgs& a
     return launch_f32_tiles(phase_b_f32_kernel<TM, TN, TY>, 16 * TY, tn_smem<TM, TN, TY>(), once,
                             dim3((s.d_in + s.d_out) / (16 * TN), s.d_hid / (TY * TM), w.nc), a, st);
 }
-constexpr long long F32_SMS = 152;
 }  // namespace
 
 cudaError_t launch_phase_a_f32(const DevState& s, const SegWork& w, cudaStream_t st) {
     const F32SegArgs a = make_f32_args(s, w);
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
     const long long g64 = (long long)(s.T / 64) * (s.d_hid / 64) * w.nc;  // 64 x 64 tiles (T, d_hid multiples of 64)
     // 32 x 64 tiles, but 64 x 64 (8 x 4 outputs a thread) where halving the tiles saves nothing of the last wave.
     // 1024 -> 1024 -> 1024, T = 256, 32 x 64 and 64 x 64 tiles: one chain (64 tiles of 64 x 64) 48 and 73 us,
     // three 102 and 123, four (256) 135 and 123, five 163 and 180, eight 223 and 234
-    const auto waves = [](long long tiles) { return (tiles + F32_SMS - 1) / F32_SMS; };
-    if (g64 > F32_SMS && waves(2 * g64) == 2 * waves(g64)) return phase_a_f32<8, 4, 8>(s, w, a, st);
+    const auto waves = [&](long long tiles) { return (tiles + sms - 1) / sms; };
+    if (g64 > sms && waves(2 * g64) == 2 * waves(g64)) return phase_a_f32<8, 4, 8>(s, w, a, st);
     return phase_a_f32<4, 4, 8>(s, w, a, st);
 }
 
 cudaError_t launch_phase_b_f32(const DevState& s, const SegWork& w, cudaStream_t st) {
     const F32SegArgs a = make_f32_args(s, w);
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
     // a tile lies in W1 or in one half of W2: widths are multiples of 64, for the large tile of 128, which
     // is taken from two thirds of the SMs on
     const bool wide = s.d_in % 128 == 0 && (s.d_out / 2) % 128 == 0 && s.d_hid % 128 == 0;
-    if (wide && (long long)(s.d_hid / 128) * ((s.d_in + s.d_out) / 128) * w.nc >= 100) return phase_b_f32<8, 8, 16>(s, w, a, st);
+    if (wide && (long long)(s.d_hid / 128) * ((s.d_in + s.d_out) / 128) * w.nc >= sms * 2 / 3)
+        return phase_b_f32<8, 8, 16>(s, w, a, st);
     // 64 x 64 tiles from two to an SM on (2 chains of 1024 -> 512 -> 512, T = 512: 49 us, 32 x 64 tiles 53), else 32 x
     // 64 (one chain, T = 64: 13.9 and 11.9 us); with 256 threads of 4 x 4 outputs 64 x 64 tiles take 55 and 12.2
-    if ((long long)(s.d_hid / 64) * ((s.d_in + s.d_out) / 64) * w.nc > 2 * F32_SMS) return phase_b_f32<8, 4, 8>(s, w, a, st);
+    if ((long long)(s.d_hid / 64) * ((s.d_in + s.d_out) / 64) * w.nc > 2 * sms) return phase_b_f32<8, 4, 8>(s, w, a, st);
     return phase_b_f32<4, 4, 8>(s, w, a, st);
 }
 

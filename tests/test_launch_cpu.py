@@ -86,3 +86,26 @@ def test_bf16_calls_on_either_device(fake, d_in, d_hid, d_out, T, layers, kw):
             mone.mone_attention(h, P, d_out // 128, Lq, P, P, mone.kv_strides(layers, d_out // 128, Lq + 8, 64), 8, P, 0)
         assert {x["dev"] for x in fake.drain()[0]} == {dev}
         mone.mone_mem_free(h)
+
+
+def test_tile_rules_follow_the_devices_sm_count(fake):
+    """Each rule at a size where 152 and 100 SMs decide differently."""
+    want = {0: {}, 1: {}}
+    for dev in (0, 1):
+        fake.device(dev)
+        h = init(3, 1024, 1024, 1024, 256, mone.MONE_FP32)  # 192 tiles of 64 x 64 in phase A
+        mone.mone_ttl_context(h, P, P, P, 256, 0)
+        want[dev]["phase_a"] = [x["grid"] for x in fake.drain()[0] if "phase_a_f32" in x["name"]]
+        h = init(1, 1024, 1024, 512, 64, mone.MONE_FP32)    # 96 tiles of 128 x 128 in phase B
+        mone.mone_ttl_context(h, P, P, P, 64, 0)
+        want[dev]["phase_b"] = [x["grid"] for x in fake.drain()[0] if "phase_b_f32" in x["name"]]
+        h = init(1, 512, 512, 512, 128, mone.MONE_BF16, mone.MONE_PAPER)
+        mone.mone_ttl_context(h, P, P, P, 4000, 0)          # 250 CTAs of 16 rows in the input transform
+        want[dev]["transform"] = [x["grid"] for x in fake.drain()[0] if "prepass" in x["name"]]
+        h = init(16, 512, 512, 512, 128, mone.MONE_BF16)    # decode over 64 heads in all
+        mone.mone_attention(h, P, 4, 1, P, P, mone.kv_strides(16, 4, 2048, 64), 2047, P, 0)
+        want[dev]["decode"] = [x["cluster"] for x in fake.drain()[0] if "decode" in x["name"]]
+    assert want[0]["phase_a"] == [(8, 16, 3)] and want[1]["phase_a"] == [(4, 16, 3)]
+    assert want[0]["phase_b"] == [(24, 32, 1)] and want[1]["phase_b"] == [(12, 8, 1)]
+    assert want[0]["transform"] == [(500, 1, 1)] and want[1]["transform"] == [(250, 1, 1)]
+    assert want[0]["decode"] == [8] and want[1]["decode"] == [6]
