@@ -461,7 +461,8 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                     }
                 }
             }
-            const float moff = -m_run * k2;
+            // every key so far at a score of -inf: probabilities 2^-inf = 0, as if these keys were not there
+            const float moff = m_run == -INFINITY ? 0.f : -m_run * k2;
             l += fa_probs(v, pack_f32x2(k2, k2), pack_f32x2(moff, moff), t_s + half * (NE / 2));
             tmem_wait_st();
             tc_fence_before();

@@ -59,6 +59,26 @@ def test_prefill_form(group, Lq, n_mem, hd, late_scale):
     run_case(group, Lq, n_mem, hd, n_layers=20, late_scale=late_scale)
 
 
+@pytest.mark.parametrize("hd,group,Lq,n_mem", [(64, 4, 200, 200), (128, 2, 150, 130), (64, 1, 3, 300)])
+def test_keys_at_minus_infinity_count_for_nothing(hd, group, Lq, n_mem):
+    """The memory keys, whole chunks of them, overflow to scores of -inf; the tokens' own keys are ordinary."""
+    n_kv, L = 2, 20
+    run = DeviceRun(wk.Workload("attn_forms", 43, 1, L, 256, 256, 2 * n_kv * hd, n_kv, hd, 128, 128, 8, "bf16", wk.PLAIN))
+    g = torch.Generator(device="cuda").manual_seed(hd + Lq)
+    rn = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()  # noqa: E731
+    K, V, Q = rn(1, L, n_kv, n_mem + Lq, hd), rn(1, L, n_kv, n_mem + Lq, hd), rn(1, L, group * n_kv, Lq, hd)
+    K[..., 0] = 0
+    K[..., :n_mem, 0] = -1e25
+    Q[..., 0] = 1e25
+    out = torch.full_like(Q, 7.0)
+    mone.mone_attention(run.h, Q, group * n_kv, Lq, K, V, K.stride()[:4], n_mem, out)
+    mone.mone_mem_sync(run.h)
+    run.close()
+    for layer in (0, L - 1):
+        ref = O.attention(Q[0, layer].cpu(), K[0, layer].cpu(), V[0, layer].cpu(), n_mem)
+        assert rel_fro(out[0, layer].float().cpu(), ref) <= 1e-2, layer
+
+
 def test_prefill_form_many_tiles_repeat():
     """More CTAs than the SMs hold at once, repeated: every wait is met and the output repeats bit for bit."""
     n_kv, group, hd, Lq, n_mem, L = 8, 4, 128, 400, 64, 16
