@@ -15,6 +15,7 @@
 // are reduced once per item, and the probabilities pass through shared memory into the
 // value accumulation, where a lane owns hd / 32 dimensions.
 #include <algorithm>
+#include <cfloat>
 #include <mutex>
 
 #include "mone_common.cuh"
@@ -36,6 +37,8 @@ struct AttnArgs {
     long long s0, s1, s2, s3;
     int L, n_q, n_kv, group, Lq, n_mem, rows;  // rows: query tokens per CTA (group * rows <= ATT_ITEMS)
     float scale;            // 1 / sqrt(hd)
+    int tile_tok, per_block;  // decode form: tokens of a block, 16-row tiles that cut it
+    int group_inv;            // decode form: 65536 / group + 1
     int vec;                // caches 16-byte aligned (base and every stride): stage with 16-byte loads
     int* status;            // device status word (bounded waits of the prefill form)
 };
@@ -253,8 +256,8 @@ struct FaSmem {
     static constexpr int Q_OFF = 0;
     static constexpr int KV_OFF = Q_OFF + (HD / 64) * Q_SLAB;
     static constexpr int X_OFF = KV_OFF + NS * TILE;       // [2][2][128] floats: row max (or sum) of each half
-    static constexpr int BAR_OFF = X_OFF + 2 * 2 * 128 * 4;  // qfull full[NS] empty[NS] sfull[2] odone[2] pready[2]
-    static constexpr int SLOT_OFF = BAR_OFF + (2 * NS + 7) * 8;
+    static constexpr int BAR_OFF = X_OFF + 2 * 2 * 128 * 4;  // qfull full[NS] empty[NS] sfull[2] odone[2] pready[2] vlast
+    static constexpr int SLOT_OFF = BAR_OFF + (2 * NS + 8) * 8;
     static constexpr int DYN = SLOT_OFF + 16 + 1024;       // + TMEM slot, + alignment slack
 };
 static_assert(2 * (FaSmem<64>::DYN + 1024) <= 228 * 1024 && 2 * (FaSmem<128>::DYN + 1024) <= 228 * 1024,
@@ -296,10 +299,12 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
     auto sfull = [&](int j) { return bars + 8 * (1 + 2 * NS + (j & 1)); };
     auto odone = [&](int j) { return bars + 8 * (3 + 2 * NS + (j & 1)); };
     auto pready = [&](int j) { return bars + 8 * (5 + 2 * NS + (j & 1)); };
+    const uint32_t vlast = bars + 8 * (7 + 2 * NS);
     uint32_t* slot = reinterpret_cast<uint32_t*>(base + SM::SLOT_OFF);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         mbar_init(qfull, 1);
+        mbar_init(vlast, 1);
         for (int s = 0; s < NS; ++s) {
             mbar_init(full(s), 1);
             mbar_init(empty(s), 1);
@@ -322,9 +327,13 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
 
     // token tiles: the last first (causal: it has the most keys)
     const int c = blockIdx.z, g = blockIdx.y, rt = a.rows, r0 = (gridDim.x - 1 - blockIdx.x) * rt;
-    const int n = (a.n_mem + min(a.Lq, r0 + rt) + NK - 1) / NK;  // chunks the tile's last token sees
+    const int keys = a.n_mem + min(a.Lq, r0 + rt), n = (keys + NK - 1) / NK;  // keys the tile's last token sees, in chunks
+    // The last chunk may hold later tokens' rows (past the cache's last row TMA writes zeros). No probability of theirs is
+    // added up, but 0 times a non-finite value would be: their value rows are cleared.
+    const bool clear = keys < a.n_mem + a.Lq && keys < n * NK;
 
     if (warp == SM::LOAD_WARP) {
+        bool landed = false;
         if (lane == 0) {
             tma_prefetch_map(&tmQ);
             tma_prefetch_map(&tmK);
@@ -350,9 +359,30 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
             };
             // K0 K1 V0 K2 V1 .. K(n-1) V(n-2) V(n-1)
             bool ok = load(&tmK, 0);
-            for (int j = 0; ok && j < n; ++j) ok = (j + 1 >= n || load(&tmK, j + 1)) && load(&tmV, j);
+            for (int j = 0; ok && j < n - 1; ++j) ok = load(&tmK, j + 1) && load(&tmV, j);
+            if (!clear) {
+                ok = ok && load(&tmV, n - 1);
+            } else if (ok && mbar_wait(empty(s), ph, a.status)) {  // on a barrier of its own: it counts as loaded once cleared
+                mbar_expect_tx(vlast, SM::TILE);
+#pragma unroll
+                for (int kb = 0; kb < HD / 64; ++kb)
+                    tma_load_5d(smem_u32(base + SM::KV_OFF + s * SM::TILE) + kb * SM::SLAB, &tmV, vlast, 64 * kb, (n - 1) * NK, g,
+                                layer, ctx);
+                landed = mbar_wait(vlast, 0, a.status);
+            }
         }
         __syncwarp();
+        if (clear && __shfl_sync(0xffffffffu, landed, 0)) {
+            const int slot_v = (2 * n - 1) % NS;  // of the last of the 2 n loads
+            uint8_t* v = base + SM::KV_OFF + slot_v * SM::TILE;
+#pragma unroll 1
+            for (int e = (keys - (n - 1) * NK) * 8 + lane; e < NK * 8; e += 32)  // 16-byte pieces, exchanged within a row
+#pragma unroll
+                for (int kb = 0; kb < HD / 64; ++kb) *reinterpret_cast<uint4*>(v + kb * SM::SLAB + e * 16) = make_uint4(0, 0, 0, 0);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full(slot_v));
+        }
     } else if (warp == SM::MMA_WARP) {
         if (lane == 0) {
             const uint32_t id_s = idesc_bf16_f32(128, NK, false, false), id_o = idesc_bf16_f32(128, HD, false, true);
@@ -440,7 +470,7 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
             tc_fence_after();
             cm = fmaxf(cm, x[(half ^ 1) * 128 + row]);
             if (j == 0) {
-                m_run = cm;
+                m_run = fmaxf(cm, -FLT_MAX);  // finite: where every key so far scores -inf, probabilities of 0
             } else {
                 const bool grown = cm > m_run;
                 if (__any_sync(0xffffffffu, grown)) {  // the same in both warps: each rescales its half of O
@@ -461,8 +491,7 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                     }
                 }
             }
-            // every key so far at a score of -inf: probabilities 2^-inf = 0, as if these keys were not there
-            const float moff = m_run == -INFINITY ? 0.f : -m_run * k2;
+            const float moff = -m_run * k2;
             l += fa_probs(v, pack_f32x2(k2, k2), pack_f32x2(moff, moff), t_s + half * (NE / 2));
             tmem_wait_st();
             tc_fence_before();
@@ -501,8 +530,8 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
 // ---------------------------------------------------------------- decode form (bf16, few rows)
 // Few (query head, token) rows per key/value head: the caches are read once and little is computed,
 // so the kernel is a stream over keys and values, bound by HBM, or at short caches by latency.  A
-// cluster of `splits` CTAs takes (chain, key/value head, 16 rows); the keys' 32-position blocks are
-// split over the CTAs and their warps.  Each warp runs an online softmax of its own with
+// cluster of `splits` CTAs takes (chain, key/value head, 16 rows); the keys' blocks of 32 (hd 128: 16)
+// positions are split over the CTAs and their warps.  Each warp runs an online softmax of its own with
 // mma.m16n8k16 on operands loaded from global memory straight into fragment order (a 128-row
 // tcgen05 tile would be 1/8 to 1/32 full, and its staging would cost more than the arithmetic): the
 // contraction over hd and the order of output columns are free, so they are permuted to let every
@@ -521,6 +550,33 @@ struct DeSmem {
     // per warp, then once for the CTA: O [16][HD], then max and sum per row
     static constexpr int PART = DE_ROWS * HD + 2 * DE_ROWS;
     static constexpr int FLOATS = (DE_WARPS + 1) * PART;
+};
+
+// Row tiles of the decode form.  The tokens go in blocks of 128 / group, the tokens of a tile of the prefill form,
+// whose (token, head of the group) rows, heads innermost, are cut into tiles of 16: a tile sees the keys up to its
+// last token's only, and a non-finite value row reaches (as 0 times it) no token outside the later one's block.
+struct DeTile {
+    int rr0, tok0, ntok, keys;  // first row within the block; the block's tokens; keys the tile's last token sees
+    static int count(int group, int Lq) {
+        const int bt = 128 / group, per = (bt * group + DE_ROWS - 1) / DE_ROWS;
+        return Lq / bt * per + (Lq % bt * group + DE_ROWS - 1) / DE_ROWS;
+    }
+    // r / group for 0 <= r < 1024 and group <= 64: the factor's error adds less than r / 65536 < 1 / group
+    static __device__ int over_group(const AttnArgs& a, int r) { return (r * a.group_inv) >> 16; }
+    __device__ DeTile(const AttnArgs& a, int t) {
+        const int b = a.Lq > a.tile_tok ? t / a.per_block : 0;
+        rr0 = (t - b * a.per_block) * DE_ROWS;
+        tok0 = b * a.tile_tok;
+        ntok = min(a.tile_tok, a.Lq - tok0);
+        keys = a.n_mem + tok0 + min(over_group(a, rr0 + DE_ROWS - 1), ntok - 1) + 1;
+    }
+    // row r of the tile; false past its last (the others then point at some valid row)
+    __device__ bool row(const AttnArgs& a, int r, int& head, int& tok) const {
+        const int i = over_group(a, rr0 + r);
+        head = (rr0 + r) - i * a.group;
+        tok = tok0 + min(i, ntok - 1);
+        return i < ntok;
+    }
 };
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&A)[4], uint32_t b0, uint32_t b1) {
@@ -542,22 +598,24 @@ __global__ void __launch_bounds__(DE_WARPS * 32, HD == 64 ? 4 : 3) attention_dec
     constexpr int KB = HD == 64 ? 32 : 16;     // keys per step
     extern __shared__ float de_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gq = lane >> 2, t = lane & 3;
-    const int c = blockIdx.z, g = blockIdx.y, rank = blockIdx.x % splits, row0 = blockIdx.x / splits * DE_ROWS;
-    const int R = a.group * a.Lq, keys = a.n_mem + a.Lq;
+    const int c = blockIdx.z, g = blockIdx.y, rank = (int)cluster_ctarank();
+    const DeTile tile(a, (int)cluster_id_x());
+    const int keys = __shfl_sync(0xffffffffu, tile.keys, 0);  // the same in every lane, and known to be
     const long long kv_off = (long long)(c / a.L) * a.s0 + (long long)(c % a.L) * a.s1 + (long long)g * a.s2;
     const bf16* Kc = static_cast<const bf16*>(a.K) + kv_off + 8 * t;
     const bf16* Vc = static_cast<const bf16*>(a.V) + kv_off + 8 * gq;
-    // rows row0 + gq and + 8: row r is token r % Lq of the group's head r / Lq
+    // rows gq and gq + 8 of the tile
     uint32_t qa[HD / 16][4];
     int vis[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int r = row0 + gq + 8 * h;
-        vis[h] = r < R ? a.n_mem + r % a.Lq + 1 : 0;
-        const bf16* q = static_cast<const bf16*>(a.Q) + ((size_t)c * a.n_q + (size_t)g * a.group) * a.Lq * HD + (size_t)r * HD + 8 * t;
+        int head, tok;
+        const bool live = tile.row(a, gq + 8 * h, head, tok);
+        vis[h] = live ? a.n_mem + tok + 1 : 0;
+        const bf16* q = static_cast<const bf16*>(a.Q) + (((size_t)c * a.n_q + (size_t)g * a.group + head) * a.Lq + tok) * HD + 8 * t;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            const uint4 v = r < R ? *reinterpret_cast<const uint4*>(q + 32 * p) : make_uint4(0, 0, 0, 0);
+            const uint4 v = live ? *reinterpret_cast<const uint4*>(q + 32 * p) : make_uint4(0, 0, 0, 0);
             qa[2 * p][h] = v.x;
             qa[2 * p][2 + h] = v.y;
             qa[2 * p + 1][h] = v.z;
@@ -698,10 +756,12 @@ __global__ void __launch_bounds__(DE_WARPS * 32, HD == 64 ? 4 : 3) attention_dec
         cluster_sync();
     else
         __syncthreads();
+    const DeTile tile_o(a, (int)cluster_id_x());  // made again: kept over the loop it costs registers that the loop needs
     // every CTA of the cluster finishes a share of the rows' outputs, two dimensions a thread
     for (int e = 2 * (rank * DE_WARPS * 32 + threadIdx.x); e < DE_ROWS * HD; e += 2 * splits * DE_WARPS * 32) {
         const int r = e / HD, d = e - r * HD;
-        if (row0 + r >= R) break;
+        int head, tok;
+        if (!tile_o.row(a, r, head, tok)) break;
         float mx = -INFINITY, lt = 0.f, o0 = 0.f, o1 = 0.f;
         for (int k = 0; k < splits; ++k) mx = fmaxf(mx, ld_cluster_f32(sum + DE_ROWS * HD + r, k));
         for (int k = 0; k < splits; ++k) {
@@ -712,7 +772,7 @@ __global__ void __launch_bounds__(DE_WARPS * 32, HD == 64 ? 4 : 3) attention_dec
             o1 = fmaf(f, ld_cluster_f32(sum + e + 1, k), o1);
         }
         const float inv = 1.f / lt;
-        bf16* out = static_cast<bf16*>(a.out) + ((size_t)c * a.n_q + (size_t)g * a.group) * a.Lq * HD + (size_t)(row0 + r) * HD + d;
+        bf16* out = static_cast<bf16*>(a.out) + (((size_t)c * a.n_q + (size_t)g * a.group + head) * a.Lq + tok) * HD + d;
         *reinterpret_cast<uint32_t*>(out) = pack_bf16(o0 * inv, o1 * inv);
     }
     if (splits > 1) cluster_sync();  // no CTA leaves while another reads its shared memory
@@ -757,12 +817,15 @@ cudaError_t launch_prefill(AttnArgs a, int n_ctx, int C, cudaStream_t st) {
 }
 
 template <int HD>
-cudaError_t launch_decode(const AttnArgs& a, int C, cudaStream_t st) {
+cudaError_t launch_decode(AttnArgs a, int C, cudaStream_t st) {
+    a.tile_tok = 128 / a.group;
+    a.per_block = (a.tile_tok * a.group + DE_ROWS - 1) / DE_ROWS;
+    a.group_inv = 65536 / a.group + 1;
     static PerDevice<SmemOptIn> once;
     constexpr size_t smem = DeSmem<HD>::FLOATS * sizeof(float);
     cudaError_t e = smem_opt_in(reinterpret_cast<const void*>(attention_decode_kernel<HD>), smem, once);
     if (e != cudaSuccess) return e;
-    const int row_tiles = (a.group * a.Lq + DE_ROWS - 1) / DE_ROWS;
+    const int row_tiles = DeTile::count(a.group, a.Lq);
     // split the keys over a cluster until the grid fills the SMs' CTA slots, or a CTA's warps would
     // have no block of keys each
     const long long ctas = (long long)row_tiles * a.n_kv * C;

@@ -79,6 +79,39 @@ def test_keys_at_minus_infinity_count_for_nothing(hd, group, Lq, n_mem):
         assert rel_fro(out[0, layer].float().cpu(), ref) <= 1e-2, layer
 
 
+@pytest.mark.parametrize("group,Lq,n_mem,hd,n_layers", [
+    (4, 200, 70, 64, 20),    # prefill: 32-token tiles; the tiles' last chunks hold later tokens' rows
+    (3, 150, 0, 128, 20),    # 42-token tiles
+    (1, 300, 77, 64, 20),    # 128-token tiles
+    (1, 300, 31, 64, 1),     # decode: 16-row tiles of one head
+    (7, 40, 500, 128, 1),    # rows of the group's heads, 18-token blocks
+    (20, 40, 60, 64, 1),     # 6-token blocks
+])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_non_finite_value_rows_stay_with_their_tile(group, Lq, n_mem, hd, n_layers, bad):
+    """A token's non-finite value and key rows reach no token of an earlier tile of 128 / group tokens."""
+    n_kv = 2
+    run = DeviceRun(wk.Workload("attn_forms", 44, 1, n_layers, 256, 256, 2 * n_kv * hd, n_kv, hd, 128, 128, 8, "bf16", wk.PLAIN))
+    g = torch.Generator(device="cuda").manual_seed(group + Lq)
+    rn = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()  # noqa: E731
+    K, V, Q = (rn(1, n_layers, h, t, hd) for h, t in ((n_kv, n_mem + Lq), (n_kv, n_mem + Lq), (group * n_kv, Lq)))
+    outs = []
+    tile = 128 // group
+    first = tile * ((Lq - 1) // tile)  # first token of the last tile
+    for t in range(first, Lq, 3):
+        V[..., n_mem + t, :] = bad
+        K[..., n_mem + t, ::2] = bad
+        outs.append(torch.full_like(Q, 7.0))
+        mone.mone_attention(run.h, Q, group * n_kv, Lq, K, V, K.stride()[:4], n_mem, outs[-1])
+    mone.mone_mem_sync(run.h)
+    run.close()
+    for layer in (0, n_layers - 1):
+        sl = slice(0, n_mem + first)
+        ref = O.attention(Q[0, layer, :, :first].cpu(), K[0, layer, :, sl].cpu(), V[0, layer, :, sl].cpu(), n_mem)
+        for out in outs:
+            assert rel_fro(out[0, layer, :, :first].float().cpu(), ref) <= 1e-2, layer
+
+
 def test_prefill_form_many_tiles_repeat():
     """More CTAs than the SMs hold at once, repeated: every wait is met and the output repeats bit for bit."""
     n_kv, group, hd, Lq, n_mem, L = 8, 4, 128, 400, 64, 16
