@@ -817,7 +817,7 @@ cudaError_t launch_prefill(AttnArgs a, int n_ctx, int C, cudaStream_t st) {
 }
 
 template <int HD>
-cudaError_t launch_decode(AttnArgs a, int C, cudaStream_t st) {
+cudaError_t launch_decode(AttnArgs a, int C, int sms, cudaStream_t st) {
     a.tile_tok = 128 / a.group;
     a.per_block = (a.tile_tok * a.group + DE_ROWS - 1) / DE_ROWS;
     a.group_inv = 65536 / a.group + 1;
@@ -830,8 +830,6 @@ cudaError_t launch_decode(AttnArgs a, int C, cudaStream_t st) {
     // have no block of keys each
     const long long ctas = (long long)row_tiles * a.n_kv * C;
     const int blocks = (a.n_mem + a.Lq + 31) / 32;
-    int sms = 0;
-    if ((e = sm_count(&sms)) != cudaSuccess) return e;
     const int slots = (HD == 64 ? 4 : 3) * sms;
     const int splits = (int)std::max(1ll, std::min({8ll, slots / ctas, (long long)blocks / DE_WARPS}));
     cudaLaunchConfig_t cfg = {};
@@ -870,7 +868,7 @@ cudaError_t launch_attention(const DevState& s, int n_layers, const void* Q, int
     if (a.vec && ((reinterpret_cast<uintptr_t>(Q) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0) {
         const long long row_tiles = ((long long)a.group * Lq + DE_ROWS - 1) / DE_ROWS;
         if (row_tiles == 1 || row_tiles * a.n_kv * s.C <= DE_MAX_TILES)
-            return s.hd == 64 ? launch_decode<64>(a, s.C, st) : launch_decode<128>(a, s.C, st);
+            return s.hd == 64 ? launch_decode<64>(a, s.C, s.sms, st) : launch_decode<128>(a, s.C, s.sms, st);
         return s.hd == 64 ? launch_prefill<64>(a, s.C / n_layers, s.C, st) : launch_prefill<128>(a, s.C / n_layers, s.C, st);
     }
     return s.hd == 64 ? launch_t<bf16, 64>(a, s.C, st) : launch_t<bf16, 128>(a, s.C, st);

@@ -13,6 +13,7 @@
 
 #include "mone.h"
 #include "mone_internal.h"
+#include "per_device.h"
 
 using namespace mone;
 
@@ -623,6 +624,9 @@ mone_status mone_mem_init(const mone_config* cfg, const float* W1_0, const float
     const size_t r1 = w1_rows(s);  // rows of W1 over all chains (and heads): sizes the row tables
     mone_status rc = MONE_OK;
     auto step = [&](mone_status r) { if (rc == MONE_OK) rc = r; };
+    // the device's facts and the kernels' opt-ins, for every launch of the handle
+    step(cuda_status(sm_count(&s.sms)));
+    if (s.dtype == MONE_BF16) step(cuda_status(s.memory == MONE_MEM_SWIGLU ? swiglu_opt_in() : tc_device(&s.tc)));
     // the momentum of a matrix follows its weights in one allocation: one tensor map covers both
     step(dalloc(&s.W1, n1 * (s.momentum ? 2 : 1)));
     step(dalloc(&s.W2, n2 * (s.momentum ? 2 : 1)));

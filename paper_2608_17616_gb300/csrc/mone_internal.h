@@ -21,7 +21,11 @@ enum : int { DS_PHASE_A_TILE = 1, DS_PHASE_B_TILE = 2, DS_READ_TILE = 3, DS_RESI
              DS_TMA_X = 5 };
 
 // Device-resident state of all chains (see mone_mem_init).
+struct TcDevice;  // what the tensor-core launches need to know of a device
+
 struct DevState {
+    int sms;                      // multiprocessors of the handle's device
+    const TcDevice* tc;           // bf16 MLP memory
     int C, d_in, d_hid, d_out, n_kv, hd, T, dtype, mode, momentum, renorm, loss;
     int memory, heads;            // MLP (heads 1) or per-head SwiGLU (d_hid = hidden units per head)
     float lr, rms_eps;
@@ -155,6 +159,8 @@ struct SwInputMaps {
     CUtensorMap Xa, Xb;        // caller's X of a group (dh, heads, rows, chains): K-major and MN boxes
     CUtensorMap Ka, Kb, Va, Vb;  // caller's K, V (dh, heads per half, rows, chains)
 };
+// Opt the SwiGLU kernels in to their shared memory on the current device (once per device).
+cudaError_t swiglu_opt_in();
 cudaError_t launch_swiglu_phase_a(const DevState& s, const SwMaps& m, const SwInputMaps& in, const SegWork& w,
                                   cudaStream_t st);
 cudaError_t launch_swiglu_phase_b(const DevState& s, const SwMaps& m, const SwInputMaps& in, const SegWork& w,
@@ -194,6 +200,9 @@ struct TcInputMaps {
     // per call: K-major {64,128} (a), MN-major blocks (b): 256 columns of X, 128 of X (b2, CTA pairs), K and V
     CUtensorMap Xa, Xb, Xb2, Ka, Kb, Va, Vb;
 };
+// The current device's TcDevice (valid until the process ends); the first call for a device opts the kernels of
+// ttl_tc.cu in to their shared memory.
+cudaError_t tc_device(const TcDevice** out);
 cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                               cudaStream_t st);
 cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,

@@ -828,26 +828,6 @@ __global__ void __launch_bounds__(256) swiglu_rows_kernel(SwArgs a, int mode, in
     }
 }
 
-// The current device's SM count; the first call for a device opts every kernel in to its shared memory.
-cudaError_t sw_device(int* sms) {
-    static PerDevice<int> devices;
-    const int* n;
-    const cudaError_t r = devices.get(&n, [](int& v) {
-        cudaError_t e = sm_count(&v);
-        auto opt_in = [&](auto kernel, int dyn) {
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-        };
-        opt_in(swiglu_b_kernel<false>, SwLayoutB::DYN);
-        opt_in(swiglu_b_kernel<true>, SwLayoutB::DYN);
-        opt_in(swiglu_a_kernel, SwLayout::DYN);
-        opt_in(swiglu_rh_kernel, SwLayout::DYN);
-        opt_in(swiglu_ro_kernel, SwLayout::DYN);
-        return e;
-    });
-    if (r == cudaSuccess) *sms = *n;
-    return r;
-}
-
 SwArgs sw_args(const DevState& s, const SegWork& w) {
     SwArgs a{};
     a.H = s.heads; a.dh = s.d_in / s.heads; a.Hk = (s.d_out / 2) / a.dh; a.F = s.d_hid; a.T = s.T; a.Tp = w.Tp;
@@ -871,15 +851,29 @@ SwArgs sw_args(const DevState& s, const SegWork& w) {
 
 }  // namespace
 
+cudaError_t swiglu_opt_in() {
+    static PerDevice<SmemOptIn> once;
+    const SmemOptIn* v;
+    return once.get(&v, [](SmemOptIn&) {
+        cudaError_t e = cudaSuccess;
+        auto opt_in = [&](auto kernel, int dyn) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+        };
+        opt_in(swiglu_b_kernel<false>, SwLayoutB::DYN);
+        opt_in(swiglu_b_kernel<true>, SwLayoutB::DYN);
+        opt_in(swiglu_a_kernel, SwLayout::DYN);
+        opt_in(swiglu_rh_kernel, SwLayout::DYN);
+        opt_in(swiglu_ro_kernel, SwLayout::DYN);
+        return e;
+    });
+}
+
 cudaError_t launch_swiglu_phase_a(const DevState& s, const SwMaps& m, const SwInputMaps& in, const SegWork& w,
                                   cudaStream_t st) {
-    int n_sms;
-    cudaError_t e = sw_device(&n_sms);
-    if (e != cudaSuccess) return e;
     SwArgs a = sw_args(s, w);
     a.nc_launch = w.nc;
     const int ntiles = (s.T / 128) * ((a.F + 127) / 128) * w.nc * a.H;
-    const int sms = n_sms - s.reserve_sms;  // leave the host-input gather's SMs free
+    const int sms = s.sms - s.reserve_sms;  // leave the host-input gather's SMs free
     const int grid = ntiles < sms ? ntiles : sms;
     swiglu_a_kernel<<<grid, SW_THREADS, SwLayout::DYN, st>>>(s.mode == 1 ? m.Ua : in.Xa, in.Ka, in.Va, m.W1a, m.W2a, a);
     return cudaGetLastError();
@@ -887,13 +881,10 @@ cudaError_t launch_swiglu_phase_a(const DevState& s, const SwMaps& m, const SwIn
 
 cudaError_t launch_swiglu_phase_b(const DevState& s, const SwMaps& m, const SwInputMaps& in, const SegWork& w,
                                   cudaStream_t st) {
-    int n_sms;
-    cudaError_t e = sw_device(&n_sms);
-    if (e != cudaSuccess) return e;
     SwArgs a = sw_args(s, w);
     a.nc_launch = w.nc;
     const int ntiles = w.nc * a.H * 3 * ((a.F + SWB_N - 1) / SWB_N) * ((a.dh + 127) / 128);
-    const int sms = n_sms - s.reserve_sms;  // leave the host-input gather's SMs free
+    const int sms = s.sms - s.reserve_sms;  // leave the host-input gather's SMs free
     const int grid = ntiles < sms ? ntiles : sms;
     if (a.step_sq)
         swiglu_b_kernel<true><<<grid, SWB_THREADS, SwLayoutB::DYN, st>>>(s.mode == 1 ? m.Ub : in.Xb, in.Kb, in.Vb, m.PG,
@@ -914,9 +905,7 @@ cudaError_t launch_swiglu_rows(const DevState& s, int mode, int parity, int c0, 
 }
 
 cudaError_t launch_swiglu_read(const DevState& s, const SwMaps& m, const void* Uq, void* Zq, int Q, cudaStream_t st) {
-    int n_sms;
-    cudaError_t e = sw_device(&n_sms);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     SegWork w{};
     w.c0 = 0;
     w.nc = s.C;

@@ -13,7 +13,6 @@
 #include <algorithm>
 
 #include "mone_common.cuh"
-#include "per_device.h"
 
 namespace mone {
 
@@ -265,12 +264,9 @@ __global__ void __launch_bounds__(256) prepass_kernel(const PrepassArgs a) {
 }
 
 template <typename Tin, typename Tout>
-cudaError_t launch_one(const PrepassArgs& a, int nchains, cudaStream_t st) {
+cudaError_t launch_one(const PrepassArgs& a, int nchains, int sms, cudaStream_t st) {
     // two rows a warp share the meta-parameter loads; few rows (less than two CTAs an SM that way) are spread
     // one a warp instead (512 rows of one chain, d_in = 2048, caches cold: 11.1 -> 9.2 us)
-    int sms = 0;
-    const cudaError_t e = sm_count(&sms);
-    if (e != cudaSuccess) return e;
     if ((long long)((a.rows + 15) / 16) * nchains >= 2 * sms)
         prepass_kernel<Tin, Tout, 2><<<dim3((a.rows + 15) / 16, nchains), 256, 0, st>>>(a);
     else
@@ -306,7 +302,7 @@ cudaError_t launch_prepass(const DevState& s, const SegWork& w, cudaStream_t st)
     a.dbeta = s.dbeta;
     a.zero = w.zero_loss;
     a.zinv = s.dtype == 1 ? s.zinv : nullptr;  // bf16 path: unnormalised z + row scale
-    return s.dtype == 0 ? launch_one<float, float>(a, w.nc, st) : launch_one<bf16, bf16>(a, w.nc, st);
+    return s.dtype == 0 ? launch_one<float, float>(a, w.nc, s.sms, st) : launch_one<bf16, bf16>(a, w.nc, s.sms, st);
 }
 
 // Query side of the read on the bf16 path, in one pass: a warp to one or two query tokens of a chain.
@@ -490,8 +486,8 @@ cudaError_t launch_query_transform(const DevState& s, const void* Xq, int Q, voi
     a.alpha = s.alpha;
     a.gamma = s.gamma;
     a.U = U;
-    if (s.dtype == 0) return launch_one<float, float>(a, s.C, st);
-    return bf16_out ? launch_one<bf16, bf16>(a, s.C, st) : launch_one<bf16, float>(a, s.C, st);
+    if (s.dtype == 0) return launch_one<float, float>(a, s.C, s.sms, st);
+    return bf16_out ? launch_one<bf16, bf16>(a, s.C, s.sms, st) : launch_one<bf16, float>(a, s.C, s.sms, st);
 }
 
 }  // namespace mone

@@ -1114,31 +1114,25 @@ cudaError_t phase_b_f32(const DevState& s, const SegWork& w, const F32SegArgs& a
 
 cudaError_t launch_phase_a_f32(const DevState& s, const SegWork& w, cudaStream_t st) {
     const F32SegArgs a = make_f32_args(s, w);
-    int sms = 0;
-    const cudaError_t e = sm_count(&sms);
-    if (e != cudaSuccess) return e;
     const long long g64 = (long long)(s.T / 64) * (s.d_hid / 64) * w.nc;  // 64 x 64 tiles (T, d_hid multiples of 64)
     // 32 x 64 tiles, but 64 x 64 (8 x 4 outputs a thread) where halving the tiles saves nothing of the last wave.
     // 1024 -> 1024 -> 1024, T = 256, 32 x 64 and 64 x 64 tiles: one chain (64 tiles of 64 x 64) 48 and 73 us,
     // three 102 and 123, four (256) 135 and 123, five 163 and 180, eight 223 and 234
-    const auto waves = [&](long long tiles) { return (tiles + sms - 1) / sms; };
-    if (g64 > sms && waves(2 * g64) == 2 * waves(g64)) return phase_a_f32<8, 4, 8>(s, w, a, st);
+    const auto waves = [&](long long tiles) { return (tiles + s.sms - 1) / s.sms; };
+    if (g64 > s.sms && waves(2 * g64) == 2 * waves(g64)) return phase_a_f32<8, 4, 8>(s, w, a, st);
     return phase_a_f32<4, 4, 8>(s, w, a, st);
 }
 
 cudaError_t launch_phase_b_f32(const DevState& s, const SegWork& w, cudaStream_t st) {
     const F32SegArgs a = make_f32_args(s, w);
-    int sms = 0;
-    const cudaError_t e = sm_count(&sms);
-    if (e != cudaSuccess) return e;
     // a tile lies in W1 or in one half of W2: widths are multiples of 64, for the large tile of 128, which
     // is taken from two thirds of the SMs on
     const bool wide = s.d_in % 128 == 0 && (s.d_out / 2) % 128 == 0 && s.d_hid % 128 == 0;
-    if (wide && (long long)(s.d_hid / 128) * ((s.d_in + s.d_out) / 128) * w.nc >= sms * 2 / 3)
+    if (wide && (long long)(s.d_hid / 128) * ((s.d_in + s.d_out) / 128) * w.nc >= s.sms * 2 / 3)
         return phase_b_f32<8, 8, 16>(s, w, a, st);
     // 64 x 64 tiles from two to an SM on (2 chains of 1024 -> 512 -> 512, T = 512: 49 us, 32 x 64 tiles 53), else 32 x
     // 64 (one chain, T = 64: 13.9 and 11.9 us); with 256 threads of 4 x 4 outputs 64 x 64 tiles take 55 and 12.2
-    if ((long long)(s.d_hid / 64) * ((s.d_in + s.d_out) / 64) * w.nc > 2 * sms) return phase_b_f32<8, 4, 8>(s, w, a, st);
+    if ((long long)(s.d_hid / 64) * ((s.d_in + s.d_out) / 64) * w.nc > 2 * s.sms) return phase_b_f32<8, 4, 8>(s, w, a, st);
     return phase_b_f32<4, 4, 8>(s, w, a, st);
 }
 
@@ -1175,15 +1169,14 @@ cudaError_t launch_resident_f32(const DevState& s, const SegWork& w, long long n
     a.step_sq = w.step0;
     a.m_sstride = w.loss0 || w.step0 ? w.mstride : 0;
     a.status = s.status;
-    int sms = 0;
-    cudaError_t e = sm_count(&sms);
+    cudaError_t e = cudaSuccess;
     // four rows a CTA while that still fits the chains in one wave, else eight (less re-streaming)
     const int D = s.d_in + s.d_out;
     static PerDevice<SmemOptIn> once4, once8;
     if (e == cudaSuccess) e = smem_opt_in(reinterpret_cast<const void*>(ttl_resident_f32_kernel<4>), res_smem_bytes<4>(512), once4);
     if (e == cudaSuccess) e = smem_opt_in(reinterpret_cast<const void*>(ttl_resident_f32_kernel<8>), res_smem_bytes<8>(512), once8);
     if (e != cudaSuccess) return e;
-    if ((long long)w.nc * (s.d_hid / 4) <= sms)
+    if ((long long)w.nc * (s.d_hid / 4) <= s.sms)
         ttl_resident_f32_kernel<4><<<dim3(s.d_hid / 4, w.nc), RES_NT, res_smem_bytes<4>(D), st>>>(a);
     else
         ttl_resident_f32_kernel<8><<<dim3(s.d_hid / 8, w.nc), RES_NT, res_smem_bytes<8>(D), st>>>(a);

@@ -35,6 +35,14 @@
 
 namespace mone {
 
+// What the launches need to know of a device.
+struct TcDevice {
+    int sms;
+    int pair_clusters;   // co-resident CTA pairs of the phase A pair kernel (0: use the one-CTA kernel)
+    int pairb_clusters;  // the same for the phase B pair kernel
+    int split4, split2;  // co-resident clusters of the phase A split kernels
+};
+
 namespace {
 
 constexpr int BK = 64;                    // 64 bf16 = one 128-byte swizzle row
@@ -2063,15 +2071,6 @@ tc_read_t_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     if (warp == 0) tmem_dealloc(tmem, RT_MAX_NT);
 }
 
-// What the launches need to know of a device.
-struct TcDevice {
-    int sms;
-    int pair_clusters;   // co-resident CTA pairs of the phase A pair kernel (0: use the one-CTA kernel)
-    int pairb_clusters;  // the same for the phase B pair kernel
-    int split4, split2;  // co-resident clusters of the phase A split kernels
-};
-PerDevice<TcDevice> g_devices;
-
 // Launch a read-structured kernel with the stage count that suits its grid (see LRT).
 template <int MODE>
 cudaError_t launch_read_kernel(const TcDevice& dev, dim3 grid, const CUtensorMap& A, const CUtensorMap& B, const ReadArgs& a,
@@ -2095,9 +2094,16 @@ cudaError_t launch_read_many(const TcDevice& dev, dim3 grid, const CUtensorMap& 
                          LRP::DYN, st, false, 2, A, B, a);
 }
 
-// The current device's TcDevice; the first call for a device opts every kernel in to its shared memory.
+// Whether phase A runs on CTA pairs (256-token x 256-hidden tiles) for this handle's shape.
+bool phase_a_pairs(const DevState& s, const TcDevice& dev) {
+    return (s.T / A_BM) % 2 == 0 && s.d_hid % P_BN == 0 && dev.pair_clusters > 0;
+}
+
+}  // namespace
+
 cudaError_t tc_device(const TcDevice** out) {
-    return g_devices.get(out, [](TcDevice& d) {
+    static PerDevice<TcDevice> devices;
+    return devices.get(out, [](TcDevice& d) {
         cudaError_t e = sm_count(&d.sms);
         auto opt_in = [&](auto kernel, int dyn) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
@@ -2145,18 +2151,9 @@ cudaError_t tc_device(const TcDevice** out) {
     });
 }
 
-// Whether phase A runs on CTA pairs (256-token x 256-hidden tiles) for this handle's shape.
-bool phase_a_pairs(const DevState& s, const TcDevice& dev) {
-    return (s.T / A_BM) % 2 == 0 && s.d_hid % P_BN == 0 && dev.pair_clusters > 0;
-}
-
-}  // namespace
-
 cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                               cudaStream_t st) {
-    const TcDevice* dev;
-    cudaError_t e = tc_device(&dev);
-    if (e != cudaSuccess) return e;
+    const TcDevice& dev = *s.tc;
     TcArgs a = make_args(s, w);
     if (s.fault_stall > 0) {  // test knob: this launch's waits run out after 1 ms with nothing in flight
         --s.fault_stall;
@@ -2168,24 +2165,24 @@ cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputM
     // few tiles of a call on one stream (its other kernels leave the SMs to this one): clusters of 4 or 2 a tile
     const int tiles = w.nc * (s.T / A_BM) * (s.d_hid / A_BN);
     if (w.single && s.loss == 0) {
-        if (tiles <= dev->split4 && s.d_in >= 4 * BK && s.d_out >= 4 * BK)
+        if (tiles <= dev.split4 && s.d_in >= 4 * BK && s.d_out >= 4 * BK)
             return launch_kernel(tc_phase_a_split_kernel<4>, dim3(4 * tiles), dim3(THREADS), LSplit<4>::DYN, st, pdl, 4, U,
                                  in.Ka, in.Va, m.W1b, m.W2b, a);
-        if (tiles <= dev->split2)
+        if (tiles <= dev.split2)
             return launch_kernel(tc_phase_a_split_kernel<2>, dim3(2 * tiles), dim3(THREADS), LSplit<2>::DYN, st, pdl, 2, U,
                                  in.Ka, in.Va, m.W1b, m.W2b, a);
     }
-    if (phase_a_pairs(s, *dev)) {
+    if (phase_a_pairs(s, dev)) {
         // squared-error segments: the pre-pass wrote At and c SiLU'(x) / |z|, only R is left
         a.r_only = (s.loss == 1) ? 1 : 0;  // 1: MONE_LOSS_MSE
         // CTA pairs over 256-token x 256-hidden tiles
         const int npairs = w.nc * (s.T / (2 * A_BM)) * (s.d_hid / P_BN);
-        const int maxc = dev->pair_clusters - (s.reserve_sms + 1) / 2;  // leave reserved SMs free
+        const int maxc = dev.pair_clusters - (s.reserve_sms + 1) / 2;  // leave reserved SMs free
         const int clusters = npairs < maxc ? npairs : maxc;
         return launch_kernel(tc_phase_a_pair_kernel, dim3(2 * clusters), dim3(THREADS), LP::DYN, st, pdl && !a.r_only, 2, U,
                              in.Ka, in.Va, m.W1b, m.W2b, a);
     }
-    const int sms = dev->sms - s.reserve_sms;
+    const int sms = dev.sms - s.reserve_sms;
     const int grid = tiles < sms ? tiles : sms;
     return launch_kernel(tc_phase_a_kernel, dim3(grid), dim3(THREADS), LA::DYN, st, pdl && s.loss == 0, 1, U, in.Ka, in.Va,
                          m.W1b, m.W2b, a);
@@ -2193,15 +2190,13 @@ cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputM
 
 cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                               cudaStream_t st) {
-    const TcDevice* dev;
-    cudaError_t e = tc_device(&dev);
-    if (e != cudaSuccess) return e;
+    const TcDevice& dev = *s.tc;
     TcArgs a = make_args(s, w);
     // CTA pairs over 256-hidden x 256-column tiles (a tile's columns all live) from T = 1024 on:
     // there a tile's operand stream (768 KB a CTA) rivals its state stream, and the pair takes a
     // third off it.  At T = 512 the pair's coupled loads and accumulator release cost more than they save.
     constexpr int PAIR_MIN_T = 1024;
-    const bool pairs = s.T >= PAIR_MIN_T && s.d_in % B_BN == 0 && dev->pairb_clusters > 0;
+    const bool pairs = s.T >= PAIR_MIN_T && s.d_in % B_BN == 0 && dev.pairb_clusters > 0;
     // When the state ring's slots are handed back, by what was fastest: how stores and loads alternate
     // decides how much of HBM the stream gets.  With no momentum, on CTA pairs, for one chain, or with W and mu of
     // the whole handle in L2, two at a time, one store later (ms, against one by one three stores later: 64 plain chains of
@@ -2218,14 +2213,14 @@ cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputM
     const int col_tiles = b_col_tiles(s.d_in, s.d_out);
     if (pairs) {
         const int npairs = w.nc * col_tiles * (s.d_hid / (2 * B_BM));
-        const int maxc = dev->pairb_clusters - (s.reserve_sms + 1) / 2;
+        const int maxc = dev.pairb_clusters - (s.reserve_sms + 1) / 2;
         const int clusters = npairs < maxc ? npairs : maxc;
         return launch_kernel(a.step_sq ? tc_phase_b_kernel<true, true> : tc_phase_b_kernel<true, false>, dim3(2 * clusters),
                              dim3(B_THREADS), LayoutB2::DYN, st, w.single != 0, 2, U2, in.Kb, in.Vb, m.dH, m.At, m.W1s,
                              m.W2s, a);
     }
     const int ntiles = w.nc * col_tiles * (s.d_hid / B_BM);
-    const int sms = dev->sms - s.reserve_sms;
+    const int sms = dev.sms - s.reserve_sms;
     const int grid = ntiles < sms ? ntiles : sms;
     return launch_kernel(a.step_sq ? tc_phase_b_kernel<false, true> : tc_phase_b_kernel<false, false>, dim3(grid),
                          dim3(B_THREADS), LayoutB::DYN, st, w.single != 0, 1, U, in.Kb, in.Vb, m.dH, m.At, m.W1s, m.W2s, a);
@@ -2235,9 +2230,7 @@ int tc_kernels_per_segment() { return 2; }
 
 cudaError_t launch_mse_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                           cudaStream_t st) {
-    const TcDevice* dev;
-    cudaError_t e = tc_device(&dev);
-    if (e != cudaSuccess) return e;
+    const TcDevice& dev = *s.tc;
     const bool paper = s.mode == 1;
     ReadArgs a{};
     a.d_in = s.d_in; a.d_hid = s.d_hid; a.d_out = s.d_out; a.n_kv = s.n_kv;
@@ -2250,7 +2243,7 @@ cudaError_t launch_mse_tc(const DevState& s, const TcMaps& m, const TcInputMaps&
     a.Kres = s.Kres; a.Vres = s.Vres;
     a.loss = w.loss;
     a.Aq = s.Amse;
-    if (phase_a_pairs(s, *dev)) {  // phase A runs in its R-only form: write At and c SiLU'(x) / |z| here
+    if (phase_a_pairs(s, dev)) {  // phase A runs in its R-only form: write At and c SiLU'(x) / |z| here
         a.At = reinterpret_cast<bf16*>(s.Att);
         a.Sp = reinterpret_cast<bf16*>(s.dHt);
         a.paper = paper ? 1 : 0;
@@ -2264,22 +2257,21 @@ cudaError_t launch_mse_tc(const DevState& s, const TcMaps& m, const TcInputMaps&
     a.a_row0 = paper ? (int)w.u_off : (int)w.row0;
     a.a_chain0 = paper ? w.c0 : 0;
     a.b_chain0 = w.c0;
-    e = launch_read_kernel<MSE_HIDDEN>(*dev, dim3(s.T / 128, s.d_hid / 128, w.nc), paper ? m.Ua : in.Xa, m.W1b, a, st);
+    cudaError_t e = launch_read_kernel<MSE_HIDDEN>(dev, dim3(s.T / 128, s.d_hid / 128, w.nc), paper ? m.Ua : in.Xa, m.W1b, a, st);
     if (e != cudaSuccess) return e;
     // out: the activations of the same chains (absolute), W2 MN-major
     a.a_row0 = 0;
     a.a_chain0 = w.c0;
-    return launch_read_kernel<MSE_OUT>(*dev, dim3(s.T / 128, s.d_out / 128, w.nc), m.Amse, m.W2m, a, st);
+    return launch_read_kernel<MSE_OUT>(dev, dim3(s.T / 128, s.d_out / 128, w.nc), m.Amse, m.W2m, a, st);
 }
 
 cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, void* Uq, void* Aq, float* zq, int Q,
                            int n_layers, void* K_out, void* V_out, const long long* strides, cudaStream_t st) {
-    const TcDevice* dev;
-    cudaError_t e = tc_device(&dev);
-    if (e != cudaSuccess) return e;
+    const TcDevice& dev = *s.tc;
     if (s.hd != 64 && s.hd != 128) return cudaErrorInvalidValue;
     // the query side: unnormalised z and 1/|z|, which the hidden kernel applies
-    if ((e = launch_query_z(s, Xq, Q, Uq, zq, st)) != cudaSuccess) return e;
+    cudaError_t e = launch_query_z(s, Xq, Q, Uq, zq, st);
+    if (e != cudaSuccess) return e;
     ReadArgs a{};
     a.Q = Q; a.d_in = s.d_in; a.d_hid = s.d_hid; a.d_out = s.d_out; a.n_kv = s.n_kv; a.L = n_layers;
     a.eps = s.rms_eps;
@@ -2293,8 +2285,8 @@ cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, v
     if (Q <= RT_MAX_NT) {  // weights as the 128-row operand, the queries as N
         const int NT = (Q + 31) / 32 * 32;
         // one CTA per SM with the deep ring when a kernel's tiles fit in one wave, else two
-        const int ring1 = (long long)(s.d_hid / 128) * s.C <= dev->sms ? RT_RING_1 : RT_RING_2;
-        const int ring2 = (long long)(s.d_out / 128) * s.C <= dev->sms ? RT_RING_1 : RT_RING_2;
+        const int ring1 = (long long)(s.d_hid / 128) * s.C <= dev.sms ? RT_RING_1 : RT_RING_2;
+        const int ring2 = (long long)(s.d_out / 128) * s.C <= dev.sms ? RT_RING_1 : RT_RING_2;
         const int k1 = rt_kblocks(NT, ring1), k2 = rt_kblocks(NT, ring2);
         CUtensorMap tu, ta;
         if (!encode_map_bf16_blocks(&tu, Uq, s.d_in, Q, s.C, NT, k1) || !encode_map_bf16_blocks(&ta, Aq, s.d_hid, Q, s.C, NT, k2))
@@ -2321,9 +2313,9 @@ cudaError_t launch_read_tc(const DevState& s, const TcMaps& m, const void* Xq, v
     if (!encode_map_bf16_3d(&mu, Uq, s.d_in, Q, s.C, 64, 128) || !encode_map_bf16_3d(&ma, Aq, s.d_hid, Q, s.C, 64, 128))
         return cudaErrorInvalidValue;
     const int nq = (Q + 127) / 128;
-    if ((e = launch_read_many<READ_HIDDEN>(*dev, dim3(nq, s.d_hid / 128, s.C), mu, m.W1b, a, st)) != cudaSuccess) return e;
-    if (s.hd == 64) return launch_read_many<64>(*dev, dim3(nq, s.d_out / 128, s.C), ma, m.W2m, a, st);
-    return launch_read_many<128>(*dev, dim3(nq, s.d_out / 128, s.C), ma, m.W2m, a, st);
+    if ((e = launch_read_many<READ_HIDDEN>(dev, dim3(nq, s.d_hid / 128, s.C), mu, m.W1b, a, st)) != cudaSuccess) return e;
+    if (s.hd == 64) return launch_read_many<64>(dev, dim3(nq, s.d_out / 128, s.C), ma, m.W2m, a, st);
+    return launch_read_many<128>(dev, dim3(nq, s.d_out / 128, s.C), ma, m.W2m, a, st);
 }
 
 // ------------------------------------------------------------------ tensor maps

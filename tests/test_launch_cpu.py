@@ -109,3 +109,14 @@ def test_tile_rules_follow_the_devices_sm_count(fake):
     assert want[0]["phase_b"] == [(24, 16, 1)] and want[1]["phase_b"] == [(12, 8, 1)]
     assert want[0]["transform"] == [(512, 1, 1)] and want[1]["transform"] == [(256, 1, 1)]
     assert want[0]["decode"] == [8] and want[1]["decode"] == [6]
+
+
+@pytest.mark.parametrize("memory", [mone.MONE_MEM_MLP, mone.MONE_MEM_SWIGLU])
+def test_a_failed_bf16_opt_in_fails_the_init_and_is_tried_again(fake, memory):
+    args = (2, 512, 256, 512, 128, mone.MONE_BF16)
+    fake.fail_opt_ins(1)
+    with pytest.raises(mone.MoneError):
+        init(*args, memory=memory, mem_heads=2)
+    h = init(*args, memory=memory, mem_heads=2)
+    mone.mone_ttl_context(h, P, P, P, 1000, 0)
+    mone.mone_mem_free(h)
