@@ -342,7 +342,8 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
 #pragma unroll
             for (int kb = 0; kb < HD / 64; ++kb)  // the query rows, [head of the group][token]
                 tma_load_4d(smem_u32(base + SM::Q_OFF) + kb * SM::Q_SLAB, &tmQ, qfull, 64 * kb, r0, g * a.group, c);
-            const int ctx = c / a.L, layer = c % a.L;
+            // a dimension that the caches share (stride 0) has one element in the maps
+            const int ctx = a.s0 ? c / a.L : 0, layer = a.s1 ? c % a.L : 0, head = a.s2 ? g : 0;
             int s = 0, ph = 1;  // slot, and the phase of its release (the first round passes)
             auto load = [&](const CUtensorMap* m, int j) {
                 if (!mbar_wait(empty(s), ph, a.status)) return false;
@@ -350,7 +351,7 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                 mbar_expect_tx(full(s), SM::TILE);
 #pragma unroll
                 for (int kb = 0; kb < HD / 64; ++kb)
-                    tma_load_5d(dst + kb * SM::SLAB, m, full(s), 64 * kb, j * NK, g, layer, ctx);
+                    tma_load_5d(dst + kb * SM::SLAB, m, full(s), 64 * kb, j * NK, head, layer, ctx);
                 if (++s == NS) {
                     s = 0;
                     ph ^= 1;
@@ -366,7 +367,7 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                 mbar_expect_tx(vlast, SM::TILE);
 #pragma unroll
                 for (int kb = 0; kb < HD / 64; ++kb)
-                    tma_load_5d(smem_u32(base + SM::KV_OFF + s * SM::TILE) + kb * SM::SLAB, &tmV, vlast, 64 * kb, (n - 1) * NK, g,
+                    tma_load_5d(smem_u32(base + SM::KV_OFF + s * SM::TILE) + kb * SM::SLAB, &tmV, vlast, 64 * kb, (n - 1) * NK, head,
                                 layer, ctx);
                 landed = mbar_wait(vlast, 0, a.status);
             }
@@ -800,15 +801,14 @@ cudaError_t launch_prefill(AttnArgs a, int n_ctx, int C, cudaStream_t st) {
     CUtensorMap mq, mk, mv;
     const uint64_t qd[4] = {HD, Lq, (uint64_t)a.n_q, (uint64_t)C}, qs[3] = {HD * 2, Lq * HD * 2, a.n_q * Lq * HD * 2};
     const uint32_t qb[4] = {64, (uint32_t)a.rows, (uint32_t)a.group, 1};
-    // the caller's strides (a dimension of one element takes any stride)
-    const uint64_t kd[5] = {HD, keys, (uint64_t)a.n_kv, (uint64_t)a.L, (uint64_t)n_ctx};
+    // the caller's strides; a dimension that the caches share (stride 0) has one element, which takes any stride
+    const uint64_t kd[5] = {HD, keys, a.s2 ? (uint64_t)a.n_kv : 1, a.s1 ? (uint64_t)a.L : 1, a.s0 ? (uint64_t)n_ctx : 1};
     const uint64_t s3 = a.s3 * 2;
-    const uint64_t ks[4] = {s3, a.n_kv > 1 ? a.s2 * 2 : s3, a.L > 1 ? a.s1 * 2 : s3, n_ctx > 1 ? a.s0 * 2 : s3};
+    const uint64_t ks[4] = {s3, kd[2] > 1 ? a.s2 * 2 : s3, kd[3] > 1 ? a.s1 * 2 : s3, kd[4] > 1 ? a.s0 * 2 : s3};
     const uint32_t kb[5] = {64, FaSmem<HD>::NK, 1, 1, 1};
-    const bool broadcast = std::min({ks[0], ks[1], ks[2], ks[3]}) == 0;
-    if (broadcast || !encode_map_bf16_4d(&mq, a.Q, qd, qs, qb) || !encode_map_bf16_5d(&mk, a.K, kd, ks, kb) ||
+    if (!encode_map_bf16_4d(&mq, a.Q, qd, qs, qb) || !encode_map_bf16_5d(&mk, a.K, kd, ks, kb) ||
         !encode_map_bf16_5d(&mv, a.V, kd, ks, kb)) {
-        a.rows = rows0;  // strides a tensor map does not take (0, or past its range): the CUDA-core form
+        a.rows = rows0;  // strides past a tensor map's range (2^40 bytes): the CUDA-core form
         return launch_t<bf16, HD>(a, C, st);
     }
     dim3 grid((a.Lq + a.rows - 1) / a.rows, a.n_kv, C);

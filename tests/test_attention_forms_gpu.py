@@ -59,6 +59,46 @@ def test_prefill_form(group, Lq, n_mem, hd, late_scale):
     run_case(group, Lq, n_mem, hd, n_layers=20, late_scale=late_scale)
 
 
+def strided(kind, n_ctx, L, n_kv, S, hd, g):
+    """A [n_ctx, L, n_kv, S, hd] cache with the strides of `kind`."""
+    rn = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()  # noqa: E731
+    if kind == "dense":
+        return rn(n_ctx, L, n_kv, S, hd)
+    if kind == "padded":  # rows of a wider buffer, spare positions after the last key
+        return rn(n_ctx, L, n_kv, S + 37, hd + 24)[..., :S, :hd]
+    if kind == "heads inner":  # [position][head]
+        return rn(n_ctx, L, S, n_kv, hd).transpose(2, 3)
+    if kind == "layers inner":  # [head][position][layer]
+        return rn(n_ctx, n_kv, S, L, hd).permute(0, 3, 1, 2, 4)
+    one = dict(zip(("context", "layer", "head"), range(3)))
+    shape = [n_ctx, L, n_kv, S, hd]
+    for name in kind.split("+"):  # shared by every context, layer or head
+        shape[one[name]] = 1
+    return rn(*shape).expand(n_ctx, L, n_kv, S, hd)
+
+
+@pytest.mark.parametrize("kind", ["dense", "padded", "heads inner", "layers inner", "context", "layer", "head",
+                                  "context+layer", "layer+head", "context+layer+head"])
+@pytest.mark.parametrize("n_ctx,group,Lq,n_mem,hd", [(2, 2, 150, 200, 64), (3, 4, 70, 130, 128), (2, 1, 3, 300, 64)])
+def test_cache_strides(kind, n_ctx, group, Lq, n_mem, hd):
+    """Several contexts over several chunks of keys, through the tensor maps of the prefill form and the plain loads
+    of the decode form; a shared dimension has stride 0."""
+    n_kv, L = 2, 12
+    run = DeviceRun(wk.Workload("attn_forms", 45, n_ctx, L, 256, 256, 2 * n_kv * hd, n_kv, hd, 128, 128, 8, "bf16", wk.PLAIN))
+    g = torch.Generator(device="cuda").manual_seed(Lq + hd)
+    K, V = (strided(kind, n_ctx, L, n_kv, n_mem + Lq, hd, g) for _ in range(2))
+    assert K.stride() == V.stride() and K.stride(4) == 1
+    Q = torch.randn(n_ctx, L, group * n_kv, Lq, hd, generator=g, device="cuda").bfloat16()
+    out = torch.full_like(Q, 7.0)
+    mone.mone_attention(run.h, Q, group * n_kv, Lq, K, V, K.stride()[:4], n_mem, out)
+    mone.mone_mem_sync(run.h)
+    run.close()
+    for c in {0, n_ctx - 1}:
+        for layer in {0, L - 1}:
+            ref = O.attention(Q[c, layer].cpu(), K[c, layer].cpu(), V[c, layer].cpu(), n_mem)
+            assert rel_fro(out[c, layer].float().cpu(), ref) <= 1e-2, (c, layer)
+
+
 @pytest.mark.parametrize("hd,group,Lq,n_mem", [(64, 4, 200, 200), (128, 2, 150, 130), (64, 1, 3, 300)])
 def test_keys_at_minus_infinity_count_for_nothing(hd, group, Lq, n_mem):
     """The memory keys, whole chunks of them, overflow to scores of -inf; the tokens' own keys are ordinary."""

@@ -120,3 +120,20 @@ def test_a_failed_bf16_opt_in_fails_the_init_and_is_tried_again(fake, memory):
     h = init(*args, memory=memory, mem_heads=2)
     mone.mone_ttl_context(h, P, P, P, 1000, 0)
     mone.mone_mem_free(h)
+
+
+@pytest.mark.parametrize("strides", [(1, 1, 1), (0, 1, 1), (1, 0, 1), (1, 1, 0), (0, 0, 1), (0, 1, 0), (1, 0, 0), (0, 0, 0)])
+def test_attention_over_shared_caches_stays_on_the_tensor_cores(fake, strides):
+    """A cache that contexts, layers or heads share (stride 0) takes the prefill form, with one element of that dimension
+    in its maps."""
+    n_ctx, L, n_kv, hd, Lq, n_mem = 3, 8, 4, 64, 1000, 64
+    h = init(L, 512, 256, 2 * n_kv * hd, 128, mone.MONE_BF16, n_ctx=n_ctx)
+    dense = mone.kv_strides(L, n_kv, n_mem + Lq, hd)
+    fake.drain()
+    mone.mone_attention(h, P, n_kv, Lq, P, P + 4096, [s * k for s, k in zip(dense, strides)] + [hd], n_mem, P, 0)
+    launches, maps = fake.drain()
+    assert [x["name"] for x in launches if "prefill" in x["name"]] and len(launches) == 1
+    for base, dims in maps[1:]:  # K and V: (dimension, stride in bytes, box)
+        assert [d for d, _, _ in dims] == [hd, n_mem + Lq, n_kv if strides[2] else 1, L if strides[1] else 1, n_ctx if strides[0] else 1]
+        assert [s for (d, s, _), keep in zip(dims[2:], strides[::-1]) if keep] == [2 * s for s, keep in zip(dense[2::-1], strides[::-1]) if keep]
+    mone.mone_mem_free(h)
