@@ -241,6 +241,9 @@ bool encode_map_bf16_4d(CUtensorMap* map, const void* base, const uint64_t dims[
 bool encode_map_bf16_5d(CUtensorMap* map, const void* base, const uint64_t dims[5], const uint64_t strides[4],
                         const uint32_t box[5]);
 
+// Set the address of an encoded map (16-byte aligned).
+bool retarget_map(CUtensorMap* map, const void* base);
+
 // Launch a kernel; pdl: with programmatic stream serialisation (it may start before the kernel ahead
 // of it in the stream ends, and waits for it with griddepcontrol.wait); cluster: CTAs per cluster (x).
 template <typename... P, typename... A>

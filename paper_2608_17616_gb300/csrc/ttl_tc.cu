@@ -2324,17 +2324,24 @@ namespace {
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+typedef CUresult (*ReplaceAddressFn)(CUtensorMap*, void*);
 EncodeTiledFn g_encode = nullptr;
+ReplaceAddressFn g_replace = nullptr;
 std::once_flag g_encode_once;
+
+void* driver_entry(const char* name) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    return cudaGetDriverEntryPointByVersion(name, &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+                   q == cudaDriverEntryPointSuccess
+               ? fn
+               : nullptr;
+}
 
 EncodeTiledFn encoder() {
     std::call_once(g_encode_once, [] {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            g_encode = reinterpret_cast<EncodeTiledFn>(fn);
+        g_encode = reinterpret_cast<EncodeTiledFn>(driver_entry("cuTensorMapEncodeTiled"));
+        g_replace = reinterpret_cast<ReplaceAddressFn>(driver_entry("cuTensorMapReplaceAddress"));
     });
     return g_encode;
 }
@@ -2394,6 +2401,10 @@ bool encode_map_bf16_5d(CUtensorMap* map, const void* base, const uint64_t dims[
     return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), d, st, b, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool retarget_map(CUtensorMap* map, const void* base) {
+    return encoder() && g_replace && g_replace(map, const_cast<void*>(base)) == CUDA_SUCCESS;
 }
 
 bool encode_map_plain_3d(CUtensorMap* map, const void* base, bool f32, uint64_t inner, uint64_t rows,

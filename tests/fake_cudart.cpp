@@ -2,7 +2,7 @@
 // place of the real one.  Two devices with different SM counts; addresses are made up and nothing is
 // copied or run.  What the host code can get wrong is checked as on a device: a launch with more than 48 KB of
 // dynamic shared memory fails unless that kernel was opted in to as much on the current device.  Launches
-// and tensor maps are logged, one line each (fake_log).
+// and tensor maps (each encoding, and each address set) are logged, one line each (fake_log).
 #include <cuda.h>
 #include <cuda_runtime_api.h>
 
@@ -32,18 +32,31 @@ cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, int cluster, int 
     return cudaSuccess;
 }
 
-CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t rank, void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+std::map<int, std::string> g_maps;  // dimensions of an encoded map, by the number written into it
+
+CUresult replace(CUtensorMap* m, void* base) {
+    if ((uintptr_t)base & 15) return CUDA_ERROR_INVALID_VALUE;
+    int id;
+    std::memcpy(&id, m, sizeof(id));
+    g_log += "map " + std::to_string((uintptr_t)base) + g_maps.at(id) + "\n";
+    return CUDA_SUCCESS;
+}
+
+CUresult encode(CUtensorMap* m, CUtensorMapDataType, cuuint32_t rank, void* base, const cuuint64_t* dims, const cuuint64_t* strides,
                 const cuuint32_t* box, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                 CUtensorMapFloatOOBfill) {
     if ((uintptr_t)base & 15) return CUDA_ERROR_INVALID_VALUE;
-    g_log += "map " + std::to_string((uintptr_t)base);
+    std::string text;
     for (cuuint32_t i = 0; i < rank; ++i) {
         if (!dims[i] || dims[i] > 1ull << 32 || !box[i] || box[i] > 256) return CUDA_ERROR_INVALID_VALUE;
         if (i && (strides[i - 1] % 16 || strides[i - 1] >= 1ull << 40)) return CUDA_ERROR_INVALID_VALUE;
-        g_log += " " + std::to_string(dims[i]) + ":" + std::to_string(i ? strides[i - 1] : 0) + ":" + std::to_string(box[i]);
+        text += " " + std::to_string(dims[i]) + ":" + std::to_string(i ? strides[i - 1] : 0) + ":" + std::to_string(box[i]);
     }
-    g_log += "\n";
-    return CUDA_SUCCESS;
+    const int id = (int)g_maps.size();
+    g_maps[id] = text;
+    std::memcpy(m, &id, sizeof(id));
+    g_log += "encode\n";
+    return replace(m, base);
 }
 }  // namespace
 
@@ -99,8 +112,8 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, 
 cudaError_t cudaMemset(void*, int, size_t) { return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaGetSymbolAddress(void** p, const void*) { return cudaMalloc(p, 1 << 24); }
-cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned, unsigned long long, cudaDriverEntryPointQueryResult* q) {
-    *f = (void*)encode; *q = cudaDriverEntryPointSuccess;
+cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** f, unsigned, unsigned long long, cudaDriverEntryPointQueryResult* q) {
+    *f = std::strstr(name, "Replace") ? (void*)replace : (void*)encode; *q = cudaDriverEntryPointSuccess;
     return cudaSuccess;
 }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {  // every address: page-locked, device view = itself

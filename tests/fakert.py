@@ -24,13 +24,16 @@ class Fake:
         self.raw.fake_fail_opt_ins(n)
 
     def drain(self):
-        """The log since the last call: launches as dicts, tensor maps as (base, [(dim, stride, box), ..])."""
-        launches, maps = [], []
+        """The log since the last call: launches as dicts, tensor maps as (base, [(dim, stride, box), ..]) each time their
+        address is set; self.encoded counts the encodings."""
+        launches, maps, self.encoded = [], [], 0
         for line in self.raw.fake_log().decode().splitlines():
             f = line.split()
             if f[0] == "launch":
                 launches.append(dict(dev=int(f[1]), name=f[2], grid=tuple(map(int, f[3:6])), block=int(f[6]),
                                      smem=int(f[7]), cluster=int(f[8]), pdl=int(f[9])))
+            elif f[0] == "encode":
+                self.encoded += 1
             else:
                 maps.append((int(f[1]), [tuple(map(int, p.split(":"))) for p in f[2:]]))
         self.raw.fake_clear()

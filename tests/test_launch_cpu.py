@@ -133,7 +133,28 @@ def test_attention_over_shared_caches_stays_on_the_tensor_cores(fake, strides):
     mone.mone_attention(h, P, n_kv, Lq, P, P + 4096, [s * k for s, k in zip(dense, strides)] + [hd], n_mem, P, 0)
     launches, maps = fake.drain()
     assert [x["name"] for x in launches if "prefill" in x["name"]] and len(launches) == 1
-    for base, dims in maps[1:]:  # K and V: (dimension, stride in bytes, box)
+    assert [m[0] for m in maps[-3:]] == [P, P, P + 4096]
+    for base, dims in maps[-2:]:  # K and V: (dimension, stride in bytes, box)
         assert [d for d, _, _ in dims] == [hd, n_mem + Lq, n_kv if strides[2] else 1, L if strides[1] else 1, n_ctx if strides[0] else 1]
         assert [s for (d, s, _), keep in zip(dims[2:], strides[::-1]) if keep] == [2 * s for s, keep in zip(dense[2::-1], strides[::-1]) if keep]
+    mone.mone_mem_free(h)
+
+
+def test_attention_maps_follow_the_calls_addresses_and_shape(fake):
+    h = init(8, 512, 256, 512, 128, mone.MONE_BF16)
+
+    def call(q, k, v, Lq=1000, n_mem=64, pad=0):
+        fake.drain()
+        mone.mone_attention(h, q, 4, Lq, k, v, mone.kv_strides(8, 4, n_mem + Lq + pad, 64), n_mem, P, 0)
+        _, maps = fake.drain()
+        assert [m[0] for m in maps[-3:]] == [q, k, v]
+        assert maps[-3][1][1][0] == Lq and maps[-2][1] == maps[-1][1] and maps[-1][1][1][0] == n_mem + Lq
+        assert maps[-1][1][2][1] == 2 * 64 * (n_mem + Lq + pad)
+        return fake.encoded
+
+    assert call(P, P + 256, P + 512) == 2
+    assert call(P + 1024, P + 2048, P + 4096) == 0  # the same shape elsewhere
+    assert call(P, P + 256, P + 512, n_mem=65) == 2
+    assert call(P, P + 256, P + 512, n_mem=65, pad=8) == 2
+    assert call(P, P + 256, P + 512) == 2
     mone.mone_mem_free(h)
