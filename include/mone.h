@@ -173,8 +173,9 @@ mone_status mone_ttl_context(mone_mem* m, const void* X, const void* K, const vo
  * the library choose: about an eighth of the context, at least two segments and 32 MB of
  * X, K and V, at most 512 MB): the library gathers chunk k+1 into one of two device windows
  * (owned by the handle, grown on demand; growing synchronises the stream) on its own
- * staging stream while chunk k is learned on `stream`, so the result equals
- * mone_ttl_context on the same tokens.  Asynchronous:
+ * staging stream while chunk k is learned on `stream`.  The result is that of mone_ttl_context:
+ * with chunk_tokens 0 of one call on all N tokens, else of one call per chunk in turn (a call
+ * ends with the rescaled weights rounded to the operands' type).  Asynchronous:
  * the host buffers must stay valid and unchanged until `stream` has passed the call
  * (mone_mem_sync or a stream synchronisation).  Kernel kind 8 times the gathers.
  * Errors: INVALID_ARG (null or unaligned pointer, device or managed memory, a range

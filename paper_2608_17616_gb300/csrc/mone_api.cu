@@ -426,8 +426,8 @@ mone_status run_segment_loop(mone_mem* m, SegWork* gw, TcInputMaps* gin, TcInput
             const cudaStream_t sg = gs[g];
             x.row0 = row0;
             x.Tp = (int)std::min<long long>(s.T, N - row0);
-            x.parity = (int)(i & 1);
-            x.renorm_pending = (s.renorm && i > 0) ? 1 : 0;
+            x.parity = (int)((w.seg0 + i) & 1);
+            x.renorm_pending = (s.renorm && w.seg0 + i > 0) ? 1 : 0;
             x.u_off = u_off;
             x.first = i == 0 && s.mode != MONE_PAPER;  // paper mode: the input transform comes first
             if (x.loss0) x.loss = x.loss0 + i * x.mstride;
@@ -463,8 +463,8 @@ mone_status run_segment_loop(mone_mem* m, SegWork* gw, TcInputMaps* gin, TcInput
         }
     }
     MONE_TRY(join());
-    if (s.renorm) {
-        const int par = (int)((S - 1) & 1);
+    if (s.renorm && !w.more) {
+        const int par = (int)((w.seg0 + S - 1) & 1);
         if (s.memory == MONE_MEM_SWIGLU)
             MONE_TRY(timed(m, K_FINALIZE, st, 1, [&] { return launch_swiglu_rows(s, 1, par, w.c0, w.nc, st); }));
         else
@@ -555,8 +555,7 @@ mone_status host_device_view(const void* p, size_t bytes, const void** out) {
 
 // Chunks when the caller leaves their length to the library: an eighth of the context, so that little
 // of it is gathered before any is learned, but at least two segments and about 32 MB of X, K and V (a
-// chunk's learning ends with the renormalisation pass over the weights, and its launches do not
-// overlap the last chunk's), and at most about 512 MB.  4096 tokens of 16 chains of 2048 -> 1024 -> 1024
+// chunk's launches do not overlap the last chunk's), and at most about 512 MB.  4096 tokens of 16 chains of 2048 -> 1024 -> 1024
 // (402 MB, gathered in 1.9 ms and learned in 1.75): 4.08 ms with its copies in one chunk, 3.03 in four.
 constexpr long long kHostChunkBytes = 512ll << 20, kHostChunkMinBytes = 32ll << 20, kHostChunks = 8;
 
@@ -808,8 +807,9 @@ mone_status mone_ttl_context(mone_mem* m, const void* X, const void* K, const vo
 
 // Test-time learning of a context held in host memory: chunks of whole segments are gathered
 // into two device windows on the staging stream while the previous chunk is learned on the
-// caller's stream (the learning of each chunk is the call mone_ttl_context makes, continuing
-// the state, so the chunks together equal one call on all N tokens).
+// caller's stream.  A chunk of the caller's length is learned by the call mone_ttl_context makes,
+// continuing the state; the library's own chunks are parts of one such call on all N tokens: the row
+// renormalisation stays pending from one to the next and is applied after the last.
 mone_status mone_ttl_context_host(mone_mem* m, const void* X, const void* K, const void* V, long long N,
                                   long long chunk_tokens, void* stream) {
     if (!is_live(m)) return MONE_ERR_INVALID_ARG;
@@ -882,6 +882,10 @@ mone_status mone_ttl_context_host(mone_mem* m, const void* X, const void* K, con
         w.x_cstride = nr * s.d_in;
         w.y_cstride = nr * (s.d_out / 2);
         w.n_rows = nr;
+        if (chunk_tokens == 0) {  // the library's chunks are parts of one call
+            w.seg0 = r0 / s.T;
+            w.more = r0 + nr < N;
+        }
         MONE_TRY(run_segments(m, w, nr, st));
         MONE_CUDA(cudaEventRecord(m->hfree[b], st));
     }

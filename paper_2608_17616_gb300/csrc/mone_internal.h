@@ -100,6 +100,10 @@ struct SegWork {
     // per-segment metrics of a whole call: segment i of chain c at [i * mstride + c], or null
     float *loss0, *step0;
     long long mstride;
+    // a call that learns in several parts: index of this part's first segment within the call (its row renormalisation
+    // carries on from the part before), and whether a part follows (which then applies the pending one)
+    long long seg0;
+    int more;
     int single;                  // the call runs on one stream: its kernels may chain by programmatic launch
     int first;                   // ... and this segment's first kernel is the call's first
     int y_scratch;               // targets are the residual scratch (rows from 0), not the caller's K, V

@@ -192,3 +192,27 @@ def test_host_context_at_the_bench_size_sampled_chains():
         assert rel_fro(Vg[ctx, layer].float(), Vo) <= BF16_TOL
     run.close()
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("memory,dtype,mode,tol", [("mlp", "bf16", wk.PAPER, 3e-4), ("swiglu", "bf16", wk.PAPER, 3e-4),
+                                                   ("mlp", "f32", wk.PAPER, 1e-6), ("mlp", "bf16", wk.PLAIN, 0.0)])
+def test_the_librarys_chunks_equal_one_device_call(memory, dtype, mode, tol):
+    """Three gathers of four segments: the same arithmetic as mone_ttl_context on the whole context, without
+    a rounding of the rescaled weights at a chunk's end.  Bounds: in paper mode float atomics add up the row sums of
+    squares in another order on every run, which moves a row's scale by some 2^-23 and now and then tips a bf16 operand over
+    (2^-8 of one product in thousands of a sum); rescaled weights rounded anew would show as 2e-3
+    or more of the momentum."""
+    if memory == "swiglu":
+        wl = swiglu(d=512, n_kv=4, T=2048, N=20000)
+    else:
+        T, N = (1024, 10000) if dtype == "f32" else (2048, 20000)
+        wl = wk.Workload("host_default", 46, 1, 2, 512, 512, 512, 4, 64, T, N, 8, dtype, mode, 0.1 if mode == wk.PAPER else 1e-2)
+    a, b = DeviceRun(wl), DeviceRun(wl)
+    mone.mone_mem_set_timing(a.h, 1)
+    mone.mone_ttl_context_host(a.h, pinned(a.X), pinned(a.K), pinned(a.V), a.N)
+    mone.mone_mem_sync(a.h)
+    assert mone.mone_mem_kernel_time(a.h, mone.KERNEL_KINDS.index("stage"))[1] == 3
+    b.ttl_context()
+    assert_same_state(a, b, tol)
+    a.close()
+    b.close()

@@ -158,3 +158,21 @@ def test_attention_maps_follow_the_calls_addresses_and_shape(fake):
     assert call(P, P + 256, P + 512, n_mem=65, pad=8) == 2
     assert call(P, P + 256, P + 512) == 2
     mone.mone_mem_free(h)
+
+
+@pytest.mark.parametrize("layers,mode,kw", [(2, mone.MONE_PAPER, {}), (1, mone.MONE_PAPER, {}), (2, mone.MONE_PLAIN, {}),
+                                            (2, mone.MONE_PAPER, dict(memory=mone.MONE_MEM_SWIGLU, mem_heads=2))])
+def test_a_host_context_in_the_librarys_chunks_renormalises_once(fake, layers, mode, kw):
+    """The learning kernels of one mone_ttl_context, and its one pass over the weights at the end."""
+    T, N = 128, 2 * (32 << 20) // (layers * 2048) + 3  # 2 KB a token and layer: chunks of 32 MB
+    h = init(layers, 512, 256, 512, T, mone.MONE_BF16, mode, **kw)
+    fake.drain()
+    mone.mone_ttl_context(h, P, P, P, N, 0)
+    one = [x["name"] for x in fake.drain()[0]]
+    mone.mone_ttl_context_host(h, P, P, P, N, 0, 0)
+    chunks = [x["name"] for x in fake.drain()[0]]
+    for part in ("phase", "swiglu_a", "swiglu_b", "finalize", "swiglu_rows"):
+        assert sum(part in n for n in chunks) == sum(part in n for n in one), part
+    assert sum("stage" in n for n in chunks) == 3
+    assert sum("finalize" in n or "swiglu_rows" in n for n in chunks) == (mode == mone.MONE_PAPER)
+    mone.mone_mem_free(h)
