@@ -94,7 +94,7 @@ struct TcArgs {
     int* status;
     int r_only;                 // phase A pairs: At and c SiLU'(x) / |z| come from the squared-error
                                 // pre-pass (the latter in dH); accumulate R only and form dH in place
-    int store_mode;             // phase B: when the state ring's slots are handed back (S_LAG3, ..)
+    int store_mode;             // phase B: when the state ring's slots are handed back (S_PAIRS1, ..)
     unsigned long long wait_ns; // limit of every mbarrier wait of the launch (kWaitLimitNs)
     int stall;                  // test knob (phase A): the producer issues no loads, so the first
                                 // wait for a full stage runs out; nothing is in flight when it does
@@ -939,8 +939,9 @@ tc_phase_a_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_co
 
 constexpr int S_ROWS = 32, S_COLS = 64;                    // state chunk: hidden rows x weight columns
 constexpr int S_SLOTS = 8;
-// when slots are handed back: one, three stores later; two at a time, three or one later
-enum { S_LAG3 = 0, S_PAIRS3 = 1, S_PAIRS1 = 2 };
+// when the store warp hands slots back to the loads: by twos one store later, one by one three stores later, by twos
+// three stores later, by fours two stores later (each leaves fewer loads in flight than the one before)
+enum { S_PAIRS1, S_LAG3, S_PAIRS3, S_QUADS2 };
 constexpr int S_F32 = S_ROWS * S_COLS * 4;                 // 8 KB
 constexpr int S_SLOT = 2 * S_F32;                          // W and mu: 16 KB
 constexpr int B_THREADS = 12 * 32;
@@ -1206,23 +1207,25 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
                     tma_store_5d(x.m ? &tmW2s : &tmW1s, smem_u32(base + L::STATE + k * S_SLOT), 0,
                                  x.h0 + chunk_row(i), (x.col + chunk_col(i)) / 32, a.c0 + x.cz, 0);
                     bulk_commit();
-                    // hand slots back whose stores have read them: the ring's slots are split between stores
-                    // and loads in flight
+                    // hand slots back whose stores have read them: `done` is the last such chunk, `n` of them at once
+                    auto hand_back = [&](uint32_t done, int n) {
+                        for (int u = n - 1; u >= 0; --u) mbar_arrive(sempty((done - u) % S_SLOTS));
+                    };
                     if (a.store_mode == S_LAG3) {
                         bulk_wait_read<3>();
-                        if (seq >= 3) mbar_arrive(sempty((seq - 3) % S_SLOTS));
-                    } else if (!(seq & 1) && seq) {  // two slots at a time
-                        uint32_t done;  // stores up to this one have been read
+                        if (seq >= 3) hand_back(seq - 3, 1);
+                    } else if (a.store_mode == S_QUADS2) {
+                        if ((seq & 3) == 1 && seq > 1) {
+                            bulk_wait_read<2>();
+                            hand_back(seq - 2, 4);
+                        }
+                    } else if (!(seq & 1) && seq) {
                         if (a.store_mode == S_PAIRS3) {
                             bulk_wait_read<3>();
-                            done = seq - 3;
+                            if (seq > 3) hand_back(seq - 3, 2);
                         } else {
                             bulk_wait_read<1>();
-                            done = seq - 1;
-                        }
-                        if ((int)done > 0) {
-                            mbar_arrive(sempty((done - 1) % S_SLOTS));
-                            mbar_arrive(sempty(done % S_SLOTS));
+                            hand_back(seq - 1, 2);
                         }
                     }
                 }
@@ -2197,17 +2200,18 @@ cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputM
     // third off it.  At T = 512 the pair's coupled loads and accumulator release cost more than they save.
     constexpr int PAIR_MIN_T = 1024;
     const bool pairs = s.T >= PAIR_MIN_T && s.d_in % B_BN == 0 && dev.pairb_clusters > 0;
-    // When the state ring's slots are handed back, by what was fastest: how stores and loads alternate
-    // decides how much of HBM the stream gets.  With no momentum, on CTA pairs, for one chain, or with W and mu of
-    // the whole handle in L2, two at a time, one store later (ms, against one by one three stores later: 64 plain chains of
-    // 2048 -> 1024 -> 1024, T = 256: 7.68 and 8.13; 28 chains, T = 1024, 4K tokens: 7.91 and 7.99; 4 chains 1.33 and
-    // 1.36).  With a large state from T = 256 on two at a time, three stores later (56 chains, T = 512: 9.81 and
-    // 10.41; 30 chains 3.86 and 3.98), else one by one (16 chains, T = 512: 5.22 and 5.39; 28 chains, T = 128: 9.74
-    // and 10.1).
-    const long long state = (long long)s.C * s.d_hid * (s.d_in + s.d_out) * 8;
-    a.store_mode = pairs || !s.momentum || w.single || state < 128000000 ? S_PAIRS1
-                   : s.T >= 256 && state > (s.T >= 512 ? 740000000 : 800000000) ? S_PAIRS3
-                                                                               : S_LAG3;
+    // When the state ring's slots are handed back, that is how many of its loads are in flight. A launch of few tiles a CTA
+    // is mostly ramp, and without momentum a slot carries half the bytes: hand back at once. The longer a launch runs
+    // (tiles a CTA) and the more operands stream beside the state (T), the fewer state loads in flight serve it best: they
+    // queue before the operands' and the stores. Measured over 70 contexts of 8 to 224 chains, the steps where the
+    // faster of two neighbours changes; whole contexts, ms, with S_PAIRS1, S_LAG3, S_PAIRS3, S_QUADS2: 8 chains of 2048 -> 1024 ->
+    // 1024, T = 128 (T * tiles 323): 1.75 1.79 1.86 1.92; 28 of 2432 -> 1280 -> 768, T = 128 (1533): 6.99 6.77 7.02 7.35; 64 of
+    // 2048 -> 1024 -> 1024, T = 512 (10,348): 5.15 5.16 4.78 4.93; 20 of 3072 -> 2048 -> 2048, T = 768 (16,168): 4.56 4.54 4.54 4.42.
+    const auto store_mode = [&](int tiles, int ctas) {
+        const double per_cta = (double)tiles / ctas, run = per_cta * s.T;
+        if (!s.momentum || per_cta <= 4) return S_PAIRS1;
+        return run < 4400 ? S_LAG3 : run < 16000 ? S_PAIRS3 : S_QUADS2;
+    };
     const CUtensorMap& U = s.mode == 1 ? m.Ub : in.Xb;
     const CUtensorMap& U2 = s.mode == 1 ? m.Ub2 : in.Xb2;
     const int col_tiles = b_col_tiles(s.d_in, s.d_out);
@@ -2215,6 +2219,8 @@ cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputM
         const int npairs = w.nc * col_tiles * (s.d_hid / (2 * B_BM));
         const int maxc = dev.pairb_clusters - (s.reserve_sms + 1) / 2;
         const int clusters = npairs < maxc ? npairs : maxc;
+        // on pairs the operand streams are smaller; by twos one store later was within 1% of the best nearly everywhere
+        a.store_mode = S_PAIRS1;
         return launch_kernel(a.step_sq ? tc_phase_b_kernel<true, true> : tc_phase_b_kernel<true, false>, dim3(2 * clusters),
                              dim3(B_THREADS), LayoutB2::DYN, st, w.single != 0, 2, U2, in.Kb, in.Vb, m.dH, m.At, m.W1s,
                              m.W2s, a);
@@ -2222,6 +2228,7 @@ cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputM
     const int ntiles = w.nc * col_tiles * (s.d_hid / B_BM);
     const int sms = dev.sms - s.reserve_sms;
     const int grid = ntiles < sms ? ntiles : sms;
+    a.store_mode = store_mode(ntiles, grid);
     return launch_kernel(a.step_sq ? tc_phase_b_kernel<false, true> : tc_phase_b_kernel<false, false>, dim3(grid),
                          dim3(B_THREADS), LayoutB::DYN, st, w.single != 0, 1, U, in.Kb, in.Vb, m.dH, m.At, m.W1s, m.W2s, a);
 }

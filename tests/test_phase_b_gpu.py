@@ -26,8 +26,11 @@ def _built():
     (128, 256, 256, 128, 2, 300, wk.PAPER),      # a narrow tile of W1, one of W2 from K and V
     (384, 256, 768, 128, 30, 300, wk.PAPER),     # 256 + 128 columns in W1; 150 tiles a launch, two launches
     (384, 256, 768, 512, 30, 700, wk.PAPER),     # the same in longer segments
-    (384, 768, 768, 256, 20, 600, wk.PAPER),     # a state above 128 MB: slots one by one; several tiles a CTA
-    (1152, 2048, 1280, 256, 22, 513, wk.PAPER),  # a state above 800 MB: slots two at a time, three stores later
+    (384, 768, 768, 256, 20, 600, wk.PAPER),     # two tiles a CTA: slots by twos, one store later
+    (1152, 2048, 1280, 256, 22, 513, wk.PAPER),  # 11.6 tiles a CTA: slots one by one, three stores later
+    (512, 512, 512, 128, 80, 300, wk.PAPER),     # 4.2 tiles a CTA: the same
+    (512, 512, 512, 512, 168, 513, wk.PAPER),    # 8.8 tiles a CTA at T = 512: slots by twos, three stores later
+    (384, 256, 256, 4096, 204, 4096 + 5, wk.PAPER),  # 4.03 tiles a CTA at T = 4096: slots by fours, two stores later
     (640, 256, 256, 256, 3, 513, wk.PLAIN),      # W alone in the ring; a last segment of one token
     (512, 256, 512, 1024, 3, 1024 + 65, wk.PAPER),  # CTA pairs
     (512, 256, 768, 1024, 3, 1024 + 65, wk.PAPER),  # CTA pairs, a tile from K and V
