@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(256) mse_out_f32_kernel(const F32SegArgs a, fl
 // 512 threads.  Forward: a warp takes two tokens of a chunk, lane l the columns 4 l + 128 i of [U | Y], with
 // the W values of these columns in registers (RB = 4; from shared memory for RB = 8) and even and odd columns
 // as packed pairs; the partial sums of H and R over the lanes are added by a transpose-reduction (16 shuffles
-// for 16 sums), and the same warp finishes the epilogue.  Backward: a thread takes two columns of [W1 | W2]
+// for 16 sums), and the same warp finishes the epilogue.  Narrow chains with RB = 8 give each token 16 lanes instead.  Backward: a thread takes two columns of [W1 | W2]
 // for all RB rows and one half of the chunk's tokens.  So a staged value is read from shared memory once in
 // each direction.  The two phases of a chunk, each a chain of shared-memory and shuffle latencies between
 // barriers with four warps a scheduler, bound it (49% of the issue slots used, 44% of the shared-memory rate).
@@ -576,9 +576,12 @@ __device__ __forceinline__ float block_sum_res(float v, float* red) {
     return t;
 }
 
-template <int RB>
+// LPT: lanes to a token of the forward, 32 (two tokens a lane) or 16 (one); widths up to DMAX.
+template <int RB, int LPT, int DMAX>
 __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResArgs a) {
-    constexpr int RC = RES_RC, NW = RES_NW, NV = 4 * RB;  // NV: sums of a warp's two tokens (H and R)
+    // tokens of a lane, sums of a lane (H and R), 16-byte column pieces of a lane
+    constexpr int RC = RES_RC, NW = RES_NW, TPL = LPT / 16, NV = 2 * TPL * RB, NI = DMAX / (4 * LPT);
+    static_assert(LPT == 32 || (LPT == 16 && RB == 8), "lanes to a token");
     static_assert(RB == 4 || RB == 8, "rows per CTA");
     static_assert(RC == 2 * NW, "two tokens a warp");
     extern __shared__ float4 res_smem[];
@@ -667,23 +670,23 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
 #pragma unroll
     for (int r = 0; r < RB; ++r) acc[r] = 0;
     __syncthreads();
-    // forward: the lane's weights, columns 4 lane + 128 i
-    constexpr int NI = 4;  // D <= 512
+    // forward: LPT lanes to a token, a lane's columns 4 (lane % LPT) + 4 LPT i
     int fo[NI];
+    const int fl = 4 * (lane % LPT);
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
         int stride;
-        fo[i] = x_col(4 * lane + 128 * i, stride);
-        fo[i] += 2 * warp * stride;
+        fo[i] = x_col(fl + 4 * LPT * i, stride);
+        fo[i] += (2 * warp + lane / LPT) * stride;
     }
     ulonglong2 w[RB == 4 ? NI : 1][RB == 4 ? RB : 1];  // two packed pairs each
     auto load_w = [&]() {
         if constexpr (RB == 4) {
 #pragma unroll
             for (int i = 0; i < NI; ++i)
-                if (4 * lane + 128 * i < D)
+                if (fl + 4 * LPT * i < D)
 #pragma unroll
-                    for (int r = 0; r < RB; ++r) w[i][r] = *reinterpret_cast<const ulonglong2*>(Ws + r * LD + 4 * lane + 128 * i);
+                    for (int r = 0; r < RB; ++r) w[i][r] = *reinterpret_cast<const ulonglong2*>(Ws + r * LD + fl + 4 * LPT * i);
         }
     };
     load_w();
@@ -706,16 +709,17 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
                 issue(seg + 1, 0, buf ^ 1);
             cp_async_commit();
             const float* Xb = Xs + buf * RC * D;
-            {   // ---- forward of tokens 2 warp, 2 warp + 1: v[(matrix 2 + token) RB + row]
+            {   // ---- forward of tokens 2 warp, 2 warp + 1: v[(matrix TPL + token) RB + row]
                 uint64_t p[NV] = {};  // even and odd columns packed
 #pragma unroll
                 for (int i = 0; i < NI; ++i) {
-                    const int c = 4 * lane + 128 * i;
+                    const int c = fl + 4 * LPT * i;
                     if (c >= D) continue;
                     const ulonglong2 xa = *reinterpret_cast<const ulonglong2*>(Xb + fo[i]);
-                    const ulonglong2 xb = *reinterpret_cast<const ulonglong2*>(Xb + fo[i] + (c < a.d_in ? a.d_in : dh));
+                    ulonglong2 xb;
+                    if constexpr (TPL == 2) xb = *reinterpret_cast<const ulonglong2*>(Xb + fo[i] + (c < a.d_in ? a.d_in : dh));
                     auto add = [&](auto mat) {
-                        constexpr int o = decltype(mat)::value * 2 * RB;
+                        constexpr int o = decltype(mat)::value * TPL * RB;
 #pragma unroll
                         for (int r = 0; r < RB; ++r) {
                             ulonglong2 wr;
@@ -724,7 +728,7 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
                             else
                                 wr = *reinterpret_cast<const ulonglong2*>(Ws + r * LD + c);
                             p[o + r] = fma_f32x2(xa.y, wr.y, fma_f32x2(xa.x, wr.x, p[o + r]));
-                            p[o + RB + r] = fma_f32x2(xb.y, wr.y, fma_f32x2(xb.x, wr.x, p[o + RB + r]));
+                            if constexpr (TPL == 2) p[o + RB + r] = fma_f32x2(xb.y, wr.y, fma_f32x2(xb.x, wr.x, p[o + RB + r]));
                         }
                     };
                     if (c < a.d_in)
@@ -738,9 +742,9 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
                     const float2 f = unpack_f32x2(p[u]);
                     v[u] = f.x + f.y;
                 }
-                // add the lanes' sums: afterwards the lanes whose top bits spell j hold sum j
+                // add the token's lanes' sums: afterwards the lanes whose top bits (of LPT) spell j hold sum j
 #pragma unroll
-                for (int n = NV, sft = 16; n > 1; n >>= 1, sft >>= 1) {
+                for (int n = NV, sft = LPT / 2; n > 1; n >>= 1, sft >>= 1) {
                     const bool upper = (lane & sft) != 0;
 #pragma unroll
                     for (int u = 0; u < n / 2; ++u) {
@@ -748,13 +752,13 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
                         v[u] = keep + __shfl_xor_sync(0xffffffffu, send, sft);
                     }
                 }
-                if (NV == 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+                if (NV < LPT) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
                 // epilogue of output (token, row): c_t = -eta_t / T' (Eq. 10), A = SiLU(H); H is in the
-                // lower lanes, R sixteen above
-                const float rv = __shfl_down_sync(0xffffffffu, v[0], 16);
-                constexpr int LPV = 32 / NV;  // lanes holding a sum
-                const int j = lane / LPV, t = 2 * warp + j / RB, r = j % RB, ts = ch * RC + t;
-                if (lane < 16 && lane % LPV == 0) {
+                // lower half of the token's lanes, R LPT / 2 above
+                const float rv = __shfl_down_sync(0xffffffffu, v[0], LPT / 2);
+                constexpr int LPV = LPT / NV;  // lanes holding a sum
+                const int j = lane % LPT / LPV, t = 2 * warp + j / RB + lane / LPT, r = j % RB, ts = ch * RC + t;
+                if (lane % LPT < LPT / 2 && lane % LPV == 0) {
                     const float hv = v[0];
                     const float ct = ts < Tp ? -etaS[buf * RC + t] / (float)Tp : 0.f;
                     const float sg = sigmoidf_(hv);
@@ -861,7 +865,7 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
                 *reinterpret_cast<float2*>(Ws + r * LD + cb) = wv;
             }
         }
-        __syncthreads();
+        if (RB == 4 || seg + 1 == a.n_seg) __syncthreads();  // eight rows: the next chunk's barrier, before W is read
         load_w();
     }
     cp_async_wait<0>();
@@ -1169,18 +1173,22 @@ cudaError_t launch_resident_f32(const DevState& s, const SegWork& w, long long n
     a.step_sq = w.step0;
     a.m_sstride = w.loss0 || w.step0 ? w.mstride : 0;
     a.status = s.status;
-    cudaError_t e = cudaSuccess;
     // four rows a CTA while that still fits the chains in one wave, else eight (less re-streaming)
     const int D = s.d_in + s.d_out;
-    static PerDevice<SmemOptIn> once4, once8;
-    if (e == cudaSuccess) e = smem_opt_in(reinterpret_cast<const void*>(ttl_resident_f32_kernel<4>), res_smem_bytes<4>(512), once4);
-    if (e == cudaSuccess) e = smem_opt_in(reinterpret_cast<const void*>(ttl_resident_f32_kernel<8>), res_smem_bytes<8>(512), once8);
-    if (e != cudaSuccess) return e;
+    auto launch = [&](auto kernel, int rows, size_t most, size_t smem, PerDevice<SmemOptIn>& once) {
+        const cudaError_t e = smem_opt_in(reinterpret_cast<const void*>(kernel), most, once);
+        if (e != cudaSuccess) return e;
+        kernel<<<dim3(s.d_hid / rows, w.nc), RES_NT, smem, st>>>(a);
+        return cudaGetLastError();
+    };
+    static PerDevice<SmemOptIn> once[3];
     if ((long long)w.nc * (s.d_hid / 4) <= s.sms)
-        ttl_resident_f32_kernel<4><<<dim3(s.d_hid / 4, w.nc), RES_NT, res_smem_bytes<4>(D), st>>>(a);
-    else
-        ttl_resident_f32_kernel<8><<<dim3(s.d_hid / 8, w.nc), RES_NT, res_smem_bytes<8>(D), st>>>(a);
-    return cudaGetLastError();
+        return launch(ttl_resident_f32_kernel<4, 32, 512>, 4, res_smem_bytes<4>(512), res_smem_bytes<4>(D), once[0]);
+    // Eight rows: the 32 sums of two tokens cost a lane 31 shuffles and their selects, more than the contraction of a narrow
+    // chain; 16 lanes to a token halve them and read W twice. 1500 tokens, 32 and 16 lanes: D = 192 (8 chains of 64 -> 320 ->
+    // 128) 444 and 397 us, 320 (4 of 192 -> 448 -> 128) 408 and 394, 384 (256 -> 768 -> 128) 234 and 252, 512 814 and 925
+    if (D <= 320) return launch(ttl_resident_f32_kernel<8, 16, 320>, 8, res_smem_bytes<8>(320), res_smem_bytes<8>(D), once[1]);
+    return launch(ttl_resident_f32_kernel<8, 32, 512>, 8, res_smem_bytes<8>(512), res_smem_bytes<8>(D), once[2]);
 }
 
 cudaError_t launch_mse_f32(const DevState& s, const SegWork& w, cudaStream_t st) {

@@ -32,6 +32,10 @@ def _built():
     (192, 128, 256, 128, 3, 2 * 128 + 33, wk.PAPER, "neg_inner"),  # resident: W1 ends inside a warp's columns
     (384, 704, 128, 64, 1, 2 * 64 + 32, wk.PLAIN, "neg_inner"),    # resident, eight rows a CTA
     (320, 256, 128, 64, 3, 3 * 64 + 1, wk.PAPER, "neg_inner"),     # resident, eight rows a CTA, W1 ends inside
+    (64, 704, 128, 64, 1, 3 * 64 + 1, wk.PAPER, "neg_inner"),      # eight rows, 16 lanes to a token: three pieces a lane
+    (128, 256, 128, 128, 3, 2 * 128 + 33, wk.PLAIN, "neg_inner"),  # four
+    (192, 256, 128, 192, 3, 2 * 192 + 17, wk.PAPER, "neg_inner"),  # five, the most
+    (64, 256, 384, 64, 3, 3 * 64 + 33, wk.PAPER, "neg_inner"),     # eight rows, 32 lanes again (448 columns)
 ])
 def test_f32_tiles(d_in, d_hid, d_out, T, n_layers, N, mode, loss):
     wl = wk.Workload("f32_tiles", 13, 1, n_layers, d_in, d_hid, d_out, d_out // 128, 64, T, N, 8, "f32", mode,
