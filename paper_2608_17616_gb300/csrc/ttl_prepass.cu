@@ -265,9 +265,10 @@ __global__ void __launch_bounds__(256) prepass_kernel(const PrepassArgs a) {
 
 template <typename Tin, typename Tout>
 cudaError_t launch_one(const PrepassArgs& a, int nchains, int sms, cudaStream_t st) {
-    // two rows a warp share the meta-parameter loads; few rows (less than two CTAs an SM that way) are spread
-    // one a warp instead (512 rows of one chain, d_in = 2048, caches cold: 11.1 -> 9.2 us)
-    if ((long long)((a.rows + 15) / 16) * nchains >= 2 * sms)
+    // Two rows a warp share the meta-parameter loads; one row a warp spreads few rows over more SMs, as long as that is one
+    // wave (three CTAs an SM). Caches cold, d = 2048, one and two rows a warp: 512 rows 11.8 and 13.9 us, 3072 rows (384 CTAs
+    // of one row a warp) 15.9 and 15.9, 4096 rows (512) 22.0 and 16.4
+    if ((long long)((a.rows + 7) / 8) * nchains > 3 * sms)
         prepass_kernel<Tin, Tout, 2><<<dim3((a.rows + 15) / 16, nchains), 256, 0, st>>>(a);
     else
         prepass_kernel<Tin, Tout, 1><<<dim3((a.rows + 7) / 8, nchains), 256, 0, st>>>(a);

@@ -100,14 +100,14 @@ def test_tile_rules_follow_the_devices_sm_count(fake):
         mone.mone_ttl_context(h, P, P, P, 64, 0)
         want[dev]["phase_b"] = [x["grid"] for x in fake.drain()[0] if "phase_b_f32" in x["name"]]
         h = init(1, 512, 512, 512, 128, mone.MONE_BF16, mone.MONE_PAPER)
-        mone.mone_ttl_context(h, P, P, P, 4000, 0)          # 256 CTAs of 16 rows in the input transform
+        mone.mone_ttl_context(h, P, P, P, 3000, 0)          # 384 CTAs of 8 rows in the input transform
         want[dev]["transform"] = [x["grid"] for x in fake.drain()[0] if "prepass" in x["name"]]
         h = init(16, 512, 512, 512, 128, mone.MONE_BF16)    # decode over 64 heads in all
         mone.mone_attention(h, P, 4, 1, P, P, mone.kv_strides(16, 4, 2048, 64), 2047, P, 0)
         want[dev]["decode"] = [x["cluster"] for x in fake.drain()[0] if "decode" in x["name"]]
     assert want[0]["phase_a"] == [(8, 16, 3)] and want[1]["phase_a"] == [(4, 16, 3)]
     assert want[0]["phase_b"] == [(24, 16, 1)] and want[1]["phase_b"] == [(12, 8, 1)]
-    assert want[0]["transform"] == [(512, 1, 1)] and want[1]["transform"] == [(256, 1, 1)]
+    assert want[0]["transform"] == [(384, 1, 1)] and want[1]["transform"] == [(192, 1, 1)]
     assert want[0]["decode"] == [8] and want[1]["decode"] == [6]
 
 
