@@ -428,6 +428,7 @@ attention_prefill_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                 // S of chunk j + 2 goes over the P that P V has to have read
                 if (j + 2 < n) ok = mbar_wait(odone(j), (j >> 1) & 1, a.status) && issue_s(j + 2);
             }
+            if (!ok) drain_copies();
         }
         __syncwarp();
     } else {

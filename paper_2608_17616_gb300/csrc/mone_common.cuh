@@ -137,6 +137,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* st
     }
 }
 
+// After a wait that ran out: some time for the copies that this CTA still has in flight to land, before it leaves and its
+// shared memory becomes another's.
+__device__ __forceinline__ void drain_copies() {
+    const uint64_t t0 = globaltimer_ns();
+    while (globaltimer_ns() - t0 < 200000) __nanosleep(1000);
+}
+
 // ------------------------------------------------------------------ cp.async (16-byte copies on the LSU path)
 // Copy 16 bytes global -> shared (`dst` in the shared window); src_bytes 0 writes 16 zero
 // bytes and reads nothing (src must still be a valid global address).

@@ -702,7 +702,10 @@ __global__ void __launch_bounds__(RES_NT, 1) ttl_resident_f32_kernel(const ResAr
         for (int ch = 0; ch < nch; ++ch) {
             cp_async_wait<0>();
             const bool landed = mbar_wait(full + 8 * buf, phase, a.status);
-            if (!__syncthreads_and(landed)) return;  // the chunk has landed; everyone is done with the other buffer and Gs
+            if (!__syncthreads_and(landed)) {  // the chunk has landed; everyone is done with the other buffer and Gs
+                drain_copies();
+                return;
+            }
             if (ch + 1 < nch)
                 issue(seg, ch + 1, buf ^ 1);
             else if (seg + 1 < a.n_seg)

@@ -545,12 +545,6 @@ struct LP {
 static_assert(LP::DYN <= 227 * 1024, "shared memory budget");
 static_assert(LP::STG % 16 == 0, "staging buffers hold 16-byte pieces");
 
-// Spin for about `ns` nanoseconds (abort path: lets copies already issued land first).
-__device__ __forceinline__ void pause_ns(uint64_t ns) {
-    const uint64_t t0 = globaltimer_ns();
-    while (globaltimer_ns() - t0 < ns) __nanosleep(1000);
-}
-
 __global__ void __launch_bounds__(THREADS, 1)
 tc_phase_a_pair_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmK,
                        const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmW1,
@@ -624,7 +618,7 @@ tc_phase_a_pair_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_con
                     }
                 }
             }
-            if (!ok) pause_ns(200000);
+            if (!ok) drain_copies();
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -661,7 +655,7 @@ tc_phase_a_pair_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_con
                 if (!ok) break;
                 umma_commit_pair(c.tfull(0, P_STAGES), 0x3);
             }
-            if (!ok) pause_ns(200000);
+            if (!ok) drain_copies();
         }
         __syncwarp();
     } else {
@@ -752,7 +746,10 @@ tc_phase_a_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_co
             const uint64_t wpol = l2_evict_last_policy();  // the bf16 W copy phase B wrote
             for (int i = 0; i < n && !a.stall; ++i) {
                 const int s = i % A_STAGES;
-                if (i >= A_STAGES && !mbar_wait(c.empty(s, A_STAGES), ((i / A_STAGES) - 1) & 1, a.status, a.wait_ns)) break;
+                if (i >= A_STAGES && !mbar_wait(c.empty(s, A_STAGES), ((i / A_STAGES) - 1) & 1, a.status, a.wait_ns)) {
+                    drain_copies();
+                    break;
+                }
                 const uint32_t sa = smem_u32(c.base + s * A_STAGE), sb = sa + A_BM * BK * 2, fb = c.full(s);
                 mbar_expect_tx(fb, A_STAGE);
                 if (i < n1) {
@@ -787,7 +784,10 @@ tc_phase_a_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_co
                               ((i == 0 || i == n1) && k == 0) ? 0u : 1u);
                 umma_commit(c.empty(s, A_STAGES));
             }
-            if (ok) umma_commit(c.tfull(0, A_STAGES));
+            if (ok)
+                umma_commit(c.tfull(0, A_STAGES));
+            else
+                drain_copies();
         }
         __syncwarp();
     } else {
@@ -1118,7 +1118,7 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
                     }
                 }
             }
-            if (PAIR && !ok) pause_ns(200000);
+            if (PAIR && !ok) drain_copies();
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -1159,7 +1159,7 @@ tc_phase_b_kernel(const __grid_constant__ CUtensorMap tmUb, const __grid_constan
                 else
                     umma_commit(tfull(b));
             }
-            if (PAIR && !ok) pause_ns(200000);
+            if (PAIR && !ok) drain_copies();
         }
         __syncwarp();
     } else if (warp == B_STATE_WARP) {
@@ -1765,7 +1765,7 @@ tc_read_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     }
                 }
             }
-            if (!ok) pause_ns(200000);
+            if (!ok) drain_copies();
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -1799,7 +1799,7 @@ tc_read_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (!ok) break;
                 umma_commit_pair(c.tfull(b, RP_STAGES), 0x3);
             }
-            if (!ok) pause_ns(200000);
+            if (!ok) drain_copies();
         }
         __syncwarp();
     } else {

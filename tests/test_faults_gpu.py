@@ -123,3 +123,30 @@ def test_bounded_wait_runs_out_and_the_handle_recovers(T):
         st, _ = oracle_chain(run, c)
         assert rel_fro(W1[c], st.W["W1"]) <= 2e-2 and rel_fro(W2[c], st.W["W2"]) <= 2e-2, c
     run.close()
+
+
+@pytest.mark.parametrize("d_in", [256, 128])  # phase A of one chain over clusters of four CTAs a tile, and of two
+def test_bounded_wait_runs_out_in_a_cluster_and_the_handle_recovers(d_in):
+    # The same knob with one chain: the launch's CTAs exchange their partial sums through the cluster. Those whose waits ran
+    # out say so, none of the cluster's CTAs writes dH, At or a loss, and phase B, chained by programmatic launch, still ends.
+    T = 256
+    wl = wk.Workload(f"fault_stall_split_{d_in}", 47, 1, 1, d_in, 256, 256, 2, 64, T, 2 * T, 16, "bf16", wk.PAPER, 0.1)
+    os.environ["MONE_FAULT_STALL"] = "1"
+    try:
+        run = DeviceRun(wl)
+    finally:
+        del os.environ["MONE_FAULT_STALL"]
+    loss = torch.full((1,), 7.0, device="cuda")
+    t0 = time.time()
+    mone.mone_ttl_segment(run.h, 0, 0, run.X[0, 0, :T], run.K[0, 0, :T], run.V[0, 0, :T], T, loss_out=loss)
+    assert code_of(mone.mone_mem_sync, run.h) == 5  # MONE_ERR_TIMEOUT
+    assert time.time() - t0 < 1.5                  # the launch's 1 ms limit, not the default 2 s
+    assert loss.item() == 0.0                      # zeroed by the input transform, nothing added
+    mone.mone_mem_sync(run.h)                      # the latch is cleared once reported
+    zero = torch.zeros_like(run.W1_0), torch.zeros_like(run.W2_0)
+    mone.mone_mem_write_state(run.h, run.W1_0, run.W2_0, *zero)
+    run.ttl_context()
+    W1, W2, _, _ = run.state()
+    st, _ = oracle_chain(run, 0)
+    assert rel_fro(W1[0], st.W["W1"]) <= 2e-2 and rel_fro(W2[0], st.W["W2"]) <= 2e-2
+    run.close()
