@@ -140,7 +140,6 @@ cudaError_t launch_col_targets(const DevState& s, cudaStream_t st);
 cudaError_t launch_gate_silu(float* gate, size_t n, int from_one, cudaStream_t st);
 cudaError_t launch_read(const DevState& s, int Q, int n_layers, void* K_out, void* V_out,
                         const long long* strides, cudaStream_t st);
-cudaError_t launch_zero_f32(float* p, size_t n, cudaStream_t st);
 
 // Allocation-free read (mone_mem_generate_kv_noalloc): fixed device scratch of
 // kNoAllocScratchFloats floats, shared by every call on a device.
@@ -211,7 +210,6 @@ cudaError_t launch_phase_a_tc(const DevState& s, const TcMaps& m, const TcInputM
                               cudaStream_t st);
 cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                               cudaStream_t st);
-int tc_kernels_per_segment();
 // The whole memory read on the tensor cores (bf16 path), query side included: Xq bf16
 // [C][Q][d_in]; Uq, Aq bf16 scratch [C][Q][d_in], [C][Q][d_hid]; zq fp32 scratch [C][Q]; writes
 // K/V (bf16) with the caller's strides.

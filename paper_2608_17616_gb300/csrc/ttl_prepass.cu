@@ -389,14 +389,14 @@ cudaError_t launch_query_z(const DevState& s, const void* Xq, int Q, void* Z, fl
                                                  static_cast<bf16*>(Z), zinv, groups);
         return cudaGetLastError();
     };
-    // Two rows a warp once that leaves enough warps to fill the GPU.  Whole reads, one and two rows a warp: 4112
+    // Two rows a warp once that leaves enough warps to fill the GPU (30 rows an SM).  Whole reads, one and two rows a warp: 4112
     // rows of 2048 70.7 and 70.9 us, 5200 rows 72.7 and 71.6, 16,000 rows 134 and 127, 28,000 rows of 3072 457
     // and 438, 128,000 rows of 256 207 and 162; 1000 rows of 2048 36.9 and 39.0.
-    if (Q > 1 && (long long)s.C * Q > 4608) return run(query_z_kernel<2, 1>, 2);
+    if (Q > 1 && (long long)s.C * Q > 30 * s.sms) return run(query_z_kernel<2, 1>, 2);
     return run(query_z_kernel<1, 4>, 1);
 }
 
-// Query side of the read, normalised (the SwiGLU read, the fp32 read and the 128-query form):
+// Query side of the read, normalised (the SwiGLU read and the fp32 read):
 // one warp per (chain, query token), d_in <= 2048.  A lane keeps its z values in registers, so
 // the row is read once: z = SiLU(alpha x + gamma), then u = z / sqrt(|z|^2 + 1e-12) (paper mode),
 // u = x in plain mode.  The loads of a 4-vector group are issued before any arithmetic.

@@ -1312,8 +1312,4 @@ cudaError_t launch_read_noalloc(const DevState& s, const TcMaps* tc, const void*
     return e != cudaSuccess ? e : launch_read(t, Q, n_layers, K_out, V_out, strides, st);
 }
 
-cudaError_t launch_zero_f32(float* p, size_t n, cudaStream_t st) {
-    return cudaMemsetAsync(p, 0, n * sizeof(float), st);
-}
-
 }  // namespace mone

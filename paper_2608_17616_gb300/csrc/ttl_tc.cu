@@ -68,7 +68,7 @@ struct Layout {
     static constexpr int END = TAB + TABLE * 4;
     static constexpr int DYN = END + 1024;                // + alignment slack
 };
-// phase A table: [2 parity][2 matrix][A_BN] scales; phase B: [2][B_BN] scales + [2][8] beta partials
+// table: [2 parity][2 matrix][A_BN] scales
 using LA = Layout<A_STAGES, A_STAGE, 4 * A_BN>;
 static_assert(LA::DYN <= 227 * 1024, "shared memory budget");
 
@@ -84,7 +84,6 @@ struct TcArgs {
     const float* dbeta;         // [C][T]
     const float* zinv;          // [C][T] 1/|z_t| (paper mode), or null
     const float* b_beta;        // [C]
-    float *W1, *W2, *mu1, *mu2;
     bf16 *W1b, *W2b;
     const float *n1, *n2;
     float* sumsq;               // [2 parity][2 matrix][C][d_hid]
@@ -1364,7 +1363,7 @@ TcArgs make_args(const DevState& s, const SegWork& w) {
     a.eta_cstride = w.eta_cstride;
     a.eta = s.eta; a.dbeta = s.dbeta; a.b_beta = s.b_beta;
     a.zinv = a.paper ? s.zinv : nullptr;
-    a.W1 = s.W1; a.W2 = s.W2; a.mu1 = s.mu1; a.mu2 = s.mu2; a.W1b = s.W1b; a.W2b = s.W2b;
+    a.W1b = s.W1b; a.W2b = s.W2b;
     a.n1 = s.n1; a.n2 = s.n2; a.sumsq = s.sumsq;
     a.dH = reinterpret_cast<bf16*>(s.dHt); a.At = reinterpret_cast<bf16*>(s.Att);
     a.loss = w.loss; a.step_sq = w.step_sq; a.status = s.status;
@@ -2232,8 +2231,6 @@ cudaError_t launch_phase_b_tc(const DevState& s, const TcMaps& m, const TcInputM
     return launch_kernel(a.step_sq ? tc_phase_b_kernel<false, true> : tc_phase_b_kernel<false, false>, dim3(grid),
                          dim3(B_THREADS), LayoutB::DYN, st, w.single != 0, 1, U, in.Kb, in.Vb, m.dH, m.At, m.W1s, m.W2s, a);
 }
-
-int tc_kernels_per_segment() { return 2; }
 
 cudaError_t launch_mse_tc(const DevState& s, const TcMaps& m, const TcInputMaps& in, const SegWork& w,
                           cudaStream_t st) {
