@@ -266,9 +266,11 @@ __global__ void __launch_bounds__(256) prepass_kernel(const PrepassArgs a) {
 template <typename Tin, typename Tout>
 cudaError_t launch_one(const PrepassArgs& a, int nchains, int sms, cudaStream_t st) {
     // Two rows a warp share the meta-parameter loads; one row a warp spreads few rows over more SMs, as long as that is one
-    // wave (three CTAs an SM). Caches cold, d = 2048, one and two rows a warp: 512 rows 11.8 and 13.9 us, 3072 rows (384 CTAs
-    // of one row a warp) 15.9 and 15.9, 4096 rows (512) 22.0 and 16.4
-    if ((long long)((a.rows + 7) / 8) * nchains > 3 * sms)
+    // wave (three CTAs an SM, in fp32 four: registers). Caches cold, bf16, d = 2048, one and two rows a warp: 512 rows 11.8 and
+    // 13.9 us, 3072 rows (384 CTAs of one row a warp) 15.9 and 15.9, 4096 rows (512) 22.0 and 16.4; 960 rows of 4 fp32 chains,
+    // d = 704 (480 CTAs): a context of 3 segments 401 and 407 us
+    constexpr int CTAS = sizeof(Tin) == 4 ? 4 : 3;
+    if ((long long)((a.rows + 7) / 8) * nchains > CTAS * sms)
         prepass_kernel<Tin, Tout, 2><<<dim3((a.rows + 15) / 16, nchains), 256, 0, st>>>(a);
     else
         prepass_kernel<Tin, Tout, 1><<<dim3((a.rows + 7) / 8, nchains), 256, 0, st>>>(a);
