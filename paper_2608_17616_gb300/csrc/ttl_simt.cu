@@ -1187,10 +1187,12 @@ cudaError_t launch_resident_f32(const DevState& s, const SegWork& w, long long n
     static PerDevice<SmemOptIn> once[3];
     if ((long long)w.nc * (s.d_hid / 4) <= s.sms)
         return launch(ttl_resident_f32_kernel<4, 32, 512>, 4, res_smem_bytes<4>(512), res_smem_bytes<4>(D), once[0]);
-    // Eight rows: the 32 sums of two tokens cost a lane 31 shuffles and their selects, more than the contraction of a narrow
-    // chain; 16 lanes to a token halve them and read W twice. 1500 tokens, 32 and 16 lanes: D = 192 (8 chains of 64 -> 320 ->
-    // 128) 444 and 397 us, 320 (4 of 192 -> 448 -> 128) 408 and 394, 384 (256 -> 768 -> 128) 234 and 252, 512 814 and 925
-    if (D <= 320) return launch(ttl_resident_f32_kernel<8, 16, 320>, 8, res_smem_bytes<8>(320), res_smem_bytes<8>(D), once[1]);
+    // Eight rows: the 32 sums of two tokens cost a lane 31 shuffles and their selects; 16 lanes to a token halve them and read
+    // W twice, which is the better form for a narrow chain whose columns leave some of 32 lanes idle. 1500 tokens, 32 and
+    // 16 lanes: D = 192 (8 chains of 64 -> 320 -> 128) 444 and 386 us, 256 (8 of 128 -> 448 -> 128) 735 and 758, 320 (4 of 192 ->
+    // 448 -> 128) 408 and 388, 384 (256 -> 768 -> 128) 234 and 252, 512 814 and 925
+    if (D <= 320 && D % 128)
+        return launch(ttl_resident_f32_kernel<8, 16, 320>, 8, res_smem_bytes<8>(320), res_smem_bytes<8>(D), once[1]);
     return launch(ttl_resident_f32_kernel<8, 32, 512>, 8, res_smem_bytes<8>(512), res_smem_bytes<8>(D), once[2]);
 }
 

@@ -33,8 +33,8 @@ def _built():
     (384, 704, 128, 64, 1, 2 * 64 + 32, wk.PLAIN, "neg_inner"),    # resident, eight rows a CTA
     (320, 256, 128, 64, 3, 3 * 64 + 1, wk.PAPER, "neg_inner"),     # resident, eight rows a CTA, W1 ends inside
     (64, 704, 128, 64, 1, 3 * 64 + 1, wk.PAPER, "neg_inner"),      # eight rows, 16 lanes to a token: three pieces a lane
-    (128, 256, 128, 128, 3, 2 * 128 + 33, wk.PLAIN, "neg_inner"),  # four
-    (192, 256, 128, 192, 3, 2 * 192 + 17, wk.PAPER, "neg_inner"),  # five, the most
+    (192, 256, 128, 192, 3, 2 * 192 + 17, wk.PLAIN, "neg_inner"),  # five, the most
+    (128, 256, 128, 128, 3, 2 * 128 + 33, wk.PAPER, "neg_inner"),  # eight rows, 32 lanes (256 columns)
     (64, 256, 384, 64, 3, 3 * 64 + 33, wk.PAPER, "neg_inner"),     # eight rows, 32 lanes again (448 columns)
 ])
 def test_f32_tiles(d_in, d_hid, d_out, T, n_layers, N, mode, loss):
