@@ -4,8 +4,9 @@ The caches hold memory tokens at positions [0, n_mem) and the query tokens' own 
 values after them.  Where the case says so, the memory tokens are the library's own read
 (mone_mem_generate_kv after a test-time-learning pass); otherwise they are random.
 Tolerances: bf16 path 1e-2 (outputs rounded to bf16, fp32 accumulation), fp32 path 1e-5.
-bf16 caches whose rows are 16-byte aligned take the tensor-core kernel (keys in chunks of 256
-positions); other bf16 layouts and fp32 take the CUDA-core kernel.  Both are covered here.
+bf16 caches whose rows are 16-byte aligned take a tensor-core kernel, for few rows over all heads the decode form and
+else the prefill form (test_attention_forms_gpu.py has their tile edges); other bf16 layouts and fp32 take the
+CUDA-core kernel.  All three are covered here; the comments name the form that a case reaches.
 """
 import pytest
 import torch
@@ -61,12 +62,12 @@ def check(wl, Qt, Kc, Vc, out, n_mem, Lq, tol):
 
 
 @pytest.mark.parametrize("group,Lq,n_mem", [
-    (2, 40, 40),      # query heads in pairs, memory = the read of 40 query tokens
-    (1, 70, 0),       # no memory: causal self-attention; 70 tokens = two tiles, the last ragged
-    (7, 20, 150),     # 7 heads per KV head (tiles of 9 tokens), memory over three 64-position chunks
-    (2, 1, 300),      # one decode token over a long memory: two key chunks on the tensor cores
-    (1, 130, 400),    # 128-token tiles, the second ragged; up to 530 keys = three chunks
-    (64, 5, 10),      # the largest group: 2 tokens x 64 heads per 128-row tile
+    (2, 40, 40),      # decode; query heads in pairs, memory = the read of 40 query tokens
+    (1, 70, 0),       # decode; no memory: causal self-attention, five row tiles
+    (7, 20, 150),     # decode; 7 heads per KV head, blocks of 18 tokens
+    (2, 1, 300),      # decode; one token over a long memory, one row tile
+    (1, 130, 400),    # decode; two blocks of 128 tokens, the second of two
+    (64, 5, 10),      # prefill; the largest group: 2 tokens x 64 heads per 128-row tile, one chunk of keys
 ])
 def test_attention_bf16(group, Lq, n_mem):
     wl = small(n_ctx=2)
@@ -84,8 +85,8 @@ def test_attention_bf16_unaligned_cache_rows(group, Lq, n_mem):
 
 
 @pytest.mark.parametrize("Lq,n_mem", [
-    (33, 77),    # one key chunk
-    (5, 400),    # two key chunks: at hd 128 the probabilities take the key buffer, restaged per chunk
+    (33, 77),    # decode; seven row tiles
+    (5, 400),    # decode; one row tile, the keys over a cluster
 ])
 def test_attention_bf16_head_dim_128_random_memory(Lq, n_mem):
     wl = small(d_out=512, hd=128)

@@ -2,7 +2,7 @@
 tiles on large grids, 32 x 64 and 64 x 64 where a width is an odd multiple of 64, 32 x 64 on small grids; ragged last
 segments (rows of a tile absent, a contraction over few tokens) and plain mode; and of the resident kernel
 (d_in + d_out <= 512) at widths that end inside a warp's 128 columns, with four and with eight rows a CTA
-(more than 152 CTAs of four), and a last segment of one token, of one chunk and one token.  fp32 bound 1e-4 on the
+(more than 152 CTAs of four; 16 or 32 lanes to a token), and a last segment of one token, of one chunk and one token.  fp32 bound 1e-4 on the
 weights, their change and the momentum (test_parity_gpu.py)."""
 import pytest
 import torch

@@ -1,8 +1,8 @@
 """GPU parity of phase B where its column tiles and state ring can go wrong: widths that leave a
 128-column tile in W1, tiles of W2 that take half their columns from K and half from V, launches of
-more than one tile per CTA (wide and narrow tiles through the same ring), the three ways the ring's slots
-are handed back (plain mode, CTA pairs and a small state; a large state; the rest) and the CTA-pair form.  Bounds as in test_parity_gpu.py: 2e-2 on the weights and on
-their change."""
+more than one tile per CTA (wide and narrow tiles through the same ring), the four ways the ring's slots
+are handed back (by tiles a CTA and T; plain mode and CTA pairs as few tiles) and the CTA-pair form.  Bounds as in
+test_parity_gpu.py: 2e-2 on the weights and on their change."""
 import pytest
 import torch
 
