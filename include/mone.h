@@ -133,6 +133,8 @@ typedef struct {
  * per head) and W2_0 [chains][mem_heads][d_hid][dh] (Wout); mone_mem_read_state /
  * mone_mem_write_state use the same layouts.  Momentum starts at 0; renormalisation targets are the row norms of
  * W_0.  meta may be NULL in MONE_PLAIN mode.  On success *out owns the state.
+ * The handle belongs to the device that is current at this call; its calls are made with that
+ * device current (a process may have handles on several).
  * Errors: INVALID_ARG, UNSUPPORTED_SHAPE, OOM, CUDA.
  */
 mone_status mone_mem_init(const mone_config* cfg, const float* W1_0, const float* W2_0,
