@@ -970,10 +970,13 @@ static_assert(LayoutB::DYN <= 227 * 1024 && LayoutB2::DYN <= 227 * 1024, "phase 
 // from V: d_out is a multiple of 256, its half of 128).
 __host__ __device__ constexpr int b_col_tiles(int d_in, int d_out) { return (d_in + B_BN - 1) / B_BN + d_out / B_BN; }
 
-// The tiles one CTA of phase B walks: t = first, first + step, ... < count.
+// The tiles one CTA of phase B walks: t = first, first + step, ... < count.  The narrow tiles (128 columns, one to a
+// stripe of hidden rows where d_in leaves that remainder) come after all others: in their place between them they
+// would all fall to the same CTAs wherever step and the stripe's tiles share a factor, and the launch would take as
+// long as with whole tiles (1000 tokens of 56 chains of 640 -> 1536 -> 1792, T = 128: 7.04 ms so, 6.90 with them last).
 template <bool PAIR>
 struct BTiles {
-    int first, step, count, n_ht, n_ct, n1, rank, d_in;
+    int first, step, count, n_ht, n_ct, n1, n_wide, rank, d_in;
     __device__ BTiles(const TcArgs& a) {
         d_in = a.d_in;
         n_ht = a.d_hid / (PAIR ? 2 * B_BM : B_BM);
@@ -983,6 +986,11 @@ struct BTiles {
         rank = PAIR ? (int)cluster_ctarank() : 0;
         first = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
         step = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+        n_wide = n_ct;
+        if (!PAIR && d_in % B_BN) {
+            n1 -= 1;  // wide tiles of W1
+            n_wide -= 1;
+        }
     }
     // tile t: chain of the launch, this CTA's first hidden row, matrix (0: U, W1; 1: Y, W2), first column within
     // it, live columns
@@ -991,12 +999,14 @@ struct BTiles {
     };
     __device__ Tile decode(int t) const {
         Tile x;
-        x.cz = t / (n_ht * n_ct);
-        x.h0 = ((t / n_ct) % n_ht) * (PAIR ? 2 * B_BM : B_BM) + rank * B_BM;
-        const int c = t % n_ct;
-        x.m = c < n1 ? 0 : 1;
+        const int wide = n_wide * (count / n_ct);  // count / n_ct: stripes of hidden rows over all chains
+        const bool narrow = !PAIR && t >= wide;
+        const int stripe = narrow ? t - wide : t / n_wide, c = narrow ? n1 : t - stripe * n_wide;
+        x.cz = stripe / n_ht;
+        x.h0 = (stripe - x.cz * n_ht) * (PAIR ? 2 * B_BM : B_BM) + rank * B_BM;
+        x.m = c < n1 || narrow ? 0 : 1;
         x.col = (x.m ? c - n1 : c) * B_BN;
-        x.ncol = x.m ? B_BN : min(B_BN, d_in - x.col);
+        x.ncol = narrow ? B_BN / 2 : B_BN;
         return x;
     }
 };
